@@ -957,7 +957,8 @@ int build_level_geometry(LevelGeo& L, const LevelGeo* finer, bool finest, bool c
     L.bref = (int*)mem.get(sizeof(int) * nb1 * D);
     L.ban = (double*)mem.get(sizeof(double) * nb1 * D);
     L.ban32 = (float*)mem.get(sizeof(float) * nb1 * D);
-    int* bpos = (int*)mem.get(sizeof(int) * nn);
+    L.bpos = (int*)mem.get(sizeof(int) * nn);
+    int* bpos = L.bpos;
     if (!L.bref || !L.ban || !L.ban32 || !bpos) {
         err = "out of device memory";
         return SULF_ENOMEM;

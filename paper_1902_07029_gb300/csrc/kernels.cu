@@ -53,14 +53,10 @@ std::string take_launch_error() {
     return m;
 }
 
-namespace {
-
-constexpr int kT = 256;
-
 // Launch shape of a one-thread-per-node kernel over n nodes.  On this GPU one
 // SM issues two FP64 lanes per clock, so a short list in 256-thread CTAs would
 // run on a few SMs at their FP64 rate: CTAs shrink (down to one warp) until the
-// list covers every SM, and grow to kT threads only for long lists.
+// list covers every SM, and grow to kNodeThreads threads only for long lists.
 int sm_count() {
     static std::atomic<int> cached[64];
     int dev = 0;
@@ -72,39 +68,23 @@ int sm_count() {
     return v;
 }
 
-inline unsigned block_for(long long n) {
+unsigned block_for(long long n) {
     const long long sms = sm_count();
     long long per = (n + sms - 1) / sms;
     long long b = (per + 31) / 32 * 32;
-    return (unsigned)(b < 32 ? 32 : (b > kT ? kT : b));
+    return (unsigned)(b < 32 ? 32 : (b > kNodeThreads ? kNodeThreads : b));
 }
 
-inline unsigned grid_for(long long n) {
+unsigned grid_for(long long n) {
     const unsigned b = block_for(n);
     return (unsigned)((n + b - 1) / b);
 }
 
-// max over the block of non-negative doubles held as bit patterns (NaN, whose
-// pattern exceeds +inf, propagates), then one atomicMax per block
-__device__ __forceinline__ void block_max(unsigned long long v, unsigned long long* out) {
-    __shared__ unsigned long long sm[32];
-    for (int o = 16; o > 0; o >>= 1) {
-        unsigned long long w = __shfl_down_sync(0xffffffffu, v, o);
-        v = v > w ? v : w;
-    }
-    int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    if (lane == 0) sm[warp] = v;
-    __syncthreads();
-    if (warp == 0) {
-        int nw = (blockDim.x + 31) >> 5;
-        v = lane < nw ? sm[lane] : 0ULL;
-        for (int o = 16; o > 0; o >>= 1) {
-            unsigned long long w = __shfl_down_sync(0xffffffffu, v, o);
-            v = v > w ? v : w;
-        }
-        if (lane == 0 && v) atomicMax(out, v);
-    }
-}
+namespace {
+
+constexpr int kT = kNodeThreads;
+
+using stages::block_max;
 
 template <int D>
 struct Offs {
@@ -1535,7 +1515,7 @@ int launch_to_float(const LevelGeo& L, const double2* src, float2* dst, cudaStre
 // records its defect norm and sets the enclosing conditional node to run
 // another cycle unless the defect met the threshold, is not a number, the
 // coarsest Jacobian was singular or the cycle cap is reached.
-__global__ void k_cycle_check(cudaGraphConditionalHandle h, const unsigned long long* __restrict__ norm,
+__global__ void k_cycle_check(cudaGraphConditionalHandle h, unsigned long long* __restrict__ norm,
                               const int* __restrict__ singular, const double* __restrict__ thr, int max_cycles,
                               int* cycles, double* rnorms) {
     pdl_enter();
@@ -1543,12 +1523,13 @@ __global__ void k_cycle_check(cudaGraphConditionalHandle h, const unsigned long 
     const int c = *cycles + 1;
     *cycles = c;
     const double rn = __longlong_as_double((long long)norm[0]);
+    norm[0] = 0;  // for the next cycle's maximum
     rnorms[c - 1] = rn;
     const bool more = *singular == 0 && rn == rn && rn > *thr && c < max_cycles;
     cudaGraphSetConditional(h, more ? 1u : 0u);
 }
 
-int launch_cycle_check(cudaGraphConditionalHandle h, const unsigned long long* norm, const int* singular,
+int launch_cycle_check(cudaGraphConditionalHandle h, unsigned long long* norm, const int* singular,
                        const double* thr, int max_cycles, int* cycles, double* rnorms, cudaStream_t s) {
     launch_k(k_cycle_check, 1, 32, 0, s, h, norm, singular, thr, max_cycles, cycles, rnorms);
     return 1;

@@ -43,6 +43,28 @@ __device__ __forceinline__ unsigned long long abs_bits(T v) {
     return (unsigned long long)__double_as_longlong(d);
 }
 
+// max over the block of non-negative doubles held as bit patterns (NaN, whose
+// pattern exceeds +inf, propagates), then one atomicMax per block
+__device__ __forceinline__ void block_max(unsigned long long v, unsigned long long* out) {
+    __shared__ unsigned long long sm[32];
+    for (int o = 16; o > 0; o >>= 1) {
+        unsigned long long w = __shfl_down_sync(0xffffffffu, v, o);
+        v = v > w ? v : w;
+    }
+    int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    if (lane == 0) sm[warp] = v;
+    __syncthreads();
+    if (warp == 0) {
+        int nw = (blockDim.x + 31) >> 5;
+        v = lane < nw ? sm[lane] : 0ULL;
+        for (int o = 16; o > 0; o >>= 1) {
+            unsigned long long w = __shfl_down_sync(0xffffffffu, v, o);
+            v = v > w ? v : w;
+        }
+        if (lane == 0 && v) atomicMax(out, v);
+    }
+}
+
 // node of list position t in the concatenation (inside colour 0, inside
 // colour 1, ghosts); kind 1 inside, 2 ghost
 struct Lists {

@@ -1,0 +1,1362 @@
+// Kernels and per-level data of the multigrid cycle on the equation for s
+// (schur.cuh).
+#include <mutex>
+
+#include <cooperative_groups.h>
+
+#include "schur.cuh"
+
+namespace sulf {
+
+using stages::abs_bits;
+using stages::block_max;
+using stages::fmadd;
+using stages::kGopLanes;
+
+namespace {
+
+constexpr int kT = kNodeThreads;
+constexpr int kRowLanes = 4;  // lanes that share a ghost's row of the defect
+
+// node coordinates of a half index
+template <int D>
+__device__ __forceinline__ void half_coords(int h, int a, int H, int n, int* ii) {
+    const unsigned row = (unsigned)h / (unsigned)H;
+    ii[0] = 2 * (int)((unsigned)h - row * (unsigned)H) + a;
+    if (D == 3) {
+        const unsigned k = row / (unsigned)n;
+        ii[1] = (int)(row - k * (unsigned)n);
+        ii[2] = (int)k;
+    } else {
+        ii[1] = (int)row;
+        ii[2] = 0;
+    }
+}
+
+template <int D>
+__device__ __forceinline__ int slot_of(int i, int j, int k, int H, int P, int Hn) {
+    return ((i + j + (D == 3 ? k : 0)) & 1) * Hn + (i >> 1) + H * j + (D == 3 ? P * k : 0);
+}
+
+// the node at list position t (inside nodes, then ghosts): its slot and box node
+template <int D, typename T>
+__device__ __forceinline__ int list_slot(const SLev<D, T>& L, int t, int& p) {
+    if (t < L.n0 + L.n1) {
+        const int e = L.hl[t], h = e >> kEntHalf;
+        int ii[3];
+        half_coords<D>(h, e & 1, L.H, L.n, ii);
+        p = ii[0] + L.n * (ii[1] + (D == 3 ? L.n * ii[2] : 0));
+        return (t >= L.n0 ? L.Hn : 0) + h;
+    }
+    const int g = t - L.n0 - L.n1;
+    p = L.gidx[g];
+    return L.gslot[g];
+}
+
+// half-index offsets of the axis neighbours (all of the other colour) of a
+// node whose x index has parity a
+template <int D, typename T>
+__device__ __forceinline__ void nbr_offsets(const SLev<D, T>& L, int a, int* o) {
+    o[0] = a;
+    o[1] = a - 1;
+    o[2] = L.H;
+    o[3] = -L.H;
+    if (D == 3) {
+        o[4 % (2 * D)] = L.P;
+        o[5 % (2 * D)] = -L.P;
+    }
+}
+
+// ---------------------------------------------------------------------------
+// set-up of a linear solve
+
+template <typename T>
+__device__ __forceinline__ void c_row(const Coef<T>& c, T s, T cp, T& ph, T& pcs, T& pcc) {
+    ph = c.alpha * cp + c.beta;
+    pcs = c.a2ms * ph * cp;
+    pcc = c.idt + c.a2ms * (c.alpha * s * cp + ph * s);
+}
+
+// FINE: the finest level of a linear solve (T = double), U the FP32 finest
+// level of mixed precision (MIXED)
+template <int D, typename T, bool FINE, bool MIXED>
+__global__ void __launch_bounds__(kT) k_s_rho(SLev<D, T> L, SLev<D, float> U, const typename V2<T>::t* __restrict__ Wc,
+                                               Coef<T> c, const double2* __restrict__ F, double* __restrict__ tt) {
+    pdl_enter();
+    const int t = blockIdx.x * blockDim.x + threadIdx.x;
+    const int nin = L.n0 + L.n1;
+    if (t >= nin + L.ng) return;
+    int p;
+    const int sl = list_slot<D, T>(L, t, p);
+    const typename V2<T>::t w = Wc[p];
+    T ph, pcs, pcc;
+    c_row<T>(c, w.x, w.y, ph, pcs, pcc);
+    const T inv = (T)1 / pcc;
+    const T rho = pcs * inv, C = c.kap * c.alpha * w.x;
+    L.rho[sl] = rho;
+    L.cs[sl] = C;
+    if (FINE) {
+        const double2 f = F[p];
+        const double t0 = f.y * (double)inv;
+        tt[sl] = t0;
+        if (MIXED) {
+            U.rho[sl] = (float)rho;
+            U.cs[sl] = (float)C;
+            L.X[sl] = 0;
+            if (t >= nin) {
+                L.b[t] = (T)f.x;
+                U.b[t] = (float)f.x;
+                U.X[sl] = 0.f;
+                U.D2[sl] = make_float2((float)-t0, (float)(-(double)C * t0));
+            }
+        } else if (t >= nin) {
+            // x = 0 is off the ghosts' c rows by -t in the first sweep
+            typename V2<T>::t d;
+            d.x = (T)-t0;
+            d.y = (T)(-(double)C * t0);
+            L.D2[sl] = d;
+            L.X[sl] = 0;
+            L.b[t] = (T)f.x;
+        }
+    }
+}
+
+template <int D, typename T, bool FINE, bool MIXED>
+__global__ void __launch_bounds__(kT) k_s_coefs(SLev<D, T> L, SLev<D, float> U,
+                                                 const typename V2<T>::t* __restrict__ Wc, Coef<T> c,
+                                                 const double2* __restrict__ F, const double* __restrict__ tt) {
+    pdl_enter();
+    typedef typename V2<T>::t T2;
+    const int t = blockIdx.x * blockDim.x + threadIdx.x;
+    if (t >= L.n0 + L.n1) return;
+    const int colour = t >= L.n0;
+    const int e = L.hl[t], h = e >> kEntHalf;
+    int ii[3], o[2 * D];
+    half_coords<D>(h, e & 1, L.H, L.n, ii);
+    nbr_offsets<D, T>(L, e & 1, o);
+    const int p = ii[0] + L.n * (ii[1] + (D == 3 ? L.n * ii[2] : 0));
+    const int st[3] = {1, L.n, L.n * L.n};
+    const int sl = colour * L.Hn + h, so = (1 - colour) * L.Hn + h;
+    const T2 w = Wc[p];
+    const T s = w.x, cp = w.y;
+    T ph, pcs, pcc;
+    c_row<T>(c, s, cp, ph, pcs, pcc);
+    T sg = 0, se = 0, et = 0;
+    T2 wq[2 * D];
+    T rq[2 * D];
+    double tq[2 * D];
+#pragma unroll
+    for (int q = 0; q < 2 * D; q++) {
+        wq[q] = Wc[(q & 1) ? p - st[q >> 1] : p + st[q >> 1]];
+        rq[q] = L.rho[so + o[q]];
+        if (FINE) tq[q] = tt[so + o[q]];
+    }
+    T g[2 * D];
+#pragma unroll
+    for (int q = 0; q < 2 * D; q++) {
+        const T gq = c.kap * ((c.alpha * wq[q].y + c.beta) + ph);
+        const T eq = c.kap * c.alpha * (s - wq[q].x);
+        sg += gq;
+        se += eq;
+        g[q] = fmadd(eq, rq[q], gq);
+        if (FINE) et = fmadd(eq, (T)tq[q], et);
+        L.gt[q * L.gs + t] = g[q];
+    }
+    const T Pss = ph * c.idt + c.a2mc * ph * cp + sg;
+    const T Psc = c.alpha * s * c.idt + c.a2mc * (c.alpha * s * cp + ph * s) + se;
+    const T dd = Pss - Psc * L.rho[sl];
+    const T di = (T)1 / dd;
+    L.dd[t] = dd;
+    L.di[t] = di;
+    if (FINE) {
+        const T bs = (T)F[p].x - Psc * (T)tt[sl];
+        const T b = bs - et;
+        L.b[t] = b;
+        if (MIXED) {
+#pragma unroll
+            for (int q = 0; q < 2 * D; q++) U.gt[q * U.gs + t] = (float)g[q];
+            const float bf = (float)b, df = (float)di;
+            U.dd[t] = (float)dd;
+            U.di[t] = df;
+            U.b[t] = bf;
+            // the first red half-sweep from zero, the neighbours' x^c = 0 off their c rows
+            if (!colour) U.X[sl] = (float)bs * df;
+        } else if (!colour) {
+            L.X[sl] = bs * di;
+        }
+    }
+}
+
+// ---------------------------------------------------------------------------
+// relaxation
+
+template <int D, typename T, bool DELTA>
+__global__ void __launch_bounds__(kT) k_s_relax(SLev<D, T> L, int colour, int snap, const int* skip, double* acc) {
+    typedef typename V2<T>::t T2;
+    const int t = blockIdx.x * blockDim.x + threadIdx.x;
+    const int cnt = colour ? L.n1 : L.n0, pos = (colour ? L.n0 : 0) + t;
+    // the row is fixed during the linear solve: fetched while the previous
+    // kernel is still running
+    int e = 0, o[2 * D];
+    T g[2 * D], di = 0, cp = 0;
+    if (t < cnt) {
+        e = L.hl[pos];
+#pragma unroll
+        for (int q = 0; q < 2 * D; q++) g[q] = L.gt[q * L.gs + pos];
+        di = L.di[pos];
+        if (DELTA) cp = L.cs[colour * L.Hn + (e >> kEntHalf)];
+    }
+    nbr_offsets<D, T>(L, e & 1, o);
+    const int sg = snap && t < L.ng ? L.gslot[t] : 0;
+    pdl_enter();
+    if (skip && *skip) return;
+    if (snap && t < L.ng) L.snap[t] = L.X[sg];
+    if (t >= cnt) return;
+    const int h = e >> kEntHalf, so = (1 - colour) * L.Hn + h, sl = colour * L.Hn + h;
+    T r = L.b[pos];
+    T x[2 * D];
+#pragma unroll
+    for (int q = 0; q < 2 * D; q++) x[q] = L.X[so + o[q]];
+    if (DELTA) {
+        // red inside nodes are on their c rows (their entries of D2 stay
+        // zero): only a black node next to a ghost has terms
+        if (colour == 0 || (e & 2)) {
+            T2 d[2 * D];
+#pragma unroll
+            for (int q = 0; q < 2 * D; q++) d[q] = L.D2[so + o[q]];
+            T sd = d[0].x, sc = d[0].y;
+#pragma unroll
+            for (int q = 1; q < 2 * D; q++) {
+                sd += d[q].x;
+                sc += d[q].y;
+            }
+            r = fmadd(-cp, sd, r + sc);
+        }
+    }
+#pragma unroll
+    for (int q = 0; q < 2 * D; q++) r = fmadd(g[q], x[q], r);
+    r *= di;
+    L.X[sl] = r;
+    if (acc) acc[sl] += (double)r;
+}
+
+template <int D, typename T>
+__device__ __forceinline__ T ghost_input(const SLev<D, T>& L, int code) {
+    if (code >= 0) return L.X[code];
+    const unsigned u = ~(unsigned)code;
+    return (u & 1u) ? L.b[L.n0 + L.n1 + (u >> 1)] : L.snap[u >> 1];
+}
+
+// all passes of a sweep's ghost relaxation, one composed row per ghost
+constexpr int kGopPre = 4;
+template <int D, typename T>
+__global__ void __launch_bounds__(kT) k_s_ghosts(SLev<D, T> L, const int* skip, double* acc) {
+    const int t = blockIdx.x * blockDim.x + threadIdx.x;
+    const int gi = t / kGopLanes, ln = t % kGopLanes;
+    const bool on = gi < L.ng;
+    int beg = 0, end = 0, sl = 0;
+    int cd[kGopPre];
+    T w[kGopPre];
+    if (on) {
+        beg = L.gptr[gi] + ln;
+        end = L.gptr[gi + 1];
+#pragma unroll
+        for (int i = 0; i < kGopPre; i++) {
+            const int j = beg + i * kGopLanes;
+            cd[i] = j < end ? L.gcode[j] : 0;
+            w[i] = j < end ? L.gval[j] : (T)0;
+        }
+        sl = L.gslot[gi];
+    }
+    pdl_enter();
+    if (skip && *skip) return;
+    T v = 0;
+    if (on) {
+        T u[kGopPre];
+#pragma unroll
+        for (int i = 0; i < kGopPre; i++) u[i] = beg + i * kGopLanes < end ? ghost_input<D, T>(L, cd[i]) : (T)0;
+#pragma unroll
+        for (int i = 0; i < kGopPre; i++)
+            if (beg + i * kGopLanes < end) v = fmadd(w[i], u[i], v);
+        for (int j = beg + kGopPre * kGopLanes; j < end; j += kGopLanes)
+            v = fmadd(L.gval[j], ghost_input<D, T>(L, L.gcode[j]), v);
+    }
+    v = stages::gop_reduce<T>(v);
+    if (!on || ln != 0) return;
+    L.X[sl] = v;
+    if (acc) acc[sl] += (double)v;
+}
+
+// ---------------------------------------------------------------------------
+// defect
+
+template <int D, typename T>
+__device__ __forceinline__ T inside_defect(const SLev<D, T>& L, int pos, int colour, int h, int a, const T* g, T dd) {
+    int o[2 * D];
+    nbr_offsets<D, T>(L, a, o);
+    const int so = (1 - colour) * L.Hn + h;
+    T x[2 * D];
+#pragma unroll
+    for (int q = 0; q < 2 * D; q++) x[q] = L.X[so + o[q]];
+    T r = fmadd(-dd, L.X[colour * L.Hn + h], L.b[pos]);
+#pragma unroll
+    for (int q = 0; q < 2 * D; q++) r = fmadd(g[q], x[q], r);
+    return r;
+}
+
+// b - row . x of ghost gi by the kRowLanes lanes of its group; every lane of
+// the warp calls it, lane 0 of the group holds the result
+template <int D, typename T>
+__device__ __forceinline__ T ghost_defect(const SLev<D, T>& L, bool on, int gi, int ln) {
+    T v = 0;
+    if (on) {
+        const int end = L.rptr[gi + 1];
+        for (int j = L.rptr[gi] + ln; j < end; j += kRowLanes) v = fmadd(L.rval[j], L.X[L.rslot[j]], v);
+    }
+#pragma unroll
+    for (int d = kRowLanes / 2; d > 0; d >>= 1) v += __shfl_xor_sync(0xffffffffu, v, d);
+    return on && ln == 0 ? L.b[L.n0 + L.n1 + gi] - v : (T)0;
+}
+
+template <int D, typename T, bool NORM>
+__global__ void __launch_bounds__(kT) k_s_residual(SLev<D, T> L, int nrow, unsigned long long* norm, int* clear) {
+    const int t = blockIdx.x * blockDim.x + threadIdx.x;
+    const int nin = L.n0 + L.nga;  // rows of inside nodes; nrow: rounded up to whole warps
+    int e = 0, pos = 0, colour = 0;
+    T g[2 * D], dd = 0;
+    if (t < nin) {
+        colour = t >= L.n0;
+        pos = colour ? L.n1 - L.nga + t : t;
+        e = L.hl[pos];
+#pragma unroll
+        for (int q = 0; q < 2 * D; q++) g[q] = L.gt[q * L.gs + pos];
+        dd = L.dd[pos];
+    }
+    pdl_enter();
+    if (clear && t == 0) *clear = 0;
+    T r = 0;
+    if (t < nrow) {
+        if (t < nin) {
+            r = inside_defect<D, T>(L, pos, colour, e >> kEntHalf, e & 1, g, dd);
+            if (!NORM) L.R[colour * L.Hn + (e >> kEntHalf)] = r;
+        }
+    } else {
+        const int gi = (t - nrow) / kRowLanes, ln = (t - nrow) % kRowLanes;
+        r = ghost_defect<D, T>(L, gi < L.ng, gi, ln);
+        if (!NORM && gi < L.ng && ln == 0) L.R[L.gslot[gi]] = r;
+    }
+    if (NORM) block_max(abs_bits(r), norm);
+}
+
+// mixed precision: the FP64 defect of every row into the FP32 right-hand
+// side; the FP32 error starts with its red half-sweep from zero
+template <int D>
+__global__ void __launch_bounds__(kT) k_s_outer(SLev<D, double> L, SLev<D, float> U, int nrow,
+                                                 unsigned long long* norm, int* clear) {
+    const int t = blockIdx.x * blockDim.x + threadIdx.x;
+    const int nin = L.n0 + L.n1;
+    int e = 0;
+    double g[2 * D], dd = 0;
+    float df = 0;
+    const int colour = t >= L.n0;
+    if (t < nin) {
+        e = L.hl[t];
+#pragma unroll
+        for (int q = 0; q < 2 * D; q++) g[q] = L.gt[q * L.gs + t];
+        dd = L.dd[t];
+        if (!colour) df = U.di[t];
+    }
+    pdl_enter();
+    if (t == 0) *clear = 0;
+    double r = 0;
+    if (t < nrow) {
+        if (t < nin) {
+            const int h = e >> kEntHalf;
+            r = inside_defect<D, double>(L, t, colour, h, e & 1, g, dd);
+            U.b[t] = (float)r;
+            if (!colour) U.X[h] = (float)r * df;
+        }
+    } else {
+        const int gi = (t - nrow) / kRowLanes, ln = (t - nrow) % kRowLanes;
+        r = ghost_defect<D, double>(L, gi < L.ng, gi, ln);
+        if (gi < L.ng && ln == 0) {
+            U.b[nin + gi] = (float)r;
+            U.X[L.gslot[gi]] = 0.f;
+        }
+    }
+    block_max(abs_bits(r), norm);
+}
+
+// ---------------------------------------------------------------------------
+// transfers
+
+// boundary-aware full weighting of the finer level's defect (Eqs. Fstencil,
+// Fstencilgen) at a coarse inside node whose fine neighbourhood holds nodes
+// that are not inside, or black nodes with a defect of their own
+template <int D, typename T>
+__device__ __forceinline__ T restrict_near(const SLev<D, T>& F, const int* ci) {
+    const int n = F.n;
+    int f[3] = {2 * ci[0], 2 * ci[1], D == 3 ? 2 * ci[2] : 0};
+    const int st[3] = {1, n, n * n};
+    const int p = f[0] + n * (f[1] + (D == 3 ? n * f[2] : 0));
+    int w[3][3];  // per-axis weights times 4
+#pragma unroll
+    for (int a = 0; a < D; a++) {
+        const bool vl = F.type[p - st[a]] == T_IN, vr = F.type[p + st[a]] == T_IN;
+        w[a][0] = vl ? (vr ? 1 : 2) : 0;
+        w[a][1] = vl || vr ? 2 : 4;
+        w[a][2] = vr ? (vl ? 1 : 2) : 0;
+    }
+    T acc = 0;
+    int wc = 0;
+    for (int kk = 0; kk < (D == 2 ? 9 : 27); kk++) {
+        const int k0 = kk % 3, k1 = (kk / 3) % 3, k2 = D == 3 ? kk / 9 : 1;
+        const int iw = w[0][k0] * w[1][k1] * (D == 3 ? w[2][k2] : 1);
+        if (iw == 0) continue;
+        const int q = p + (k0 - 1) + (k1 - 1) * st[1] + (D == 3 ? (k2 - 1) * st[2] : 0);
+        const bool centre = k0 == 1 && k1 == 1 && k2 == 1;
+        if (centre || F.type[q] != T_IN)
+            wc += iw;
+        else
+            acc = fmadd((T)iw, F.R[slot_of<D>(f[0] + k0 - 1, f[1] + k1 - 1, f[2] + k2 - 1, F.H, F.P, F.Hn)], acc);
+    }
+    acc = fmadd((T)wc, F.R[slot_of<D>(f[0], f[1], f[2], F.H, F.P, F.Hn)], acc);
+    return acc / (T)(D == 2 ? 16 : 64);
+}
+
+// the finer level's defect onto the coarse level's right-hand side; the coarse
+// error starts with its red half-sweep from zero
+template <int D, typename T>
+__global__ void __launch_bounds__(kT) k_s_restrict(SLev<D, T> F, SLev<D, T> C, int nrow) {
+    const int t = blockIdx.x * blockDim.x + threadIdx.x;
+    const int nin = C.n0 + C.n1;
+    int e = 0, tw = -1;
+    T di = 0;
+    if (t < nin) {
+        e = C.hl[t];
+        tw = C.twin[t];
+        if (t < C.n0) di = C.di[t];
+    }
+    pdl_enter();
+    if (t < nrow) {
+        if (t >= nin) return;
+        T r;
+        if (tw >= 0) {
+            // black members (weights of the faces and corners) have no defect
+            const T* R = F.R + tw;
+            const int H = F.H, P = F.P;
+            const T c0 = R[0];
+            T s = (R[H] + R[H - 1]) + (R[-H] + R[-H - 1]);
+            if (D == 3) {
+                s += (R[P] + R[P - 1]) + (R[-P] + R[-P - 1]);
+                s += (R[P + H] + R[P - H]) + (R[H - P] + R[-H - P]);
+                r = (T)0.125 * c0 + (T)0.03125 * s;
+            } else {
+                r = (T)0.25 * c0 + (T)0.0625 * s;
+            }
+        } else {
+            int ci[3];
+            half_coords<D>(e >> kEntHalf, e & 1, C.H, C.n, ci);
+            r = restrict_near<D, T>(F, ci);
+        }
+        C.b[t] = r;
+        C.X[(t >= C.n0 ? C.Hn : 0) + (e >> kEntHalf)] = t < C.n0 ? r * di : (T)0;
+    } else {
+        const int gi = (t - nrow) / kGopLanes, ln = (t - nrow) % kGopLanes;
+        T v = 0;
+        if (gi < C.ng) {
+            const int end = C.cptr[gi + 1];
+            for (int j = C.cptr[gi] + ln; j < end; j += kGopLanes) v = fmadd(C.cval[j], F.R[C.cslot[j]], v);
+        }
+        v = stages::gop_reduce<T>(v);
+        if (gi < C.ng && ln == 0) {
+            C.b[nin + gi] = v;
+            C.X[C.gslot[gi]] = 0;
+        }
+    }
+}
+
+// (bi/tri)linear interpolation of the coarse error, renormalised over the
+// active corners (Sec. 3.5.3), at the black nodes and the ghosts; the
+// corners' x^c is -rho x^s
+template <int D, typename T>
+__global__ void __launch_bounds__(kT) k_s_prolong(SLev<D, T> F, SLev<D, T> C) {
+    typedef typename V2<T>::t T2;
+    const int t = blockIdx.x * blockDim.x + threadIdx.x;
+    const bool on = t < F.n1 + F.ng;
+    int cn[1 << D];
+    T cr[1 << D];
+    unsigned use = 0;
+    int sl = 0;
+    T rho = 0, Cs = 0;
+    if (on) {
+        int ii[3];
+        bool all = false;
+        if (t < F.n1) {
+            const int e = F.hl[F.n0 + t];
+            sl = F.Hn + (e >> kEntHalf);
+            half_coords<D>(e >> kEntHalf, e & 1, F.H, F.n, ii);
+            all = e & 4;
+        } else {
+            sl = F.gslot[t - F.n1];
+            stages::box_coords<D>(F.gidx[t - F.n1], F.n, ii);
+        }
+        rho = F.rho[sl];
+        Cs = F.cs[sl];
+#pragma unroll
+        for (int cc = 0; cc < (1 << D); cc++) {
+            int q[3] = {0, 0, 0};
+            bool dup = false;
+#pragma unroll
+            for (int a = 0; a < D; a++) {
+                const int up = (cc >> a) & 1;
+                if (up && !(ii[a] & 1)) dup = true;
+                q[a] = (ii[a] >> 1) + (up && (ii[a] & 1) ? 1 : 0);
+            }
+            cn[cc] = slot_of<D>(q[0], q[1], q[2], C.H, C.P, C.Hn);
+            if (dup) continue;
+            if (!all) {
+                const int8_t ty = C.type[q[0] + C.n * (q[1] + (D == 3 ? C.n * q[2] : 0))];
+                if (ty != T_IN && ty != T_GHOST) continue;
+            }
+            use |= 1u << cc;
+            cr[cc] = C.rho[cn[cc]];
+        }
+    }
+    pdl_enter();
+    if (!on) return;
+    T2 d;
+    d.x = 0;
+    d.y = 0;
+    if (use) {
+        T v[1 << D];
+#pragma unroll
+        for (int cc = 0; cc < (1 << D); cc++) v[cc] = (use >> cc) & 1u ? C.X[cn[cc]] : (T)0;
+        T x = F.X[sl];
+        T ps = 0, pc = 0;
+#pragma unroll
+        for (int cc = 0; cc < (1 << D); cc++)
+            if ((use >> cc) & 1u) {
+                ps += v[cc];
+                pc = fmadd(-cr[cc], v[cc], pc);
+            }
+        const T r = stages::inv_count<T>(__popc(use));
+        F.X[sl] = fmadd(ps, r, x);
+        // off the c row by delta = x^c + rho x^s of the correction
+        d.x = fmadd(rho, ps, pc) * r;
+        d.y = Cs * d.x;
+    }
+    F.D2[sl] = d;
+}
+
+// coarse (s, c) by injection; a coarse ghost whose fine twin is inactive takes
+// the mean over the active fine 3^d neighbourhood
+template <int D, typename TF, typename T>
+__global__ void __launch_bounds__(kT) k_inject_to(stages::Lists ls, int cn, const int8_t* __restrict__ ftype, int fn,
+                                                   const typename V2<TF>::t* __restrict__ fW,
+                                                   typename V2<T>::t* __restrict__ cW) {
+    pdl_enter();
+    const int t = blockIdx.x * blockDim.x + threadIdx.x;
+    if (t >= ls.n0 + ls.n1 + ls.ng) return;
+    int kind, gi, ii[3];
+    const long long I = stages::list_node(ls, t, kind, gi);
+    stages::box_coords<D>(I, cn, ii);
+    const int f = 2 * ii[0] + fn * (2 * ii[1] + (D == 3 ? fn * 2 * ii[2] : 0));
+    typename V2<T>::t out;
+    const int8_t tf = ftype[f];
+    if (tf == T_IN || tf == T_GHOST) {
+        const typename V2<TF>::t v = fW[f];
+        out.x = (T)v.x;
+        out.y = (T)v.y;
+        cW[I] = out;
+        return;
+    }
+    TF ss = 0, sc = 0;
+    int cnt = 0;
+    for (int kk = 0; kk < (D == 2 ? 9 : 27); kk++) {
+        const int k[3] = {kk % 3 - 1, (kk / 3) % 3 - 1, D == 3 ? kk / 9 - 1 : 0};
+        bool ok = true;
+        for (int a = 0; a < D; a++) ok = ok && 2 * ii[a] + k[a] >= 0 && 2 * ii[a] + k[a] < fn;
+        if (!ok) continue;
+        const int q = f + k[0] + fn * (k[1] + (D == 3 ? fn * k[2] : 0));
+        if (ftype[q] != T_IN && ftype[q] != T_GHOST) continue;
+        const typename V2<TF>::t v = fW[q];
+        ss += v.x;
+        sc += v.y;
+        cnt++;
+    }
+    out.x = (T)(cnt ? ss / (TF)cnt : (TF)0);
+    out.y = (T)(cnt ? sc / (TF)cnt : (TF)0);
+    cW[I] = out;
+}
+
+// ---------------------------------------------------------------------------
+// coarsest level
+
+// The dense Schur complement in list order (inside nodes, then ghosts)
+// assembled and inverted by Gauss-Jordan elimination with partial pivoting on
+// a thread-block cluster: CTA r of C owns the columns j with j % C == r, in
+// its shared memory where they fit (SMEM) or in A.  Step k: the owner of
+// column k finds the pivot row (first of largest magnitude, i >= k) and writes
+// the interchanged column, its pivot's reciprocal and the pivot row index into
+// every CTA's shared memory (double-buffered by the parity of k); one cluster
+// barrier; then each CTA interchanges, scales and eliminates in its own
+// columns.  The row interchanges are undone as column interchanges at the end.
+// Eliminating c first halves the order of the matrix: half the pivot steps.
+constexpr int kFacCluster = 8;
+constexpr int kFacThreads = 512;
+
+template <typename T>
+inline size_t factor_smem(int m, bool columns) {
+    const size_t mc = ((size_t)m + kFacCluster - 1) / kFacCluster;
+    return sizeof(T) * ((columns ? (size_t)m * mc : 0) + 2 * ((size_t)m + 1)) + sizeof(int) * 3 * (size_t)m;
+}
+
+template <int D, typename T, bool SMEM>
+__global__ void __launch_bounds__(kFacThreads) k_s_factor(SLev<D, T> L, const int* __restrict__ spos, T* Ag, T* Ainv,
+                                                          int* singular) {
+    namespace cg = cooperative_groups;
+    pdl_enter();
+    cg::cluster_group cl = cg::this_cluster();
+    const int C = (int)cl.num_blocks(), me = (int)cl.block_rank();
+    const int nin = L.n0 + L.n1, m = nin + L.ng;
+    const int mc = (m + C - 1) / C;  // local column jl is global column jl * C + me
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    T* A = SMEM ? reinterpret_cast<T*>(smem_raw) : Ag + (size_t)me * m * mc;  // m x mc, row-major
+    T* fac = reinterpret_cast<T*>(smem_raw) + (SMEM ? (size_t)m * mc : 0);    // two buffers of m + 1
+    int* piv = reinterpret_cast<int*>(fac + 2 * (m + 1));
+    int* idx = piv + m;
+    int* pos = idx + m;
+    for (int i = threadIdx.x; i < m * mc; i += blockDim.x) A[i] = 0;
+    __syncthreads();
+    auto add = [&](int i, int j, T v) {
+        if (j % C == me) A[(size_t)i * mc + j / C] += v;
+    };
+    for (int r = threadIdx.x; r < m; r += blockDim.x) {
+        if (r < nin) {
+            const int colour = r >= L.n0, e = L.hl[r];
+            int o[2 * D];
+            nbr_offsets<D, T>(L, e & 1, o);
+            const int so = (1 - colour) * L.Hn + (e >> kEntHalf);
+            for (int q = 0; q < 2 * D; q++) add(r, spos[so + o[q]], -L.gt[q * L.gs + r]);
+            add(r, r, L.dd[r]);
+        } else {
+            for (int j = L.rptr[r - nin]; j < L.rptr[r - nin + 1]; j++) add(r, spos[L.rslot[j]], L.rval[j]);
+        }
+    }
+    __syncthreads();
+    __shared__ int s_piv;
+    __shared__ T s_inv;
+    for (int k = 0; k < m; k++) {
+        T* fb = fac + (size_t)(k & 1) * (m + 1);
+        if (k % C == me) {
+            const int kl = k / C;
+            __syncthreads();  // this CTA's updates of column k in the previous step
+            if (threadIdx.x < 32) {
+                const int lane = threadIdx.x;
+                T bv = -1;
+                int bi = k;
+                for (int i = k + lane; i < m; i += 32) {
+                    const T v = fabs(A[(size_t)i * mc + kl]);
+                    if (v > bv) {
+                        bv = v;
+                        bi = i;
+                    }
+                }
+                for (int o = 16; o > 0; o >>= 1) {
+                    const T ov = __shfl_down_sync(0xffffffffu, bv, o);
+                    const int oi = __shfl_down_sync(0xffffffffu, bi, o);
+                    if (ov > bv || (ov == bv && oi < bi)) {
+                        bv = ov;
+                        bi = oi;
+                    }
+                }
+                if (lane == 0) {
+                    s_piv = bi;
+                    s_inv = (T)1 / A[(size_t)bi * mc + kl];
+                    if (!(bv > (T)0)) *singular = 1;
+                }
+            }
+            __syncthreads();
+            const int pr = s_piv;
+            for (int t = threadIdx.x; t < m * C; t += blockDim.x) {
+                const int rk = t / m, i = t % m;
+                const int src = i == k ? pr : (i == pr ? k : i);
+                T* dst = cl.map_shared_rank(fb, rk);
+                dst[i] = A[(size_t)src * mc + kl];
+                if (i == 0) {
+                    dst[m] = s_inv;
+                    cl.map_shared_rank(piv, rk)[k] = pr;
+                }
+            }
+        }
+        cl.sync();
+        const int pr = piv[k];
+        const T inv = fb[m];
+        for (int jl = threadIdx.x; jl < mc; jl += blockDim.x) {
+            const int j = jl * C + me;
+            if (j >= m) continue;
+            T rowk = A[(size_t)k * mc + jl];
+            if (pr != k) {
+                const T rowp = A[(size_t)pr * mc + jl];
+                A[(size_t)pr * mc + jl] = rowk;
+                rowk = rowp;
+            }
+            A[(size_t)k * mc + jl] = j == k ? inv : rowk * inv;
+        }
+        __syncthreads();
+        for (int t = threadIdx.x; t < m * mc; t += blockDim.x) {
+            const int i = t / mc, jl = t % mc;
+            const int j = jl * C + me;
+            if (i == k || j >= m) continue;
+            if (j == k)
+                A[(size_t)i * mc + jl] = -fb[i] * inv;
+            else
+                A[(size_t)i * mc + jl] -= fb[i] * A[(size_t)k * mc + jl];
+        }
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        for (int j = 0; j < m; j++) idx[j] = j;
+        for (int k = m - 1; k >= 0; k--) {
+            const int p = piv[k], t = idx[k];
+            idx[k] = idx[p];
+            idx[p] = t;
+        }
+        for (int j = 0; j < m; j++) pos[idx[j]] = j;
+    }
+    __syncthreads();
+    for (int t = threadIdx.x; t < m * mc; t += blockDim.x) {
+        const int i = t / mc, jl = t % mc;
+        const int j = jl * C + me;
+        if (j < m) Ainv[(size_t)i * m + pos[j]] = A[(size_t)i * mc + jl];
+    }
+    cl.sync();  // no CTA leaves while another may still write its shared memory
+}
+
+// x = A^{-1} b: one warp per row
+template <int D, typename T>
+__global__ void __launch_bounds__(256) k_s_solve(SLev<D, T> L, const T* __restrict__ Ainv) {
+    const int nin = L.n0 + L.n1, m = nin + L.ng;
+    const int r = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+    pdl_enter();
+    if (r >= m) return;
+    const T* row = Ainv + (size_t)r * m;
+    T v = 0;
+    for (int j = lane; j < m; j += 32) v = fmadd(row[j], L.b[j], v);
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
+    if (lane == 0) {
+        int p;
+        L.X[list_slot<D, T>(L, r, p)] = v;
+    }
+}
+
+// ---------------------------------------------------------------------------
+// end of a linear solve
+
+template <int D>
+__global__ void __launch_bounds__(kT) k_s_update(SLev<D, double> L, const double* __restrict__ tt,
+                                                  double2* __restrict__ W, unsigned long long* norms) {
+    pdl_enter();
+    const int t = blockIdx.x * blockDim.x + threadIdx.x;
+    unsigned long long nx = 0, nw = 0;
+    if (t < L.n0 + L.n1 + L.ng) {
+        int p;
+        const int sl = list_slot<D, double>(L, t, p);
+        double2 w = W[p];
+        const double xs = L.X[sl], xc = fmadd(-L.rho[sl], xs, tt[sl]);
+        unsigned long long a0 = abs_bits(w.x), a1 = abs_bits(w.y);
+        nw = a0 > a1 ? a0 : a1;
+        a0 = abs_bits(xs);
+        a1 = abs_bits(xc);
+        nx = a0 > a1 ? a0 : a1;
+        w.x -= xs;
+        w.y -= xc;
+        W[p] = w;
+    }
+    block_max(nx, norms);
+    __syncthreads();
+    block_max(nw, norms + 1);
+}
+
+template <int D>
+__global__ void __launch_bounds__(kT) k_s_export(SLev<D, double> L, const double* __restrict__ tt, double2* x) {
+    pdl_enter();
+    const int t = blockIdx.x * blockDim.x + threadIdx.x;
+    if (t >= L.n0 + L.n1 + L.ng) return;
+    int p;
+    const int sl = list_slot<D, double>(L, t, p);
+    x[p] = make_double2(L.X[sl], fmadd(-L.rho[sl], L.X[sl], tt[sl]));
+}
+
+// ---------------------------------------------------------------------------
+// per-level data
+
+constexpr int kChunk = 1024;
+
+__device__ __forceinline__ bool near_ghost(const int8_t* type, int p, int n, int dim) {
+    bool g = type[p - 1] == T_GHOST || type[p + 1] == T_GHOST || type[p - n] == T_GHOST || type[p + n] == T_GHOST;
+    if (dim == 3) g = g || type[p - n * n] == T_GHOST || type[p + n * n] == T_GHOST;
+    return g;
+}
+
+// nodes of a colour's list without a ghost neighbour, per chunk
+__global__ void k_away_count(const int* __restrict__ list, int cnt, const int8_t* __restrict__ type, int n, int dim,
+                             int* __restrict__ out) {
+    const int t = blockIdx.x * kChunk + threadIdx.x;
+    const int c = __syncthreads_count(t < cnt && !near_ghost(type, list[t], n, dim));
+    if (threadIdx.x == 0) out[blockIdx.x] = c;
+}
+
+// entries of a colour's nodes, those next to a ghost (at `away` and on) last
+__global__ void k_entries(const int* __restrict__ list, int cnt, const int8_t* __restrict__ type, int n, int dim,
+                          const int8_t* __restrict__ ctype, int cn, const int* __restrict__ off, int away, int H,
+                          int* __restrict__ hl) {
+    __shared__ int wsum[32];
+    const int t = blockIdx.x * kChunk + threadIdx.x;
+    const bool on = t < cnt;
+    const int p = on ? list[t] : 0;
+    const bool a = on && !near_ghost(type, p, n, dim);
+    const unsigned m = __ballot_sync(0xffffffffu, a);
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    if (lane == 0) wsum[warp] = __popc(m);
+    __syncthreads();
+    if (!on) return;
+    int r = off[blockIdx.x] + __popc(m & ((1u << lane) - 1u));
+    for (int w = 0; w < warp; w++) r += wsum[w];
+    const int ii[3] = {p % n, (p / n) % n, dim == 3 ? p / (n * n) : 0};
+    bool all = ctype != nullptr;
+    for (int cc = 0; cc < (1 << dim) && all; cc++) {
+        int q = 0, st = 1;
+        for (int d = 0; d < dim; d++) {
+            q += ((ii[d] + ((cc >> d) & 1)) >> 1) * st;
+            st *= cn;
+        }
+        all = ctype[q] == T_IN || ctype[q] == T_GHOST;
+    }
+    const int h = (ii[0] >> 1) + H * (ii[1] + n * ii[2]);
+    hl[a ? r : away + t - r] = (h << kEntHalf) | (all ? 4 : 0) | (a ? 0 : 2) | (ii[0] & 1);
+}
+
+__device__ __forceinline__ int box_slot(int p, int n, int dim, int H, int Hn) {
+    const int i = p % n, j = (p / n) % n, k = dim == 3 ? p / (n * n) : 0;
+    return ((i + j + k) & 1) * Hn + (i >> 1) + H * (j + n * k);
+}
+
+__global__ void k_ghost_slots(const int* __restrict__ gidx, int ng, int n, int dim, int H, int Hn,
+                              int* __restrict__ gslot) {
+    const int g = blockIdx.x * blockDim.x + threadIdx.x;
+    if (g < ng) gslot[g] = box_slot(gidx[g], n, dim, H, Hn);
+}
+
+__global__ void k_gop_codes(const int* __restrict__ code, int nnz, const int* __restrict__ gpos, int n, int dim,
+                            int H, int Hn, int* __restrict__ out) {
+    const int j = blockIdx.x * blockDim.x + threadIdx.x;
+    if (j >= nnz) return;
+    const int c = code[j];
+    if (c >= 0) {
+        out[j] = box_slot(c, n, dim, H, Hn);
+        return;
+    }
+    const unsigned u = ~(unsigned)c;
+    out[j] = (u & 1u) ? ~(int)(2u * (unsigned)gpos[u >> 1] + 1u) : c;
+}
+
+// members of the ghosts' rows: count, then fill
+__global__ void k_rows(int ng, int K, const double* __restrict__ wk, const float* __restrict__ wk32,
+                       const int* __restrict__ node, const int* __restrict__ ptr, int n, int dim, int H, int Hn,
+                       int* __restrict__ cnt, int* __restrict__ slot, double* __restrict__ val,
+                       float* __restrict__ val32) {
+    const int g = blockIdx.x * blockDim.x + threadIdx.x;
+    if (g >= ng) return;
+    int j = ptr ? ptr[g] : 0;
+    for (int kk = 0; kk < K; kk++) {
+        const long long o = (long long)kk * ng + g;
+        if (wk[o] == 0.0 && wk32[o] == 0.f) continue;
+        if (ptr) {
+            slot[j] = box_slot(node[o], n, dim, H, Hn);
+            val[j] = wk[o];
+            val32[j] = wk32[o];
+        }
+        j++;
+    }
+    if (!ptr) cnt[g] = j;
+}
+
+// slot of the fine twin of a coarse inside node all of whose 3^d fine members
+// are inside nodes, its black ones (odd index sum) away from the ghosts
+__global__ void k_twins(const int* __restrict__ hl, int n0, int nin, int cn, int cH, const int8_t* __restrict__ ftype,
+                        int fn, int fH, int dim, int* __restrict__ twin) {
+    const int t = blockIdx.x * blockDim.x + threadIdx.x;
+    if (t >= nin) return;
+    const int e = hl[t], h = e >> kEntHalf, row = h / cH;
+    const int f[3] = {2 * (2 * (h - row * cH) + (e & 1)), 2 * (row % cn), dim == 3 ? 2 * (row / cn) : 0};
+    bool ok = true;
+    for (int kk = 0; kk < (dim == 2 ? 9 : 27) && ok; kk++) {
+        const int k[3] = {kk % 3 - 1, (kk / 3) % 3 - 1, dim == 3 ? kk / 9 - 1 : 0};
+        int q = 0, st = 1;
+        for (int a = 0; a < dim; a++) {
+            if (f[a] + k[a] < 0 || f[a] + k[a] >= fn) ok = false;
+            q += (f[a] + k[a]) * st;
+            st *= fn;
+        }
+        if (!ok) break;
+        ok = ftype[q] == T_IN;
+        if (ok && ((k[0] + k[1] + k[2]) & 1)) ok = !near_ghost(ftype, q, fn, dim);
+    }
+    // (2I, 2J, 2K) is a red node: slot = half index
+    twin[t] = ok ? (f[0] >> 1) + fH * (f[1] + fn * f[2]) : -1;
+}
+
+// A coarse ghost's right-hand side: the outside weighting (Sec. 3.5.2) of the
+// fine ghosts' defects and of their extension into the band, as one row over
+// the fine ghosts (entries of one ghost merged).  Workspace in shared memory.
+constexpr int kOutCap = 192;
+struct OutWork {
+    double w[kOutCap];
+    int g[kOutCap];
+};
+constexpr int kOutThreads = 16;
+
+__global__ void k_outside_rows(const int* __restrict__ cgidx, int cng, int cn, const int8_t* __restrict__ ftype,
+                               int fn, int dim, const int* __restrict__ bpos, const int* __restrict__ eptr,
+                               const int* __restrict__ eidx, const double* __restrict__ eval, int fH, int fHn,
+                               const int* __restrict__ ptr, int* __restrict__ cnt, int* __restrict__ slot,
+                               double* __restrict__ val, float* __restrict__ val32) {
+    extern __shared__ OutWork out_ws[];
+    const int gi = blockIdx.x * blockDim.x + threadIdx.x;
+    if (gi >= cng) return;
+    OutWork& W = out_ws[threadIdx.x];
+    int m = 0;
+    bool over = false;
+    auto add = [&](int g, double w) {
+        int j = 0;
+        while (j < m && W.g[j] != g) j++;
+        if (j == m) {
+            if (m == kOutCap) {
+                over = true;
+                return;
+            }
+            W.g[m] = g;
+            W.w[m] = 0.0;
+            m++;
+        }
+        W.w[j] += w;
+    };
+    auto node = [&](int q, double w) {
+        if (ftype[q] == T_GHOST)
+            add(q, w);
+        else if (ftype[q] == T_BAND)
+            for (int j = eptr[bpos[q]]; j < eptr[bpos[q] + 1]; j++) add(eidx[j], w * eval[j]);
+    };
+    const int I = cgidx[gi];
+    const int ci[3] = {I % cn, (I / cn) % cn, dim == 3 ? I / (cn * cn) : 0};
+    const int st[3] = {1, fn, fn * fn};
+    int p = 0;
+    for (int a = 0; a < dim; a++) p += 2 * ci[a] * st[a];
+    auto outside = [&](int q) { return ftype[q] == T_GHOST || ftype[q] == T_BAND; };
+    int w[3][3] = {{0, 1, 0}, {0, 1, 0}, {0, 1, 0}};
+    for (int a = 0; a < dim; a++) {
+        const bool vl = ci[a] > 0 && outside(p - st[a]), vr = 2 * ci[a] < fn - 1 && outside(p + st[a]);
+        w[a][0] = vl ? (vr ? 1 : 2) : (vr ? 0 : 0);
+        w[a][1] = vl || vr ? 2 : 4;
+        w[a][2] = vr ? (vl ? 1 : 2) : 0;
+    }
+    const double scale = dim == 2 ? 1.0 / 16 : 1.0 / 64;
+    int wc = 0;
+    for (int kk = 0; kk < (dim == 2 ? 9 : 27); kk++) {
+        const int k[3] = {kk % 3, (kk / 3) % 3, dim == 3 ? kk / 9 : 1};
+        const int iw = w[0][k[0]] * w[1][k[1]] * w[2][k[2]];
+        if (iw == 0) continue;
+        int q = p;
+        for (int a = 0; a < dim; a++) q += (k[a] - 1) * st[a];
+        if (q == p || !outside(q))
+            wc += iw;
+        else
+            node(q, iw * scale);
+    }
+    node(p, wc * scale);
+    if (!ptr) {
+        cnt[gi] = over ? -1 : m;
+        return;
+    }
+    for (int j = 0; j < m; j++) {
+        slot[ptr[gi] + j] = box_slot(W.g[j], fn, dim, fH, fHn);
+        val[ptr[gi] + j] = W.w[j];
+        val32[ptr[gi] + j] = (float)W.w[j];
+    }
+}
+
+__global__ void k_positions(const int* __restrict__ hl, int n0, int nin, const int* __restrict__ gslot, int ng, int Hn,
+                            int* __restrict__ spos) {
+    const int t = blockIdx.x * blockDim.x + threadIdx.x;
+    if (t < nin)
+        spos[(t >= n0 ? Hn : 0) + (hl[t] >> kEntHalf)] = t;
+    else if (t < nin + ng)
+        spos[gslot[t - nin]] = t;
+}
+
+inline unsigned nblk(long long n, int t = 256) { return (unsigned)((n + t - 1) / t); }
+
+// host scan of n counts at dcnt into offsets (in place, dcnt has n + 1
+// entries); the total, or -1 on a negative count or error
+long long host_scan(int* dcnt, int n, cudaStream_t s, bool& bad) {
+    std::vector<int> c(n + 1, 0);
+    bad = false;
+    if (cudaMemcpyAsync(c.data(), dcnt, sizeof(int) * n, cudaMemcpyDeviceToHost, s) != cudaSuccess ||
+        cudaStreamSynchronize(s) != cudaSuccess)
+        return -1;
+    long long tot = 0;
+    for (int i = 0; i < n; i++) {
+        if (c[i] < 0) bad = true;
+        const int v = c[i];
+        c[i] = (int)tot;
+        tot += v;
+    }
+    c[n] = (int)tot;
+    if (bad) return 0;
+    if (cudaMemcpyAsync(dcnt, c.data(), sizeof(int) * (n + 1), cudaMemcpyHostToDevice, s) != cudaSuccess ||
+        cudaStreamSynchronize(s) != cudaSuccess)
+        return -1;
+    return tot;
+}
+
+}  // namespace
+
+int build_sgeo(SGeo& S, const LevelGeo& L, const LevelGeo* finer, const SGeo* sfiner, const LevelGeo* coarser,
+               DevMem& mem, cudaStream_t s, std::string& err, long long& launches, bool& ok) {
+    ok = false;
+    auto oom = [&] {
+        err = "out of device memory";
+        return SULF_ENOMEM;
+    };
+    auto fail = [&] {
+        err = "level lists failed";
+        return SULF_EDEVICE;
+    };
+    if (L.nn >= (1LL << 28)) return SULF_OK;  // entries hold 29-bit half indices
+    S.H = (L.n + 1) / 2;
+    S.P = S.H * L.n;
+    S.Hn = L.dim == 3 ? S.P * L.n : S.P;
+    S.n0 = L.nin[0];
+    S.n1 = L.nin[1];
+    const int nin = S.n0 + S.n1;
+    S.hl = (int*)mem.get(sizeof(int) * (nin + 1));
+    S.gslot = (int*)mem.get(sizeof(int) * (L.ng + 1));
+    const int nch = (int)nblk(S.n0 > S.n1 ? S.n0 : S.n1, kChunk);
+    int* dc = (int*)mem.get(sizeof(int) * 2 * (nch + 1));
+    if (!S.hl || !S.gslot || !dc) return oom();
+    std::vector<int> c(2 * (nch + 1), 0);
+    for (int k = 0; k < 2; k++)
+        if (L.nin[k] > 0) {
+            k_away_count<<<nblk(L.nin[k], kChunk), kChunk, 0, s>>>(L.inl[k], L.nin[k], L.type, L.n, L.dim,
+                                                                   dc + k * (nch + 1));
+            launches++;
+        }
+    if (cudaMemcpyAsync(c.data(), dc, sizeof(int) * c.size(), cudaMemcpyDeviceToHost, s) != cudaSuccess ||
+        cudaStreamSynchronize(s) != cudaSuccess)
+        return fail();
+    int away[2] = {0, 0};
+    for (int k = 0; k < 2; k++) {
+        const int nk = (int)nblk(L.nin[k], kChunk);
+        int tot = 0;
+        for (int b = 0; b < nk; b++) {
+            const int v = c[k * (nch + 1) + b];
+            c[k * (nch + 1) + b] = tot;
+            tot += v;
+        }
+        away[k] = tot;
+    }
+    S.nga = S.n1 - away[1];
+    if (cudaMemcpyAsync(dc, c.data(), sizeof(int) * c.size(), cudaMemcpyHostToDevice, s) != cudaSuccess) return fail();
+    for (int k = 0; k < 2; k++)
+        if (L.nin[k] > 0) {
+            k_entries<<<nblk(L.nin[k], kChunk), kChunk, 0, s>>>(
+                L.inl[k], L.nin[k], L.type, L.n, L.dim, coarser ? coarser->type : nullptr, coarser ? coarser->n : 0,
+                dc + k * (nch + 1), away[k], S.H, S.hl + (k ? S.n0 : 0));
+            launches++;
+        }
+    if (L.ng > 0) {
+        k_ghost_slots<<<nblk(L.ng), 256, 0, s>>>(L.gidx, L.ng, L.n, L.dim, S.H, S.Hn, S.gslot);
+        launches++;
+    }
+    if (finer) {
+        S.twin = (int*)mem.get(sizeof(int) * (nin + 1));
+        S.cptr = (int*)mem.get(sizeof(int) * (L.ng + 1));
+        if (!S.twin || !S.cptr) return oom();
+        k_twins<<<nblk(nin), 256, 0, s>>>(S.hl, S.n0, nin, L.n, S.H, finer->type, finer->n, sfiner->H, L.dim, S.twin);
+        launches++;
+        long long tot = 0;
+        const size_t shm = sizeof(OutWork) * kOutThreads;
+        if (L.ng > 0) {
+            k_outside_rows<<<nblk(L.ng, kOutThreads), kOutThreads, shm, s>>>(
+                L.gidx, L.ng, L.n, finer->type, finer->n, L.dim, finer->bpos, finer->eptr, finer->eidx, finer->eval,
+                sfiner->H, sfiner->Hn, nullptr, S.cptr, nullptr, nullptr, nullptr);
+            launches++;
+            bool bad;
+            tot = host_scan(S.cptr, L.ng, s, bad);
+            if (tot < 0) return fail();
+            if (bad) return SULF_OK;
+        }
+        S.cslot = (int*)mem.get(sizeof(int) * (tot + 1));
+        S.cval = (double*)mem.get(sizeof(double) * (tot + 1));
+        S.cval32 = (float*)mem.get(sizeof(float) * (tot + 1));
+        if (!S.cslot || !S.cval || !S.cval32) return oom();
+        if (L.ng > 0) {
+            k_outside_rows<<<nblk(L.ng, kOutThreads), kOutThreads, shm, s>>>(
+                L.gidx, L.ng, L.n, finer->type, finer->n, L.dim, finer->bpos, finer->eptr, finer->eidx, finer->eval,
+                sfiner->H, sfiner->Hn, S.cptr, nullptr, S.cslot, S.cval, S.cval32);
+            launches++;
+        }
+    }
+    if (!coarser) {
+        S.spos = (int*)mem.get(sizeof(int) * 2 * (size_t)S.Hn);
+        if (!S.spos) return oom();
+        if (cudaMemsetAsync(S.spos, 0, sizeof(int) * 2 * (size_t)S.Hn, s) != cudaSuccess) return fail();
+        k_positions<<<nblk(nin + L.ng), 256, 0, s>>>(S.hl, S.n0, nin, S.gslot, L.ng, S.Hn, S.spos);
+        launches++;
+    }
+    if (cudaStreamSynchronize(s) != cudaSuccess) return fail();
+    ok = true;
+    return SULF_OK;
+}
+
+int build_sgeo_rows(SGeo& S, const LevelGeo& L, DevMem& mem, cudaStream_t s, std::string& err, long long& launches) {
+    auto oom = [&] {
+        err = "out of device memory";
+        return SULF_ENOMEM;
+    };
+    S.bc = L.gop_bc;
+    S.passes = L.gop_passes;
+    S.tau = L.gop_tau;
+    if (L.ng == 0) return SULF_OK;
+    if (L.gop_nnz > S.gcap) {
+        S.gcode = (int*)mem.get(sizeof(int) * (L.gop_nnz + 1));
+        if (!S.gcode) return oom();
+        S.gcap = L.gop_nnz;
+    }
+    k_gop_codes<<<nblk(L.gop_nnz), 256, 0, s>>>(L.gop_code, (int)L.gop_nnz, L.gpos, L.n, L.dim, S.H, S.Hn, S.gcode);
+    const int K = L.dim == 2 ? 9 : 27;
+    if (!S.rptr) {
+        S.rptr = (int*)mem.get(sizeof(int) * (L.ng + 1));
+        // at most K members a row: sized once, the boundary condition may change
+        S.rslot = (int*)mem.get(sizeof(int) * (size_t)K * (L.ng + 1));
+        S.rval = (double*)mem.get(sizeof(double) * (size_t)K * (L.ng + 1));
+        S.rval32 = (float*)mem.get(sizeof(float) * (size_t)K * (L.ng + 1));
+        if (!S.rptr || !S.rslot || !S.rval || !S.rval32) return oom();
+    }
+    k_rows<<<nblk(L.ng), 256, 0, s>>>(L.ng, K, L.gwk, L.gwk32, L.gnode, nullptr, L.n, L.dim, S.H, S.Hn, S.rptr,
+                                      nullptr, nullptr, nullptr);
+    bool bad;
+    if (host_scan(S.rptr, L.ng, s, bad) < 0 || bad) {
+        err = "ghost rows failed";
+        return SULF_EDEVICE;
+    }
+    k_rows<<<nblk(L.ng), 256, 0, s>>>(L.ng, K, L.gwk, L.gwk32, L.gnode, S.rptr, L.n, L.dim, S.H, S.Hn, nullptr,
+                                      S.rslot, S.rval, S.rval32);
+    launches += 3;
+    if (cudaStreamSynchronize(s) != cudaSuccess) {
+        err = "ghost rows failed";
+        return SULF_EDEVICE;
+    }
+    return SULF_OK;
+}
+
+// ---------------------------------------------------------------------------
+// launchers
+
+template <int D, typename T>
+int launch_s_rho(const SLev<D, T>& L, const typename V2<T>::t* Wc, const Coef<T>& c, cudaStream_t s) {
+    const int tot = L.n0 + L.n1 + L.ng;
+    launch_k(k_s_rho<D, T, false, false>, grid_for(tot), block_for(tot), 0, s, L, SLev<D, float>{}, Wc, c,
+             (const double2*)nullptr, (double*)nullptr);
+    return 1;
+}
+
+template <int D>
+int launch_s_rho_fine(const SLev<D, double>& L, const double2* Wc, const Coef<double>& c, const double2* F, double* tt,
+                      const SLev<D, float>* U, cudaStream_t s) {
+    const int tot = L.n0 + L.n1 + L.ng;
+    if (U)
+        launch_k(k_s_rho<D, double, true, true>, grid_for(tot), block_for(tot), 0, s, L, *U, Wc, c, F, tt);
+    else
+        launch_k(k_s_rho<D, double, true, false>, grid_for(tot), block_for(tot), 0, s, L, SLev<D, float>{}, Wc, c, F,
+                 tt);
+    return 1;
+}
+
+template <int D, typename T>
+int launch_s_coefs(const SLev<D, T>& L, const typename V2<T>::t* Wc, const Coef<T>& c, cudaStream_t s) {
+    const int tot = L.n0 + L.n1;
+    launch_k(k_s_coefs<D, T, false, false>, grid_for(tot), block_for(tot), 0, s, L, SLev<D, float>{}, Wc, c,
+             (const double2*)nullptr, (const double*)nullptr);
+    return 1;
+}
+
+template <int D>
+int launch_s_coefs_fine(const SLev<D, double>& L, const double2* Wc, const Coef<double>& c, const double2* F,
+                        const double* tt, const SLev<D, float>* U, cudaStream_t s) {
+    const int tot = L.n0 + L.n1;
+    if (U)
+        launch_k(k_s_coefs<D, double, true, true>, grid_for(tot), block_for(tot), 0, s, L, *U, Wc, c, F, tt);
+    else
+        launch_k(k_s_coefs<D, double, true, false>, grid_for(tot), block_for(tot), 0, s, L, SLev<D, float>{}, Wc, c, F,
+                 tt);
+    return 1;
+}
+
+template <int D, typename T>
+int launch_s_relax(const SLev<D, T>& L, int colour, bool delta, bool snap, const int* skip, double* acc,
+                   cudaStream_t s) {
+    const int cnt = colour ? L.n1 : L.n0, tot = snap && L.ng > cnt ? L.ng : cnt;
+    if (tot == 0) return 0;
+    launch_k(delta ? k_s_relax<D, T, true> : k_s_relax<D, T, false>, grid_for(tot), block_for(tot), 0, s, L, colour,
+             snap ? 1 : 0, skip, acc);
+    return 1;
+}
+
+template <int D, typename T>
+int launch_s_ghosts(const SLev<D, T>& L, const int* skip, double* acc, cudaStream_t s) {
+    if (L.ng == 0) return 0;
+    const long long nt = (long long)L.ng * kGopLanes;
+    launch_k(k_s_ghosts<D, T>, grid_for(nt), block_for(nt), 0, s, L, skip, acc);
+    return 1;
+}
+
+template <int D, typename T>
+int launch_s_residual(const SLev<D, T>& L, unsigned long long* norm, int* clear, cudaStream_t s) {
+    const int nrow = (L.n0 + L.nga + 31) / 32 * 32;
+    const long long tot = nrow + (long long)L.ng * kRowLanes;
+    launch_k(norm ? k_s_residual<D, T, true> : k_s_residual<D, T, false>, grid_for(tot), block_for(tot), 0, s, L, nrow,
+             norm, clear);
+    return 1;
+}
+
+template <int D>
+int launch_s_outer(const SLev<D, double>& L, const SLev<D, float>& U, unsigned long long* norm, int* clear,
+                   cudaStream_t s) {
+    const int nrow = (L.n0 + L.n1 + 31) / 32 * 32;
+    const long long tot = nrow + (long long)L.ng * kRowLanes;
+    launch_k(k_s_outer<D>, grid_for(tot), block_for(tot), 0, s, L, U, nrow, norm, clear);
+    return 1;
+}
+
+template <int D, typename T>
+int launch_s_restrict(const SLev<D, T>& F, const SLev<D, T>& C, cudaStream_t s) {
+    const int nrow = (C.n0 + C.n1 + 31) / 32 * 32;
+    const long long tot = nrow + (long long)C.ng * kGopLanes;
+    launch_k(k_s_restrict<D, T>, grid_for(tot), block_for(tot), 0, s, F, C, nrow);
+    return 1;
+}
+
+template <int D, typename T>
+int launch_s_prolong(const SLev<D, T>& F, const SLev<D, T>& C, cudaStream_t s) {
+    const int tot = F.n1 + F.ng;
+    if (tot == 0) return 0;
+    launch_k(k_s_prolong<D, T>, grid_for(tot), block_for(tot), 0, s, F, C);
+    return 1;
+}
+
+template <int D, typename T>
+int launch_s_factor(const SLev<D, T>& L, const int* spos, T* A, T* Ainv, int* singular, cudaStream_t s) {
+    const int m = L.n0 + L.n1 + L.ng;
+    constexpr size_t kMaxSmem = 220 * 1024;
+    const bool smem = factor_smem<T>(m, true) <= kMaxSmem;
+    auto kern = smem ? k_s_factor<D, T, true> : k_s_factor<D, T, false>;
+    // set once to the largest size ever used (a per-launch value would race
+    // with other threads' launches of different sizes)
+    static std::mutex mu;
+    static bool raised[2][64] = {};
+    int dev = 0;
+    cudaGetDevice(&dev);
+    {
+        std::lock_guard<std::mutex> lock(mu);
+        if (dev < 0 || dev >= 64 || !raised[smem][dev]) {
+            cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMaxSmem);
+            if (dev >= 0 && dev < 64) raised[smem][dev] = true;
+        }
+    }
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(kFacCluster);
+    cfg.blockDim = dim3(kFacThreads);
+    cfg.dynamicSmemBytes = factor_smem<T>(m, smem);
+    cfg.stream = s;
+    cudaLaunchAttribute at[2];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = kFacCluster;
+    at[0].val.clusterDim.y = 1;
+    at[0].val.clusterDim.z = 1;
+    at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[1].val.programmaticStreamSerializationAllowed = launch_pdl() ? 1 : 0;
+    cfg.attrs = at;
+    cfg.numAttrs = 2;
+    cudaError_t e = cudaLaunchKernelEx(&cfg, kern, L, spos, A, Ainv, singular);
+    if (e != cudaSuccess) note_launch_error(e, kFacCluster, kFacThreads, cfg.dynamicSmemBytes);
+    return 1;
+}
+
+template <int D, typename T>
+int launch_s_solve(const SLev<D, T>& L, const T* Ainv, cudaStream_t s) {
+    const int m = L.n0 + L.n1 + L.ng;
+    launch_k(k_s_solve<D, T>, (m + 7) / 8, 256, 0, s, L, Ainv);
+    return 1;
+}
+
+template <int D>
+int launch_s_update(const SLev<D, double>& L, const double* tt, double2* W, unsigned long long* norms,
+                    cudaStream_t s) {
+    const int tot = L.n0 + L.n1 + L.ng;
+    launch_k(k_s_update<D>, grid_for(tot), block_for(tot), 0, s, L, tt, W, norms);
+    return 1;
+}
+
+template <int D>
+int launch_s_export(const SLev<D, double>& L, const double* tt, double2* x, cudaStream_t s) {
+    const int tot = L.n0 + L.n1 + L.ng;
+    launch_k(k_s_export<D>, grid_for(tot), block_for(tot), 0, s, L, tt, x);
+    return 1;
+}
+
+template <int D, typename TF, typename T>
+int launch_inject_to(const LevelGeo& F, const typename V2<TF>::t* fW, const LevelGeo& C, typename V2<T>::t* cW,
+                     cudaStream_t s) {
+    stages::Lists ls = stages::make_lists(C);
+    const int tot = ls.n0 + ls.n1 + ls.ng;
+    launch_k(k_inject_to<D, TF, T>, grid_for(tot), block_for(tot), 0, s, ls, C.n, F.type, F.n, fW, cW);
+    return 1;
+}
+
+#define SULF_INST_S(D, T)                                                                                          \
+    template int launch_s_rho<D, T>(const SLev<D, T>&, const typename V2<T>::t*, const Coef<T>&, cudaStream_t);     \
+    template int launch_s_coefs<D, T>(const SLev<D, T>&, const typename V2<T>::t*, const Coef<T>&, cudaStream_t);   \
+    template int launch_s_relax<D, T>(const SLev<D, T>&, int, bool, bool, const int*, double*, cudaStream_t);      \
+    template int launch_s_ghosts<D, T>(const SLev<D, T>&, const int*, double*, cudaStream_t);                      \
+    template int launch_s_residual<D, T>(const SLev<D, T>&, unsigned long long*, int*, cudaStream_t);              \
+    template int launch_s_restrict<D, T>(const SLev<D, T>&, const SLev<D, T>&, cudaStream_t);                      \
+    template int launch_s_prolong<D, T>(const SLev<D, T>&, const SLev<D, T>&, cudaStream_t);                       \
+    template int launch_s_factor<D, T>(const SLev<D, T>&, const int*, T*, T*, int*, cudaStream_t);                 \
+    template int launch_s_solve<D, T>(const SLev<D, T>&, const T*, cudaStream_t);
+SULF_INST_S(2, double)
+SULF_INST_S(2, float)
+SULF_INST_S(3, double)
+SULF_INST_S(3, float)
+#define SULF_INST_SD(D)                                                                                            \
+    template int launch_s_rho_fine<D>(const SLev<D, double>&, const double2*, const Coef<double>&, const double2*, \
+                                      double*, const SLev<D, float>*, cudaStream_t);                               \
+    template int launch_s_coefs_fine<D>(const SLev<D, double>&, const double2*, const Coef<double>&,               \
+                                        const double2*, const double*, const SLev<D, float>*, cudaStream_t);       \
+    template int launch_s_outer<D>(const SLev<D, double>&, const SLev<D, float>&, unsigned long long*, int*,       \
+                                   cudaStream_t);                                                                  \
+    template int launch_s_update<D>(const SLev<D, double>&, const double*, double2*, unsigned long long*,          \
+                                    cudaStream_t);                                                                 \
+    template int launch_s_export<D>(const SLev<D, double>&, const double*, double2*, cudaStream_t);                \
+    template int launch_inject_to<D, double, double>(const LevelGeo&, const double2*, const LevelGeo&, double2*,   \
+                                                     cudaStream_t);                                                \
+    template int launch_inject_to<D, double, float>(const LevelGeo&, const double2*, const LevelGeo&, float2*,     \
+                                                    cudaStream_t);                                                 \
+    template int launch_inject_to<D, float, float>(const LevelGeo&, const float2*, const LevelGeo&, float2*,       \
+                                                   cudaStream_t);
+SULF_INST_SD(2)
+SULF_INST_SD(3)
+
+}  // namespace sulf

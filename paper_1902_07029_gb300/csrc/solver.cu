@@ -14,6 +14,7 @@
 
 #include "../../include/sulfmg_debug.h"
 #include "lockstep.cuh"
+#include "schur.cuh"
 #include "sulf_internal.cuh"
 
 using namespace sulf;
@@ -81,7 +82,15 @@ struct sulf_domain {
     LevelGeo geo[SULF_MAXLEV];
     LevelVec<double> v64[SULF_MAXLEV];
     LevelVec<float> v32[SULF_MAXLEV];
-    bool have32 = false;
+    bool have64 = false, have32 = false;  // the two-unknown kernels' vectors (on first use)
+    // the cycle on the equation for s (schur.cuh): built on first use;
+    // s_geo -1 where the geometry does not fit its form
+    SGeo sgeo[SULF_MAXLEV];
+    SVec<double> s64[SULF_MAXLEV];
+    SVec<float> s32[SULF_MAXLEV];
+    int s_geo = 0;
+    bool s_on = false;     // the current linear solve runs that cycle
+    int* dskip = nullptr;  // device flag: the first sweep of the cycle has been done
     int bc = 0;  // boundary condition for s: 0 Dirichlet (Eq. BCs), 1 Neumann (Eq. BCsN)
     double2* W = nullptr;   // state, = v64[0].Wc
     double2* Wn = nullptr;  // state at t_n
@@ -124,6 +133,7 @@ struct sulf_domain {
         cudaGraphExec_t exec = nullptr;
         double dt = 0;
         sulf_solver sv{};
+        bool s_on = false;
         int prof = 0;
         long long kernels = 0;
         size_t ev0 = 0, ev1 = 0;
@@ -137,6 +147,7 @@ struct sulf_domain {
         cudaGraphExec_t exec = nullptr;
         double dt = 0;
         sulf_solver sv{};
+        bool s_on = false;
         int max_cycles = 0;
         long long kernels = 0;  // per cycle
     } loop[2];
@@ -243,15 +254,47 @@ FConst make_fconst(const sulf_domain* d) {
     return f;
 }
 
+// forget the captured cycles (they hold pointers and parameters that changed)
+void drop_graphs(sulf_domain* d) {
+    for (auto& g : d->graph)
+        if (g.exec) {
+            cudaGraphExecDestroy(g.exec);
+            g.exec = nullptr;
+        }
+    for (auto& g : d->loop)
+        if (g.exec) {
+            cudaGraphExecDestroy(g.exec);
+            g.exec = nullptr;
+        }
+}
+
+// what every path uses: the coefficient source of each level (the finest one
+// is the state) and the finest right-hand side F
+int alloc_core(sulf_domain* d) {
+    for (int l = 0; l < d->L; l++) {
+        LevelVec<double>& v = d->v64[l];
+        const size_t nb2 = sizeof(double2) * d->geo[l].nn;
+        v.Wc = (double2*)d->mem.get(nb2);
+        if (!v.Wc) return sulf_fail(SULF_ENOMEM, "out of device memory");
+        SULF_CUDA_TRY(cudaMemsetAsync(v.Wc, 0, nb2, d->stream));
+    }
+    d->v64[0].rhs = (double2*)d->mem.get(sizeof(double2) * d->geo[0].nn);
+    if (!d->v64[0].rhs) return sulf_fail(SULF_ENOMEM, "out of device memory");
+    SULF_CUDA_TRY(cudaMemsetAsync(d->v64[0].rhs, 0, sizeof(double2) * d->geo[0].nn, d->stream));
+    return SULF_OK;
+}
+
+// the vectors of the two-unknown kernels
 template <typename T>
-int alloc_vectors(sulf_domain* d, LevelVec<T>* V, bool share_state) {
+int alloc_vectors(sulf_domain* d, LevelVec<T>* V) {
     typedef typename V2<T>::t T2;
     for (int l = 0; l < d->L; l++) {
         const LevelGeo& G = d->geo[l];
         LevelVec<T>& v = V[l];
         size_t nb2 = sizeof(T2) * G.nn;
-        if (!(share_state && l == 0)) v.Wc = (T2*)d->mem.get(nb2);
-        v.rhs = (T2*)d->mem.get(nb2);
+        const bool wc = !v.Wc, rhs = !v.rhs;
+        if (wc) v.Wc = (T2*)d->mem.get(nb2);
+        if (rhs) v.rhs = (T2*)d->mem.get(nb2);
         v.x = (T2*)d->mem.get(nb2);
         v.res = (T2*)d->mem.get(nb2);
         for (int k = 0; k < 2; k++) v.gbuf[k] = (T*)d->mem.get(sizeof(T) * (G.ng + 1));
@@ -272,13 +315,10 @@ int alloc_vectors(sulf_domain* d, LevelVec<T>* V, bool share_state) {
             SULF_CUDA_TRY(cudaMemsetAsync(v.rhsc, 0, nl, d->stream));
         }
         if (!v.Pa || !v.Pb || !v.Ia || !v.Ib || !v.Pc || !v.Ic || !v.gc || !v.gci || !v.edge[0] || !v.edge[1] ||
-            (G.dim == 3 && !v.edge[2]))
+            (G.dim == 3 && !v.edge[2]) || !v.Wc || !v.rhs || !v.x || !v.res || !v.gbuf[0] || !v.gbuf[1])
             return sulf_fail(SULF_ENOMEM, "out of device memory");
-        if ((!share_state || l > 0) && !v.Wc) return sulf_fail(SULF_ENOMEM, "out of device memory");
-        if (!v.rhs || !v.x || !v.res || !v.gbuf[0] || !v.gbuf[1])
-            return sulf_fail(SULF_ENOMEM, "out of device memory");
-        if (v.Wc) SULF_CUDA_TRY(cudaMemsetAsync(v.Wc, 0, nb2, d->stream));
-        SULF_CUDA_TRY(cudaMemsetAsync(v.rhs, 0, nb2, d->stream));
+        if (wc) SULF_CUDA_TRY(cudaMemsetAsync(v.Wc, 0, nb2, d->stream));
+        if (rhs) SULF_CUDA_TRY(cudaMemsetAsync(v.rhs, 0, nb2, d->stream));
         SULF_CUDA_TRY(cudaMemsetAsync(v.x, 0, nb2, d->stream));
         SULF_CUDA_TRY(cudaMemsetAsync(v.res, 0, nb2, d->stream));
         if (l == d->L - 1) {
@@ -291,11 +331,132 @@ int alloc_vectors(sulf_domain* d, LevelVec<T>* V, bool share_state) {
     return SULF_OK;
 }
 
+int ensure64(sulf_domain* d) {
+    if (d->have64) return SULF_OK;
+    int rc = alloc_vectors<double>(d, d->v64);
+    if (rc) return rc;
+    // a residual F computed before has no list-ordered copy yet
+    d->launches += launch_gather_list(d->geo[0], d->v64[0].rhs, d->v64[0].rhsc, d->stream);
+    d->have64 = true;
+    return SULF_OK;
+}
+
 int ensure32(sulf_domain* d) {
     if (d->have32) return SULF_OK;
-    int rc = alloc_vectors<float>(d, d->v32, false);
+    int rc = alloc_vectors<float>(d, d->v32);
     if (rc) return rc;
     d->have32 = true;
+    return SULF_OK;
+}
+
+// ---- the cycle on the equation for s (schur.cuh) ----
+
+// whether the solver controls allow it: collective red-black V- or W-cycles
+// with pre- and post-relaxation and the composed ghost relaxation (and in
+// mixed precision not the stored-coefficient or tiled FP32 sweeps).  Small
+// mixed-precision domains stay with the two-unknown kernels, whose coarse
+// levels run as one single-CTA launch (13 k active nodes, 257^2 star: 9.8 ms
+// for two CN steps against 10.9; 104 k nodes, 65^3 box: 26.7 against 28.2 the
+// other way)
+constexpr long long kSchurMinMixed = 50000;
+bool schur_wanted(const sulf_domain* d) {
+    const sulf_solver& v = d->solver;
+    if (v.precision == 1 && (long long)d->geo[0].nin[0] + d->geo[0].nin[1] < kSchurMinMixed) return false;
+    return d->L >= 2 && v.smoother == 0 && v.cycle != 3 && v.nu1 >= 1 && v.nu2 >= 1 && v.ghost_compose &&
+           (v.precision == 0 || v.relax_matrix_free == 1);
+}
+
+// levels 0 .. nl-1; outer: only what the FP64 defect of mixed precision uses
+template <typename T>
+int alloc_schur(sulf_domain* d, SVec<T>* V, int nl, bool outer) {
+    const bool f32 = std::is_same<T, float>::value;
+    bool ok = true;
+    auto get = [&](auto*& p, size_t n, bool zero) {
+        if (p || !ok) return;
+        const size_t nb = sizeof(*p) * (n + 1);
+        p = (std::remove_reference_t<decltype(p)>)d->mem.get(nb);
+        ok = p && (!zero || cudaMemsetAsync(p, 0, nb, d->stream) == cudaSuccess);
+    };
+    for (int l = 0; l < nl; l++) {
+        const LevelGeo& G = d->geo[l];
+        const SGeo& S = d->sgeo[l];
+        SVec<T>& v = V[l];
+        const size_t ns = 2 * (size_t)S.Hn, nin = (size_t)S.n0 + S.n1;
+        get(v.X, ns, true);
+        get(v.rho, ns, false);
+        get(v.cs, ns, false);
+        get(v.gt, nin * 2 * G.dim, false);
+        get(v.dd, nin, false);
+        get(v.di, nin, false);
+        get(v.b, nin + G.ng, false);
+        if (!f32 && l == 0) get(v.tt, ns, false);
+        if (outer) continue;
+        get(v.snap, (size_t)G.ng, false);
+        // zero where never written: defects of the black nodes away from the
+        // ghosts, and the red nodes' (delta, C delta)
+        get(v.R, ns, true);
+        get(v.D2, ns, true);
+        if (f32 && l > 0) get(v.Wc, (size_t)G.nn, false);
+        if (l == d->L - 1) {
+            const size_t m = nin + G.ng;
+            get(v.A, m * (m + 8), false);
+            get(v.Ainv, m * m, false);
+        }
+    }
+    return ok ? SULF_OK : sulf_fail(SULF_ENOMEM, "out of device memory");
+}
+
+// decides d->s_on for the next linear solve and builds what it needs
+int ensure_schur(sulf_domain* d);
+int ensure_path(sulf_domain* d) {
+    if (int rc = ensure_schur(d)) return rc;
+    if (d->s_on) return SULF_OK;
+    if (int rc = ensure64(d)) return rc;
+    return d->solver.precision == 1 ? ensure32(d) : SULF_OK;
+}
+
+int ensure_schur(sulf_domain* d) {
+    d->s_on = false;
+    if (!schur_wanted(d) || d->s_geo < 0) return SULF_OK;
+    for (int l = 0; l < d->L; l++) {
+        const LevelGeo& G = d->geo[l];
+        if (G.ng > 0 && !(G.gop_on && G.gop_bc == d->bc && G.gop_passes == d->solver.ghost_sweeps &&
+                          G.gop_tau == level_tau(d, l)))
+            return SULF_OK;
+    }
+    std::string err;
+    if (!d->s_geo) {
+        for (int l = 0; l < d->L; l++) {
+            bool ok = false;
+            int rc = build_sgeo(d->sgeo[l], d->geo[l], l ? &d->geo[l - 1] : nullptr, l ? &d->sgeo[l - 1] : nullptr,
+                                l + 1 < d->L ? &d->geo[l + 1] : nullptr, d->mem, d->stream, err, d->launches, ok);
+            if (rc) return sulf_fail(rc, err);
+            if (!ok) {
+                d->s_geo = -1;
+                return SULF_OK;
+            }
+        }
+        d->dskip = (int*)d->mem.get(sizeof(int));
+        if (!d->dskip) return sulf_fail(SULF_ENOMEM, "out of device memory");
+        d->s_geo = 1;
+    }
+    bool changed = false;
+    for (int l = 0; l < d->L; l++) {
+        SGeo& S = d->sgeo[l];
+        const LevelGeo& G = d->geo[l];
+        if (S.bc == G.gop_bc && S.passes == G.gop_passes && S.tau == G.gop_tau) continue;
+        int rc = build_sgeo_rows(S, G, d->mem, d->stream, err, d->launches);
+        if (rc) return sulf_fail(rc, err);
+        changed = true;
+    }
+    if (changed) drop_graphs(d);
+    if (d->solver.precision == 0) {
+        if (int rc = alloc_schur<double>(d, d->s64, d->L, false)) return rc;
+    } else {
+        if (int rc = alloc_schur<double>(d, d->s64, 1, true)) return rc;
+        if (int rc = alloc_schur<float>(d, d->s32, d->L, false)) return rc;
+    }
+    d->s_on = true;
     return SULF_OK;
 }
 
@@ -341,20 +502,6 @@ int ensure_tail(sulf_domain* d, const LevelVec<T>* V) {
     if (rc) return rc;
     d->tail_ready[p] = true;
     return SULF_OK;
-}
-
-// forget the captured cycles (they hold pointers and parameters that changed)
-void drop_graphs(sulf_domain* d) {
-    for (auto& g : d->graph)
-        if (g.exec) {
-            cudaGraphExecDestroy(g.exec);
-            g.exec = nullptr;
-        }
-    for (auto& g : d->loop)
-        if (g.exec) {
-            cudaGraphExecDestroy(g.exec);
-            g.exec = nullptr;
-        }
 }
 
 // (re)build the composed ghost relaxation of every level whose map was built
@@ -517,6 +664,109 @@ struct MG {
     }
 };
 
+// ---- the same cycle on the equation for s (schur.cuh), precision T ----
+template <int D, typename T>
+struct SMG {
+    sulf_domain* d;
+    SVec<T>* V;
+    double* acc = nullptr;  // mixed precision: the FP64 update the finest error is added to
+    int fine_sweeps = 0;
+
+    SLev<D, T> lev(int l) { return make_slev<D, T>(d->geo[l], d->sgeo[l], V[l]); }
+
+    // delta: the sweep follows a prolongation; a: see launch_s_relax
+    void relax(int l, bool skip_red, bool delta, const int* skip, double* a) {
+        const SLev<D, T> L = lev(l);
+        // timed sweeps: both colours launched and not skipped on a flag
+        const bool whole = l == 0 && !skip_red && !skip;
+        const bool timed = whole && (d->prof == 2 || (d->prof == 1 && fine_sweeps == 0));
+        if (whole) fine_sweeps++;
+        const unsigned fl = d->capturing ? cudaEventRecordExternal : cudaEventRecordDefault;
+        if (timed) cudaEventRecordWithFlags(next_event(d), d->stream, fl);
+        if (!skip_red) d->launches += launch_s_relax<D, T>(L, 0, delta, false, skip, a, d->stream);
+        d->launches += launch_s_relax<D, T>(L, 1, delta, true, skip, a, d->stream);
+        if (timed) cudaEventRecordWithFlags(next_event(d), d->stream, fl);
+        d->launches += launch_s_ghosts<D, T>(L, skip, a, d->stream);
+    }
+
+    // red_done: the first red half-sweep (from zero) came with the
+    // right-hand side; first: device flag, set where the whole first sweep
+    // has been done
+    int cycle(int l, bool red_done, const int* first) {
+        if (l == d->L - 1) {
+            d->launches += launch_s_solve<D, T>(lev(l), V[l].Ainv, d->stream);
+            return SULF_OK;
+        }
+        const sulf_solver& sv = d->solver;
+        for (int k = 0; k < sv.nu1; k++) relax(l, red_done && k == 0, false, k == 0 ? first : nullptr, nullptr);
+        d->launches += launch_s_residual<D, T>(lev(l), nullptr, nullptr, d->stream);
+        d->launches += launch_s_restrict<D, T>(lev(l), lev(l + 1), d->stream);
+        for (int g = 0; g < (sv.cycle == 2 ? 2 : 1); g++)
+            if (int rc = cycle(l + 1, g == 0, nullptr)) return rc;
+        d->launches += launch_s_prolong<D, T>(lev(l), lev(l + 1), d->stream);
+        for (int k = 0; k < sv.nu2; k++)
+            relax(l, false, k == 0, nullptr, l == 0 && k == sv.nu2 - 1 ? acc : nullptr);
+        return SULF_OK;
+    }
+
+    // coarse levels: (s, c) by injection and the rows; the coarsest inverse
+    int prepare_coarse() {
+        for (int l = 1; l < d->L; l++) {
+            if (std::is_same<T, float>::value && l == 1)
+                d->launches += launch_inject_to<D, double, T>(d->geo[0], d->W, d->geo[1], wc(1), d->stream);
+            else
+                d->launches += launch_inject_to<D, T, T>(d->geo[l - 1], wc(l - 1), d->geo[l], wc(l), d->stream);
+            const Coef<T> c = make_coef<T>(d, l);
+            d->launches += launch_s_rho<D, T>(lev(l), wc(l), c, d->stream);
+            d->launches += launch_s_coefs<D, T>(lev(l), wc(l), c, d->stream);
+        }
+        SULF_CUDA_TRY(cudaMemsetAsync(d->dsing, 0, sizeof(int), d->stream));
+        const int lc = d->L - 1;
+        d->launches += launch_s_factor<D, T>(lev(lc), d->sgeo[lc].spos, V[lc].A, V[lc].Ainv, d->dsing, d->stream);
+        return SULF_OK;
+    }
+
+    typename V2<T>::t* wc(int l) {
+        if constexpr (std::is_same<T, double>::value)
+            return d->v64[l].Wc;
+        else
+            return V[l].Wc;
+    }
+};
+
+template <int D>
+SLev<D, double> fine_slev(sulf_domain* d) {
+    return make_slev<D, double>(d->geo[0], d->sgeo[0], d->s64[0]);
+}
+
+// set-up of a linear solve J dW = F in this form: the rows of every level, the
+// coarsest inverse, and the first sweep of the first cycle, which runs from a
+// zero that is off the c rows
+template <int D>
+int schur_prepare(sulf_domain* d) {
+    const SLev<D, double> L0 = fine_slev<D>(d);
+    const Coef<double> c0 = make_coef<double>(d, 0);
+    const double2* F = d->v64[0].rhs;
+    double* tt = d->s64[0].tt;
+    if (d->solver.precision == 1) {
+        const SLev<D, float> U = make_slev<D, float>(d->geo[0], d->sgeo[0], d->s32[0]);
+        d->launches += launch_s_rho_fine<D>(L0, d->W, c0, F, tt, &U, d->stream);
+        d->launches += launch_s_coefs_fine<D>(L0, d->W, c0, F, tt, &U, d->stream);
+        if (int rc = SMG<D, float>{d, d->s32}.prepare_coarse()) return rc;
+        d->launches += launch_s_relax<D, float>(U, 1, true, true, nullptr, nullptr, d->stream);
+        d->launches += launch_s_ghosts<D, float>(U, nullptr, nullptr, d->stream);
+    } else {
+        d->launches += launch_s_rho_fine<D>(L0, d->W, c0, F, tt, nullptr, d->stream);
+        d->launches += launch_s_coefs_fine<D>(L0, d->W, c0, F, tt, nullptr, d->stream);
+        if (int rc = SMG<D, double>{d, d->s64}.prepare_coarse()) return rc;
+        d->launches += launch_s_relax<D, double>(L0, 1, true, true, nullptr, nullptr, d->stream);
+        d->launches += launch_s_ghosts<D, double>(L0, nullptr, nullptr, d->stream);
+    }
+    SULF_CUDA_TRY(cudaMemsetAsync(d->dskip, 1, sizeof(int), d->stream));
+    SULF_CUDA_TRY(cudaMemsetAsync(d->dnorm, 0, sizeof(unsigned long long) * 2, d->stream));
+    return SULF_OK;
+}
+
 // sum the device time of the event pairs [from, to) of the pool
 int accumulate_prof(sulf_domain* d, size_t from, size_t to) {
     for (size_t k = from; k + 1 < to; k += 2) {
@@ -537,6 +787,19 @@ bool same_solver(const sulf_solver& a, const sulf_solver& b) {
            a.relax_matrix_free == b.relax_matrix_free;
 }
 
+// the end of a cycle: its defect norm and the coarsest level's singularity flag
+// to the host, or the device loop's test
+int cycle_end(sulf_domain* d, const cudaGraphConditionalHandle* loop, int max_cycles) {
+    if (loop) {
+        d->launches +=
+            launch_cycle_check(*loop, d->dnorm, d->dsing, d->dthr, max_cycles, d->dcyc, d->drn, d->stream);
+        return SULF_OK;
+    }
+    SULF_CUDA_TRY(cudaMemcpyAsync(d->hnorm, d->dnorm, sizeof(unsigned long long), cudaMemcpyDeviceToHost, d->stream));
+    SULF_CUDA_TRY(cudaMemcpyAsync(d->hnorm + 6, d->dsing, sizeof(int), cudaMemcpyDeviceToHost, d->stream));
+    return SULF_OK;
+}
+
 // One cycle of the linear solve on the finest level, then the FP64 defect
 // r = F - J dW, its max-norm and the coarsest-level singularity flag copied to
 // pinned host memory.  FP64: a multigrid cycle on J dW = F.  Mixed: an FP32
@@ -546,6 +809,20 @@ int cycle_body(sulf_domain* d, const cudaGraphConditionalHandle* loop = nullptr,
     const LevelGeo& G0 = d->geo[0];
     LevelVec<double>& V0 = d->v64[0];
     const bool fmg = d->fmg_now && d->L > 1;
+    if (d->s_on) {
+        // the norm's slot is zeroed by the set-up and by the loop's test
+        if (!loop) SULF_CUDA_TRY(cudaMemsetAsync(d->dnorm, 0, sizeof(unsigned long long) * 2, d->stream));
+        const SLev<D, double> L0 = fine_slev<D>(d);
+        if (d->solver.precision == 0) {
+            if (int rc = SMG<D, double>{d, d->s64}.cycle(0, false, d->dskip)) return rc;
+            d->launches += launch_s_residual<D, double>(L0, d->dnorm, d->dskip, d->stream);
+        } else {
+            if (int rc = SMG<D, float>{d, d->s32, d->s64[0].X}.cycle(0, true, d->dskip)) return rc;
+            d->launches += launch_s_outer<D>(L0, make_slev<D, float>(G0, d->sgeo[0], d->s32[0]), d->dnorm, d->dskip,
+                                             d->stream);
+        }
+        return cycle_end(d, loop, max_cycles);
+    }
     if (d->solver.precision == 0) {
         if (d->L == 1)
             d->launches += launch_coarsest_solve<D, double>(G0, V0, d->stream);
@@ -565,13 +842,7 @@ int cycle_body(sulf_domain* d, const cudaGraphConditionalHandle* loop = nullptr,
         d->launches += launch_residual_to32<D>(G0, V0, d->v32[0].rhs, d->dnorm, d->stream);
     else
         d->launches += launch_residual<D, double>(G0, V0, make_coef<double>(d, 0), d->dnorm, d->stream);
-    if (!loop) {
-        SULF_CUDA_TRY(
-            cudaMemcpyAsync(d->hnorm, d->dnorm, sizeof(unsigned long long), cudaMemcpyDeviceToHost, d->stream));
-        SULF_CUDA_TRY(cudaMemcpyAsync(d->hnorm + 6, d->dsing, sizeof(int), cudaMemcpyDeviceToHost, d->stream));
-    }
-    if (loop) d->launches += launch_cycle_check(*loop, d->dnorm, d->dsing, d->dthr, max_cycles, d->dcyc, d->drn, d->stream);
-    return SULF_OK;
+    return cycle_end(d, loop, max_cycles);
 }
 
 constexpr int kLoopMaxCycles = 256;
@@ -646,6 +917,7 @@ bool build_loop(sulf_domain* d, int max_cycles) {
     }
     g.dt = d->dt;
     g.sv = d->solver;
+    g.s_on = d->s_on;
     g.max_cycles = max_cycles;
     return true;
 }
@@ -659,7 +931,7 @@ int device_loop(sulf_domain* d, double fnorm, int max_cycles, double rtol, doubl
     if (d->loop_off || !d->solver.graphs || d->prof || max_cycles > kLoopMaxCycles || d->solver.cycle == 3) return 0;
     const int p = d->solver.precision;
     sulf_domain::LoopGraph& g = d->loop[p];
-    if (!g.exec || g.dt != d->dt || !same_solver(g.sv, d->solver) || g.max_cycles != max_cycles)
+    if (!g.exec || g.dt != d->dt || !same_solver(g.sv, d->solver) || g.s_on != d->s_on || g.max_cycles != max_cycles)
         if (!build_loop<D>(d, max_cycles)) return 0;
     d->hloop[0] = rtol * fnorm;
     SULF_CUDA_TRY(cudaMemcpyAsync(d->dthr, d->hloop, sizeof(double), cudaMemcpyHostToDevice, d->stream));
@@ -715,7 +987,7 @@ int run_cycle(sulf_domain* d) {
     sulf_domain::CycleGraph& g = d->graph[p];
     // an instantiated graph may be launched on any stream: a new stream alone
     // needs no recapture
-    if (!g.exec || g.dt != d->dt || !same_solver(g.sv, d->solver) || g.prof != d->prof) {
+    if (!g.exec || g.dt != d->dt || !same_solver(g.sv, d->solver) || g.s_on != d->s_on || g.prof != d->prof) {
         if (g.exec) cudaGraphExecDestroy(g.exec);
         g.exec = nullptr;
         d->evused = 0;
@@ -740,6 +1012,7 @@ int run_cycle(sulf_domain* d) {
         g.ev1 = d->evused;
         g.dt = d->dt;
         g.sv = d->solver;
+        g.s_on = d->s_on;
         g.prof = d->prof;
     }
     SULF_CUDA_TRY(cudaGraphLaunch(g.exec, d->stream));
@@ -755,9 +1028,12 @@ int run_cycle(sulf_domain* d) {
 template <int D>
 int linear_solve(sulf_domain* d, double fnorm, int max_cycles, double rtol, double* rnorms) {
     const LevelGeo& G0 = d->geo[0];
-    SULF_CUDA_TRY(cudaMemsetAsync(d->v64[0].x, 0, sizeof(double2) * G0.nn, d->stream));
-    int rc;
-    if (d->solver.precision == 0) {
+    int rc = ensure_path(d);
+    if (rc) return rc;
+    if (!d->s_on) SULF_CUDA_TRY(cudaMemsetAsync(d->v64[0].x, 0, sizeof(double2) * G0.nn, d->stream));
+    if (d->s_on) {
+        rc = schur_prepare<D>(d);
+    } else if (d->solver.precision == 0) {
         rc = ensure_tail<D, double>(d, d->v64);
         if (rc) return rc;
         rc = MG<D, double>{d, d->v64}.prepare();
@@ -832,7 +1108,10 @@ int cn_step(sulf_domain* d) {
         d->cycles_last += nc;
         d->cycles_total += nc;
         SULF_CUDA_TRY(cudaMemsetAsync(d->dnorm, 0, sizeof(unsigned long long) * 4, d->stream));
-        d->launches += launch_newton_update(G0, d->W, V0.x, d->dnorm, d->stream);
+        if (d->s_on)
+            d->launches += launch_s_update<D>(fine_slev<D>(d), d->s64[0].tt, d->W, d->dnorm, d->stream);
+        else
+            d->launches += launch_newton_update(G0, d->W, V0.x, d->dnorm, d->stream);
         d->launches += launch_newton_F<D>(G0, d->W, d->G, V0.rhs, V0.rhsc, fc, d->dnorm + 2, d->stream);
         rc = read_norms(d, 3);
         if (rc) return rc;
@@ -1026,7 +1305,7 @@ int sulf_create_domain(const double* levelset, int dim, const double* box, int N
                                   d->launches);
         if (rc) sulf_fail(rc, err);
     }
-    if (rc == SULF_OK) rc = alloc_vectors<double>(d, d->v64, false);
+    if (rc == SULF_OK) rc = alloc_core(d);
     if (rc == SULF_OK) {
         long long nn = d->geo[0].nn;
         d->W = d->v64[0].Wc;
@@ -1081,9 +1360,9 @@ int sulf_set_solver(sulf_handle h, const sulf_solver* s) {
     if (int rc = refresh_ghost_ops(h)) return rc;
     if (v.smoother == 2)
         if (int rc = ensure_lex(h)) return rc;
-    if (v.precision == 1) {
+    if (v.precision == 1 && v.relax_matrix_free == 2) {
         if (int rc = ensure32(h)) return rc;
-        if (v.relax_matrix_free == 2) return ensure_tiles(h);
+        return ensure_tiles(h);
     }
     return SULF_OK;
 }
@@ -1342,6 +1621,7 @@ static int dbg_copy_out(sulf_handle h, int l, const double2* src, double* dst, b
 
 int sulf_dbg_eval_F(sulf_handle h, double dt, const double* W, const double* Wn, double* F) {
     if (!valid(h) || !W || !Wn || !F || !(dt > 0)) return sulf_fail(SULF_EINVAL, "invalid arguments");
+    if (int rc = ensure64(h)) return rc;
     const LevelGeo& G0 = h->geo[0];
     h->dt = dt;
     int rc = copy_in(h, h->W, W, sizeof(double2) * G0.nn);
@@ -1361,6 +1641,7 @@ int sulf_dbg_eval_F(sulf_handle h, double dt, const double* W, const double* Wn,
 
 int sulf_dbg_apply_J(sulf_handle h, int l, double dt, const double* Wc, const double* x, double* out) {
     if (!dbg_level_ok(h, l) || !Wc || !x || !out || !(dt > 0)) return sulf_fail(SULF_EINVAL, "invalid arguments");
+    if (int rc = ensure64(h)) return rc;
     const LevelGeo& G = h->geo[l];
     LevelVec<double>& V = h->v64[l];
     h->dt = dt;
@@ -1385,6 +1666,7 @@ int sulf_dbg_apply_J(sulf_handle h, int l, double dt, const double* Wc, const do
 int sulf_dbg_smooth(sulf_handle h, int l, double dt, const double* Wc, const double* rhs, double* x, int sweeps) {
     if (!dbg_level_ok(h, l) || !Wc || !rhs || !x || !(dt > 0) || sweeps < 0)
         return sulf_fail(SULF_EINVAL, "invalid arguments");
+    if (int rc = ensure64(h)) return rc;
     const LevelGeo& G = h->geo[l];
     LevelVec<double>& V = h->v64[l];
     h->dt = dt;
@@ -1408,6 +1690,7 @@ int sulf_dbg_smooth(sulf_handle h, int l, double dt, const double* Wc, const dou
 
 int sulf_dbg_restrict(sulf_handle h, int l, double* res, double* rhs_coarse) {
     if (!valid(h) || l < 0 || l + 1 >= h->L || !res || !rhs_coarse) return sulf_fail(SULF_EINVAL, "invalid arguments");
+    if (int rc = ensure64(h)) return rc;
     const LevelGeo& G = h->geo[l];
     int rc = copy_in(h, h->v64[l].res, res, sizeof(double2) * G.nn);
     if (rc) return rc;
@@ -1425,6 +1708,7 @@ int sulf_dbg_restrict(sulf_handle h, int l, double* res, double* rhs_coarse) {
 
 int sulf_dbg_prolong(sulf_handle h, int l, const double* xc, double* xf) {
     if (!valid(h) || l < 0 || l + 1 >= h->L || !xc || !xf) return sulf_fail(SULF_EINVAL, "invalid arguments");
+    if (int rc = ensure64(h)) return rc;
     int rc = copy_in(h, h->v64[l + 1].x, xc, sizeof(double2) * h->geo[l + 1].nn);
     if (!rc) rc = copy_in(h, h->v64[l].x, xf, sizeof(double2) * h->geo[l].nn);
     if (rc) return rc;
@@ -1437,6 +1721,7 @@ int sulf_dbg_prolong(sulf_handle h, int l, const double* xc, double* xf) {
 
 int sulf_dbg_inject(sulf_handle h, const double* Wc0, int l, double* Wc_out) {
     if (!dbg_level_ok(h, l) || !Wc0 || !Wc_out) return sulf_fail(SULF_EINVAL, "invalid arguments");
+    if (int rc = ensure64(h)) return rc;
     int rc = copy_in(h, h->v64[0].Wc, Wc0, sizeof(double2) * h->geo[0].nn);
     if (rc) return rc;
     for (int k = 1; k <= l; k++) {
@@ -1450,6 +1735,7 @@ int sulf_dbg_inject(sulf_handle h, const double* Wc0, int l, double* Wc_out) {
 
 int sulf_dbg_coarsest_solve(sulf_handle h, double dt, const double* Wc0, const double* rhs_c, double* x_c) {
     if (!valid(h) || !Wc0 || !rhs_c || !x_c || !(dt > 0)) return sulf_fail(SULF_EINVAL, "invalid arguments");
+    if (int rc = ensure64(h)) return rc;
     h->dt = dt;
     int lc = h->L - 1;
     int rc = copy_in(h, h->W, Wc0, sizeof(double2) * h->geo[0].nn);
@@ -2006,6 +2292,7 @@ int lockstep_run(const std::vector<sulf_domain*>& hs, double dt, int nsteps, int
     C.mem = &mem;
     for (sulf_domain* d : hs) {
         d->dt = dt;
+        if (int rc = ensure64(d)) return rc;
         if (d->solver.precision == 1)
             if (int rc = ensure32(d)) return rc;
         if (int rc = refresh_ghost_ops(d)) return rc;
@@ -2236,6 +2523,7 @@ int sulf_autotune(sulf_handle h, double dt, int use_cache, sulf_tune_result* out
 int sulf_dbg_cycles(sulf_handle h, double dt, const double* Wc0, const double* rhs, double* x, int ncycles,
                     double* rnorms) {
     if (!valid(h) || !Wc0 || !rhs || !x || ncycles < 1 || !(dt > 0)) return sulf_fail(SULF_EINVAL, "invalid arguments");
+    if (int rc = ensure64(h)) return rc;
     const LevelGeo& G0 = h->geo[0];
     h->dt = dt;
     int rc = copy_in(h, h->W, Wc0, sizeof(double2) * G0.nn);
@@ -2251,6 +2539,9 @@ int sulf_dbg_cycles(sulf_handle h, double dt, const double* Wc0, const double* r
     PdlScope pdl(h->solver.pdl != 0, h->solver.relax_occupancy, h->solver.relax_matrix_free);
     int nc = h->dim == 2 ? linear_solve<2>(h, 1.0, ncycles, 0.0, rnorms) : linear_solve<3>(h, 1.0, ncycles, 0.0, rnorms);
     if (nc < 0) return nc;
+    if (h->s_on)
+        h->launches += h->dim == 2 ? launch_s_export<2>(fine_slev<2>(h), h->s64[0].tt, h->v64[0].x, h->stream)
+                                   : launch_s_export<3>(fine_slev<3>(h), h->s64[0].tt, h->v64[0].x, h->stream);
     return dbg_copy_out(h, 0, h->v64[0].x, x, false);
 }
 

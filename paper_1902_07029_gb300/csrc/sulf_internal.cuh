@@ -69,6 +69,7 @@ struct LevelGeo {
     int* gsrc = nullptr;
     int nb = 0;
     int* bidx = nullptr;     // band nodes, box order
+    int* bpos = nullptr;     // node -> band index (nb > 0)
     int* bref = nullptr;     // nb*dim: >=0 band index, -1 none, <=-2 ghost node -(idx+2)
     double* ban = nullptr;   // nb*dim |n_a|
     float* ban32 = nullptr;
@@ -276,7 +277,7 @@ int launch_average_sources(long long nn, const double* f4, double2* src, cudaStr
 // the convergence test at the end of a cycle of the device-side loop
 // (conditional graph node h): cycles counts, rnorms[cycle-1] records the
 // defect norm
-int launch_cycle_check(cudaGraphConditionalHandle h, const unsigned long long* norm, const int* singular,
+int launch_cycle_check(cudaGraphConditionalHandle h, unsigned long long* norm, const int* singular,
                        const double* thr, int max_cycles, int* cycles, double* rnorms, cudaStream_t s);
 
 // mixed precision transfers on the finest level (active nodes)
@@ -323,6 +324,12 @@ __device__ __forceinline__ void pdl_enter() {
     asm volatile("griddepcontrol.wait;" ::: "memory");
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 }
+
+// launch shape of a one-thread-per-node kernel (kernels.cu)
+constexpr int kNodeThreads = 256;
+int sm_count();
+unsigned block_for(long long n);
+unsigned grid_for(long long n);
 
 // launches made by the calling thread use the attribute while on (solver.cu
 // switches it per call from sulf_solver::pdl)
