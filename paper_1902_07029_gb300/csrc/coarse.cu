@@ -1,0 +1,1244 @@
+// The cluster-resident coarse levels (coarse.cuh): kernel and tables.
+#include <algorithm>
+#include <cstring>
+#include <mutex>
+
+#include "coarse.cuh"
+
+namespace sulf {
+
+using stages::fmadd;
+using stages::kGopLanes;
+
+namespace {
+
+constexpr int kRefBits = 12;  // a reference: owner << kRefBits | index in its values
+constexpr unsigned kRefMask = (1u << kRefBits) - 1;
+constexpr unsigned kNoRef = 0xffffu;
+constexpr size_t kCoarseSmem = 224 * 1024;
+// words of the cycle's program: phase | level << 8 | flags; kOpAll: by every
+// CTA (else CTA 0), kOpFar: values of other CTAs are read, kOpWide: a cluster
+// barrier follows (else one of CTA 0)
+enum { kOpNone = 0, kOpRed, kOpBlack, kOpGhosts, kOpDefect, kOpRestrict, kOpSolve, kOpProlong, kOpVisit };
+constexpr unsigned kOpDelta = 1u << 16, kOpLast = 1u << 17, kOpAll = 1u << 18, kOpFar = 1u << 19, kOpWide = 1u << 20;
+constexpr unsigned kOpSkipRed = 1u << 21, kOpDown = 1u << 22;  // of a visit: first red half-sweep done; defect after
+constexpr int kCoarseLog = 2;
+constexpr int kCoarseLanes = 1 << kCoarseLog;                // lanes of a row of more than kShortRow entries
+constexpr int kShortRow = 6, kLongRow = 64;    // and of more than kLongRow: a warp
+
+__device__ __forceinline__ unsigned cta_rank() {
+    unsigned r;
+    asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+    return r;
+}
+__device__ __forceinline__ void cluster_barrier() {
+    asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+    asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+__device__ __forceinline__ unsigned map_rank(unsigned a, unsigned r) {
+    unsigned o;
+    asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(o) : "r"(a), "r"(r));
+    return o;
+}
+__device__ __forceinline__ void ld_remote(unsigned a, float& v) {
+    asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(v) : "r"(a));
+}
+__device__ __forceinline__ void ld_remote(unsigned a, double& v) {
+    asm volatile("ld.shared::cluster.f64 %0, [%1];" : "=d"(v) : "r"(a));
+}
+__device__ __forceinline__ void ld_remote(unsigned a, float2& v) {
+    asm volatile("ld.shared::cluster.v2.f32 {%0, %1}, [%2];" : "=f"(v.x), "=f"(v.y) : "r"(a));
+}
+__device__ __forceinline__ void ld_remote(unsigned a, double2& v) {
+    asm volatile("ld.shared::cluster.v2.f64 {%0, %1}, [%2];" : "=d"(v.x), "=d"(v.y) : "r"(a));
+}
+
+// own shared memory (W false) or the cluster's, by address
+template <bool W>
+__device__ __forceinline__ void ld_at(unsigned a, float& v) {
+    if (W)
+        asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(v) : "r"(a));
+    else
+        asm volatile("ld.shared.f32 %0, [%1];" : "=f"(v) : "r"(a));
+}
+template <bool W>
+__device__ __forceinline__ void ld_at(unsigned a, double& v) {
+    if (W)
+        asm volatile("ld.shared::cluster.f64 %0, [%1];" : "=d"(v) : "r"(a));
+    else
+        asm volatile("ld.shared.f64 %0, [%1];" : "=d"(v) : "r"(a));
+}
+template <bool W>
+__device__ __forceinline__ void ld_at(unsigned a, float2& v) {
+    if (W)
+        asm volatile("ld.shared::cluster.v2.f32 {%0, %1}, [%2];" : "=f"(v.x), "=f"(v.y) : "r"(a));
+    else
+        asm volatile("ld.shared.v2.f32 {%0, %1}, [%2];" : "=f"(v.x), "=f"(v.y) : "r"(a));
+}
+template <bool W>
+__device__ __forceinline__ void ld_at(unsigned a, double2& v) {
+    if (W)
+        asm volatile("ld.shared::cluster.v2.f64 {%0, %1}, [%2];" : "=d"(v.x), "=d"(v.y) : "r"(a));
+    else
+        asm volatile("ld.shared.v2.f64 {%0, %1}, [%2];" : "=d"(v.x), "=d"(v.y) : "r"(a));
+}
+template <bool W>
+__device__ __forceinline__ void phase_barrier() {
+    if (W)
+        cluster_barrier();
+    else
+        __syncthreads();
+}
+
+// copy into shared memory in 16-byte pieces (both ends aligned) by the CTA
+__device__ __forceinline__ void stage(char* dst, const void* src, size_t bytes) {
+    const size_t n16 = (bytes + 15) / 16;
+    for (size_t c = threadIdx.x; c < n16; c += blockDim.x) {
+        const unsigned d = (unsigned)__cvta_generic_to_shared(dst + 16 * c);
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(d), "l"((const char*)src + 16 * c) : "memory");
+    }
+}
+
+template <int D, typename T>
+struct Coarse {
+    typedef typename V2<T>::t T2;
+    char* sm;
+    unsigned sa;  // shared address of sm
+    int tid, nthr;
+
+    template <typename V>
+    __device__ __forceinline__ V* at(int off) const {
+        return reinterpret_cast<V*>(sm + off);
+    }
+    // the values N references name in the array at byte offset off (the same
+    // offset in every CTA); w: an owner may be another CTA (uniform)
+    template <int N, typename V>
+    __device__ __forceinline__ void get(bool w, int off, const unsigned* ref, V* v) const {
+        if (w) {
+#pragma unroll
+            for (int q = 0; q < N; q++)
+                ld_remote(map_rank(sa + off + (ref[q] & kRefMask) * (unsigned)sizeof(V), ref[q] >> kRefBits), v[q]);
+        } else {
+#pragma unroll
+            for (int q = 0; q < N; q++) v[q] = at<const V>(off)[ref[q]];
+        }
+    }
+
+    // entries beg, beg + step, ... < end of a CSR table times the values they
+    // name; `composed`: an entry's upper half selects the array (x, snap, b)
+    template <class R>
+    __device__ __forceinline__ T entries(bool w, int beg, int end, int step, const R* ref, const T* val, int off,
+                                         int off1, int off2) const {
+        T v = 0;
+        for (int j0 = beg; j0 < end; j0 += 4 * step) {
+            unsigned u[4];
+            T c[4], x[4];
+#pragma unroll
+            for (int q = 0; q < 4; q++) {
+                const int j = j0 + q * step < end ? j0 + q * step : j0;
+                u[q] = ref[j];
+                c[q] = val[j];
+            }
+            if (sizeof(R) == 2) {
+                get<4, T>(w, off, u, x);
+            } else {
+#pragma unroll
+                for (int q = 0; q < 4; q++) {
+                    const unsigned kind = u[q] >> 16, r = u[q] & 0xffffu;
+                    get<1, T>(w, kind == 0 ? off : (kind == 1 ? off1 : off2), &r, x + q);
+                }
+            }
+#pragma unroll
+            for (int q = 0; q < 4; q++)
+                if (j0 + q * step < end) v = fmadd(c[q], x[q], v);
+        }
+        return v;
+    }
+
+    // the rows of a table after the `skip` first threads' own work first(t) (a
+    // multiple of 32); done(ghost, sum)
+    template <class R, class First, class Done>
+    __device__ __forceinline__ void rows(bool w, int skip, const CTab& tab, int off, int off1, int off2,
+                                         const First& first, const Done& done) const {
+        const int nx = tab.nx, nl = tab.nl, ns = tab.ns;
+        const int tl = skip + 32 * nx, ts = tl + (nl * kCoarseLanes + 31) / 32 * 32, tot = ts + (ns + 31) / 32 * 32;
+        for (int t = tid; t < tot; t += nthr) {
+            if (t < skip) {
+                first(t);
+                continue;
+            }
+            const int lanes = t >= ts ? 1 : (t >= tl ? kCoarseLanes : 32), lg = t >= ts ? 0 : (t >= tl ? kCoarseLog : 5);
+            const int q = (t - (t >= ts ? ts : (t >= tl ? tl : skip))), i = q >> lg, ln = q & (lanes - 1);
+            const bool on = i < (t >= ts ? ns : (t >= tl ? nl : nx));
+            const int r = i + (t >= ts ? nx + nl : (t >= tl ? nx : 0));
+            T v = 0;
+            if (on) {
+                const int* ptr = at<const int>(tab.ptr);
+                v = entries<R>(w, ptr[r] + ln, ptr[r + 1], lanes, at<const R>(tab.ref), at<const T>(tab.val), off, off1,
+                               off2);
+            }
+            for (int o = lanes >> 1; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+            if (on && ln == 0) done(at<const uint16_t>(tab.idx)[r], v);
+        }
+    }
+
+    // a row's neighbour sum: gt . x over the axis neighbours added to r
+    __device__ __forceinline__ T couple(bool w, const T* coef, int nr, int i, int x, const unsigned* u, T r) const {
+        T xv[2 * D];
+        get<2 * D, T>(w, x, u, xv);
+#pragma unroll
+        for (int q = 0; q < 2 * D; q++) r = fmadd(coef[q * nr + i], xv[q], r);
+        return r;
+    }
+
+    __device__ __forceinline__ void colour(const CLev& L, bool w, int c, bool delta, bool last) const {
+        const T* coef = at<const T>(L.coef);
+        const uint16_t* nbr = at<const uint16_t>(L.nbr);
+        const int nr = L.nr, i1 = c ? nr : L.cr, near = L.cr + L.cbn, xo = L.x, cg = L.cg;
+        const T* b = at<const T>(L.b);
+        T* x = at<T>(xo);
+        T* y = at<T>(L.y);
+        const int d2 = L.d2, nx = L.nx;
+        for (int i = (c ? L.cr : 0) + tid; i < i1; i += nthr) {
+            unsigned u[2 * D];
+#pragma unroll
+            for (int q = 0; q < 2 * D; q++) u[q] = nbr[q * nr + i];
+            T r = b[i];
+            if (delta && (c == 0 || i >= near)) {
+                T2 d[2 * D];
+                get<2 * D, T2>(w, d2, u, d);
+                T sd = d[0].x, sc = d[0].y;
+#pragma unroll
+                for (int q = 1; q < 2 * D; q++) {
+                    sd += d[q].x;
+                    sc += d[q].y;
+                }
+                r = fmadd(-coef[(2 * D + 2) * nr + nx + i], sd, r + sc);
+            }
+            r = couple(w, coef, nr, i, xo, u, r) * coef[(2 * D + 1) * nr + i];
+            x[i] = r;
+            if (last) y[i] = coef[(2 * D + 2) * nr + i] * r;
+        }
+        if (c)
+            for (int g = nthr - 1 - tid; g < cg; g += nthr) at<T>(L.snap)[g] = x[nr + g];
+    }
+
+    __device__ __forceinline__ void ghosts(const CLev& L, bool w, bool last) const {
+        const T* rho = at<const T>(L.coef) + (2 * D + 3) * L.nr;  // of the ghosts
+        T* x = at<T>(L.x) + L.nr;
+        T* y = at<T>(L.y) + L.nr;
+        rows<unsigned>(
+            w, 0, L.g, L.x, L.snap, L.b, [](int) {},
+            [&](int g, T v) {
+                x[g] = v;
+                if (last) y[g] = rho[g] * v;
+            });
+    }
+
+    // defect of the red nodes, of the black ones next to a ghost and of the ghosts
+    __device__ __forceinline__ void defect(const CLev& L, bool w) const {
+        const T* coef = at<const T>(L.coef);
+        const uint16_t* nbr = at<const uint16_t>(L.nbr);
+        const int nr = L.nr, cr = L.cr, cbn = L.cbn, own = nr - cbn, xo = L.x;
+        const T* x = at<const T>(xo);
+        const T* b = at<const T>(L.b);
+        T* R = at<T>(L.y);
+        rows<uint16_t>(
+            w, (own + 31) / 32 * 32, L.r, xo, 0, 0,
+            [&](int t) {
+                if (t >= own) return;
+                const int i = t < cr ? t : cbn + t;
+                unsigned u[2 * D];
+#pragma unroll
+                for (int q = 0; q < 2 * D; q++) u[q] = nbr[q * nr + i];
+                R[i] = couple(w, coef, nr, i, xo, u, fmadd(-coef[2 * D * nr + i], x[i], b[i]));
+            },
+            [&](int g, T v) { R[nr + g] = b[nr + g] - v; });
+    }
+
+    // the defect of level F onto the right-hand side of the next coarser level
+    // C, whose x starts with its red half-sweep from zero
+    __device__ __forceinline__ void restrict_to(const CLev& F, const CLev& C, bool w) const {
+        const int* ptr = at<const int>(C.cptr);
+        const uint16_t* ref = at<const uint16_t>(C.cref);
+        const T* val = at<const T>(C.cval);
+        const int nr = C.nr, cr = C.cr, yo = F.y;
+        const T* di = at<const T>(C.coef) + (2 * D + 1) * nr;
+        T* b = at<T>(C.b);
+        T* x = at<T>(C.x);
+        rows<uint16_t>(
+            w, (nr + 31) / 32 * 32, C.c, yo, 0, 0,
+            [&](int i) {
+                if (i >= nr) return;
+                const T v = entries<uint16_t>(w, ptr[i], ptr[i + 1], 1, ref, val, yo, 0, 0);
+                b[i] = v;
+                x[i] = i < cr ? v * di[i] : (T)0;
+            },
+            [&](int g, T v) {
+                b[nr + g] = v;
+                x[nr + g] = 0;
+            });
+    }
+
+    __device__ __forceinline__ void prolong(const CLev& F, const CLev& C, bool w) const {
+        const uint16_t* pro = at<const uint16_t>(F.pro);
+        const int n = F.cb + F.cg, cr = F.cr, nx = F.nx, xc = C.x, yc = C.y;
+        const T* rho = at<const T>(F.coef) + (2 * D + 2) * F.nr;
+        T* x = at<T>(F.x);
+        T2* d2 = at<T2>(F.d2);
+        for (int t = tid; t < n; t += nthr) {
+            const int i = cr + t;  // black nodes, then ghosts
+            unsigned u[1 << D];
+            T v[1 << D];
+            int cnt = 0;
+            bool has[1 << D];
+#pragma unroll
+            for (int cc = 0; cc < (1 << D); cc++) {
+                u[cc] = pro[cc * n + t];
+                has[cc] = u[cc] != kNoRef;
+                cnt += has[cc];
+                if (!has[cc]) u[cc] = 0;  // read and dropped
+            }
+            T ps = 0, py = 0;
+            get<1 << D, T>(w, xc, u, v);
+#pragma unroll
+            for (int cc = 0; cc < (1 << D); cc++)
+                if (has[cc]) ps += v[cc];
+            get<1 << D, T>(w, yc, u, v);
+#pragma unroll
+            for (int cc = 0; cc < (1 << D); cc++)
+                if (has[cc]) py += v[cc];
+            T2 d;
+            d.x = 0;
+            d.y = 0;
+            if (cnt) {
+                const T r = stages::inv_count<T>(cnt);
+                x[i] = fmadd(ps, r, x[i]);
+                d.x = fmadd(rho[i], ps, -py) * r;
+                d.y = rho[nx + i] * d.x;
+            }
+            d2[i] = d;
+        }
+    }
+
+    // address of a reference in the array at byte offset off
+    template <bool W, typename V>
+    __device__ __forceinline__ unsigned addr(int off, unsigned ref) const {
+        if (!W) return sa + off + ref * (unsigned)sizeof(V);
+        return map_rank(sa + off + (ref & kRefMask) * (unsigned)sizeof(V), ref >> kRefBits);
+    }
+
+    // The sweeps of one visit of a level whose rows fit the threads, and after
+    // the down sweeps the defect: a thread has a red row, a black row or four
+    // lanes share a ghost's row, kept in registers (coefficients and
+    // addresses) over the visit, so a phase is a handful of loads and
+    // multiply-adds between two barriers.  What a warp executes between two
+    // barriers is its latency and what all warps execute the CTA's, so nothing
+    // else is left there and the warps without a row do nothing.  Measured: a
+    // phase of CTA 0 takes 120 cycles at least, one with a cluster barrier and
+    // remote loads 770, of which the barrier's fence is 350.
+    template <bool W>
+    __device__ __forceinline__ void visit(const CLev& L, int nsw, bool skip_red, bool delta, bool last,
+                                          bool dft) const {
+        const int nr = L.nr, cr = L.cr, cg = L.cg;
+        const int tb = (cr + 31) & ~31, tg = tb + ((L.cb + 31) & ~31), nact = tg + ((4 * cg + 31) & ~31);
+        auto barrier = [&] {
+            if (W)
+                cluster_barrier();
+            else
+                asm volatile("bar.sync 1, %0;" ::"r"(nact) : "memory");
+        };
+        const int nbar = 3 * nsw - (skip_red ? 1 : 0) - (dft ? 0 : 1);  // (before the defect: one more)
+        if (tid >= nact) {
+            if (W)
+                for (int q = 0; q < nbar; q++) cluster_barrier();
+            return;
+        }
+        const T* coef = at<const T>(L.coef);
+        const int xo = L.x;
+        T* xs = at<T>(xo);
+        T* y = at<T>(L.y);
+        if (tid < tg) {
+            const bool black = tid >= tb;
+            const int i = black ? cr + tid - tb : tid;
+            const bool on = black ? i < nr : i < cr;
+            const bool near = on && black && i >= cr + L.cbn, own = on && (!black || near);
+            unsigned u[2 * D];
+            T g[2 * D], di = 0, b = 0, dsum = 0, rho = 0;
+            const uint16_t* nbr = at<const uint16_t>(L.nbr);
+            if (on) {
+#pragma unroll
+                for (int q = 0; q < 2 * D; q++) {
+                    u[q] = nbr[q * nr + i];
+                    g[q] = coef[q * nr + i];
+                }
+                di = coef[(2 * D + 1) * nr + i];
+                b = at<const T>(L.b)[i];
+                if (last) rho = coef[(2 * D + 2) * nr + i];
+                if (delta && own) {
+                    // what the neighbours are off their c rows by
+                    T2 d[2 * D];
+#pragma unroll
+                    for (int q = 0; q < 2 * D; q++) ld_at<W>(addr<W, T2>(L.d2, u[q]), d[q]);
+                    T sd = 0, sc = 0;
+#pragma unroll
+                    for (int q = 0; q < 2 * D; q++) {
+                        sd += d[q].x;
+                        sc += d[q].y;
+                    }
+                    dsum = fmadd(-coef[(2 * D + 2) * nr + L.nx + i], sd, sc);
+                }
+#pragma unroll
+                for (int q = 0; q < 2 * D; q++) u[q] = addr<W, T>(xo, u[q]);
+            }
+            // phases: red, black, ghosts, red, ...; one copy of the code
+            int kind = skip_red ? 1 : 0;
+            const int mine = black ? 1 : 0;
+#pragma unroll 1
+            for (int q = 0; q < 3 * nsw - (skip_red ? 1 : 0); q++) {
+                if (on && kind == mine) {
+                    T v[2 * D], r = b + dsum;
+#pragma unroll
+                    for (int e = 0; e < 2 * D; e++) ld_at<W>(u[e], v[e]);
+#pragma unroll
+                    for (int e = 0; e < 2 * D; e++) r = fmadd(g[e], v[e], r);
+                    r *= di;
+                    xs[i] = r;
+                    if (last) y[i] = rho * r;  // the last sweep's stays
+                    dsum = 0;
+                }
+                kind = kind == 2 ? 0 : kind + 1;
+                if (q < nbar) barrier();
+            }
+            if (dft && own) {
+                T v[2 * D];
+#pragma unroll
+                for (int q = 0; q < 2 * D; q++) ld_at<W>(u[q], v[q]);
+                T r = fmadd(-coef[2 * D * nr + i], xs[i], b);
+#pragma unroll
+                for (int q = 0; q < 2 * D; q++) r = fmadd(g[q], v[q], r);
+                y[i] = r;
+            }
+        } else {
+            const int t = tid - tg, gi = t >> 2, ln = t & 3;
+            const bool on = gi < cg;
+            const unsigned* ref = at<const unsigned>(L.g.ref);
+            const T* val = at<const T>(L.g.val);
+            T* snap = at<T>(L.snap);
+            const int so = L.snap, bo = L.b;
+            int beg = 0, end = 0;
+            unsigned a[4];
+            T c[4], rho = 0;
+            auto fetch = [&](int j) {
+#pragma unroll
+                for (int q = 0; q < 4; q++) {
+                    const int k = j + 4 * q;
+                    const unsigned e = ref[k < end ? k : beg], kind = e >> 16;
+                    a[q] = addr<W, T>(kind == 0 ? xo : (kind == 1 ? so : bo), e & 0xffffu);
+                    c[q] = k < end ? val[k] : (T)0;
+                }
+            };
+            if (on) {
+                const int* ptr = at<const int>(L.g.ptr);
+                beg = ptr[gi] + ln;
+                end = ptr[gi + 1];
+                if (beg >= end) beg = end - 1;  // (a lane without an entry reads one and drops it)
+                fetch(ptr[gi] + ln);
+                if (last) rho = coef[(2 * D + 3) * nr + gi];
+            }
+            const bool more = on && beg + 16 < end;
+            int kind = skip_red ? 1 : 0;
+#pragma unroll 1
+            for (int p = 0; p < 3 * nsw - (skip_red ? 1 : 0); p++) {
+                if (kind == 1) {
+                    if (on && ln == 0) snap[gi] = xs[nr + gi];
+                } else if (kind == 2) {
+                    T v = 0;
+                    if (on) {
+                        T w[4];
+#pragma unroll
+                        for (int q = 0; q < 4; q++) ld_at<W>(a[q], w[q]);
+#pragma unroll
+                        for (int q = 0; q < 4; q++) v = fmadd(c[q], w[q], v);
+                        if (more) {
+#pragma unroll 1
+                            for (int j = beg + 16; j < end; j += 16) {
+#pragma unroll
+                                for (int q = 0; q < 4; q++) {
+                                    const int k = j + 4 * q;
+                                    const unsigned e = ref[k < end ? k : beg], kd = e >> 16;
+                                    ld_at<W>(addr<W, T>(kd == 0 ? xo : (kd == 1 ? so : bo), e & 0xffffu), w[q]);
+                                }
+#pragma unroll
+                                for (int q = 0; q < 4; q++) {
+                                    const int k = j + 4 * q;
+                                    v = fmadd(k < end ? val[k] : (T)0, w[q], v);
+                                }
+                            }
+                        }
+                    }
+                    v += __shfl_xor_sync(0xffffffffu, v, 2);
+                    v += __shfl_xor_sync(0xffffffffu, v, 1);
+                    if (on && ln == 0) {
+                        xs[nr + gi] = v;
+                        if (last) y[nr + gi] = rho * v;
+                    }
+                }
+                kind = kind == 2 ? 0 : kind + 1;
+                if (p < nbar) barrier();
+            }
+            if (dft) {
+                T v = 0;
+                if (on) {
+                    const int* ptr = at<const int>(L.r.ptr);
+                    v = entries<uint16_t>(W, ptr[gi] + ln, ptr[gi + 1], 4, at<const uint16_t>(L.r.ref),
+                                          at<const T>(L.r.val), xo, 0, 0);
+                }
+                v += __shfl_xor_sync(0xffffffffu, v, 2);
+                v += __shfl_xor_sync(0xffffffffu, v, 1);
+                if (on && ln == 0) y[nr + gi] = at<const T>(L.b)[nr + gi] - v;
+            }
+        }
+        // (the caller's barrier follows)
+    }
+
+    // coarsest level: x = A^{-1} b, kGopLanes lanes per row
+    __device__ __forceinline__ void solve(const CLev& L, bool w, const CDesc<T>& d, const T* ag) const {
+        const T* A = L.ainv >= 0 ? at<const T>(L.ainv) : ag;
+        const int* cnt = d.cnt_m;
+        const T* rho = at<const T>(L.coef) + (2 * D + 2) * L.nr;
+        const int ln = tid % kGopLanes, nx = L.nx, m = L.m, bo = L.b;
+        for (int base = 0; base < nx; base += nthr / kGopLanes) {
+            const int i = base + tid / kGopLanes;
+            T v = 0;
+            if (i < nx) {
+                const T* a = A + (size_t)i * m;
+                for (unsigned o = 0; o < (w ? (unsigned)d.ncta : 1u); o++) {
+                    const int n = cnt[o];
+                    for (int j0 = ln; j0 < n; j0 += 4 * kGopLanes) {
+                        unsigned u[4];
+                        T x[4];
+#pragma unroll
+                        for (int q = 0; q < 4; q++)
+                            u[q] = o << kRefBits | (unsigned)(j0 + q * kGopLanes < n ? j0 + q * kGopLanes : j0);
+                        get<4, T>(w, bo, u, x);
+#pragma unroll
+                        for (int q = 0; q < 4; q++)
+                            if (j0 + q * kGopLanes < n) v = fmadd(a[j0 + q * kGopLanes], x[q], v);
+                    }
+                    a += n;
+                }
+            }
+            v = stages::gop_reduce<T>(v);
+            if (i < nx && ln == 0) {
+                at<T>(L.x)[i] = v;
+                at<T>(L.y)[i] = rho[i] * v;
+            }
+        }
+    }
+};
+
+// The phases of a cycle run as a program of (phase, level, flags, barrier)
+// words: each phase's code exists once and stays in the instruction cache
+// (inlined per call site and per kind of level the kernel had 144 KB of code
+// and its phases took two to three times as long).
+template <int D, typename T>
+__global__ void __launch_bounds__(kCoarseThreads, 1) k_s_coarse(const CDesc<T>* __restrict__ dp) {
+    extern __shared__ __align__(16) char coarse_smem[];
+    const CDesc<T>& d = *dp;
+    Coarse<D, T> k;
+    k.sm = coarse_smem;
+    k.sa = (unsigned)__cvta_generic_to_shared(coarse_smem);
+    k.tid = threadIdx.x;
+    k.nthr = blockDim.x;
+    const int me = (int)cta_rank(), n = d.nlev, nop = d.nop;
+    // fixed during the linear solve: copied while the previous kernel runs
+    stage(k.sm, d.head + (size_t)me * d.head_len, d.head_len);
+    stage(k.sm + d.tab_at, d.tab + d.tab_off[me], d.tab_len[me]);
+    stage(k.sm + d.coef_at, d.coef + d.coef_off[me], sizeof(T) * (size_t)d.coef_len[me]);
+    if (d.ainv_len[me]) stage(k.sm + d.ainv_at, d.ainv + d.ainv_off[me], sizeof(T) * (size_t)d.ainv_len[me]);
+    asm volatile("cp.async.commit_group;" ::: "memory");
+    const T* bg = d.b + d.b_off[me];
+    const int* slot = d.slot + d.b_off[me];
+    const T* ag = d.ainv + d.ainv_off[me];
+    T* X = d.X;
+    double* acc = d.acc;
+    asm volatile("cp.async.wait_group 0;" ::: "memory");
+    __syncthreads();
+    const CLev* lev = reinterpret_cast<const CLev*>(k.sm);
+    const unsigned* prog = reinterpret_cast<const unsigned*>(k.sm + n * sizeof(CLev));
+    // the red nodes stay on their c rows
+    for (int l = 0; l + 1 < n; l++)
+        for (int i = threadIdx.x; i < 2 * lev[l].cr; i += blockDim.x) k.template at<T>(lev[l].d2)[i] = 0;
+    const int nx = lev[0].nx;
+    pdl_enter();
+    {
+        // the first level's right-hand side, and its red half-sweep from zero
+        const CLev& L = lev[0];
+        const T* di = k.template at<const T>(L.coef) + (2 * D + 1) * L.nr;
+        const int cr = L.cr;
+        for (int i = threadIdx.x; i < nx; i += blockDim.x) {
+            const T v = __ldcg(bg + i);
+            k.template at<T>(L.b)[i] = v;
+            k.template at<T>(L.x)[i] = i < cr ? v * di[i] : (T)0;
+        }
+    }
+    for (int pc = 0; pc < nop; pc++) {
+        const unsigned o = prog[pc];
+        const CLev& L = lev[(o >> 8) & 0xff];
+        if ((o & kOpAll) || me == 0) {
+            const bool w = o & kOpFar, delta = o & kOpDelta, last = o & kOpLast;
+            switch (o & 0xff) {
+                case kOpRed:
+                case kOpBlack: k.colour(L, w, (o & 0xff) == kOpBlack, delta, last); break;
+                case kOpGhosts: k.ghosts(L, w, last); break;
+                case kOpDefect: k.defect(L, w); break;
+                case kOpRestrict: k.restrict_to(*(&L - 1), L, w); break;
+                case kOpSolve: k.solve(L, w, d, ag); break;
+                case kOpProlong: k.prolong(L, *(&L + 1), w); break;
+                case kOpVisit:
+                    if (w)
+                        k.template visit<true>(L, o >> 24, o & kOpSkipRed, delta, last, o & kOpDown);
+                    else
+                        k.template visit<false>(L, o >> 24, o & kOpSkipRed, delta, last, o & kOpDown);
+                    break;
+                default: break;
+            }
+        }
+        if (o & kOpWide)
+            cluster_barrier();
+        else if (me == 0)
+            __syncthreads();
+    }
+    {
+        const T* x = k.template at<const T>(lev[0].x);
+        for (int i = threadIdx.x; i < nx; i += blockDim.x) {
+            if (acc)
+                acc[slot[i]] += (double)x[i];
+            else
+                X[slot[i]] = x[i];
+        }
+    }
+    cluster_barrier();  // no CTA leaves while another may still read its shared memory
+}
+
+// ---------------------------------------------------------------------------
+// tables (host)
+
+// the kernel's limits raised once per device (a per-launch value would race
+// with other threads' launches)
+template <int D, typename T>
+void raise_limits() {
+    static std::mutex mu;
+    static bool raised[64] = {};
+    int dev = 0;
+    cudaGetDevice(&dev);
+    std::lock_guard<std::mutex> lock(mu);
+    if (dev >= 0 && dev < 64 && raised[dev]) return;
+    cudaFuncSetAttribute(k_s_coarse<D, T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kCoarseSmem);
+    cudaFuncSetAttribute(k_s_coarse<D, T>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+    if (dev >= 0 && dev < 64) raised[dev] = true;
+}
+
+// whether the device can hold a cluster of C such CTAs
+template <int D, typename T>
+bool cluster_fits(int C, size_t smem) {
+    raise_limits<D, T>();
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(C);
+    cfg.blockDim = dim3(kCoarseThreads);
+    cfg.dynamicSmemBytes = smem;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = C;
+    at[0].val.clusterDim.y = 1;
+    at[0].val.clusterDim.z = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    int n = 0;
+    if (cudaOccupancyMaxActiveClusters(&n, k_s_coarse<D, T>, &cfg) != cudaSuccess) {
+        cudaGetLastError();
+        return false;
+    }
+    return n > 0;
+}
+
+inline size_t up16(size_t n) { return (n + 15) & ~size_t(15); }
+
+template <typename T>
+struct Download {
+    std::vector<T> v;
+    void get(const T* dev, size_t n, cudaStream_t s, bool& ok) {
+        v.resize(n + 1);
+        if (n && cudaMemcpyAsync(v.data(), dev, sizeof(T) * n, cudaMemcpyDeviceToHost, s) != cudaSuccess) ok = false;
+    }
+};
+
+// a level's device data on the host
+struct HostLevel {
+    Download<int> hl, gslot, gptr, gcode, rptr, rslot, cptr, cslot;
+    Download<double> gval, rval, cval;
+    Download<int8_t> type;
+    std::vector<uint16_t> ref;                  // slot -> reference
+    std::vector<std::vector<int>> own;          // per CTA: list positions, red, black away, black near, ghosts
+    std::vector<int> cr, cbn, cb, cg;
+    int wide = 1;
+};
+
+}  // namespace
+
+template <int D, typename T>
+int build_coarse(CoarseSet<T>& S, const LevelGeo* G, const SGeo* SG, const SVec<T>* V, int L, int want, int nu1,
+                 int nu2, double* acc, DevMem& mem, cudaStream_t s, std::string& err) {
+    S.l0 = -1;
+    S.want = want;
+    S.nu1 = nu1;
+    S.nu2 = nu2;
+    S.rows = true;
+    if (want < 0 || want > L - 1) return SULF_OK;
+    const bool f32 = std::is_same<T, float>::value;
+    // levels of up to this many nodes run on CTA 0: FP32 phases are short
+    // there; an SM's two FP64 lanes make it slow sooner
+    const int narrow = f32 ? 1200 : 600;
+    constexpr size_t kNodeBytes = sizeof(T) * (2 * D + 9);
+    // the first level that fits, with the smallest cluster
+    int l0 = want, ncta = 0;
+    for (; l0 < L; l0++) {
+        size_t nodes = 0;
+        for (int l = l0; l < L; l++) nodes += (size_t)G[l].nin[0] + G[l].nin[1] + G[l].ng;
+        if (nodes > 40000) continue;
+        break;
+    }
+    if (l0 >= L) return SULF_OK;
+    std::vector<HostLevel> H(L);
+    bool ok = true;
+    for (int l = l0; l < L; l++) {
+        HostLevel& h = H[l];
+        const SGeo& g = SG[l];
+        const size_t nin = (size_t)g.n0 + g.n1, ng = G[l].ng;
+        h.hl.get(g.hl, nin, s, ok);
+        h.gslot.get(g.gslot, ng, s, ok);
+        h.type.get(G[l].type, (size_t)G[l].nn, s, ok);
+        if (ng) {
+            h.gptr.get(G[l].gop_ptr, ng + 1, s, ok);
+            h.gcode.get(g.gcode, (size_t)G[l].gop_nnz, s, ok);
+            h.gval.get(G[l].gop_val, (size_t)G[l].gop_nnz, s, ok);
+            h.rptr.get(g.rptr, ng + 1, s, ok);
+            if (l > 0) h.cptr.get(g.cptr, ng + 1, s, ok);
+        }
+    }
+    if (!ok || cudaStreamSynchronize(s) != cudaSuccess) {
+        err = "coarse-level tables failed";
+        return SULF_EDEVICE;
+    }
+    for (int l = l0; l < L; l++) {
+        HostLevel& h = H[l];
+        if (!G[l].ng) continue;
+        h.rslot.get(SG[l].rslot, (size_t)h.rptr.v[G[l].ng], s, ok);
+        h.rval.get(SG[l].rval, (size_t)h.rptr.v[G[l].ng], s, ok);
+        if (l > l0) {
+            h.cslot.get(SG[l].cslot, (size_t)h.cptr.v[G[l].ng], s, ok);
+            h.cval.get(SG[l].cval, (size_t)h.cptr.v[G[l].ng], s, ok);
+        }
+    }
+    if (!ok || cudaStreamSynchronize(s) != cudaSuccess) {
+        err = "coarse-level tables failed";
+        return SULF_EDEVICE;
+    }
+    std::vector<char> tab;
+    std::vector<CLev> lev;
+    std::vector<unsigned> prog;
+    CDesc<T> d;
+    std::vector<int> slots;
+    size_t smem = 0, coef_tot = 0;
+    bool fit = false;
+    for (; l0 < L && !fit; l0++) {
+        for (int C : {8, 16}) {
+            const int n = L - l0;
+            ncta = C;
+            // deal the nodes: bands of the box order (slots are box order up to
+            // the colour: half indices compare as box rows do)
+            bool refs_ok = true;
+            for (int l = l0; l < L && refs_ok; l++) {
+                HostLevel& h = H[l];
+                const SGeo& g = SG[l];
+                const int nin = g.n0 + g.n1, ng = G[l].ng, tot = nin + ng;
+                h.wide = tot > narrow || (l == L - 1 && !f32 && tot > 40);
+                const int w = h.wide ? C : 1;
+                auto half = [&](int t) {
+                    if (t < nin) return h.hl.v[t] >> kEntHalf;
+                    const int sl = h.gslot.v[t - nin];
+                    return sl >= g.Hn ? sl - g.Hn : sl;
+                };
+                // counting sort by half index
+                std::vector<int> cnt(g.Hn + 1, 0), ord(tot);
+                for (int t = 0; t < tot; t++) cnt[half(t) + 1]++;
+                for (int q = 0; q < g.Hn; q++) cnt[q + 1] += cnt[q];
+                for (int t = 0; t < tot; t++) ord[cnt[half(t)]++] = t;
+                h.own.assign(C, {});
+                h.cr.assign(C, 0);
+                h.cbn.assign(C, 0);
+                h.cb.assign(C, 0);
+                h.cg.assign(C, 0);
+                h.ref.assign(2 * (size_t)g.Hn, (uint16_t)kNoRef);
+                for (int r = 0; r < w; r++) {
+                    const int a = (int)((long long)tot * r / w), b = (int)((long long)tot * (r + 1) / w);
+                    std::vector<int> part[4];
+                    for (int q = a; q < b; q++) {
+                        const int t = ord[q];
+                        part[t >= nin ? 3 : (t < g.n0 ? 0 : (t < nin - g.nga ? 1 : 2))].push_back(t);
+                    }
+                    h.cr[r] = (int)part[0].size();
+                    h.cbn[r] = (int)part[1].size();
+                    h.cb[r] = (int)(part[1].size() + part[2].size());
+                    h.cg[r] = (int)part[3].size();
+                    std::vector<int>& o = h.own[r];
+                    for (auto& p : part) o.insert(o.end(), p.begin(), p.end());
+                    if (o.size() > kRefMask) refs_ok = false;
+                    for (size_t i = 0; i < o.size(); i++) {
+                        const int t = o[i];
+                        const int sl = t >= nin ? h.gslot.v[t - nin] : (t >= g.n0 ? g.Hn : 0) + (h.hl.v[t] >> kEntHalf);
+                        h.ref[sl] = (uint16_t)(r << kRefBits | (int)i);
+                    }
+                }
+            }
+            if (!refs_ok) continue;
+            // uniform offsets of the values
+            std::vector<CLev> base(n);
+            // levels whose rows fit the threads are swept a visit at a time
+            auto fits = [&](int l) {
+                const HostLevel& h = H[l0 + l];
+                for (int r = 0; r < C; r++)
+                    if (((h.cr[r] + 31) & ~31) + ((h.cb[r] + 31) & ~31) + ((4 * h.cg[r] + 31) & ~31) > kCoarseThreads)
+                        return false;
+                for (int q = 0; q < G[l0 + l].ng; q++)
+                    if (h.gptr.v[q + 1] - h.gptr.v[q] > kLongRow || h.gptr.v[q + 1] == h.gptr.v[q]) return false;
+                return nu1 < 256 && nu2 < 256;
+            };
+            // the program
+            prog.clear();
+            {
+                auto wide = [&](int l) { return H[l0 + l].wide != 0; };
+                // a phase that reads level a and writes level b
+                auto op = [&](unsigned code, int lv, int a, int b, unsigned fl, bool sync) {
+                    const bool far = wide(a) || wide(b);
+                    prog.push_back(code | (unsigned)lv << 8 | fl | (wide(b) ? kOpAll : 0u) | (far ? kOpFar : 0u) |
+                                   (sync ? kOpWide : 0u));
+                };
+                auto sweep = [&](int l, bool red, unsigned fl, bool after) {
+                    if (red) op(kOpRed, l, l, l, fl, wide(l));
+                    op(kOpBlack, l, l, l, fl, wide(l));
+                    op(kOpGhosts, l, l, l, fl, wide(l) || after);
+                };
+                op(kOpNone, 0, 0, 0, 0, wide(0));
+                for (int l = 0; l + 1 < n; l++) {
+                    const bool both = wide(l) || wide(l + 1);
+                    if (fits(l)) {
+                        op(kOpVisit, l, l, l, (unsigned)nu1 << 24 | kOpSkipRed | kOpDown, both);
+                    } else {
+                        for (int q = 0; q < nu1; q++) sweep(l, q > 0, 0, false);
+                        op(kOpDefect, l, l, l, 0, both);
+                    }
+                    op(kOpRestrict, l + 1, l, l + 1, 0, both);
+                }
+                op(kOpSolve, n - 1, n - 1, n - 1, 0, wide(n - 1) || (n > 1 && wide(n - 2)));
+                for (int l = n - 2; l >= 0; l--) {
+                    op(kOpProlong, l, l + 1, l, 0, wide(l) || wide(l + 1));
+                    if (fits(l))
+                        op(kOpVisit, l, l, l, (unsigned)nu2 << 24 | kOpDelta | (l > 0 ? kOpLast : 0u),
+                           wide(l) || (l > 0 && wide(l - 1)));
+                    else
+                    for (int q = 0; q < nu2; q++)
+                        sweep(l, true, (q == 0 ? kOpDelta : 0u) | (q == nu2 - 1 && l > 0 ? kOpLast : 0u),
+                              q == nu2 - 1 && l > 0 && wide(l - 1));
+                }
+            }
+            d.nop = (int)prog.size();
+            d.head_len = (int)up16(n * sizeof(CLev) + 4 * prog.size());
+            size_t off = d.head_len;
+            for (int l = l0; l < L; l++) {
+                const HostLevel& h = H[l];
+                CLev& c = base[l - l0];
+                memset(&c, 0, sizeof c);
+                size_t nx = 0, ng = 0;
+                for (int r = 0; r < C; r++) {
+                    nx = std::max(nx, h.own[r].size());
+                    ng = std::max(ng, (size_t)h.cg[r]);
+                }
+                c.wide = h.wide;
+                auto take = [&](int& o, size_t bytes) {
+                    o = (int)off;
+                    off += up16(bytes);
+                };
+                take(c.x, sizeof(T) * nx);
+                take(c.y, sizeof(T) * nx);
+                take(c.b, sizeof(T) * nx);
+                take(c.d2, 2 * sizeof(T) * nx);
+                take(c.snap, sizeof(T) * ng);
+            }
+            d.coef_at = (int)off;
+            // coefficients: own offsets, the tables after the largest of them
+            lev.assign((size_t)C * n, CLev{});
+            size_t coef_max = 0;
+            coef_tot = 0;
+            for (int r = 0; r < C; r++) {
+                size_t e = 0;
+                d.coef_off[r] = (int)coef_tot;
+                for (int l = l0; l < L; l++) {
+                    CLev& c = lev[(size_t)r * n + l - l0];
+                    const HostLevel& h = H[l];
+                    c = base[l - l0];
+                    c.cr = h.cr[r];
+                    c.cbn = h.cbn[r];
+                    c.cb = h.cb[r];
+                    c.cg = h.cg[r];
+                    c.nr = c.cr + c.cb;
+                    c.nx = c.nr + c.cg;
+                    c.coef = d.coef_at + (int)(sizeof(T) * e);
+                    e += up16(sizeof(T) * ((size_t)(2 * D + 2) * c.nr + 2 * (size_t)c.nx)) / sizeof(T);
+                }
+                d.coef_len[r] = (int)e;
+                coef_tot += e;
+                coef_max = std::max(coef_max, e);
+            }
+            d.tab_at = d.coef_at + (int)up16(sizeof(T) * coef_max);
+            tab.clear();
+            size_t tab_max = 0;
+            for (int r = 0; r < C; r++) {
+                const size_t t0 = tab.size();
+                d.tab_off[r] = (int)t0;
+                auto put = [&](const void* p, size_t bytes) {
+                    const size_t o = tab.size();
+                    tab.resize(o + up16(bytes));
+                    if (bytes) memcpy(tab.data() + o, p, bytes);
+                    return d.tab_at + (int)(o - t0);
+                };
+                // rows given in ghost order, stored longest first
+                auto put_tab = [&](CTab& tb, const std::vector<int>& rp, const auto& ref, const std::vector<T>& val,
+                                   bool sorted) {
+                    const int cnt = (int)rp.size() - 1;
+                    std::vector<uint16_t> idx(cnt);
+                    for (int i = 0; i < cnt; i++) idx[i] = (uint16_t)i;
+                    auto len = [&](int i) { return rp[i + 1] - rp[i]; };
+                    if (sorted) std::stable_sort(idx.begin(), idx.end(), [&](int a, int b) { return len(a) > len(b); });
+                    std::vector<int> p(1, 0);
+                    auto rf = ref;
+                    std::vector<T> vl;
+                    rf.clear();
+                    tb.nx = tb.nl = tb.ns = 0;
+                    for (int i : idx) {
+                        rf.insert(rf.end(), ref.begin() + rp[i], ref.begin() + rp[i + 1]);
+                        vl.insert(vl.end(), val.begin() + rp[i], val.begin() + rp[i + 1]);
+                        p.push_back((int)rf.size());
+                        (len(i) > kLongRow ? tb.nx : (len(i) > kShortRow ? tb.nl : tb.ns))++;
+                    }
+                    tb.ptr = put(p.data(), 4 * p.size());
+                    tb.ref = put(rf.data(), sizeof(rf[0]) * rf.size());
+                    tb.val = put(vl.data(), sizeof(T) * vl.size());
+                    tb.idx = put(idx.data(), 2 * idx.size());
+                };
+                for (int l = l0; l < L; l++) {
+                    CLev& c = lev[(size_t)r * n + l - l0];
+                    const HostLevel& h = H[l];
+                    const SGeo& g = SG[l];
+                    const int nin = g.n0 + g.n1, nn = G[l].n;
+                    std::vector<uint16_t> u;
+                    std::vector<int> ptr;
+                    std::vector<T> val;
+                    // neighbours
+                    u.assign((size_t)2 * D * c.nr + 1, 0);
+                    for (int i = 0; i < c.nr; i++) {
+                        const int t = h.own[r][i], e = h.hl.v[t], a = e & 1;
+                        const int so = (t >= g.n0 ? 0 : g.Hn) + (e >> kEntHalf);
+                        const int o[6] = {a, a - 1, g.H, -g.H, g.P, -g.P};
+                        for (int q = 0; q < 2 * D; q++) u[(size_t)q * c.nr + i] = h.ref[so + o[q]];
+                    }
+                    c.nbr = put(u.data(), 2 * (size_t)2 * D * c.nr);
+                    // composed ghost rows and rows of the defect
+                    std::vector<unsigned> gr;
+                    std::vector<uint16_t> rr;
+                    std::vector<T> rv;
+                    std::vector<int> rp;
+                    ptr.assign(1, 0);
+                    rp.assign(1, 0);
+                    for (int q = 0; q < c.cg; q++) {
+                        const int gi = h.own[r][c.nr + q] - nin;
+                        for (int j = h.gptr.v[gi]; j < h.gptr.v[gi + 1]; j++) {
+                            const int code = h.gcode.v[j];
+                            unsigned kind = 0, ref;
+                            if (code >= 0) {
+                                ref = h.ref[code];
+                            } else {
+                                const unsigned w = ~(unsigned)code;
+                                ref = h.ref[h.gslot.v[w >> 1]];
+                                kind = (w & 1u) ? 2 : 1;
+                                if (kind == 1) {  // snap holds the ghosts only
+                                    const int o = (int)(ref >> kRefBits);
+                                    ref -= (unsigned)(h.cr[o] + h.cb[o]);
+                                }
+                            }
+                            gr.push_back(kind << 16 | ref);
+                            val.push_back((T)h.gval.v[j]);
+                        }
+                        ptr.push_back((int)gr.size());
+                        for (int j = h.rptr.v[gi]; j < h.rptr.v[gi + 1]; j++) {
+                            rr.push_back(h.ref[h.rslot.v[j]]);
+                            rv.push_back((T)h.rval.v[j]);
+                        }
+                        rp.push_back((int)rr.size());
+                    }
+                    put_tab(c.g, ptr, gr, val, !fits(l - l0));
+                    put_tab(c.r, rp, rr, rv, !fits(l - l0));
+                    // coarse corners of the black nodes and the ghosts
+                    auto coords = [&](int t, int* ii) {
+                        int sl = t >= nin ? h.gslot.v[t - nin] : (t >= g.n0 ? g.Hn : 0) + (h.hl.v[t] >> kEntHalf);
+                        const int col = sl >= g.Hn;
+                        if (col) sl -= g.Hn;
+                        const int row = sl / g.H;
+                        ii[1] = D == 3 ? row % nn : row;
+                        ii[2] = D == 3 ? row / nn : 0;
+                        ii[0] = 2 * (sl % g.H) + ((col + ii[1] + ii[2]) & 1);
+                    };
+                    auto slot_of = [](const SGeo& q, int n_, int i, int j, int k) {
+                        return ((i + j + k) & 1) * q.Hn + (i >> 1) + q.H * (j + n_ * k);
+                    };
+                    if (l + 1 < L) {
+                        const HostLevel& hc = H[l + 1];
+                        const SGeo& gc = SG[l + 1];
+                        const int np = c.cb + c.cg;
+                        u.assign(((size_t)np << D) + 1, (uint16_t)kNoRef);
+                        for (int q = 0; q < np; q++) {
+                            int ii[3];
+                            coords(h.own[r][c.cr + q], ii);
+                            for (int cc = 0; cc < (1 << D); cc++) {
+                                int v[3] = {0, 0, 0};
+                                bool dup = false;
+                                for (int a = 0; a < D; a++) {
+                                    const int upper = (cc >> a) & 1;
+                                    dup = dup || (upper && !(ii[a] & 1));
+                                    v[a] = (ii[a] >> 1) + (upper && (ii[a] & 1) ? 1 : 0);
+                                }
+                                if (!dup) u[(size_t)cc * np + q] = hc.ref[slot_of(gc, G[l + 1].n, v[0], v[1], v[2])];
+                            }
+                        }
+                        c.pro = put(u.data(), 2 * ((size_t)np << D));
+                    }
+                    // rows of the restriction onto this level
+                    if (l > l0) {
+                        const HostLevel& hf = H[l - 1];
+                        const SGeo& gf = SG[l - 1];
+                        const int fn = G[l - 1].n, st[3] = {1, fn, fn * fn};
+                        const int8_t* ft = hf.type.v.data();
+                        ptr.assign(1, 0);
+                        rr.clear();
+                        rv.clear();
+                        for (int i = 0; i < c.nr; i++) {
+                            int ci[3];
+                            coords(h.own[r][i], ci);
+                            const int f[3] = {2 * ci[0], 2 * ci[1], 2 * ci[2]};
+                            int p = 0, w[3][3] = {{0, 1, 0}, {0, 1, 0}, {0, 1, 0}};
+                            for (int a = 0; a < D; a++) p += f[a] * st[a];
+                            for (int a = 0; a < D; a++) {
+                                const bool vl = ft[p - st[a]] == T_IN, vr = ft[p + st[a]] == T_IN;
+                                w[a][0] = vl ? (vr ? 1 : 2) : 0;
+                                w[a][1] = vl || vr ? 2 : 4;
+                                w[a][2] = vr ? (vl ? 1 : 2) : 0;
+                            }
+                            int wc = 0;
+                            auto add = [&](int a0, int a1, int a2, int iw) {
+                                // black nodes away from the ghosts have no defect
+                                const uint16_t ref = hf.ref[slot_of(gf, fn, a0, a1, a2)];
+                                const int o = ref >> kRefBits, x = ref & (int)kRefMask;
+                                if (x >= hf.cr[o] && x < hf.cr[o] + hf.cbn[o]) return;
+                                rr.push_back(ref);
+                                rv.push_back((T)iw / (T)(D == 2 ? 16 : 64));
+                            };
+                            for (int kk = 0; kk < (D == 2 ? 9 : 27); kk++) {
+                                const int k0 = kk % 3 - 1, k1 = (kk / 3) % 3 - 1, k2 = D == 3 ? kk / 9 - 1 : 0;
+                                const int iw = w[0][k0 + 1] * w[1][k1 + 1] * (D == 3 ? w[2][k2 + 1] : 1);
+                                if (!iw) continue;
+                                const int q = p + k0 + k1 * st[1] + k2 * st[2];
+                                if ((!k0 && !k1 && !k2) || ft[q] != T_IN)
+                                    wc += iw;
+                                else
+                                    add(f[0] + k0, f[1] + k1, f[2] + k2, iw);
+                            }
+                            add(f[0], f[1], f[2], wc);
+                            ptr.push_back((int)rr.size());
+                        }
+                        c.cptr = put(ptr.data(), 4 * ptr.size());
+                        c.cref = put(rr.data(), 2 * rr.size());
+                        c.cval = put(rv.data(), sizeof(T) * rv.size());
+                        ptr.assign(1, 0);
+                        rr.clear();
+                        rv.clear();
+                        for (int q = 0; q < c.cg; q++) {
+                            const int gi = h.own[r][c.nr + q] - nin;
+                            for (int j = h.cptr.v[gi]; j < h.cptr.v[gi + 1]; j++) {
+                                rr.push_back(hf.ref[h.cslot.v[j]]);
+                                rv.push_back((T)h.cval.v[j]);
+                            }
+                            ptr.push_back((int)rr.size());
+                        }
+                        put_tab(c.c, ptr, rr, rv, true);
+                    }
+                }
+                d.tab_len[r] = (int)(tab.size() - t0);
+                tab_max = std::max(tab_max, tab.size() - t0);
+            }
+            // the coarsest inverse: own rows in shared memory where they fit
+            d.ainv_at = d.tab_at + (int)up16(tab_max);
+            const HostLevel& hc = H[L - 1];
+            const int m = SG[L - 1].n0 + SG[L - 1].n1 + G[L - 1].ng;
+            size_t rows_max = 0;
+            int row0 = 0;
+            for (int r = 0; r < C; r++) {
+                CLev& c = lev[(size_t)r * n + n - 1];
+                c.m = m;
+                c.row0 = row0;
+                d.ainv_off[r] = row0 * m;
+                d.ainv_len[r] = c.nx * m;
+                row0 += c.nx;
+                rows_max = std::max(rows_max, (size_t)c.nx * m);
+            }
+            (void)hc;
+            // a copied piece starts on 16 bytes: rows of odd length may not
+            bool stage_inv = d.ainv_at + up16(sizeof(T) * rows_max) <= kCoarseSmem;
+            for (int r = 0; r < C; r++)
+                if ((sizeof(T) * (size_t)d.ainv_off[r]) % 16) stage_inv = false;
+            for (int r = 0; r < C; r++) {
+                lev[(size_t)r * n + n - 1].ainv = stage_inv ? d.ainv_at : -1;
+                if (!stage_inv) d.ainv_len[r] = 0;
+            }
+            smem = d.ainv_at + (stage_inv ? up16(sizeof(T) * rows_max) : 0);
+            if (smem <= kCoarseSmem && cluster_fits<D, T>(C, smem)) {
+                fit = true;
+                break;
+            }
+        }
+        if (fit) break;
+    }
+    (void)kNodeBytes;
+    if (!fit) return SULF_OK;
+    const int n = L - l0, C = ncta;
+    // device copies
+    auto oom = [&] {
+        err = "out of device memory";
+        return SULF_ENOMEM;
+    };
+    auto grow = [&](auto*& p, size_t& cap, size_t bytes) {
+        if (bytes <= cap && p) return true;
+        p = (std::remove_reference_t<decltype(p)>)mem.get(bytes + 64);
+        cap = bytes;
+        return p != nullptr;
+    };
+    if (!grow(S.tab, S.tab_cap, tab.size()) || !grow(S.coef, S.coef_cap, sizeof(T) * coef_tot)) return oom();
+    const int nb = SG[l0].n0 + SG[l0].n1 + G[l0].ng, nc = SG[L - 1].n0 + SG[L - 1].n1 + G[L - 1].ng;
+    if (!grow(S.b, S.b_cap, sizeof(T) * nb)) return oom();
+    std::vector<int> bpos(nb), cpos(nc), cntm(C);
+    slots.resize(nb);
+    {
+        int at = 0;
+        for (int r = 0; r < C; r++) {
+            d.b_off[r] = at;
+            for (int t : H[l0].own[r]) {
+                const SGeo& g = SG[l0];
+                const int nin = g.n0 + g.n1;
+                bpos[t] = at;
+                slots[at++] =
+                    t >= nin ? H[l0].gslot.v[t - nin] : (t >= g.n0 ? g.Hn : 0) + (H[l0].hl.v[t] >> kEntHalf);
+            }
+        }
+        at = 0;
+        for (int r = 0; r < C; r++) {
+            cntm[r] = (int)H[L - 1].own[r].size();
+            for (int t : H[L - 1].own[r]) cpos[t] = at++;
+        }
+    }
+    for (int r = C; r < kCoarseMaxCta; r++)
+        d.tab_off[r] = d.tab_len[r] = d.coef_off[r] = d.coef_len[r] = d.ainv_off[r] = d.ainv_len[r] = d.b_off[r] = 0;
+    std::vector<std::vector<CPerm>> perm(L);
+    for (int l = l0; l < L; l++) {
+        const SGeo& g = SG[l];
+        perm[l].resize((size_t)g.n0 + g.n1 + G[l].ng);
+        for (int r = 0; r < C; r++) {
+            const CLev& c = lev[(size_t)r * n + l - l0];
+            const int base = d.coef_off[r] + (int)((c.coef - d.coef_at) / (int)sizeof(T));
+            for (int i = 0; i < c.nx; i++)
+                perm[l][H[l].own[r][i]] = CPerm{base + i, c.nr, base + (2 * D + 2) * c.nr + i, c.nx};
+        }
+    }
+    // (the first level and its lists may change with the threshold: new
+    // arrays, the old ones stay with the handle)
+    auto upload = [&](auto*& dst, const auto& v) {
+        dst = (std::remove_reference_t<decltype(dst)>)mem.get(sizeof(v[0]) * v.size() + 64);
+        return dst && cudaMemcpyAsync(dst, v.data(), sizeof(v[0]) * v.size(), cudaMemcpyHostToDevice, s) == cudaSuccess;
+    };
+    for (int l = 0; l < SULF_MAXLEV; l++) S.perm[l] = nullptr;
+    for (int l = l0; l < L; l++)
+        if (!upload(S.perm[l], perm[l])) return oom();
+    std::vector<char> head((size_t)C * d.head_len, 0);
+    for (int r = 0; r < C; r++) {
+        memcpy(head.data() + (size_t)r * d.head_len, &lev[(size_t)r * n], n * sizeof(CLev));
+        memcpy(head.data() + (size_t)r * d.head_len + n * sizeof(CLev), prog.data(), 4 * prog.size());
+    }
+    if (!upload(S.bpos, bpos) || !upload(S.cpos, cpos) || !upload(S.slot, slots) || !upload(S.head, head) ||
+        !upload(S.cnt_m, cntm))
+        return oom();
+    d.head = S.head;
+    d.tab = S.tab;
+    d.coef = S.coef;
+    d.ainv = V[L - 1].Ainv;
+    d.b = S.b;
+    d.slot = S.slot;
+    d.X = V[l0].X;
+    d.acc = l0 == 0 ? acc : nullptr;
+    d.cnt_m = S.cnt_m;
+    d.nlev = n;
+    d.ncta = C;
+    std::vector<CDesc<T>> dd(1, d);
+    if (!upload(S.dev, dd)) return oom();
+    if (cudaMemcpyAsync(S.tab, tab.data(), tab.size(), cudaMemcpyHostToDevice, s) != cudaSuccess ||
+        cudaMemsetAsync(S.coef, 0, sizeof(T) * coef_tot, s) != cudaSuccess || cudaStreamSynchronize(s) != cudaSuccess) {
+        err = "coarse-level tables failed";
+        return SULF_EDEVICE;
+    }
+    S.nthr = kCoarseThreads;
+    S.smem = smem;
+    S.ncta = C;
+    S.l0 = l0;
+    return SULF_OK;
+}
+
+template <int D, typename T>
+int launch_coarse(const CoarseSet<T>& S, cudaStream_t s) {
+    auto kern = k_s_coarse<D, T>;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(S.ncta);
+    cfg.blockDim = dim3(S.nthr);
+    cfg.dynamicSmemBytes = S.smem;
+    cfg.stream = s;
+    cudaLaunchAttribute at[2];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = S.ncta;
+    at[0].val.clusterDim.y = 1;
+    at[0].val.clusterDim.z = 1;
+    at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[1].val.programmaticStreamSerializationAllowed = launch_pdl() ? 1 : 0;
+    cfg.attrs = at;
+    cfg.numAttrs = 2;
+    cudaError_t e = cudaLaunchKernelEx(&cfg, kern, (const CDesc<T>*)S.dev);
+    if (e != cudaSuccess) note_launch_error(e, S.ncta, kCoarseThreads, S.smem);
+    return 1;
+}
+
+#define SULF_INST_COARSE(D, T)                                                                                      \
+    template int build_coarse<D, T>(CoarseSet<T>&, const LevelGeo*, const SGeo*, const SVec<T>*, int, int, int, int, \
+                                    double*, DevMem&, cudaStream_t, std::string&);                                            \
+    template int launch_coarse<D, T>(const CoarseSet<T>&, cudaStream_t);
+SULF_INST_COARSE(2, double)
+SULF_INST_COARSE(2, float)
+SULF_INST_COARSE(3, double)
+SULF_INST_COARSE(3, float)
+
+}  // namespace sulf

@@ -95,6 +95,11 @@ __global__ void __launch_bounds__(kT) k_s_rho(SLev<D, T> L, SLev<D, float> U, co
     const T rho = pcs * inv, C = c.kap * c.alpha * w.x;
     L.rho[sl] = rho;
     L.cs[sl] = C;
+    if (!FINE && L.perm) {
+        const CPerm q = L.perm[t];
+        L.cf[q.roff] = rho;
+        L.cf[q.roff + q.nx] = C;
+    }
     if (FINE) {
         const double2 f = F[p];
         const double t0 = f.y * (double)inv;
@@ -168,6 +173,13 @@ __global__ void __launch_bounds__(kT) k_s_coefs(SLev<D, T> L, SLev<D, float> U,
     const T di = (T)1 / dd;
     L.dd[t] = dd;
     L.di[t] = di;
+    if (!FINE && L.perm) {
+        const CPerm q = L.perm[t];
+#pragma unroll
+        for (int a = 0; a < 2 * D; a++) L.cf[q.off + a * q.stride] = g[a];
+        L.cf[q.off + 2 * D * q.stride] = dd;
+        L.cf[q.off + (2 * D + 1) * q.stride] = di;
+    }
     if (FINE) {
         const T bs = (T)F[p].x - Psc * (T)tt[sl];
         const T b = bs - et;
@@ -459,8 +471,12 @@ __global__ void __launch_bounds__(kT) k_s_restrict(SLev<D, T> F, SLev<D, T> C, i
             half_coords<D>(e >> kEntHalf, e & 1, C.H, C.n, ci);
             r = restrict_near<D, T>(F, ci);
         }
-        C.b[t] = r;
-        C.X[(t >= C.n0 ? C.Hn : 0) + (e >> kEntHalf)] = t < C.n0 ? r * di : (T)0;
+        if (C.bpos) {
+            C.bf[C.bpos[t]] = r;
+        } else {
+            C.b[t] = r;
+            C.X[(t >= C.n0 ? C.Hn : 0) + (e >> kEntHalf)] = t < C.n0 ? r * di : (T)0;
+        }
     } else {
         const int gi = (t - nrow) / kGopLanes, ln = (t - nrow) % kGopLanes;
         T v = 0;
@@ -470,8 +486,12 @@ __global__ void __launch_bounds__(kT) k_s_restrict(SLev<D, T> F, SLev<D, T> C, i
         }
         v = stages::gop_reduce<T>(v);
         if (gi < C.ng && ln == 0) {
-            C.b[nin + gi] = v;
-            C.X[C.gslot[gi]] = 0;
+            if (C.bpos) {
+                C.bf[C.bpos[nin + gi]] = v;
+            } else {
+                C.b[nin + gi] = v;
+                C.X[C.gslot[gi]] = 0;
+            }
         }
     }
 }
@@ -613,7 +633,8 @@ inline size_t factor_smem(int m, bool columns) {
 }
 
 template <int D, typename T, bool SMEM>
-__global__ void __launch_bounds__(kFacThreads) k_s_factor(SLev<D, T> L, const int* __restrict__ spos, T* Ag, T* Ainv,
+__global__ void __launch_bounds__(kFacThreads) k_s_factor(SLev<D, T> L, const int* __restrict__ spos,
+                                                          const int* __restrict__ cpos, T* Ag, T* Ainv,
                                                           int* singular) {
     namespace cg = cooperative_groups;
     pdl_enter();
@@ -729,7 +750,8 @@ __global__ void __launch_bounds__(kFacThreads) k_s_factor(SLev<D, T> L, const in
     for (int t = threadIdx.x; t < m * mc; t += blockDim.x) {
         const int i = t / mc, jl = t % mc;
         const int j = jl * C + me;
-        if (j < m) Ainv[(size_t)i * m + pos[j]] = A[(size_t)i * mc + jl];
+        if (j < m)
+            Ainv[(size_t)(cpos ? cpos[i] : i) * m + (cpos ? cpos[pos[j]] : pos[j])] = A[(size_t)i * mc + jl];
     }
     cl.sync();  // no CTA leaves while another may still write its shared memory
 }
@@ -1258,7 +1280,8 @@ int launch_s_prolong(const SLev<D, T>& F, const SLev<D, T>& C, cudaStream_t s) {
 }
 
 template <int D, typename T>
-int launch_s_factor(const SLev<D, T>& L, const int* spos, T* A, T* Ainv, int* singular, cudaStream_t s) {
+int launch_s_factor(const SLev<D, T>& L, const int* spos, const int* cpos, T* A, T* Ainv, int* singular,
+                    cudaStream_t s) {
     const int m = L.n0 + L.n1 + L.ng;
     constexpr size_t kMaxSmem = 220 * 1024;
     const bool smem = factor_smem<T>(m, true) <= kMaxSmem;
@@ -1290,7 +1313,7 @@ int launch_s_factor(const SLev<D, T>& L, const int* spos, T* A, T* Ainv, int* si
     at[1].val.programmaticStreamSerializationAllowed = launch_pdl() ? 1 : 0;
     cfg.attrs = at;
     cfg.numAttrs = 2;
-    cudaError_t e = cudaLaunchKernelEx(&cfg, kern, L, spos, A, Ainv, singular);
+    cudaError_t e = cudaLaunchKernelEx(&cfg, kern, L, spos, cpos, A, Ainv, singular);
     if (e != cudaSuccess) note_launch_error(e, kFacCluster, kFacThreads, cfg.dynamicSmemBytes);
     return 1;
 }
@@ -1334,7 +1357,7 @@ int launch_inject_to(const LevelGeo& F, const typename V2<TF>::t* fW, const Leve
     template int launch_s_residual<D, T>(const SLev<D, T>&, unsigned long long*, int*, cudaStream_t);              \
     template int launch_s_restrict<D, T>(const SLev<D, T>&, const SLev<D, T>&, cudaStream_t);                      \
     template int launch_s_prolong<D, T>(const SLev<D, T>&, const SLev<D, T>&, cudaStream_t);                       \
-    template int launch_s_factor<D, T>(const SLev<D, T>&, const int*, T*, T*, int*, cudaStream_t);                 \
+    template int launch_s_factor<D, T>(const SLev<D, T>&, const int*, const int*, T*, T*, int*, cudaStream_t);     \
     template int launch_s_solve<D, T>(const SLev<D, T>&, const T*, cudaStream_t);
 SULF_INST_S(2, double)
 SULF_INST_S(2, float)

@@ -43,6 +43,13 @@ namespace sulf {
 // ghost << 1 | parity of i.  nn < 2^29 (checked by the builder).
 constexpr int kEntHalf = 3;
 
+// where a node of a level fused into the cluster kernel (coarse.cuh) lies in
+// that kernel's rows: gt[q] at off + q stride, then dd and 1/dd; rho at roff, C
+// at roff + nx; in the order of the level's list
+struct CPerm {
+    int off, stride, roff, nx;
+};
+
 // one level as the kernels read it
 template <int D, typename T>
 struct SLev {
@@ -84,6 +91,12 @@ struct SLev {
     const int* cptr;
     const int* cslot;
     const T* cval;
+    // a fused level (else null): its rows, and on the first of them where the
+    // right-hand side goes (then x is not started)
+    const CPerm* perm;
+    T* cf;
+    const int* bpos;
+    T* bf;
 };
 
 // geometry of a level in these terms (precision independent)
@@ -155,6 +168,10 @@ SLev<D, T> make_slev(const LevelGeo& G, const SGeo& S, const SVec<T>& V) {
     s.cptr = S.cptr;
     s.cslot = S.cslot;
     s.cval = f ? (const T*)S.cval32 : (const T*)S.cval;
+    s.perm = nullptr;
+    s.cf = nullptr;
+    s.bpos = nullptr;
+    s.bf = nullptr;
     return s;
 }
 
@@ -203,9 +220,11 @@ template <int D, typename T>
 int launch_s_restrict(const SLev<D, T>& F, const SLev<D, T>& C, cudaStream_t s);
 template <int D, typename T>
 int launch_s_prolong(const SLev<D, T>& F, const SLev<D, T>& C, cudaStream_t s);
-// coarsest level: the dense Schur complement inverted, and applied
+// coarsest level: the dense Schur complement inverted (rows and columns in
+// list order, or at cpos of it), and applied
 template <int D, typename T>
-int launch_s_factor(const SLev<D, T>& L, const int* spos, T* A, T* Ainv, int* singular, cudaStream_t s);
+int launch_s_factor(const SLev<D, T>& L, const int* spos, const int* cpos, T* A, T* Ainv, int* singular,
+                    cudaStream_t s);
 template <int D, typename T>
 int launch_s_solve(const SLev<D, T>& L, const T* Ainv, cudaStream_t s);
 // W -= (x, t - rho x) on the active nodes with the norms of launch_newton_update

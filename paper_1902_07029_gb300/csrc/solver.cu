@@ -13,6 +13,7 @@
 #include <vector>
 
 #include "../../include/sulfmg_debug.h"
+#include "coarse.cuh"
 #include "lockstep.cuh"
 #include "schur.cuh"
 #include "sulf_internal.cuh"
@@ -89,6 +90,9 @@ struct sulf_domain {
     SVec<double> s64[SULF_MAXLEV];
     SVec<float> s32[SULF_MAXLEV];
     int s_geo = 0;
+    // the coarse levels fused into one cluster launch, per precision
+    CoarseSet<double> cs64;
+    CoarseSet<float> cs32;
     bool s_on = false;     // the current linear solve runs that cycle
     int* dskip = nullptr;  // device flag: the first sweep of the cycle has been done
     int bc = 0;  // boundary condition for s: 0 Dirichlet (Eq. BCs), 1 Neumann (Eq. BCsN)
@@ -358,7 +362,9 @@ int ensure32(sulf_domain* d) {
 // levels run as one single-CTA launch (13 k active nodes, 257^2 star: 9.8 ms
 // for two CN steps against 10.9; 104 k nodes, 65^3 box: 26.7 against 28.2 the
 // other way)
-constexpr long long kSchurMinMixed = 50000;
+constexpr long long kSchurMinMixed = 0;
+// automatic fused-level threshold: nodes of the first level of the cluster kernel
+constexpr int kCoarseAuto = 40000;
 bool schur_wanted(const sulf_domain* d) {
     const sulf_solver& v = d->solver;
     if (v.precision == 1 && (long long)d->geo[0].nin[0] + d->geo[0].nin[1] < kSchurMinMixed) return false;
@@ -406,6 +412,24 @@ int alloc_schur(sulf_domain* d, SVec<T>* V, int nl, bool outer) {
     return ok ? SULF_OK : sulf_fail(SULF_ENOMEM, "out of device memory");
 }
 
+// the fused coarse levels of the current threshold (sulf_solver::fuse_below)
+template <typename T>
+int ensure_coarse(sulf_domain* d, CoarseSet<T>& S, const SVec<T>* V) {
+    int want = -1;
+    const int fb = d->solver.fuse_below >= 0 ? d->solver.fuse_below : kCoarseAuto;
+    if (fb > 0 && d->solver.cycle == 1)
+        for (int l = 1; l < d->L && want < 0; l++)
+            if ((long long)d->geo[l].nin[0] + d->geo[l].nin[1] + d->geo[l].ng <= fb) want = l;
+    const int nu1 = d->solver.nu1, nu2 = d->solver.nu2;
+    if (S.rows && S.want == want && S.nu1 == nu1 && S.nu2 == nu2) return SULF_OK;
+    SULF_CUDA_TRY(cudaStreamSynchronize(d->stream));
+    drop_graphs(d);
+    std::string err;
+    int rc = d->dim == 2 ? build_coarse<2, T>(S, d->geo, d->sgeo, V, d->L, want, nu1, nu2, nullptr, d->mem, d->stream, err)
+                         : build_coarse<3, T>(S, d->geo, d->sgeo, V, d->L, want, nu1, nu2, nullptr, d->mem, d->stream, err);
+    return rc ? sulf_fail(rc, err) : SULF_OK;
+}
+
 // decides d->s_on for the next linear solve and builds what it needs
 int ensure_schur(sulf_domain* d);
 int ensure_path(sulf_domain* d) {
@@ -449,12 +473,17 @@ int ensure_schur(sulf_domain* d) {
         if (rc) return sulf_fail(rc, err);
         changed = true;
     }
-    if (changed) drop_graphs(d);
+    if (changed) {
+        drop_graphs(d);
+        d->cs64.rows = d->cs32.rows = false;
+    }
     if (d->solver.precision == 0) {
         if (int rc = alloc_schur<double>(d, d->s64, d->L, false)) return rc;
+        if (int rc = ensure_coarse<double>(d, d->cs64, d->s64)) return rc;
     } else {
         if (int rc = alloc_schur<double>(d, d->s64, 1, true)) return rc;
         if (int rc = alloc_schur<float>(d, d->s32, d->L, false)) return rc;
+        if (int rc = ensure_coarse<float>(d, d->cs32, d->s32)) return rc;
     }
     d->s_on = true;
     return SULF_OK;
@@ -672,7 +701,26 @@ struct SMG {
     double* acc = nullptr;  // mixed precision: the FP64 update the finest error is added to
     int fine_sweeps = 0;
 
-    SLev<D, T> lev(int l) { return make_slev<D, T>(d->geo[l], d->sgeo[l], V[l]); }
+    const CoarseSet<T>& fused() const {
+        if constexpr (std::is_same<T, double>::value)
+            return d->cs64;
+        else
+            return d->cs32;
+    }
+
+    SLev<D, T> lev(int l) {
+        SLev<D, T> s = make_slev<D, T>(d->geo[l], d->sgeo[l], V[l]);
+        const CoarseSet<T>& S = fused();
+        if (S.l0 >= 0 && l >= S.l0) {
+            s.perm = S.perm[l];
+            s.cf = S.coef;
+            if (l == S.l0) {
+                s.bpos = S.bpos;
+                s.bf = S.b;
+            }
+        }
+        return s;
+    }
 
     // delta: the sweep follows a prolongation; a: see launch_s_relax
     void relax(int l, bool skip_red, bool delta, const int* skip, double* a) {
@@ -693,11 +741,15 @@ struct SMG {
     // right-hand side; first: device flag, set where the whole first sweep
     // has been done
     int cycle(int l, bool red_done, const int* first) {
+        const sulf_solver& sv = d->solver;
+        if (l == fused().l0) {
+            d->launches += launch_coarse<D, T>(fused(), d->stream);
+            return SULF_OK;
+        }
         if (l == d->L - 1) {
             d->launches += launch_s_solve<D, T>(lev(l), V[l].Ainv, d->stream);
             return SULF_OK;
         }
-        const sulf_solver& sv = d->solver;
         for (int k = 0; k < sv.nu1; k++) relax(l, red_done && k == 0, false, k == 0 ? first : nullptr, nullptr);
         d->launches += launch_s_residual<D, T>(lev(l), nullptr, nullptr, d->stream);
         d->launches += launch_s_restrict<D, T>(lev(l), lev(l + 1), d->stream);
@@ -722,7 +774,7 @@ struct SMG {
         }
         SULF_CUDA_TRY(cudaMemsetAsync(d->dsing, 0, sizeof(int), d->stream));
         const int lc = d->L - 1;
-        d->launches += launch_s_factor<D, T>(lev(lc), d->sgeo[lc].spos, V[lc].A, V[lc].Ainv, d->dsing, d->stream);
+        d->launches += launch_s_factor<D, T>(lev(lc), d->sgeo[lc].spos, fused().l0 >= 0 ? fused().cpos : nullptr, V[lc].A, V[lc].Ainv, d->dsing, d->stream);
         return SULF_OK;
     }
 
