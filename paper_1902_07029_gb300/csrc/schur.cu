@@ -16,7 +16,6 @@ using stages::kGopLanes;
 namespace {
 
 constexpr int kT = kNodeThreads;
-constexpr int kRowLanes = 4;  // lanes that share a ghost's row of the defect
 
 // node coordinates of a half index
 template <int D>
@@ -216,7 +215,7 @@ __global__ void __launch_bounds__(kT) k_s_relax(SLev<D, T> L, int colour, int sn
 #pragma unroll
         for (int q = 0; q < 2 * D; q++) g[q] = L.gt[q * L.gs + pos];
         di = L.di[pos];
-        if (DELTA) cp = L.cs[colour * L.Hn + (e >> kEntHalf)];
+        if (DELTA && (colour == 0 || (e & 2))) cp = L.cs[colour * L.Hn + (e >> kEntHalf)];
     }
     nbr_offsets<D, T>(L, e & 1, o);
     const int sg = snap && t < L.ng ? L.gslot[t] : 0;
@@ -259,42 +258,92 @@ __device__ __forceinline__ T ghost_input(const SLev<D, T>& L, int code) {
     return (u & 1u) ? L.b[L.n0 + L.n1 + (u >> 1)] : L.snap[u >> 1];
 }
 
+// The threads of a kernel over the ghosts' rows: one for each of the ng1 short
+// rows, `mid` lanes for each of the ng8 next, `most` for each longer one, every
+// part rounded up to whole warps.  On the flat parts of a boundary a composed
+// row has 4 entries, on an edge of a box 50 to 500: eight lanes for all left
+// most lanes idle and the long rows as a tail (257^3 box FP64: 37.6 us).
+struct GhostPart {
+    int g, lane, lanes;
+    bool on;
+};
+__host__ __device__ __forceinline__ int up32(int n) { return (n + 31) & ~31; }
+template <int D, typename T>
+__host__ __device__ __forceinline__ int ghost_threads(const SLev<D, T>& L, int mid, int most) {
+    return up32(L.ng1) + up32(L.ng8 * mid) + up32((L.ng - L.ng1 - L.ng8) * most);
+}
+template <int D, typename T>
+__device__ __forceinline__ GhostPart ghost_part(const SLev<D, T>& L, int t, int mid, int most) {
+    GhostPart p;
+    const int t8 = up32(L.ng1), tx = t8 + up32(L.ng8 * mid);
+    if (t < t8) {
+        p.lanes = 1;
+        p.lane = 0;
+        p.g = t;
+        p.on = t < L.ng1;
+    } else if (t < tx) {
+        p.lanes = mid;
+        p.lane = (t - t8) % mid;
+        p.g = L.ng1 + (t - t8) / mid;
+        p.on = p.g < L.ng1 + L.ng8;
+    } else {
+        p.lanes = most;
+        p.lane = (t - tx) % most;
+        p.g = L.ng1 + L.ng8 + (t - tx) / most;
+        p.on = p.g < L.ng;
+    }
+    p.g = p.on ? L.gord[p.g] : 0;
+    return p;
+}
+// sum over the lanes of a part (every lane of the warp calls it)
+template <typename T>
+__device__ __forceinline__ T part_sum(T v, int lanes) {
+    for (int o = lanes >> 1; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    return v;
+}
+
 // all passes of a sweep's ghost relaxation, one composed row per ghost
 constexpr int kGopPre = 4;
 template <int D, typename T>
 __global__ void __launch_bounds__(kT) k_s_ghosts(SLev<D, T> L, const int* skip, double* acc) {
-    const int t = blockIdx.x * blockDim.x + threadIdx.x;
-    const int gi = t / kGopLanes, ln = t % kGopLanes;
-    const bool on = gi < L.ng;
+    const GhostPart p = ghost_part<D, T>(L, blockIdx.x * blockDim.x + threadIdx.x, kGopLanes, 32);
     int beg = 0, end = 0, sl = 0;
     int cd[kGopPre];
     T w[kGopPre];
-    if (on) {
-        beg = L.gptr[gi] + ln;
-        end = L.gptr[gi + 1];
+    if (p.on) {
+        beg = L.gptr[p.g] + p.lane;
+        end = L.gptr[p.g + 1];
 #pragma unroll
         for (int i = 0; i < kGopPre; i++) {
-            const int j = beg + i * kGopLanes;
+            const int j = beg + i * p.lanes;
             cd[i] = j < end ? L.gcode[j] : 0;
             w[i] = j < end ? L.gval[j] : (T)0;
         }
-        sl = L.gslot[gi];
+        sl = L.gslot[p.g];
     }
     pdl_enter();
     if (skip && *skip) return;
     T v = 0;
-    if (on) {
-        T u[kGopPre];
+    if (p.on) {
+        for (int j = beg;;) {
+            T u[kGopPre];
 #pragma unroll
-        for (int i = 0; i < kGopPre; i++) u[i] = beg + i * kGopLanes < end ? ghost_input<D, T>(L, cd[i]) : (T)0;
+            for (int i = 0; i < kGopPre; i++) u[i] = j + i * p.lanes < end ? ghost_input<D, T>(L, cd[i]) : (T)0;
 #pragma unroll
-        for (int i = 0; i < kGopPre; i++)
-            if (beg + i * kGopLanes < end) v = fmadd(w[i], u[i], v);
-        for (int j = beg + kGopPre * kGopLanes; j < end; j += kGopLanes)
-            v = fmadd(L.gval[j], ghost_input<D, T>(L, L.gcode[j]), v);
+            for (int i = 0; i < kGopPre; i++)
+                if (j + i * p.lanes < end) v = fmadd(w[i], u[i], v);
+            j += kGopPre * p.lanes;
+            if (j >= end) break;
+#pragma unroll
+            for (int i = 0; i < kGopPre; i++) {
+                const int q = j + i * p.lanes < end ? j + i * p.lanes : j;
+                cd[i] = L.gcode[q];
+                w[i] = L.gval[q];
+            }
+        }
     }
-    v = stages::gop_reduce<T>(v);
-    if (!on || ln != 0) return;
+    v = part_sum<T>(v, p.lanes);
+    if (!p.on || p.lane != 0) return;
     L.X[sl] = v;
     if (acc) acc[sl] += (double)v;
 }
@@ -316,18 +365,17 @@ __device__ __forceinline__ T inside_defect(const SLev<D, T>& L, int pos, int col
     return r;
 }
 
-// b - row . x of ghost gi by the kRowLanes lanes of its group; every lane of
-// the warp calls it, lane 0 of the group holds the result
+// b - row . x of a ghost by its lanes; every lane of the warp calls it, lane 0
+// holds the result
 template <int D, typename T>
-__device__ __forceinline__ T ghost_defect(const SLev<D, T>& L, bool on, int gi, int ln) {
+__device__ __forceinline__ T ghost_defect(const SLev<D, T>& L, const GhostPart& p) {
     T v = 0;
-    if (on) {
-        const int end = L.rptr[gi + 1];
-        for (int j = L.rptr[gi] + ln; j < end; j += kRowLanes) v = fmadd(L.rval[j], L.X[L.rslot[j]], v);
+    if (p.on) {
+        const int end = L.rptr[p.g + 1];
+        for (int j = L.rptr[p.g] + p.lane; j < end; j += p.lanes) v = fmadd(L.rval[j], L.X[L.rslot[j]], v);
     }
-#pragma unroll
-    for (int d = kRowLanes / 2; d > 0; d >>= 1) v += __shfl_xor_sync(0xffffffffu, v, d);
-    return on && ln == 0 ? L.b[L.n0 + L.n1 + gi] - v : (T)0;
+    v = part_sum<T>(v, p.lanes);
+    return p.on && p.lane == 0 ? L.b[L.n0 + L.n1 + p.g] - v : (T)0;
 }
 
 template <int D, typename T, bool NORM>
@@ -353,9 +401,9 @@ __global__ void __launch_bounds__(kT) k_s_residual(SLev<D, T> L, int nrow, unsig
             if (!NORM) L.R[colour * L.Hn + (e >> kEntHalf)] = r;
         }
     } else {
-        const int gi = (t - nrow) / kRowLanes, ln = (t - nrow) % kRowLanes;
-        r = ghost_defect<D, T>(L, gi < L.ng, gi, ln);
-        if (!NORM && gi < L.ng && ln == 0) L.R[L.gslot[gi]] = r;
+        const GhostPart p = ghost_part<D, T>(L, t - nrow, kGopLanes, kGopLanes);
+        r = ghost_defect<D, T>(L, p);
+        if (!NORM && p.on && p.lane == 0) L.R[L.gslot[p.g]] = r;
     }
     if (NORM) block_max(abs_bits(r), norm);
 }
@@ -389,11 +437,11 @@ __global__ void __launch_bounds__(kT) k_s_outer(SLev<D, double> L, SLev<D, float
             if (!colour) U.X[h] = (float)r * df;
         }
     } else {
-        const int gi = (t - nrow) / kRowLanes, ln = (t - nrow) % kRowLanes;
-        r = ghost_defect<D, double>(L, gi < L.ng, gi, ln);
-        if (gi < L.ng && ln == 0) {
-            U.b[nin + gi] = (float)r;
-            U.X[L.gslot[gi]] = 0.f;
+        const GhostPart p = ghost_part<D, double>(L, t - nrow, kGopLanes, kGopLanes);
+        r = ghost_defect<D, double>(L, p);
+        if (p.on && p.lane == 0) {
+            U.b[nin + p.g] = (float)r;
+            U.X[L.gslot[p.g]] = 0.f;
         }
     }
     block_max(abs_bits(r), norm);
@@ -404,36 +452,41 @@ __global__ void __launch_bounds__(kT) k_s_outer(SLev<D, double> L, SLev<D, float
 
 // boundary-aware full weighting of the finer level's defect (Eqs. Fstencil,
 // Fstencilgen) at a coarse inside node whose fine neighbourhood holds nodes
-// that are not inside, or black nodes with a defect of their own
+// that are not inside, or black nodes with a defect of their own; m: the
+// members that are inside nodes.  Weights are powers of two over 4^D, built
+// from their exponents (mg_stages.cuh).
 template <int D, typename T>
-__device__ __forceinline__ T restrict_near(const SLev<D, T>& F, const int* ci) {
-    const int n = F.n;
-    int f[3] = {2 * ci[0], 2 * ci[1], D == 3 ? 2 * ci[2] : 0};
-    const int st[3] = {1, n, n * n};
-    const int p = f[0] + n * (f[1] + (D == 3 ? n * f[2] : 0));
-    int w[3][3];  // per-axis weights times 4
+__device__ __forceinline__ T restrict_near(const SLev<D, T>& F, int tw, unsigned m) {
+    constexpr int K = D == 2 ? 9 : 27, mid = K / 2, pw[3] = {1, 3, 9};
+    int e[3][3];  // per axis: log2 of the weight times 4, or -16 (weight 0)
 #pragma unroll
     for (int a = 0; a < D; a++) {
-        const bool vl = F.type[p - st[a]] == T_IN, vr = F.type[p + st[a]] == T_IN;
-        w[a][0] = vl ? (vr ? 1 : 2) : 0;
-        w[a][1] = vl || vr ? 2 : 4;
-        w[a][2] = vr ? (vl ? 1 : 2) : 0;
+        const bool vl = (m >> (mid - pw[a])) & 1u, vr = (m >> (mid + pw[a])) & 1u;
+        e[a][0] = vl ? (vr ? 0 : 1) : -16;
+        e[a][1] = vl || vr ? 1 : 2;
+        e[a][2] = vr ? (vl ? 0 : 1) : -16;
+    }
+    // the twin (2I, 2J, 2K) is red at an even x index: the members along x lie
+    // at half indices -1, 0 (odd x) or 0 (even x) of its row
+    T v[K];
+#pragma unroll
+    for (int kk = 0; kk < K; kk++) {
+        const int k0 = kk % 3 - 1, k1 = (kk / 3) % 3 - 1, k2 = D == 3 ? kk / 9 - 1 : 0;
+        const int odd = (k0 + k1 + k2) & 1;
+        v[kk] = (m >> kk) & 1u ? F.R[tw + odd * F.Hn + (k0 < 0 ? -1 : 0) + k1 * F.H + (D == 3 ? k2 * F.P : 0)] : (T)0;
     }
     T acc = 0;
     int wc = 0;
-    for (int kk = 0; kk < (D == 2 ? 9 : 27); kk++) {
-        const int k0 = kk % 3, k1 = (kk / 3) % 3, k2 = D == 3 ? kk / 9 : 1;
-        const int iw = w[0][k0] * w[1][k1] * (D == 3 ? w[2][k2] : 1);
-        if (iw == 0) continue;
-        const int q = p + (k0 - 1) + (k1 - 1) * st[1] + (D == 3 ? (k2 - 1) * st[2] : 0);
-        const bool centre = k0 == 1 && k1 == 1 && k2 == 1;
-        if (centre || F.type[q] != T_IN)
-            wc += iw;
+#pragma unroll
+    for (int kk = 0; kk < K; kk++) {
+        const int s = e[0][kk % 3] + e[1][(kk / 3) % 3] + (D == 3 ? e[2][kk / 9] : 0);
+        if (s < 0) continue;
+        if (kk == mid || !((m >> kk) & 1u))
+            wc += 1 << s;
         else
-            acc = fmadd((T)iw, F.R[slot_of<D>(f[0] + k0 - 1, f[1] + k1 - 1, f[2] + k2 - 1, F.H, F.P, F.Hn)], acc);
+            acc = fmadd(stages::pow2_weight<D, T>(s), v[kk], acc);
     }
-    acc = fmadd((T)wc, F.R[slot_of<D>(f[0], f[1], f[2], F.H, F.P, F.Hn)], acc);
-    return acc / (T)(D == 2 ? 16 : 64);
+    return fmadd((T)wc * stages::pow2_weight<D, T>(0), v[mid], acc);
 }
 
 // the finer level's defect onto the coarse level's right-hand side; the coarse
@@ -441,19 +494,28 @@ __device__ __forceinline__ T restrict_near(const SLev<D, T>& F, const int* ci) {
 template <int D, typename T>
 __global__ void __launch_bounds__(kT) k_s_restrict(SLev<D, T> F, SLev<D, T> C, int nrow) {
     const int t = blockIdx.x * blockDim.x + threadIdx.x;
-    const int nin = C.n0 + C.n1;
-    int e = 0, tw = -1;
+    const int nin = C.n0 + C.n1, nreg = C.nreg0 + C.nreg1, freg = up32(nreg);
+    // regular nodes, then (from a whole warp on) the others
+    int pos = -1, tw = 0, e = 0;
+    unsigned m = 0;
     T di = 0;
-    if (t < nin) {
-        e = C.hl[t];
-        tw = C.twin[t];
-        if (t < C.n0) di = C.di[t];
+    if (t < nreg) {
+        pos = t < C.nreg0 ? t : C.n0 + t - C.nreg0;
+    } else if (t >= freg && t < nrow) {
+        const int u = t - freg, near0 = C.n0 - C.nreg0;
+        if (u < nin - nreg) pos = u < near0 ? C.nreg0 + u : C.n0 + C.nreg1 + u - near0;
+    }
+    if (pos >= 0) {
+        tw = C.twin[pos];
+        e = C.hl[pos];
+        if (t >= freg) m = (unsigned)C.mask[pos];
+        if (pos < C.n0) di = C.di[pos];
     }
     pdl_enter();
     if (t < nrow) {
-        if (t >= nin) return;
+        if (pos < 0) return;
         T r;
-        if (tw >= 0) {
+        if (t < freg) {
             // black members (weights of the faces and corners) have no defect
             const T* R = F.R + tw;
             const int H = F.H, P = F.P;
@@ -467,15 +529,13 @@ __global__ void __launch_bounds__(kT) k_s_restrict(SLev<D, T> F, SLev<D, T> C, i
                 r = (T)0.25 * c0 + (T)0.0625 * s;
             }
         } else {
-            int ci[3];
-            half_coords<D>(e >> kEntHalf, e & 1, C.H, C.n, ci);
-            r = restrict_near<D, T>(F, ci);
+            r = restrict_near<D, T>(F, tw, m);
         }
         if (C.bpos) {
-            C.bf[C.bpos[t]] = r;
+            C.bf[C.bpos[pos]] = r;
         } else {
-            C.b[t] = r;
-            C.X[(t >= C.n0 ? C.Hn : 0) + (e >> kEntHalf)] = t < C.n0 ? r * di : (T)0;
+            C.b[pos] = r;
+            C.X[(pos >= C.n0 ? C.Hn : 0) + (e >> kEntHalf)] = pos < C.n0 ? r * di : (T)0;
         }
     } else {
         const int gi = (t - nrow) / kGopLanes, ln = (t - nrow) % kGopLanes;
@@ -507,7 +567,7 @@ __global__ void __launch_bounds__(kT) k_s_prolong(SLev<D, T> F, SLev<D, T> C) {
     int cn[1 << D];
     T cr[1 << D];
     unsigned use = 0;
-    int sl = 0;
+    int sl = 0, pair = -1;  // a black node on a coarse line: the two corners along this axis
     T rho = 0, Cs = 0;
     if (on) {
         int ii[3];
@@ -517,30 +577,39 @@ __global__ void __launch_bounds__(kT) k_s_prolong(SLev<D, T> F, SLev<D, T> C) {
             sl = F.Hn + (e >> kEntHalf);
             half_coords<D>(e >> kEntHalf, e & 1, F.H, F.n, ii);
             all = e & 4;
+            if (all && (D == 2 || !(ii[0] & ii[1] & ii[2] & 1))) pair = ii[0] & 1 ? 0 : (ii[1] & 1 ? 1 : 2);
         } else {
             sl = F.gslot[t - F.n1];
             stages::box_coords<D>(F.gidx[t - F.n1], F.n, ii);
         }
         rho = F.rho[sl];
         Cs = F.cs[sl];
+        if (pair >= 0) {
+            int q[3] = {ii[0] >> 1, ii[1] >> 1, D == 3 ? ii[2] >> 1 : 0};
+            cn[0] = slot_of<D>(q[0], q[1], q[2], C.H, C.P, C.Hn);
+            cn[1] = slot_of<D>(q[0] + (pair == 0), q[1] + (pair == 1), q[2] + (pair == 2), C.H, C.P, C.Hn);
+            cr[0] = C.rho[cn[0]];
+            cr[1] = C.rho[cn[1]];
+        } else {
 #pragma unroll
-        for (int cc = 0; cc < (1 << D); cc++) {
-            int q[3] = {0, 0, 0};
-            bool dup = false;
+            for (int cc = 0; cc < (1 << D); cc++) {
+                int q[3] = {0, 0, 0};
+                bool dup = false;
 #pragma unroll
-            for (int a = 0; a < D; a++) {
-                const int up = (cc >> a) & 1;
-                if (up && !(ii[a] & 1)) dup = true;
-                q[a] = (ii[a] >> 1) + (up && (ii[a] & 1) ? 1 : 0);
+                for (int a = 0; a < D; a++) {
+                    const int up = (cc >> a) & 1;
+                    if (up && !(ii[a] & 1)) dup = true;
+                    q[a] = (ii[a] >> 1) + (up && (ii[a] & 1) ? 1 : 0);
+                }
+                cn[cc] = slot_of<D>(q[0], q[1], q[2], C.H, C.P, C.Hn);
+                if (dup) continue;
+                if (!all) {
+                    const int8_t ty = C.type[q[0] + C.n * (q[1] + (D == 3 ? C.n * q[2] : 0))];
+                    if (ty != T_IN && ty != T_GHOST) continue;
+                }
+                use |= 1u << cc;
+                cr[cc] = C.rho[cn[cc]];
             }
-            cn[cc] = slot_of<D>(q[0], q[1], q[2], C.H, C.P, C.Hn);
-            if (dup) continue;
-            if (!all) {
-                const int8_t ty = C.type[q[0] + C.n * (q[1] + (D == 3 ? C.n * q[2] : 0))];
-                if (ty != T_IN && ty != T_GHOST) continue;
-            }
-            use |= 1u << cc;
-            cr[cc] = C.rho[cn[cc]];
         }
     }
     pdl_enter();
@@ -548,19 +617,25 @@ __global__ void __launch_bounds__(kT) k_s_prolong(SLev<D, T> F, SLev<D, T> C) {
     T2 d;
     d.x = 0;
     d.y = 0;
-    if (use) {
+    T x = F.X[sl], ps = 0, pc = 0, r = 0;
+    if (pair >= 0) {
+        const T v0 = C.X[cn[0]], v1 = C.X[cn[1]];
+        ps = v0 + v1;
+        pc = fmadd(-cr[1], v1, -cr[0] * v0);
+        r = (T)0.5;
+    } else if (use) {
         T v[1 << D];
 #pragma unroll
         for (int cc = 0; cc < (1 << D); cc++) v[cc] = (use >> cc) & 1u ? C.X[cn[cc]] : (T)0;
-        T x = F.X[sl];
-        T ps = 0, pc = 0;
 #pragma unroll
         for (int cc = 0; cc < (1 << D); cc++)
             if ((use >> cc) & 1u) {
                 ps += v[cc];
                 pc = fmadd(-cr[cc], v[cc], pc);
             }
-        const T r = stages::inv_count<T>(__popc(use));
+        r = stages::inv_count<T>(__popc(use));
+    }
+    if (pair >= 0 || use) {
         F.X[sl] = fmadd(ps, r, x);
         // off the c row by delta = x^c + rho x^s of the correction
         d.x = fmadd(rho, ps, pc) * r;
@@ -822,30 +897,69 @@ __device__ __forceinline__ bool near_ghost(const int8_t* type, int p, int n, int
     return g;
 }
 
-// nodes of a colour's list without a ghost neighbour, per chunk
-__global__ void k_away_count(const int* __restrict__ list, int cnt, const int8_t* __restrict__ type, int n, int dim,
-                             int* __restrict__ out) {
-    const int t = blockIdx.x * kChunk + threadIdx.x;
-    const int c = __syncthreads_count(t < cnt && !near_ghost(type, list[t], n, dim));
-    if (threadIdx.x == 0) out[blockIdx.x] = c;
+// bits of the 3^d fine members of a coarse node (its fine twin at box node p)
+// that are inside nodes; regular: all of them are, the black ones (odd index
+// sum) away from the ghosts
+__device__ __forceinline__ int member_mask(const int8_t* ftype, int p, int fn, int dim, bool& regular) {
+    int m = 0;
+    regular = true;
+    for (int kk = 0; kk < (dim == 2 ? 9 : 27); kk++) {
+        const int k[3] = {kk % 3 - 1, (kk / 3) % 3 - 1, dim == 3 ? kk / 9 - 1 : 0};
+        const int q = p + k[0] + fn * (k[1] + fn * k[2]);
+        const bool in = ftype[q] == T_IN;
+        if (in) m |= 1 << kk;
+        if (!in || (((k[0] + k[1] + k[2]) & 1) && near_ghost(ftype, q, fn, dim))) regular = false;
+    }
+    return m;
 }
 
-// entries of a colour's nodes, those next to a ghost (at `away` and on) last
+// class of an inside node: 2 next to a ghost, else 0 where its restriction
+// from the finer level (if any) is regular, 1 where it is not
+__device__ __forceinline__ int node_class(const int8_t* type, int p, int n, int dim, const int8_t* ftype, int fn) {
+    if (near_ghost(type, p, n, dim)) return 2;
+    if (!ftype) return 0;
+    bool regular;
+    member_mask(ftype, 2 * (p % n) + fn * (2 * ((p / n) % n) + (dim == 3 ? fn * 2 * (p / (n * n)) : 0)), fn, dim,
+                regular);
+    return regular ? 0 : 1;
+}
+
+// nodes of a colour's list of class 0 and 1, per chunk
+__global__ void k_class_count(const int* __restrict__ list, int cnt, const int8_t* __restrict__ type, int n, int dim,
+                              const int8_t* __restrict__ ftype, int fn, int* __restrict__ out) {
+    const int t = blockIdx.x * kChunk + threadIdx.x;
+    const int k = t < cnt ? node_class(type, list[t], n, dim, ftype, fn) : 3;
+    const int c0 = __syncthreads_count(k == 0), c1 = __syncthreads_count(k == 1);
+    if (threadIdx.x == 0) {
+        out[2 * blockIdx.x] = c0;
+        out[2 * blockIdx.x + 1] = c1;
+    }
+}
+
+// entries of a colour's nodes by class, each class in list order; off: the
+// chunk's offsets within classes 0 and 1, first: where classes 1 and 2 begin
 __global__ void k_entries(const int* __restrict__ list, int cnt, const int8_t* __restrict__ type, int n, int dim,
-                          const int8_t* __restrict__ ctype, int cn, const int* __restrict__ off, int away, int H,
-                          int* __restrict__ hl) {
-    __shared__ int wsum[32];
+                          const int8_t* __restrict__ ftype, int fn, const int8_t* __restrict__ ctype, int cn,
+                          const int* __restrict__ off, int first1, int first2, int H, int* __restrict__ hl) {
+    __shared__ int wsum[2][32];
     const int t = blockIdx.x * kChunk + threadIdx.x;
     const bool on = t < cnt;
     const int p = on ? list[t] : 0;
-    const bool a = on && !near_ghost(type, p, n, dim);
-    const unsigned m = __ballot_sync(0xffffffffu, a);
+    const int k = on ? node_class(type, p, n, dim, ftype, fn) : 3;
+    const unsigned m0 = __ballot_sync(0xffffffffu, k == 0), m1 = __ballot_sync(0xffffffffu, k == 1);
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    if (lane == 0) wsum[warp] = __popc(m);
+    if (lane == 0) {
+        wsum[0][warp] = __popc(m0);
+        wsum[1][warp] = __popc(m1);
+    }
     __syncthreads();
     if (!on) return;
-    int r = off[blockIdx.x] + __popc(m & ((1u << lane) - 1u));
-    for (int w = 0; w < warp; w++) r += wsum[w];
+    const unsigned below = (1u << lane) - 1u;
+    int r0 = off[2 * blockIdx.x] + __popc(m0 & below), r1 = off[2 * blockIdx.x + 1] + __popc(m1 & below);
+    for (int w = 0; w < warp; w++) {
+        r0 += wsum[0][w];
+        r1 += wsum[1][w];
+    }
     const int ii[3] = {p % n, (p / n) % n, dim == 3 ? p / (n * n) : 0};
     bool all = ctype != nullptr;
     for (int cc = 0; cc < (1 << dim) && all; cc++) {
@@ -857,7 +971,8 @@ __global__ void k_entries(const int* __restrict__ list, int cnt, const int8_t* _
         all = ctype[q] == T_IN || ctype[q] == T_GHOST;
     }
     const int h = (ii[0] >> 1) + H * (ii[1] + n * ii[2]);
-    hl[a ? r : away + t - r] = (h << kEntHalf) | (all ? 4 : 0) | (a ? 0 : 2) | (ii[0] & 1);
+    hl[k == 0 ? r0 : (k == 1 ? first1 + r1 : first2 + t - r0 - r1)] =
+        (h << kEntHalf) | (all ? 4 : 0) | (k == 2 ? 2 : 0) | (ii[0] & 1);
 }
 
 __device__ __forceinline__ int box_slot(int p, int n, int dim, int H, int Hn) {
@@ -905,29 +1020,16 @@ __global__ void k_rows(int ng, int K, const double* __restrict__ wk, const float
     if (!ptr) cnt[g] = j;
 }
 
-// slot of the fine twin of a coarse inside node all of whose 3^d fine members
-// are inside nodes, its black ones (odd index sum) away from the ghosts
-__global__ void k_twins(const int* __restrict__ hl, int n0, int nin, int cn, int cH, const int8_t* __restrict__ ftype,
-                        int fn, int fH, int dim, int* __restrict__ twin) {
+// slot of a coarse inside node's fine twin (a red node) and its members
+__global__ void k_twins(const int* __restrict__ hl, int nin, int cn, int cH, const int8_t* __restrict__ ftype, int fn,
+                        int fH, int dim, int* __restrict__ twin, int* __restrict__ mask) {
     const int t = blockIdx.x * blockDim.x + threadIdx.x;
     if (t >= nin) return;
     const int e = hl[t], h = e >> kEntHalf, row = h / cH;
     const int f[3] = {2 * (2 * (h - row * cH) + (e & 1)), 2 * (row % cn), dim == 3 ? 2 * (row / cn) : 0};
-    bool ok = true;
-    for (int kk = 0; kk < (dim == 2 ? 9 : 27) && ok; kk++) {
-        const int k[3] = {kk % 3 - 1, (kk / 3) % 3 - 1, dim == 3 ? kk / 9 - 1 : 0};
-        int q = 0, st = 1;
-        for (int a = 0; a < dim; a++) {
-            if (f[a] + k[a] < 0 || f[a] + k[a] >= fn) ok = false;
-            q += (f[a] + k[a]) * st;
-            st *= fn;
-        }
-        if (!ok) break;
-        ok = ftype[q] == T_IN;
-        if (ok && ((k[0] + k[1] + k[2]) & 1)) ok = !near_ghost(ftype, q, fn, dim);
-    }
-    // (2I, 2J, 2K) is a red node: slot = half index
-    twin[t] = ok ? (f[0] >> 1) + fH * (f[1] + fn * f[2]) : -1;
+    bool regular;
+    mask[t] = member_mask(ftype, f[0] + fn * (f[1] + fn * f[2]), fn, dim, regular);
+    twin[t] = (f[0] >> 1) + fH * (f[1] + fn * f[2]);
 }
 
 // A coarse ghost's right-hand side: the outside weighting (Sec. 3.5.2) of the
@@ -1066,36 +1168,39 @@ int build_sgeo(SGeo& S, const LevelGeo& L, const LevelGeo* finer, const SGeo* sf
     S.hl = (int*)mem.get(sizeof(int) * (nin + 1));
     S.gslot = (int*)mem.get(sizeof(int) * (L.ng + 1));
     const int nch = (int)nblk(S.n0 > S.n1 ? S.n0 : S.n1, kChunk);
-    int* dc = (int*)mem.get(sizeof(int) * 2 * (nch + 1));
+    int* dc = (int*)mem.get(sizeof(int) * 4 * (nch + 1));
     if (!S.hl || !S.gslot || !dc) return oom();
-    std::vector<int> c(2 * (nch + 1), 0);
+    std::vector<int> c(4 * (nch + 1), 0);
+    const int8_t* ft = finer ? finer->type : nullptr;
+    const int fn = finer ? finer->n : 0;
     for (int k = 0; k < 2; k++)
         if (L.nin[k] > 0) {
-            k_away_count<<<nblk(L.nin[k], kChunk), kChunk, 0, s>>>(L.inl[k], L.nin[k], L.type, L.n, L.dim,
-                                                                   dc + k * (nch + 1));
+            k_class_count<<<nblk(L.nin[k], kChunk), kChunk, 0, s>>>(L.inl[k], L.nin[k], L.type, L.n, L.dim, ft, fn,
+                                                                    dc + 2 * k * (nch + 1));
             launches++;
         }
     if (cudaMemcpyAsync(c.data(), dc, sizeof(int) * c.size(), cudaMemcpyDeviceToHost, s) != cudaSuccess ||
         cudaStreamSynchronize(s) != cudaSuccess)
         return fail();
-    int away[2] = {0, 0};
-    for (int k = 0; k < 2; k++) {
-        const int nk = (int)nblk(L.nin[k], kChunk);
-        int tot = 0;
-        for (int b = 0; b < nk; b++) {
-            const int v = c[k * (nch + 1) + b];
-            c[k * (nch + 1) + b] = tot;
-            tot += v;
-        }
-        away[k] = tot;
-    }
-    S.nga = S.n1 - away[1];
+    int tot[2][2] = {{0, 0}, {0, 0}};
+    for (int k = 0; k < 2; k++)
+        for (int b = 0; b < (int)nblk(L.nin[k], kChunk); b++)
+            for (int q = 0; q < 2; q++) {
+                int& v = c[2 * k * (nch + 1) + 2 * b + q];
+                const int w = v;
+                v = tot[k][q];
+                tot[k][q] += w;
+            }
+    S.nreg0 = tot[0][0];
+    S.nreg1 = tot[1][0];
+    S.nga = S.n1 - tot[1][0] - tot[1][1];
     if (cudaMemcpyAsync(dc, c.data(), sizeof(int) * c.size(), cudaMemcpyHostToDevice, s) != cudaSuccess) return fail();
     for (int k = 0; k < 2; k++)
         if (L.nin[k] > 0) {
             k_entries<<<nblk(L.nin[k], kChunk), kChunk, 0, s>>>(
-                L.inl[k], L.nin[k], L.type, L.n, L.dim, coarser ? coarser->type : nullptr, coarser ? coarser->n : 0,
-                dc + k * (nch + 1), away[k], S.H, S.hl + (k ? S.n0 : 0));
+                L.inl[k], L.nin[k], L.type, L.n, L.dim, ft, fn, coarser ? coarser->type : nullptr,
+                coarser ? coarser->n : 0, dc + 2 * k * (nch + 1), tot[k][0], tot[k][0] + tot[k][1], S.H,
+                S.hl + (k ? S.n0 : 0));
             launches++;
         }
     if (L.ng > 0) {
@@ -1105,8 +1210,10 @@ int build_sgeo(SGeo& S, const LevelGeo& L, const LevelGeo* finer, const SGeo* sf
     if (finer) {
         S.twin = (int*)mem.get(sizeof(int) * (nin + 1));
         S.cptr = (int*)mem.get(sizeof(int) * (L.ng + 1));
-        if (!S.twin || !S.cptr) return oom();
-        k_twins<<<nblk(nin), 256, 0, s>>>(S.hl, S.n0, nin, L.n, S.H, finer->type, finer->n, sfiner->H, L.dim, S.twin);
+        S.mask = (int*)mem.get(sizeof(int) * (nin + 1));
+        if (!S.twin || !S.cptr || !S.mask) return oom();
+        k_twins<<<nblk(nin), 256, 0, s>>>(S.hl, nin, L.n, S.H, finer->type, finer->n, sfiner->H, L.dim, S.twin,
+                                          S.mask);
         launches++;
         long long tot = 0;
         const size_t shm = sizeof(OutWork) * kOutThreads;
@@ -1156,6 +1263,32 @@ int build_sgeo_rows(SGeo& S, const LevelGeo& L, DevMem& mem, cudaStream_t s, std
         S.gcode = (int*)mem.get(sizeof(int) * (L.gop_nnz + 1));
         if (!S.gcode) return oom();
         S.gcap = L.gop_nnz;
+    }
+    {
+        // the ghosts by the length of their composed row
+        if (!S.gord) S.gord = (int*)mem.get(sizeof(int) * (L.ng + 1));
+        if (!S.gord) return oom();
+        std::vector<int> p(L.ng + 1), ord(L.ng);
+        if (cudaMemcpyAsync(p.data(), L.gop_ptr, sizeof(int) * (L.ng + 1), cudaMemcpyDeviceToHost, s) != cudaSuccess ||
+            cudaStreamSynchronize(s) != cudaSuccess) {
+            err = "ghost rows failed";
+            return SULF_EDEVICE;
+        }
+        int n[4] = {0, 0, 0, 0};
+        auto part = [&](int g) {
+            const int len = p[g + 1] - p[g];
+            return len <= kGopPre ? 0 : (len <= kGopPre * kGopLanes ? 1 : 2);
+        };
+        for (int g = 0; g < L.ng; g++) n[part(g) + 1]++;
+        S.ng1 = n[1];
+        S.ng8 = n[2];
+        n[2] += n[1];
+        for (int g = 0; g < L.ng; g++) ord[n[part(g)]++] = g;
+        if (cudaMemcpyAsync(S.gord, ord.data(), sizeof(int) * L.ng, cudaMemcpyHostToDevice, s) != cudaSuccess ||
+            cudaStreamSynchronize(s) != cudaSuccess) {
+            err = "ghost rows failed";
+            return SULF_EDEVICE;
+        }
     }
     k_gop_codes<<<nblk(L.gop_nnz), 256, 0, s>>>(L.gop_code, (int)L.gop_nnz, L.gpos, L.n, L.dim, S.H, S.Hn, S.gcode);
     const int K = L.dim == 2 ? 9 : 27;
@@ -1240,7 +1373,7 @@ int launch_s_relax(const SLev<D, T>& L, int colour, bool delta, bool snap, const
 template <int D, typename T>
 int launch_s_ghosts(const SLev<D, T>& L, const int* skip, double* acc, cudaStream_t s) {
     if (L.ng == 0) return 0;
-    const long long nt = (long long)L.ng * kGopLanes;
+    const long long nt = ghost_threads<D, T>(L, kGopLanes, 32);
     launch_k(k_s_ghosts<D, T>, grid_for(nt), block_for(nt), 0, s, L, skip, acc);
     return 1;
 }
@@ -1248,7 +1381,7 @@ int launch_s_ghosts(const SLev<D, T>& L, const int* skip, double* acc, cudaStrea
 template <int D, typename T>
 int launch_s_residual(const SLev<D, T>& L, unsigned long long* norm, int* clear, cudaStream_t s) {
     const int nrow = (L.n0 + L.nga + 31) / 32 * 32;
-    const long long tot = nrow + (long long)L.ng * kRowLanes;
+    const long long tot = nrow + ghost_threads<D>(L, kGopLanes, kGopLanes);
     launch_k(norm ? k_s_residual<D, T, true> : k_s_residual<D, T, false>, grid_for(tot), block_for(tot), 0, s, L, nrow,
              norm, clear);
     return 1;
@@ -1258,14 +1391,14 @@ template <int D>
 int launch_s_outer(const SLev<D, double>& L, const SLev<D, float>& U, unsigned long long* norm, int* clear,
                    cudaStream_t s) {
     const int nrow = (L.n0 + L.n1 + 31) / 32 * 32;
-    const long long tot = nrow + (long long)L.ng * kRowLanes;
+    const long long tot = nrow + ghost_threads<D>(L, kGopLanes, kGopLanes);
     launch_k(k_s_outer<D>, grid_for(tot), block_for(tot), 0, s, L, U, nrow, norm, clear);
     return 1;
 }
 
 template <int D, typename T>
 int launch_s_restrict(const SLev<D, T>& F, const SLev<D, T>& C, cudaStream_t s) {
-    const int nrow = (C.n0 + C.n1 + 31) / 32 * 32;
+    const int nreg = C.nreg0 + C.nreg1, nrow = up32(nreg) + up32(C.n0 + C.n1 - nreg);
     const long long tot = nrow + (long long)C.ng * kGopLanes;
     launch_k(k_s_restrict<D, T>, grid_for(tot), block_for(tot), 0, s, F, C, nrow);
     return 1;

@@ -32,7 +32,9 @@
 // H = (n + 1) / 2, so that a colour's update reads whole sectors of the other
 // colour and writes whole sectors of its own.  What belongs to one row of the
 // system (gt, dd, 1/dd, b~) is stored in the order of the row list: red inside
-// nodes, black inside nodes, ghosts, each colour's nodes next to a ghost last.
+// nodes, black inside nodes, ghosts; in each colour the nodes with a regular
+// restriction first and those next to a ghost last, so that the cases of a
+// kernel fall into different warps.
 #pragma once
 
 #include "mg_stages.cuh"
@@ -57,6 +59,7 @@ struct SLev {
     int n, H, P, Hn;   // nodes per axis, row and plane pitch, half size
     int n0, n1, ng;    // red and black inside nodes, ghosts
     int nga;           // black nodes next to a ghost (the last ones)
+    int nreg0, nreg1;  // red and black nodes with a regular restriction (the first ones)
     const int* hl;     // entries of the inside nodes
     const int* gslot;  // slots of the ghosts
     const int* gidx;   // box nodes of the ghosts
@@ -79,15 +82,21 @@ struct SLev {
     const int* gptr;
     const int* gcode;
     const T* gval;
+    // the ghosts by the length of that row: ng1 of up to 4 entries, ng8 of up
+    // to 32, the longer ones
+    const int* gord;
+    int ng1, ng8;
     // ghost rows: slot and weight of the members
     const int* rptr;
     const int* rslot;
     const T* rval;
-    // restriction onto this level (from the next finer one): slot of the fine
-    // twin of an inside node whose 3^D members are inside and away from the
-    // ghosts (else -1), and the ghosts' rows over the finer level's ghost
-    // defects (extension along the normal, then outside weighting)
+    // restriction onto this level (from the next finer one): slot of an inside
+    // node's fine twin; bits of the 3^D fine members that are inside nodes (a
+    // regular node's are all, its black ones away from the ghosts); and the
+    // ghosts' rows over the finer level's ghost defects (extension along the
+    // normal, then outside weighting)
     const int* twin;
+    const int* mask;
     const int* cptr;
     const int* cslot;
     const T* cval;
@@ -102,15 +111,16 @@ struct SLev {
 // geometry of a level in these terms (precision independent)
 struct SGeo {
     bool ready = false;
-    int H = 0, P = 0, Hn = 0, n0 = 0, n1 = 0, nga = 0;
+    int H = 0, P = 0, Hn = 0, n0 = 0, n1 = 0, nga = 0, nreg0 = 0, nreg1 = 0, ng1 = 0, ng8 = 0;
     int* hl = nullptr;
     int* gslot = nullptr;
     int* gcode = nullptr;
+    int* gord = nullptr;
     long long gcap = 0;
     int *rptr = nullptr, *rslot = nullptr;
     double* rval = nullptr;
     float* rval32 = nullptr;
-    int* twin = nullptr;
+    int *twin = nullptr, *mask = nullptr;
     int *cptr = nullptr, *cslot = nullptr;
     double* cval = nullptr;
     float* cval32 = nullptr;
@@ -143,6 +153,11 @@ SLev<D, T> make_slev(const LevelGeo& G, const SGeo& S, const SVec<T>& V) {
     s.n1 = S.n1;
     s.ng = G.ng;
     s.nga = S.nga;
+    s.nreg0 = S.nreg0;
+    s.nreg1 = S.nreg1;
+    s.gord = S.gord;
+    s.ng1 = S.ng1;
+    s.ng8 = S.ng8;
     s.hl = S.hl;
     s.gslot = S.gslot;
     s.gidx = G.gidx;
@@ -165,6 +180,7 @@ SLev<D, T> make_slev(const LevelGeo& G, const SGeo& S, const SVec<T>& V) {
     s.rslot = S.rslot;
     s.rval = f ? (const T*)S.rval32 : (const T*)S.rval;
     s.twin = S.twin;
+    s.mask = S.mask;
     s.cptr = S.cptr;
     s.cslot = S.cslot;
     s.cval = f ? (const T*)S.cval32 : (const T*)S.cval;
