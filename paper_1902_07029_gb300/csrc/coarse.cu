@@ -31,6 +31,11 @@ __device__ __forceinline__ unsigned cta_rank() {
     asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
     return r;
 }
+__device__ __forceinline__ unsigned cluster_size() {
+    unsigned r;
+    asm volatile("mov.u32 %0, %%cluster_nctarank;" : "=r"(r));
+    return r;
+}
 __device__ __forceinline__ void cluster_barrier() {
     asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
     asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
@@ -543,9 +548,14 @@ struct Coarse {
 // (inlined per call site and per kind of level the kernel had 144 KB of code
 // and its phases took two to three times as long).
 template <int D, typename T>
-__global__ void __launch_bounds__(kCoarseThreads, 1) k_s_coarse(const CDesc<T>* __restrict__ dp) {
+__global__ void __launch_bounds__(kCoarseThreads, 1) k_s_coarse(const CDesc<T>* __restrict__ one,
+                                                                   const CDesc<T>* const* __restrict__ many,
+                                                                   const int* __restrict__ active) {
     extern __shared__ __align__(16) char coarse_smem[];
-    const CDesc<T>& d = *dp;
+    // many domains (lock-step batching): a cluster each, masked ones skipped
+    const int inst = many ? (int)(blockIdx.x / cluster_size()) : 0;
+    if (many && !active[inst]) return;
+    const CDesc<T>& d = many ? *many[inst] : *one;
     Coarse<D, T> k;
     k.sm = coarse_smem;
     k.sa = (unsigned)__cvta_generic_to_shared(coarse_smem);
@@ -689,11 +699,12 @@ struct HostLevel {
 
 template <int D, typename T>
 int build_coarse(CoarseSet<T>& S, const LevelGeo* G, const SGeo* SG, const SVec<T>* V, int L, int want, int nu1,
-                 int nu2, double* acc, DevMem& mem, cudaStream_t s, std::string& err) {
+                 int nu2, int max_cta, double* acc, DevMem& mem, cudaStream_t s, std::string& err) {
     S.l0 = -1;
     S.want = want;
     S.nu1 = nu1;
     S.nu2 = nu2;
+    S.max_cta = max_cta;
     S.rows = true;
     if (want < 0 || want > L - 1) return SULF_OK;
     const bool f32 = std::is_same<T, float>::value;
@@ -754,6 +765,7 @@ int build_coarse(CoarseSet<T>& S, const LevelGeo* G, const SGeo* SG, const SVec<
     bool fit = false;
     for (; l0 < L && !fit; l0++) {
         for (int C : {8, 16}) {
+            if (C > max_cta) break;
             const int n = L - l0;
             ncta = C;
             // deal the nodes: bands of the box order (slots are box order up to
@@ -1203,39 +1215,53 @@ int build_coarse(CoarseSet<T>& S, const LevelGeo* G, const SGeo* SG, const SVec<
         err = "coarse-level tables failed";
         return SULF_EDEVICE;
     }
-    S.nthr = kCoarseThreads;
     S.smem = smem;
     S.ncta = C;
     S.l0 = l0;
     return SULF_OK;
 }
 
+namespace {
 template <int D, typename T>
-int launch_coarse(const CoarseSet<T>& S, cudaStream_t s) {
-    auto kern = k_s_coarse<D, T>;
+int launch_clusters(int K, int ncta, size_t smem, const CDesc<T>* one, const CDesc<T>* const* many, const int* active,
+                    cudaStream_t s) {
+    raise_limits<D, T>();
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(S.ncta);
-    cfg.blockDim = dim3(S.nthr);
-    cfg.dynamicSmemBytes = S.smem;
+    cfg.gridDim = dim3(K * ncta);
+    cfg.blockDim = dim3(kCoarseThreads);
+    cfg.dynamicSmemBytes = smem;
     cfg.stream = s;
     cudaLaunchAttribute at[2];
     at[0].id = cudaLaunchAttributeClusterDimension;
-    at[0].val.clusterDim.x = S.ncta;
+    at[0].val.clusterDim.x = ncta;
     at[0].val.clusterDim.y = 1;
     at[0].val.clusterDim.z = 1;
     at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     at[1].val.programmaticStreamSerializationAllowed = launch_pdl() ? 1 : 0;
     cfg.attrs = at;
     cfg.numAttrs = 2;
-    cudaError_t e = cudaLaunchKernelEx(&cfg, kern, (const CDesc<T>*)S.dev);
-    if (e != cudaSuccess) note_launch_error(e, S.ncta, kCoarseThreads, S.smem);
+    cudaError_t e = cudaLaunchKernelEx(&cfg, k_s_coarse<D, T>, one, many, active);
+    if (e != cudaSuccess) note_launch_error(e, K * ncta, kCoarseThreads, smem);
     return 1;
+}
+}  // namespace
+
+template <int D, typename T>
+int launch_coarse(const CoarseSet<T>& S, cudaStream_t s) {
+    return launch_clusters<D, T>(1, S.ncta, S.smem, S.dev, nullptr, nullptr, s);
+}
+
+template <int D, typename T>
+int launch_coarse_batched(const CDesc<T>* const* descs, int K, const int* active, int ncta, size_t smem,
+                          cudaStream_t s) {
+    return launch_clusters<D, T>(K, ncta, smem, nullptr, descs, active, s);
 }
 
 #define SULF_INST_COARSE(D, T)                                                                                      \
     template int build_coarse<D, T>(CoarseSet<T>&, const LevelGeo*, const SGeo*, const SVec<T>*, int, int, int, int, \
-                                    double*, DevMem&, cudaStream_t, std::string&);                                            \
-    template int launch_coarse<D, T>(const CoarseSet<T>&, cudaStream_t);
+                                    int, double*, DevMem&, cudaStream_t, std::string&);                                            \
+    template int launch_coarse<D, T>(const CoarseSet<T>&, cudaStream_t);                                          \
+    template int launch_coarse_batched<D, T>(const CDesc<T>* const*, int, const int*, int, size_t, cudaStream_t);
 SULF_INST_COARSE(2, double)
 SULF_INST_COARSE(2, float)
 SULF_INST_COARSE(3, double)

@@ -70,10 +70,10 @@ struct CDesc {
 template <typename T>
 struct CoarseSet {
     int l0 = -1;
-    int want = -2, nu1 = 0, nu2 = 0;  // what it was built for
+    int want = -2, nu1 = 0, nu2 = 0, max_cta = 0;  // what it was built for
     bool rows = false;      // built for the current boundary rows
     size_t smem = 0;
-    int ncta = 0, nthr = 0;
+    int ncta = 0;
     CDesc<T>* dev = nullptr;
     CPerm* perm[SULF_MAXLEV] = {};  // device, per level
     T* coef = nullptr;
@@ -91,8 +91,13 @@ struct CoarseSet {
 // l0 = -1 where none does
 template <int D, typename T>
 int build_coarse(CoarseSet<T>& S, const LevelGeo* G, const SGeo* SG, const SVec<T>* V, int L, int want, int nu1,
-                 int nu2, double* acc, DevMem& mem, cudaStream_t s, std::string& err);
+                 int nu2, int max_cta, double* acc, DevMem& mem, cudaStream_t s, std::string& err);
 template <int D, typename T>
 int launch_coarse(const CoarseSet<T>& S, cudaStream_t s);
+// the fused levels of K domains (device array of their descriptors), a cluster
+// each; masked ones skipped
+template <int D, typename T>
+int launch_coarse_batched(const CDesc<T>* const* descs, int K, const int* active, int ncta, size_t smem,
+                          cudaStream_t s);
 
 }  // namespace sulf

@@ -201,10 +201,13 @@ __global__ void __launch_bounds__(kT) k_s_coefs(SLev<D, T> L, SLev<D, float> U,
 // ---------------------------------------------------------------------------
 // relaxation
 
+// Each phase of the cycle is a function of a level and a thread's place in its
+// work; one kernel takes the level of one domain, another the levels of many
+// (lock-step batching): CTA b serves the domain i with pre[i] <= b < pre[i+1].
 template <int D, typename T, bool DELTA>
-__global__ void __launch_bounds__(kT) k_s_relax(SLev<D, T> L, int colour, int snap, const int* skip, double* acc) {
+__device__ __forceinline__ void s_relax(const SLev<D, T>& L, int t, int colour, bool snap, bool use_skip,
+                                        bool use_acc) {
     typedef typename V2<T>::t T2;
-    const int t = blockIdx.x * blockDim.x + threadIdx.x;
     const int cnt = colour ? L.n1 : L.n0, pos = (colour ? L.n0 : 0) + t;
     // the row is fixed during the linear solve: fetched while the previous
     // kernel is still running
@@ -220,7 +223,7 @@ __global__ void __launch_bounds__(kT) k_s_relax(SLev<D, T> L, int colour, int sn
     nbr_offsets<D, T>(L, e & 1, o);
     const int sg = snap && t < L.ng ? L.gslot[t] : 0;
     pdl_enter();
-    if (skip && *skip) return;
+    if (use_skip && *L.skip) return;
     if (snap && t < L.ng) L.snap[t] = L.X[sg];
     if (t >= cnt) return;
     const int h = e >> kEntHalf, so = (1 - colour) * L.Hn + h, sl = colour * L.Hn + h;
@@ -248,7 +251,7 @@ __global__ void __launch_bounds__(kT) k_s_relax(SLev<D, T> L, int colour, int sn
     for (int q = 0; q < 2 * D; q++) r = fmadd(g[q], x[q], r);
     r *= di;
     L.X[sl] = r;
-    if (acc) acc[sl] += (double)r;
+    if (use_acc) L.acc[sl] += (double)r;
 }
 
 template <int D, typename T>
@@ -305,8 +308,8 @@ __device__ __forceinline__ T part_sum(T v, int lanes) {
 // all passes of a sweep's ghost relaxation, one composed row per ghost
 constexpr int kGopPre = 4;
 template <int D, typename T>
-__global__ void __launch_bounds__(kT) k_s_ghosts(SLev<D, T> L, const int* skip, double* acc) {
-    const GhostPart p = ghost_part<D, T>(L, blockIdx.x * blockDim.x + threadIdx.x, kGopLanes, 32);
+__device__ __forceinline__ void s_ghosts(const SLev<D, T>& L, int t, bool use_skip, bool use_acc) {
+    const GhostPart p = ghost_part<D, T>(L, t, kGopLanes, 32);
     int beg = 0, end = 0, sl = 0;
     int cd[kGopPre];
     T w[kGopPre];
@@ -322,7 +325,7 @@ __global__ void __launch_bounds__(kT) k_s_ghosts(SLev<D, T> L, const int* skip, 
         sl = L.gslot[p.g];
     }
     pdl_enter();
-    if (skip && *skip) return;
+    if (use_skip && *L.skip) return;
     T v = 0;
     if (p.on) {
         for (int j = beg;;) {
@@ -345,7 +348,7 @@ __global__ void __launch_bounds__(kT) k_s_ghosts(SLev<D, T> L, const int* skip, 
     v = part_sum<T>(v, p.lanes);
     if (!p.on || p.lane != 0) return;
     L.X[sl] = v;
-    if (acc) acc[sl] += (double)v;
+    if (use_acc) L.acc[sl] += (double)v;
 }
 
 // ---------------------------------------------------------------------------
@@ -379,9 +382,8 @@ __device__ __forceinline__ T ghost_defect(const SLev<D, T>& L, const GhostPart& 
 }
 
 template <int D, typename T, bool NORM>
-__global__ void __launch_bounds__(kT) k_s_residual(SLev<D, T> L, int nrow, unsigned long long* norm, int* clear) {
-    const int t = blockIdx.x * blockDim.x + threadIdx.x;
-    const int nin = L.n0 + L.nga;  // rows of inside nodes; nrow: rounded up to whole warps
+__device__ __forceinline__ void s_residual(const SLev<D, T>& L, int t, unsigned long long* norm) {
+    const int nin = L.n0 + L.nga, nrow = up32(nin);  // rows of inside nodes, in whole warps
     int e = 0, pos = 0, colour = 0;
     T g[2 * D], dd = 0;
     if (t < nin) {
@@ -393,7 +395,7 @@ __global__ void __launch_bounds__(kT) k_s_residual(SLev<D, T> L, int nrow, unsig
         dd = L.dd[pos];
     }
     pdl_enter();
-    if (clear && t == 0) *clear = 0;
+    if (NORM && t == 0) *L.skip = 0;  // the next cycle runs its first sweep
     T r = 0;
     if (t < nrow) {
         if (t < nin) {
@@ -411,10 +413,9 @@ __global__ void __launch_bounds__(kT) k_s_residual(SLev<D, T> L, int nrow, unsig
 // mixed precision: the FP64 defect of every row into the FP32 right-hand
 // side; the FP32 error starts with its red half-sweep from zero
 template <int D>
-__global__ void __launch_bounds__(kT) k_s_outer(SLev<D, double> L, SLev<D, float> U, int nrow,
-                                                 unsigned long long* norm, int* clear) {
-    const int t = blockIdx.x * blockDim.x + threadIdx.x;
-    const int nin = L.n0 + L.n1;
+__device__ __forceinline__ void s_outer(const SLev<D, double>& L, const SLev<D, float>& U, int t,
+                                        unsigned long long* norm) {
+    const int nin = L.n0 + L.n1, nrow = up32(nin);
     int e = 0;
     double g[2 * D], dd = 0;
     float df = 0;
@@ -427,7 +428,7 @@ __global__ void __launch_bounds__(kT) k_s_outer(SLev<D, double> L, SLev<D, float
         if (!colour) df = U.di[t];
     }
     pdl_enter();
-    if (t == 0) *clear = 0;
+    if (t == 0) *U.skip = 0;
     double r = 0;
     if (t < nrow) {
         if (t < nin) {
@@ -492,9 +493,8 @@ __device__ __forceinline__ T restrict_near(const SLev<D, T>& F, int tw, unsigned
 // the finer level's defect onto the coarse level's right-hand side; the coarse
 // error starts with its red half-sweep from zero
 template <int D, typename T>
-__global__ void __launch_bounds__(kT) k_s_restrict(SLev<D, T> F, SLev<D, T> C, int nrow) {
-    const int t = blockIdx.x * blockDim.x + threadIdx.x;
-    const int nin = C.n0 + C.n1, nreg = C.nreg0 + C.nreg1, freg = up32(nreg);
+__device__ __forceinline__ void s_restrict(const SLev<D, T>& F, const SLev<D, T>& C, int t) {
+    const int nin = C.n0 + C.n1, nreg = C.nreg0 + C.nreg1, freg = up32(nreg), nrow = freg + up32(nin - nreg);
     // regular nodes, then (from a whole warp on) the others
     int pos = -1, tw = 0, e = 0;
     unsigned m = 0;
@@ -560,9 +560,8 @@ __global__ void __launch_bounds__(kT) k_s_restrict(SLev<D, T> F, SLev<D, T> C, i
 // active corners (Sec. 3.5.3), at the black nodes and the ghosts; the
 // corners' x^c is -rho x^s
 template <int D, typename T>
-__global__ void __launch_bounds__(kT) k_s_prolong(SLev<D, T> F, SLev<D, T> C) {
+__device__ __forceinline__ void s_prolong(const SLev<D, T>& F, const SLev<D, T>& C, int t) {
     typedef typename V2<T>::t T2;
-    const int t = blockIdx.x * blockDim.x + threadIdx.x;
     const bool on = t < F.n1 + F.ng;
     int cn[1 << D];
     T cr[1 << D];
@@ -833,12 +832,12 @@ __global__ void __launch_bounds__(kFacThreads) k_s_factor(SLev<D, T> L, const in
 
 // x = A^{-1} b: one warp per row
 template <int D, typename T>
-__global__ void __launch_bounds__(256) k_s_solve(SLev<D, T> L, const T* __restrict__ Ainv) {
+__device__ __forceinline__ void s_solve(const SLev<D, T>& L, int t) {
     const int nin = L.n0 + L.n1, m = nin + L.ng;
-    const int r = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+    const int r = t >> 5, lane = t & 31;
     pdl_enter();
     if (r >= m) return;
-    const T* row = Ainv + (size_t)r * m;
+    const T* row = L.Ainv + (size_t)r * m;
     T v = 0;
     for (int j = lane; j < m; j += 32) v = fmadd(row[j], L.b[j], v);
     for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
@@ -849,12 +848,83 @@ __global__ void __launch_bounds__(256) k_s_solve(SLev<D, T> L, const T* __restri
 }
 
 // ---------------------------------------------------------------------------
+// the phases as kernels, of one domain and of many
+
+enum { kPhRelax = 0, kPhDelta, kPhGhosts, kPhResidual, kPhNorm, kPhRestrict, kPhProlong, kPhSolve };
+
+// flags: 1 black colour, 2 snap, 4 skip on the flag, 8 accumulate
+template <int D, typename T, int PH>
+__device__ __forceinline__ void s_phase(const SLev<D, T>& L, const SLev<D, T>& C, int t, int flags,
+                                        unsigned long long* norm) {
+    if (PH == kPhRelax) s_relax<D, T, false>(L, t, flags & 1, flags & 2, flags & 4, flags & 8);
+    if (PH == kPhDelta) s_relax<D, T, true>(L, t, flags & 1, flags & 2, flags & 4, flags & 8);
+    if (PH == kPhGhosts) s_ghosts<D, T>(L, t, flags & 4, flags & 8);
+    if (PH == kPhResidual) s_residual<D, T, false>(L, t, norm);
+    if (PH == kPhNorm) s_residual<D, T, true>(L, t, norm);
+    if (PH == kPhRestrict) s_restrict<D, T>(L, C, t);
+    if (PH == kPhProlong) s_prolong<D, T>(L, C, t);
+    if (PH == kPhSolve) s_solve<D, T>(L, t);
+}
+
+template <int D, typename T, int PH>
+__global__ void __launch_bounds__(kT) k_s_phase(const __grid_constant__ SLev<D, T> L,
+                                                 const __grid_constant__ SLev<D, T> C, int flags,
+                                                 unsigned long long* norm) {
+    s_phase<D, T, PH>(L, C, blockIdx.x * blockDim.x + threadIdx.x, flags, norm);
+}
+
+// (single-level phases: one level parameter less to copy per launch)
+template <int D, typename T, int PH>
+__global__ void __launch_bounds__(kT) k_s_phase1(const __grid_constant__ SLev<D, T> L, int flags,
+                                                  unsigned long long* norm) {
+    s_phase<D, T, PH>(L, L, blockIdx.x * blockDim.x + threadIdx.x, flags, norm);
+}
+
+template <int D>
+__global__ void __launch_bounds__(kT) k_s_outer(const __grid_constant__ SLev<D, double> L,
+                                                 const __grid_constant__ SLev<D, float> U, unsigned long long* norm) {
+    s_outer<D>(L, U, blockIdx.x * blockDim.x + threadIdx.x, norm);
+}
+
+__device__ __forceinline__ int find_instance(const int* __restrict__ pre, int K, int b) {
+    int lo = 0, hi = K;  // pre[0] = 0 <= b < pre[K]
+    while (hi - lo > 1) {
+        const int mid = (lo + hi) >> 1;
+        if (pre[mid] <= b)
+            lo = mid;
+        else
+            hi = mid;
+    }
+    return lo;
+}
+
+template <int D, typename T, int PH>
+__global__ void __launch_bounds__(kT) kb_s_phase(const SLev<D, T>* __restrict__ lv, const SLev<D, T>* __restrict__ lc,
+                                                  const int* __restrict__ pre, int K, const int* __restrict__ active,
+                                                  int flags, unsigned long long* norms) {
+    const int i = find_instance(pre, K, blockIdx.x);
+    if (!active[i]) return;
+    s_phase<D, T, PH>(lv[i], lc[i], (blockIdx.x - pre[i]) * kT + threadIdx.x, flags, norms + i);
+}
+
+template <int D>
+__global__ void __launch_bounds__(kT) kb_s_outer(const SLev<D, double>* __restrict__ l64,
+                                                  const SLev<D, float>* __restrict__ l32, const int* __restrict__ pre,
+                                                  int K, const int* __restrict__ active, unsigned long long* norms) {
+    const int i = find_instance(pre, K, blockIdx.x);
+    if (!active[i]) return;
+    s_outer<D>(l64[i], l32[i], (blockIdx.x - pre[i]) * kT + threadIdx.x, norms + i);
+}
+
+// ---------------------------------------------------------------------------
 // end of a linear solve
 
 template <int D>
 __global__ void __launch_bounds__(kT) k_s_update(SLev<D, double> L, const double* __restrict__ tt,
-                                                  double2* __restrict__ W, unsigned long long* norms) {
+                                                  double2* __restrict__ W, unsigned long long* norms,
+                                                  const int* __restrict__ on) {
     pdl_enter();
+    if (on && !*on) return;
     const int t = blockIdx.x * blockDim.x + threadIdx.x;
     unsigned long long nx = 0, nw = 0;
     if (t < L.n0 + L.n1 + L.ng) {
@@ -1360,55 +1430,124 @@ int launch_s_coefs_fine(const SLev<D, double>& L, const double2* Wc, const Coef<
     return 1;
 }
 
-template <int D, typename T>
-int launch_s_relax(const SLev<D, T>& L, int colour, bool delta, bool snap, const int* skip, double* acc,
-                   cudaStream_t s) {
-    const int cnt = colour ? L.n1 : L.n0, tot = snap && L.ng > cnt ? L.ng : cnt;
-    if (tot == 0) return 0;
-    launch_k(delta ? k_s_relax<D, T, true> : k_s_relax<D, T, false>, grid_for(tot), block_for(tot), 0, s, L, colour,
-             snap ? 1 : 0, skip, acc);
+namespace {
+template <int D, typename T, int PH>
+int launch_one(const SLev<D, T>& L, long long threads, int flags, unsigned long long* norm, cudaStream_t s) {
+    if (threads <= 0) return 0;
+    launch_k(k_s_phase1<D, T, PH>, grid_for(threads), block_for(threads), 0, s, L, flags, norm);
     return 1;
+}
+inline int relax_flags(int colour, bool snap, bool skip, bool acc) {
+    return (colour ? 1 : 0) | (snap ? 2 : 0) | (skip ? 4 : 0) | (acc ? 8 : 0);
+}
+}  // namespace
+
+template <int D, typename T>
+long long s_threads(SPhase ph, const SLev<D, T>& L, const SLev<D, T>* C) {
+    switch (ph) {
+        case SPhase::red: return L.n0;
+        case SPhase::black: return L.n1 > L.ng ? L.n1 : L.ng;
+        case SPhase::ghosts: return ghost_threads<D, T>(L, kGopLanes, 32);
+        case SPhase::residual: return up32(L.n0 + L.nga) + (long long)ghost_threads<D, T>(L, kGopLanes, kGopLanes);
+        case SPhase::outer: return up32(L.n0 + L.n1) + (long long)ghost_threads<D, T>(L, kGopLanes, kGopLanes);
+        case SPhase::restrict_to:
+            return up32(C->nreg0 + C->nreg1) + up32(C->n0 + C->n1 - C->nreg0 - C->nreg1) + (long long)C->ng * kGopLanes;
+        case SPhase::prolong_from: return (long long)L.n1 + L.ng;
+        case SPhase::solve: return 32LL * (L.n0 + L.n1 + L.ng);
+    }
+    return 0;
 }
 
 template <int D, typename T>
-int launch_s_ghosts(const SLev<D, T>& L, const int* skip, double* acc, cudaStream_t s) {
-    if (L.ng == 0) return 0;
-    const long long nt = ghost_threads<D, T>(L, kGopLanes, 32);
-    launch_k(k_s_ghosts<D, T>, grid_for(nt), block_for(nt), 0, s, L, skip, acc);
-    return 1;
+int launch_s_relax(const SLev<D, T>& L, int colour, bool delta, bool snap, bool skip, bool acc, cudaStream_t s) {
+    const long long n = colour && snap ? s_threads<D, T>(SPhase::black, L, nullptr) : (colour ? L.n1 : L.n0);
+    const int fl = relax_flags(colour, snap, skip, acc);
+    return delta ? launch_one<D, T, kPhDelta>(L, n, fl, nullptr, s) : launch_one<D, T, kPhRelax>(L, n, fl, nullptr, s);
 }
 
 template <int D, typename T>
-int launch_s_residual(const SLev<D, T>& L, unsigned long long* norm, int* clear, cudaStream_t s) {
-    const int nrow = (L.n0 + L.nga + 31) / 32 * 32;
-    const long long tot = nrow + ghost_threads<D>(L, kGopLanes, kGopLanes);
-    launch_k(norm ? k_s_residual<D, T, true> : k_s_residual<D, T, false>, grid_for(tot), block_for(tot), 0, s, L, nrow,
-             norm, clear);
-    return 1;
+int launch_s_ghosts(const SLev<D, T>& L, bool skip, bool acc, cudaStream_t s) {
+    return launch_one<D, T, kPhGhosts>(L, s_threads<D, T>(SPhase::ghosts, L, nullptr), relax_flags(0, false, skip, acc),
+                                       nullptr, s);
+}
+
+template <int D, typename T>
+int launch_s_residual(const SLev<D, T>& L, unsigned long long* norm, cudaStream_t s) {
+    const long long n = s_threads<D, T>(SPhase::residual, L, nullptr);
+    return norm ? launch_one<D, T, kPhNorm>(L, n, 0, norm, s) : launch_one<D, T, kPhResidual>(L, n, 0, norm, s);
 }
 
 template <int D>
-int launch_s_outer(const SLev<D, double>& L, const SLev<D, float>& U, unsigned long long* norm, int* clear,
-                   cudaStream_t s) {
-    const int nrow = (L.n0 + L.n1 + 31) / 32 * 32;
-    const long long tot = nrow + ghost_threads<D>(L, kGopLanes, kGopLanes);
-    launch_k(k_s_outer<D>, grid_for(tot), block_for(tot), 0, s, L, U, nrow, norm, clear);
+int launch_s_outer(const SLev<D, double>& L, const SLev<D, float>& U, unsigned long long* norm, cudaStream_t s) {
+    const long long n = s_threads<D, double>(SPhase::outer, L, nullptr);
+    launch_k(k_s_outer<D>, grid_for(n), block_for(n), 0, s, L, U, norm);
     return 1;
 }
 
 template <int D, typename T>
 int launch_s_restrict(const SLev<D, T>& F, const SLev<D, T>& C, cudaStream_t s) {
-    const int nreg = C.nreg0 + C.nreg1, nrow = up32(nreg) + up32(C.n0 + C.n1 - nreg);
-    const long long tot = nrow + (long long)C.ng * kGopLanes;
-    launch_k(k_s_restrict<D, T>, grid_for(tot), block_for(tot), 0, s, F, C, nrow);
+    const long long n = s_threads<D, T>(SPhase::restrict_to, F, &C);
+    launch_k(k_s_phase<D, T, kPhRestrict>, grid_for(n), block_for(n), 0, s, F, C, 0, (unsigned long long*)nullptr);
     return 1;
 }
 
 template <int D, typename T>
 int launch_s_prolong(const SLev<D, T>& F, const SLev<D, T>& C, cudaStream_t s) {
-    const int tot = F.n1 + F.ng;
-    if (tot == 0) return 0;
-    launch_k(k_s_prolong<D, T>, grid_for(tot), block_for(tot), 0, s, F, C);
+    const long long n = s_threads<D, T>(SPhase::prolong_from, F, &C);
+    if (n == 0) return 0;
+    launch_k(k_s_phase<D, T, kPhProlong>, grid_for(n), block_for(n), 0, s, F, C, 0, (unsigned long long*)nullptr);
+    return 1;
+}
+
+template <int D, typename T>
+int launch_s_solve(const SLev<D, T>& L, cudaStream_t s) {
+    return launch_one<D, T, kPhSolve>(L, s_threads<D, T>(SPhase::solve, L, nullptr), 0, nullptr, s);
+}
+
+template <int D, typename T>
+int launch_s_batched(SPhase ph, bool delta, const SLev<D, T>* lv, const SLev<D, T>* lc, const int* pre, int nblocks,
+                     int K, const int* active, bool skip, bool acc, unsigned long long* norms, cudaStream_t s) {
+    if (nblocks <= 0) return 0;
+    const unsigned nb = (unsigned)nblocks;
+    if (!lc) lc = lv;
+    const int fl = relax_flags(ph == SPhase::black, ph == SPhase::black, skip, acc);
+    switch (ph) {
+        case SPhase::red:
+        case SPhase::black:
+            if (delta)
+                launch_k(kb_s_phase<D, T, kPhDelta>, nb, kT, 0, s, lv, lc, pre, K, active, fl, norms);
+            else
+                launch_k(kb_s_phase<D, T, kPhRelax>, nb, kT, 0, s, lv, lc, pre, K, active, fl, norms);
+            break;
+        case SPhase::ghosts:
+            launch_k(kb_s_phase<D, T, kPhGhosts>, nb, kT, 0, s, lv, lc, pre, K, active, fl, norms);
+            break;
+        case SPhase::residual:
+            if (norms)
+                launch_k(kb_s_phase<D, T, kPhNorm>, nb, kT, 0, s, lv, lc, pre, K, active, fl, norms);
+            else
+                launch_k(kb_s_phase<D, T, kPhResidual>, nb, kT, 0, s, lv, lc, pre, K, active, fl, norms);
+            break;
+        case SPhase::restrict_to:
+            launch_k(kb_s_phase<D, T, kPhRestrict>, nb, kT, 0, s, lv, lc, pre, K, active, fl, norms);
+            break;
+        case SPhase::prolong_from:
+            launch_k(kb_s_phase<D, T, kPhProlong>, nb, kT, 0, s, lv, lc, pre, K, active, fl, norms);
+            break;
+        case SPhase::solve:
+            launch_k(kb_s_phase<D, T, kPhSolve>, nb, kT, 0, s, lv, lc, pre, K, active, fl, norms);
+            break;
+        default:
+            return 0;
+    }
+    return 1;
+}
+
+template <int D>
+int launch_s_batched_outer(const SLev<D, double>* l64, const SLev<D, float>* l32, const int* pre, int nblocks, int K,
+                           const int* active, unsigned long long* norms, cudaStream_t s) {
+    if (nblocks <= 0) return 0;
+    launch_k(kb_s_outer<D>, (unsigned)nblocks, kT, 0, s, l64, l32, pre, K, active, norms);
     return 1;
 }
 
@@ -1451,18 +1590,11 @@ int launch_s_factor(const SLev<D, T>& L, const int* spos, const int* cpos, T* A,
     return 1;
 }
 
-template <int D, typename T>
-int launch_s_solve(const SLev<D, T>& L, const T* Ainv, cudaStream_t s) {
-    const int m = L.n0 + L.n1 + L.ng;
-    launch_k(k_s_solve<D, T>, (m + 7) / 8, 256, 0, s, L, Ainv);
-    return 1;
-}
-
 template <int D>
-int launch_s_update(const SLev<D, double>& L, const double* tt, double2* W, unsigned long long* norms,
+int launch_s_update(const SLev<D, double>& L, const double* tt, double2* W, unsigned long long* norms, const int* on,
                     cudaStream_t s) {
     const int tot = L.n0 + L.n1 + L.ng;
-    launch_k(k_s_update<D>, grid_for(tot), block_for(tot), 0, s, L, tt, W, norms);
+    launch_k(k_s_update<D>, grid_for(tot), block_for(tot), 0, s, L, tt, W, norms, on);
     return 1;
 }
 
@@ -1485,13 +1617,16 @@ int launch_inject_to(const LevelGeo& F, const typename V2<TF>::t* fW, const Leve
 #define SULF_INST_S(D, T)                                                                                          \
     template int launch_s_rho<D, T>(const SLev<D, T>&, const typename V2<T>::t*, const Coef<T>&, cudaStream_t);     \
     template int launch_s_coefs<D, T>(const SLev<D, T>&, const typename V2<T>::t*, const Coef<T>&, cudaStream_t);   \
-    template int launch_s_relax<D, T>(const SLev<D, T>&, int, bool, bool, const int*, double*, cudaStream_t);      \
-    template int launch_s_ghosts<D, T>(const SLev<D, T>&, const int*, double*, cudaStream_t);                      \
-    template int launch_s_residual<D, T>(const SLev<D, T>&, unsigned long long*, int*, cudaStream_t);              \
+    template long long s_threads<D, T>(SPhase, const SLev<D, T>&, const SLev<D, T>*);                              \
+    template int launch_s_relax<D, T>(const SLev<D, T>&, int, bool, bool, bool, bool, cudaStream_t);               \
+    template int launch_s_ghosts<D, T>(const SLev<D, T>&, bool, bool, cudaStream_t);                               \
+    template int launch_s_residual<D, T>(const SLev<D, T>&, unsigned long long*, cudaStream_t);                    \
     template int launch_s_restrict<D, T>(const SLev<D, T>&, const SLev<D, T>&, cudaStream_t);                      \
     template int launch_s_prolong<D, T>(const SLev<D, T>&, const SLev<D, T>&, cudaStream_t);                       \
     template int launch_s_factor<D, T>(const SLev<D, T>&, const int*, const int*, T*, T*, int*, cudaStream_t);     \
-    template int launch_s_solve<D, T>(const SLev<D, T>&, const T*, cudaStream_t);
+    template int launch_s_solve<D, T>(const SLev<D, T>&, cudaStream_t);                                            \
+    template int launch_s_batched<D, T>(SPhase, bool, const SLev<D, T>*, const SLev<D, T>*, const int*, int, int,  \
+                                        const int*, bool, bool, unsigned long long*, cudaStream_t);
 SULF_INST_S(2, double)
 SULF_INST_S(2, float)
 SULF_INST_S(3, double)
@@ -1501,10 +1636,12 @@ SULF_INST_S(3, float)
                                       double*, const SLev<D, float>*, cudaStream_t);                               \
     template int launch_s_coefs_fine<D>(const SLev<D, double>&, const double2*, const Coef<double>&,               \
                                         const double2*, const double*, const SLev<D, float>*, cudaStream_t);       \
-    template int launch_s_outer<D>(const SLev<D, double>&, const SLev<D, float>&, unsigned long long*, int*,       \
+    template int launch_s_outer<D>(const SLev<D, double>&, const SLev<D, float>&, unsigned long long*,             \
                                    cudaStream_t);                                                                  \
+    template int launch_s_batched_outer<D>(const SLev<D, double>*, const SLev<D, float>*, const int*, int, int,    \
+                                           const int*, unsigned long long*, cudaStream_t);                         \
     template int launch_s_update<D>(const SLev<D, double>&, const double*, double2*, unsigned long long*,          \
-                                    cudaStream_t);                                                                 \
+                                    const int*, cudaStream_t);                                                     \
     template int launch_s_export<D>(const SLev<D, double>&, const double*, double2*, cudaStream_t);                \
     template int launch_inject_to<D, double, double>(const LevelGeo&, const double2*, const LevelGeo&, double2*,   \
                                                      cudaStream_t);                                                \

@@ -106,7 +106,14 @@ struct SLev {
     T* cf;
     const int* bpos;
     T* bf;
+    const T* Ainv;  // coarsest level
+    int* skip;      // finest level: set where the first sweep of the cycle has been done
+    double* acc;    // finest FP32 level: the FP64 update its error is added to
 };
+
+// phases of the cycle over a level (restriction and prolongation: a level and
+// the next coarser one)
+enum class SPhase { red, black, ghosts, residual, outer, restrict_to, prolong_from, solve };
 
 // geometry of a level in these terms (precision independent)
 struct SGeo {
@@ -188,6 +195,9 @@ SLev<D, T> make_slev(const LevelGeo& G, const SGeo& S, const SVec<T>& V) {
     s.cf = nullptr;
     s.bpos = nullptr;
     s.bf = nullptr;
+    s.Ainv = V.Ainv;
+    s.skip = nullptr;
+    s.acc = nullptr;
     return s;
 }
 
@@ -216,22 +226,23 @@ int launch_s_coefs(const SLev<D, T>& L, const typename V2<T>::t* Wc, const Coef<
 template <int D>
 int launch_s_coefs_fine(const SLev<D, double>& L, const double2* Wc, const Coef<double>& c, const double2* F,
                         const double* tt, const SLev<D, float>* U, cudaStream_t s);
+// threads of a phase
+template <int D, typename T>
+long long s_threads(SPhase ph, const SLev<D, T>& L, const SLev<D, T>* C);
 // one colour; snap: also the ghosts' s into snap; skip: return at once where
-// *skip is set; acc: FP64 array (slots) the new values are added to
+// *L.skip is set; acc: the new values are added to L.acc
 template <int D, typename T>
-int launch_s_relax(const SLev<D, T>& L, int colour, bool delta, bool snap, const int* skip, double* acc,
-                   cudaStream_t s);
+int launch_s_relax(const SLev<D, T>& L, int colour, bool delta, bool snap, bool skip, bool acc, cudaStream_t s);
 template <int D, typename T>
-int launch_s_ghosts(const SLev<D, T>& L, const int* skip, double* acc, cudaStream_t s);
+int launch_s_ghosts(const SLev<D, T>& L, bool skip, bool acc, cudaStream_t s);
 // defect of the red nodes, of the black ones next to a ghost and of the
-// ghosts into R (norm null), or its max-norm only; clear: a flag set to 0
+// ghosts into R (norm null), or its max-norm only (and *L.skip set to 0)
 template <int D, typename T>
-int launch_s_residual(const SLev<D, T>& L, unsigned long long* norm, int* clear, cudaStream_t s);
+int launch_s_residual(const SLev<D, T>& L, unsigned long long* norm, cudaStream_t s);
 // mixed precision: the FP64 defect of every row with its max-norm, stored as
-// the FP32 right-hand side, and the FP32 error's start; clear as above
+// the FP32 right-hand side, and the FP32 error's start (and *U.skip set to 0)
 template <int D>
-int launch_s_outer(const SLev<D, double>& L, const SLev<D, float>& U, unsigned long long* norm, int* clear,
-                   cudaStream_t s);
+int launch_s_outer(const SLev<D, double>& L, const SLev<D, float>& U, unsigned long long* norm, cudaStream_t s);
 template <int D, typename T>
 int launch_s_restrict(const SLev<D, T>& F, const SLev<D, T>& C, cudaStream_t s);
 template <int D, typename T>
@@ -242,10 +253,19 @@ template <int D, typename T>
 int launch_s_factor(const SLev<D, T>& L, const int* spos, const int* cpos, T* A, T* Ainv, int* singular,
                     cudaStream_t s);
 template <int D, typename T>
-int launch_s_solve(const SLev<D, T>& L, const T* Ainv, cudaStream_t s);
-// W -= (x, t - rho x) on the active nodes with the norms of launch_newton_update
+int launch_s_solve(const SLev<D, T>& L, cudaStream_t s);
+// a phase of K domains in one launch (CTAs of kNodeThreads; masked domains are
+// skipped; a residual with norms is the finest one's norms)
+template <int D, typename T>
+int launch_s_batched(SPhase ph, bool delta, const SLev<D, T>* lv, const SLev<D, T>* lc, const int* pre, int nblocks,
+                     int K, const int* active, bool skip, bool acc, unsigned long long* norms, cudaStream_t s);
 template <int D>
-int launch_s_update(const SLev<D, double>& L, const double* tt, double2* W, unsigned long long* norms,
+int launch_s_batched_outer(const SLev<D, double>* l64, const SLev<D, float>* l32, const int* pre, int nblocks, int K,
+                           const int* active, unsigned long long* norms, cudaStream_t s);
+// W -= (x, t - rho x) on the active nodes with the norms of launch_newton_update
+// (nothing where *on is zero)
+template <int D>
+int launch_s_update(const SLev<D, double>& L, const double* tt, double2* W, unsigned long long* norms, const int* on,
                     cudaStream_t s);
 // (x, t - rho x) in box order (debug outputs)
 template <int D>

@@ -412,26 +412,30 @@ int alloc_schur(sulf_domain* d, SVec<T>* V, int nl, bool outer) {
     return ok ? SULF_OK : sulf_fail(SULF_ENOMEM, "out of device memory");
 }
 
-// the fused coarse levels of the current threshold (sulf_solver::fuse_below)
+// the fused coarse levels of the current threshold (sulf_solver::fuse_below);
+// at_least: the first of them no finer than this level; max_cta: cluster size
 template <typename T>
-int ensure_coarse(sulf_domain* d, CoarseSet<T>& S, const SVec<T>* V) {
+int ensure_coarse(sulf_domain* d, CoarseSet<T>& S, const SVec<T>* V, int at_least = 1, int max_cta = kCoarseMaxCta) {
     int want = -1;
     const int fb = d->solver.fuse_below >= 0 ? d->solver.fuse_below : kCoarseAuto;
     if (fb > 0 && d->solver.cycle == 1)
-        for (int l = 1; l < d->L && want < 0; l++)
+        for (int l = at_least; l < d->L && want < 0; l++)
             if ((long long)d->geo[l].nin[0] + d->geo[l].nin[1] + d->geo[l].ng <= fb) want = l;
     const int nu1 = d->solver.nu1, nu2 = d->solver.nu2;
-    if (S.rows && S.want == want && S.nu1 == nu1 && S.nu2 == nu2) return SULF_OK;
+    if (S.rows && S.want == want && S.nu1 == nu1 && S.nu2 == nu2 && S.max_cta == max_cta) return SULF_OK;
     SULF_CUDA_TRY(cudaStreamSynchronize(d->stream));
     drop_graphs(d);
     std::string err;
-    int rc = d->dim == 2 ? build_coarse<2, T>(S, d->geo, d->sgeo, V, d->L, want, nu1, nu2, nullptr, d->mem, d->stream, err)
-                         : build_coarse<3, T>(S, d->geo, d->sgeo, V, d->L, want, nu1, nu2, nullptr, d->mem, d->stream, err);
+    int rc = d->dim == 2 ? build_coarse<2, T>(S, d->geo, d->sgeo, V, d->L, want, nu1, nu2, max_cta, nullptr, d->mem,
+                                              d->stream, err)
+                         : build_coarse<3, T>(S, d->geo, d->sgeo, V, d->L, want, nu1, nu2, max_cta, nullptr, d->mem,
+                                              d->stream, err);
     return rc ? sulf_fail(rc, err) : SULF_OK;
 }
 
-// decides d->s_on for the next linear solve and builds what it needs
-int ensure_schur(sulf_domain* d);
+// decides d->s_on for the next linear solve and builds what it needs (coarse:
+// the fused levels too)
+int ensure_schur(sulf_domain* d, bool coarse = true);
 int ensure_path(sulf_domain* d) {
     if (int rc = ensure_schur(d)) return rc;
     if (d->s_on) return SULF_OK;
@@ -439,7 +443,7 @@ int ensure_path(sulf_domain* d) {
     return d->solver.precision == 1 ? ensure32(d) : SULF_OK;
 }
 
-int ensure_schur(sulf_domain* d) {
+int ensure_schur(sulf_domain* d, bool coarse) {
     d->s_on = false;
     if (!schur_wanted(d) || d->s_geo < 0) return SULF_OK;
     for (int l = 0; l < d->L; l++) {
@@ -479,11 +483,13 @@ int ensure_schur(sulf_domain* d) {
     }
     if (d->solver.precision == 0) {
         if (int rc = alloc_schur<double>(d, d->s64, d->L, false)) return rc;
-        if (int rc = ensure_coarse<double>(d, d->cs64, d->s64)) return rc;
+        if (coarse)
+            if (int rc = ensure_coarse<double>(d, d->cs64, d->s64)) return rc;
     } else {
         if (int rc = alloc_schur<double>(d, d->s64, 1, true)) return rc;
         if (int rc = alloc_schur<float>(d, d->s32, d->L, false)) return rc;
-        if (int rc = ensure_coarse<float>(d, d->cs32, d->s32)) return rc;
+        if (coarse)
+            if (int rc = ensure_coarse<float>(d, d->cs32, d->s32)) return rc;
     }
     d->s_on = true;
     return SULF_OK;
@@ -698,7 +704,6 @@ template <int D, typename T>
 struct SMG {
     sulf_domain* d;
     SVec<T>* V;
-    double* acc = nullptr;  // mixed precision: the FP64 update the finest error is added to
     int fine_sweeps = 0;
 
     const CoarseSet<T>& fused() const {
@@ -719,11 +724,15 @@ struct SMG {
                 s.bf = S.b;
             }
         }
+        if (l == 0) {
+            s.skip = d->dskip;
+            s.acc = std::is_same<T, float>::value ? d->s64[0].X : nullptr;
+        }
         return s;
     }
 
-    // delta: the sweep follows a prolongation; a: see launch_s_relax
-    void relax(int l, bool skip_red, bool delta, const int* skip, double* a) {
+    // delta: the sweep follows a prolongation; skip, add: see launch_s_relax
+    void relax(int l, bool skip_red, bool delta, bool skip, bool add) {
         const SLev<D, T> L = lev(l);
         // timed sweeps: both colours launched and not skipped on a flag
         const bool whole = l == 0 && !skip_red && !skip;
@@ -731,33 +740,33 @@ struct SMG {
         if (whole) fine_sweeps++;
         const unsigned fl = d->capturing ? cudaEventRecordExternal : cudaEventRecordDefault;
         if (timed) cudaEventRecordWithFlags(next_event(d), d->stream, fl);
-        if (!skip_red) d->launches += launch_s_relax<D, T>(L, 0, delta, false, skip, a, d->stream);
-        d->launches += launch_s_relax<D, T>(L, 1, delta, true, skip, a, d->stream);
+        if (!skip_red) d->launches += launch_s_relax<D, T>(L, 0, delta, false, skip, add, d->stream);
+        d->launches += launch_s_relax<D, T>(L, 1, delta, true, skip, add, d->stream);
         if (timed) cudaEventRecordWithFlags(next_event(d), d->stream, fl);
-        d->launches += launch_s_ghosts<D, T>(L, skip, a, d->stream);
+        d->launches += launch_s_ghosts<D, T>(L, skip, add, d->stream);
     }
 
-    // red_done: the first red half-sweep (from zero) came with the
-    // right-hand side; first: device flag, set where the whole first sweep
-    // has been done
-    int cycle(int l, bool red_done, const int* first) {
+    // red_done: the first red half-sweep (from zero) came with the right-hand
+    // side; the finest level's first sweep is skipped where its flag is set;
+    // in FP32 its last one adds the error to the FP64 update
+    int cycle(int l, bool red_done) {
         const sulf_solver& sv = d->solver;
         if (l == fused().l0) {
             d->launches += launch_coarse<D, T>(fused(), d->stream);
             return SULF_OK;
         }
         if (l == d->L - 1) {
-            d->launches += launch_s_solve<D, T>(lev(l), V[l].Ainv, d->stream);
+            d->launches += launch_s_solve<D, T>(lev(l), d->stream);
             return SULF_OK;
         }
-        for (int k = 0; k < sv.nu1; k++) relax(l, red_done && k == 0, false, k == 0 ? first : nullptr, nullptr);
-        d->launches += launch_s_residual<D, T>(lev(l), nullptr, nullptr, d->stream);
+        for (int k = 0; k < sv.nu1; k++) relax(l, red_done && k == 0, false, l == 0 && k == 0, false);
+        d->launches += launch_s_residual<D, T>(lev(l), nullptr, d->stream);
         d->launches += launch_s_restrict<D, T>(lev(l), lev(l + 1), d->stream);
         for (int g = 0; g < (sv.cycle == 2 ? 2 : 1); g++)
-            if (int rc = cycle(l + 1, g == 0, nullptr)) return rc;
+            if (int rc = cycle(l + 1, g == 0)) return rc;
         d->launches += launch_s_prolong<D, T>(lev(l), lev(l + 1), d->stream);
         for (int k = 0; k < sv.nu2; k++)
-            relax(l, false, k == 0, nullptr, l == 0 && k == sv.nu2 - 1 ? acc : nullptr);
+            relax(l, false, k == 0, false, std::is_same<T, float>::value && l == 0 && k == sv.nu2 - 1);
         return SULF_OK;
     }
 
@@ -788,7 +797,7 @@ struct SMG {
 
 template <int D>
 SLev<D, double> fine_slev(sulf_domain* d) {
-    return make_slev<D, double>(d->geo[0], d->sgeo[0], d->s64[0]);
+    return SMG<D, double>{d, d->s64}.lev(0);
 }
 
 // set-up of a linear solve J dW = F in this form: the rows of every level, the
@@ -805,14 +814,14 @@ int schur_prepare(sulf_domain* d) {
         d->launches += launch_s_rho_fine<D>(L0, d->W, c0, F, tt, &U, d->stream);
         d->launches += launch_s_coefs_fine<D>(L0, d->W, c0, F, tt, &U, d->stream);
         if (int rc = SMG<D, float>{d, d->s32}.prepare_coarse()) return rc;
-        d->launches += launch_s_relax<D, float>(U, 1, true, true, nullptr, nullptr, d->stream);
-        d->launches += launch_s_ghosts<D, float>(U, nullptr, nullptr, d->stream);
+        d->launches += launch_s_relax<D, float>(U, 1, true, true, false, false, d->stream);
+        d->launches += launch_s_ghosts<D, float>(U, false, false, d->stream);
     } else {
         d->launches += launch_s_rho_fine<D>(L0, d->W, c0, F, tt, nullptr, d->stream);
         d->launches += launch_s_coefs_fine<D>(L0, d->W, c0, F, tt, nullptr, d->stream);
         if (int rc = SMG<D, double>{d, d->s64}.prepare_coarse()) return rc;
-        d->launches += launch_s_relax<D, double>(L0, 1, true, true, nullptr, nullptr, d->stream);
-        d->launches += launch_s_ghosts<D, double>(L0, nullptr, nullptr, d->stream);
+        d->launches += launch_s_relax<D, double>(L0, 1, true, true, false, false, d->stream);
+        d->launches += launch_s_ghosts<D, double>(L0, false, false, d->stream);
     }
     SULF_CUDA_TRY(cudaMemsetAsync(d->dskip, 1, sizeof(int), d->stream));
     SULF_CUDA_TRY(cudaMemsetAsync(d->dnorm, 0, sizeof(unsigned long long) * 2, d->stream));
@@ -866,12 +875,11 @@ int cycle_body(sulf_domain* d, const cudaGraphConditionalHandle* loop = nullptr,
         if (!loop) SULF_CUDA_TRY(cudaMemsetAsync(d->dnorm, 0, sizeof(unsigned long long) * 2, d->stream));
         const SLev<D, double> L0 = fine_slev<D>(d);
         if (d->solver.precision == 0) {
-            if (int rc = SMG<D, double>{d, d->s64}.cycle(0, false, d->dskip)) return rc;
-            d->launches += launch_s_residual<D, double>(L0, d->dnorm, d->dskip, d->stream);
+            if (int rc = SMG<D, double>{d, d->s64}.cycle(0, false)) return rc;
+            d->launches += launch_s_residual<D, double>(L0, d->dnorm, d->stream);
         } else {
-            if (int rc = SMG<D, float>{d, d->s32, d->s64[0].X}.cycle(0, true, d->dskip)) return rc;
-            d->launches += launch_s_outer<D>(L0, make_slev<D, float>(G0, d->sgeo[0], d->s32[0]), d->dnorm, d->dskip,
-                                             d->stream);
+            if (int rc = SMG<D, float>{d, d->s32}.cycle(0, true)) return rc;
+            d->launches += launch_s_outer<D>(L0, SMG<D, float>{d, d->s32}.lev(0), d->dnorm, d->stream);
         }
         return cycle_end(d, loop, max_cycles);
     }
@@ -1161,7 +1169,7 @@ int cn_step(sulf_domain* d) {
         d->cycles_total += nc;
         SULF_CUDA_TRY(cudaMemsetAsync(d->dnorm, 0, sizeof(unsigned long long) * 4, d->stream));
         if (d->s_on)
-            d->launches += launch_s_update<D>(fine_slev<D>(d), d->s64[0].tt, d->W, d->dnorm, d->stream);
+            d->launches += launch_s_update<D>(fine_slev<D>(d), d->s64[0].tt, d->W, d->dnorm, nullptr, d->stream);
         else
             d->launches += launch_newton_update(G0, d->W, V0.x, d->dnorm, d->stream);
         d->launches += launch_newton_F<D>(G0, d->W, d->G, V0.rhs, V0.rhsc, fc, d->dnorm + 2, d->stream);
@@ -1929,6 +1937,16 @@ struct LockClass {
     int ltail = -1;
     const void* const* dtail = nullptr;
     std::vector<const LevelGeo*> geos;
+    // the cycle on the equation for s (schur.cuh) where every instance runs it:
+    // the levels, work lists per phase (SPhase) and the fused coarse levels
+    bool schur = false;
+    const SLev<D, double>* s64[SULF_MAXLEV] = {};
+    const SLev<D, float>* s32[SULF_MAXLEV] = {};
+    Blocks sb[SULF_MAXLEV][8];
+    int scoarse = -1, sncta = 0;
+    size_t ssmem = 0;
+    const void* sdesc = nullptr;
+    int* dnewton = nullptr;  // instance still in its Newton loop
     // branches of the per-instance phases (instance i on aux[i % naux])
     static constexpr int kMaxAux = 8;
     cudaStream_t aux[kMaxAux] = {};
@@ -2032,8 +2050,137 @@ struct LockClass {
         return SULF_OK;
     }
 
+    template <typename T>
+    static CoarseSet<T>& coarse_of(sulf_domain* d) {
+        if constexpr (std::is_same<T, double>::value)
+            return d->cs64;
+        else
+            return d->cs32;
+    }
+    template <typename T>
+    static SVec<T>* svec_of(sulf_domain* d) {
+        if constexpr (std::is_same<T, double>::value)
+            return d->s64;
+        else
+            return d->s32;
+    }
+
+    template <typename T>
+    int upload_slevels(int nl, const SLev<D, T>** out) {
+        for (int l = 0; l < nl; l++) {
+            std::vector<SLev<D, T>> v;
+            for (int i = 0; i < K; i++) v.push_back(SMG<D, T>{h[i], svec_of<T>(h[i])}.lev(l));
+            SLev<D, T>* dv = (SLev<D, T>*)mem->get(sizeof(SLev<D, T>) * K);
+            if (!dv) return sulf_fail(SULF_ENOMEM, "out of device memory");
+            SULF_CUDA_TRY(cudaMemcpyAsync(dv, v.data(), sizeof(SLev<D, T>) * K, cudaMemcpyHostToDevice, s));
+            SULF_CUDA_TRY(cudaStreamSynchronize(s));  // the host vector goes out of scope
+            out[l] = dv;
+        }
+        return SULF_OK;
+    }
+
+    // the levels, lists and coarse clusters of the cycle in precision T
+    template <typename T>
+    int setup_schur(const SLev<D, T>** out) {
+        // all instances fuse the same levels, on clusters of 8 CTAs
+        for (int first = 1;;) {
+            int worst = 0, none = 0;
+            for (int i = 0; i < K; i++) {
+                CoarseSet<T>& S = coarse_of<T>(h[i]);
+                if (int rc = ensure_coarse<T>(h[i], S, svec_of<T>(h[i]), first, 8)) return rc;
+                none += S.l0 < 0;
+                worst = std::max(worst, S.l0);
+                ssmem = i ? std::max(ssmem, S.smem) : S.smem;
+            }
+            if (none == K) break;
+            if (none) {
+                first = L;  // one has none: none for all
+                continue;
+            }
+            bool same = true;
+            for (int i = 0; i < K; i++) same = same && coarse_of<T>(h[i]).l0 == worst;
+            if (same) {
+                scoarse = worst;
+                sncta = 8;
+                break;
+            }
+            first = worst;
+        }
+        if (int rc = upload_slevels<T>(L, out)) return rc;
+        for (int l = 0; l < L; l++)
+            for (int p = 0; p < 8; p++) {
+                const SPhase ph = (SPhase)p;
+                const bool pair = ph == SPhase::restrict_to || ph == SPhase::prolong_from;
+                if ((pair && l + 1 >= L) || (scoarse >= 0 && l >= scoarse)) continue;
+                std::vector<long long> n(K);
+                for (int i = 0; i < K; i++) {
+                    SMG<D, T> m{h[i], svec_of<T>(h[i])};
+                    const SLev<D, T> a = m.lev(l), c = m.lev(pair ? l + 1 : l);
+                    n[i] = s_threads<D, T>(ph, a, &c);
+                }
+                if (int rc = upload_blocks(sb[l][p], n, kNodeThreads)) return rc;
+            }
+        if (scoarse >= 0) {
+            std::vector<const CDesc<T>*> dd;
+            for (int i = 0; i < K; i++) dd.push_back(coarse_of<T>(h[i]).dev);
+            void* p = mem->get(sizeof(void*) * K);
+            if (!p) return sulf_fail(SULF_ENOMEM, "out of device memory");
+            SULF_CUDA_TRY(cudaMemcpyAsync(p, dd.data(), sizeof(void*) * K, cudaMemcpyHostToDevice, s));
+            SULF_CUDA_TRY(cudaStreamSynchronize(s));
+            sdesc = p;
+        }
+        return SULF_OK;
+    }
+
+    template <typename T>
+    void srun(const SLev<D, T>* const* lv, SPhase ph, int l, bool delta, bool skip, bool add) {
+        const Blocks& b = sb[l][(int)ph];
+        const bool pair = ph == SPhase::restrict_to || ph == SPhase::prolong_from;
+        launches += launch_s_batched<D, T>(ph, delta, lv[l], pair ? lv[l + 1] : nullptr, b.d, b.total, K, dactive, skip,
+                                           add, nullptr, s);
+    }
+
+    // as SMG::cycle
+    template <typename T>
+    void scycle(const SLev<D, T>* const* lv, int l, bool red_done) {
+        const sulf_solver& sv = h[0]->solver;
+        if (l == scoarse) {
+            launches += launch_coarse_batched<D, T>((const CDesc<T>* const*)sdesc, K, dactive, sncta, ssmem, s);
+            return;
+        }
+        if (l == L - 1) {
+            srun<T>(lv, SPhase::solve, l, false, false, false);
+            return;
+        }
+        auto sweep = [&](bool skip_red, bool delta, bool skip, bool add) {
+            if (!skip_red) srun<T>(lv, SPhase::red, l, delta, skip, add);
+            srun<T>(lv, SPhase::black, l, delta, skip, add);
+            srun<T>(lv, SPhase::ghosts, l, false, skip, add);
+        };
+        for (int k = 0; k < sv.nu1; k++) sweep(red_done && k == 0, false, l == 0 && k == 0, false);
+        srun<T>(lv, SPhase::residual, l, false, false, false);
+        srun<T>(lv, SPhase::restrict_to, l, false, false, false);
+        scycle<T>(lv, l + 1, true);
+        srun<T>(lv, SPhase::prolong_from, l, false, false, false);
+        for (int k = 0; k < sv.nu2; k++)
+            sweep(false, k == 0, false, std::is_same<T, float>::value && l == 0 && k == sv.nu2 - 1);
+    }
+
     int setup() {
         const bool mixed = h[0]->solver.precision == 1;
+        dnewton = (int*)mem->get(sizeof(int) * K);
+        if (!dnewton) return sulf_fail(SULF_ENOMEM, "out of memory");
+        if (schur) {
+            int rc;
+            if (mixed) {
+                rc = setup_schur<float>(s32);
+                if (!rc) rc = upload_slevels<double>(1, s64);
+            } else {
+                rc = setup_schur<double>(s64);
+            }
+            if (rc) return rc;
+            return setup_common();
+        }
         if (int rc = upload_levels<double>([](sulf_domain* d) { return d->v64; }, l64)) return rc;
         if (mixed)
             if (int rc = upload_levels<float>([](sulf_domain* d) { return d->v32; }, l32)) return rc;
@@ -2059,18 +2206,7 @@ struct LockClass {
             max_nact = std::max(max_nact, h[i]->geo[L - 1].nact);
         }
         if (int rc = upload_blocks(coarse, rows, kBatchT / 32)) return rc;
-        dactive = (int*)mem->get(sizeof(int) * K);
-        dnorm = (unsigned long long*)mem->get(sizeof(unsigned long long) * K);
-        hnorm = (unsigned long long*)mem->get_host(sizeof(unsigned long long) * K);
-        if (!dactive || !dnorm || !hnorm) return sulf_fail(SULF_ENOMEM, "out of memory");
-        active.assign(K, 0);
-        SULF_CUDA_TRY(cudaEventCreateWithFlags(&ev_fork, cudaEventDisableTiming));
-        naux = std::min(K, kMaxAux);
-        for (int j = 0; j < naux; j++) {
-            SULF_CUDA_TRY(cudaStreamCreateWithFlags(&aux[j], cudaStreamNonBlocking));
-            SULF_CUDA_TRY(cudaEventCreateWithFlags(&ev_join[j], cudaEventDisableTiming));
-        }
-        graphs = h[0]->solver.graphs != 0;
+        if (int rc = setup_common()) return rc;
         // the fused coarse levels: from the first level that every
         // instance's threshold fuses
         for (int i = 0; i < K; i++) {
@@ -2096,6 +2232,23 @@ struct LockClass {
             SULF_CUDA_TRY(cudaStreamSynchronize(s));
             dtail = (const void* const*)p;
         }
+        SULF_CUDA_TRY(cudaStreamSynchronize(s));
+        return SULF_OK;
+    }
+
+    int setup_common() {
+        dactive = (int*)mem->get(sizeof(int) * K);
+        dnorm = (unsigned long long*)mem->get(sizeof(unsigned long long) * K);
+        hnorm = (unsigned long long*)mem->get_host(sizeof(unsigned long long) * K);
+        if (!dactive || !dnorm || !hnorm) return sulf_fail(SULF_ENOMEM, "out of memory");
+        active.assign(K, 0);
+        SULF_CUDA_TRY(cudaEventCreateWithFlags(&ev_fork, cudaEventDisableTiming));
+        naux = std::min(K, kMaxAux);
+        for (int j = 0; j < naux; j++) {
+            SULF_CUDA_TRY(cudaStreamCreateWithFlags(&aux[j], cudaStreamNonBlocking));
+            SULF_CUDA_TRY(cudaEventCreateWithFlags(&ev_join[j], cudaEventDisableTiming));
+        }
+        graphs = h[0]->solver.graphs != 0;
         SULF_CUDA_TRY(cudaStreamSynchronize(s));
         return SULF_OK;
     }
@@ -2148,6 +2301,21 @@ struct LockClass {
     // defect with each instance's max-norm (copied to hnorm)
     int cycle_body() {
         const bool mixed = h[0]->solver.precision == 1;
+        if (schur) {
+            if (mixed)
+                scycle<float>(s32, 0, true);
+            else
+                scycle<double>(s64, 0, false);
+            SULF_CUDA_TRY(cudaMemsetAsync(dnorm, 0, sizeof(unsigned long long) * K, s));
+            const Blocks& b = sb[0][(int)(mixed ? SPhase::outer : SPhase::residual)];
+            if (mixed)
+                launches += launch_s_batched_outer<D>(s64[0], s32[0], b.d, b.total, K, dactive, dnorm, s);
+            else
+                launches += launch_s_batched<D, double>(SPhase::residual, false, s64[0], nullptr, b.d, b.total, K,
+                                                        dactive, false, false, dnorm, s);
+            SULF_CUDA_TRY(cudaMemcpyAsync(hnorm, dnorm, sizeof(unsigned long long) * K, cudaMemcpyDeviceToHost, s));
+            return SULF_OK;
+        }
         if (mixed) {
             launches += launch_batched_mixed<D>(BPhase::zero32, l64[0], l32[0], act[0].d, act[0].total, K, dactive,
                                                 s);
@@ -2224,14 +2392,21 @@ int lockstep_step(LockClass<D>& C, LockGraphs<D>& P, int* status, std::vector<st
         bool any = false;
         for (int i = 0; i < K; i++) any = any || inewton[i];
         if (!any) break;
+        if (C.schur) {
+            // (an instance out of its loop keeps its state: no update)
+            SULF_CUDA_TRY(cudaMemcpyAsync(C.dnewton, inewton.data(), sizeof(int) * K, cudaMemcpyHostToDevice, C.s));
+            SULF_CUDA_TRY(cudaStreamSynchronize(C.s));
+        }
         // per instance: the Jacobian of this Newton iteration on every level
         rc = C.run_phase(P.prepare, [&] {
             return C.per_instance([&](int i, cudaStream_t b) {
                 sulf_domain* d = C.h[i];
                 const LevelGeo& G0 = d->geo[0];
-                SULF_CUDA_TRY(cudaMemsetAsync(d->v64[0].x, 0, sizeof(double2) * G0.nn, b));
                 int r;
-                if (sv.precision == 0) {
+                if (!C.schur) SULF_CUDA_TRY(cudaMemsetAsync(d->v64[0].x, 0, sizeof(double2) * G0.nn, b));
+                if (C.schur) {
+                    r = schur_prepare<D>(d);
+                } else if (sv.precision == 0) {
                     r = MG<D, double>{d, d->v64}.prepare();
                 } else {
                     d->launches += launch_to_float(G0, d->W, d->v32[0].Wc, b);
@@ -2288,7 +2463,10 @@ int lockstep_step(LockClass<D>& C, LockGraphs<D>& P, int* status, std::vector<st
                 const LevelGeo& G0 = d->geo[0];
                 FConst fc = make_fconst(d);
                 SULF_CUDA_TRY(cudaMemsetAsync(d->dnorm, 0, sizeof(unsigned long long) * 4, b));
-                d->launches += launch_newton_update(G0, d->W, d->v64[0].x, d->dnorm, b);
+                if (C.schur)
+                    d->launches += launch_s_update<D>(fine_slev<D>(d), d->s64[0].tt, d->W, d->dnorm, C.dnewton + i, b);
+                else
+                    d->launches += launch_newton_update(G0, d->W, d->v64[0].x, d->dnorm, b);
                 d->launches += launch_newton_F<D>(G0, d->W, d->G, d->v64[0].rhs, d->v64[0].rhsc, fc, d->dnorm + 2, b);
                 SULF_CUDA_TRY(
                     cudaMemcpyAsync(d->hnorm, d->dnorm, sizeof(unsigned long long) * 3, cudaMemcpyDeviceToHost, b));
@@ -2342,13 +2520,19 @@ int lockstep_run(const std::vector<sulf_domain*>& hs, double dt, int nsteps, int
     C.L = hs[0]->L;
     C.s = s;
     C.mem = &mem;
+    C.schur = true;
     for (sulf_domain* d : hs) {
         d->dt = dt;
-        if (int rc = ensure64(d)) return rc;
-        if (d->solver.precision == 1)
-            if (int rc = ensure32(d)) return rc;
         if (int rc = refresh_ghost_ops(d)) return rc;
+        if (int rc = ensure_schur(d, false)) return rc;  // (its fused levels: setup_schur)
+        C.schur = C.schur && d->s_on;
     }
+    if (!C.schur)
+        for (sulf_domain* d : hs) {
+            if (int rc = ensure64(d)) return rc;
+            if (d->solver.precision == 1)
+                if (int rc = ensure32(d)) return rc;
+        }
     if (int rc = C.setup()) return rc;
     PdlScope pdl(hs[0]->solver.pdl != 0, 0, 0);
     LockGraphs<D> P;
