@@ -1047,19 +1047,20 @@ __global__ void __launch_bounds__(256) k_coarsest_solve(int nact, const int* __r
 // ---------------------------------------------------------------------------
 // Newton residual (Eqs. FDs, FDc, BCs), FP64
 
+// Written for the FP64 pipe, which bounds these kernels (two lanes per SM and
+// clock): phi_q + phi_p as one multiply-add, the reaction's phi s c once for
+// both equations: 28 FP64 instructions per 3-D node (257^3 box: 620 us with 39).
 template <int D>
-__device__ __forceinline__ double Ls_h(long long p, const double2* __restrict__ W, const Offs<D>& of,
-                                       const FConst& f, double& ph_out) {
-    double2 w = W[p];
-    double ph = f.alpha * w.y + f.beta;
+__device__ __forceinline__ double flux_sum(long long p, double2 w, double ph, const double2* __restrict__ W,
+                                           const Offs<D>& of, const FConst& f) {
+    const double bp = f.beta + ph;
+    double2 wq[2 * D];
+#pragma unroll
+    for (int q = 0; q < 2 * D; q++) wq[q] = W[p + of.o[q]];
     double flux = 0.0;
 #pragma unroll
-    for (int q = 0; q < 2 * D; q++) {
-        double2 wq = W[p + of.o[q]];
-        flux += ((f.alpha * wq.y + f.beta) + ph) * (wq.x - w.x);
-    }
-    ph_out = ph;
-    return -f.amc * ph * w.x * w.y + f.dh2 * flux;
+    for (int q = 0; q < 2 * D; q++) flux = fma(fma(f.alpha, wq[q].y, bp), wq[q].x - w.x, flux);
+    return flux;
 }
 
 // old-time part G = -M(W^n)/dt - L(W^n)/2 of the CN step (once per step)
@@ -1071,16 +1072,14 @@ __global__ void __launch_bounds__(kT) k_old_time(Lists ls, const double2* __rest
     if (t >= ls.n0 + ls.n1 + ls.ng) return;
     int kind, gi;
     long long p = list_node(ls, t, kind, gi);
-    double2 w = Wn[p];
-    double ph = f.alpha * w.y + f.beta;
-    double Lc = -f.ams * ph * w.x * w.y;
+    const double2 w = Wn[p];
+    const double ph = fma(f.alpha, w.y, f.beta), ps = ph * w.x, psc = ps * w.y;
     double2 g;
-    g.y = -w.y * f.idt - 0.5 * Lc;
+    g.y = fma(0.5 * f.ams, psc, -w.y * f.idt);
     g.x = 0.0;
     if (kind == 1) {
-        double phd;
-        double Ls = Ls_h<D>(p, Wn, of, f, phd);
-        g.x = -ph * w.x * f.idt - 0.5 * Ls;
+        const double Ls = fma(f.dh2, flux_sum<D>(p, w, ph, Wn, of, f), -f.amc * psc);
+        g.x = fma(-0.5, Ls, -ps * f.idt);
     }
     if (f.src) {  // manufactured sources: F^s -= (f1o + f1n)/2 inside, F^c -= (f2o + f2n)/2
         double2 q = f.src[p];
@@ -1097,30 +1096,44 @@ __global__ void k_average_sources(long long nn, const double* __restrict__ f4, d
     src[i] = make_double2(0.5 * (f4[i] + f4[nn + i]), 0.5 * (f4[2 * nn + i] + f4[3 * nn + i]));
 }
 
-template <int D>
-__global__ void __launch_bounds__(kT) k_newton_F(Lists ls, GhostTab<double> tb, const double2* __restrict__ W, const double2* __restrict__ G,
-                                                  double2* __restrict__ F, double2* __restrict__ Fc, Offs<D> of,
-                                                  long long st1, long long st2, FConst f, unsigned long long* norm) {
+// FIRST: at W = W^n, writing the step's old-time part too; with
+// G = -M/dt - L/2 the residual M/dt - L/2 + G there is -L (minus the sources)
+template <int D, bool FIRST>
+__global__ void __launch_bounds__(kT) k_newton_F(Lists ls, GhostTab<double> tb, const double2* __restrict__ W,
+                                                  double2* __restrict__ G, double2* __restrict__ F,
+                                                  double2* __restrict__ Fc, Offs<D> of, FConst f,
+                                                  unsigned long long* norm) {
     pdl_enter();
     int t = blockIdx.x * blockDim.x + threadIdx.x;
     unsigned long long nb = 0;
     if (t < ls.n0 + ls.n1 + ls.ng) {
         int kind, gi = 0;
         long long p = list_node(ls, t, kind, gi);
-        double2 w = W[p];
-        double2 g = G[p];
-        double ph = f.alpha * w.y + f.beta;
-        double Lc = -f.ams * ph * w.x * w.y;
-        double2 out;
-        out.y = w.y * f.idt - 0.5 * Lc + g.y;
+        const double2 w = W[p];
+        const double ph = fma(f.alpha, w.y, f.beta), ps = ph * w.x, psc = ps * w.y;
+        double2 out, g = make_double2(0.0, 0.0);
+        if (!FIRST) g = G[p];
+        double2 src = make_double2(0.0, 0.0);
+        if (FIRST && f.src) src = f.src[p];
+        if (FIRST) {
+            g.y = fma(0.5 * f.ams, psc, -w.y * f.idt) - src.y;
+            out.y = fma(f.ams, psc, -src.y);
+        } else {
+            out.y = fma(w.y, f.idt, fma(0.5 * f.ams, psc, g.y));
+        }
         if (kind == 1) {
-            double phd;
-            double Ls = Ls_h<D>(p, W, of, f, phd);
-            out.x = ph * w.x * f.idt - 0.5 * Ls + g.x;
+            const double Ls = fma(f.dh2, flux_sum<D>(p, w, ph, W, of, f), -f.amc * psc);
+            if (FIRST) {
+                g.x = fma(-0.5, Ls, -ps * f.idt) - src.x;
+                out.x = -Ls - src.x;
+            } else {
+                out.x = fma(ps, f.idt, fma(-0.5, Ls, g.x));
+            }
         } else {
             out.x = stages::row_dot<D, double, false>(tb, gi, nullptr, W, nullptr, true) - (f.sbg ? f.sbg[gi] : f.sb);
         }
         F[p] = out;
+        if (FIRST) G[p] = g;
         if (Fc) Fc[t] = out;  // the list-ordered copy
         unsigned long long a0 = abs_bits(out.x), a1 = abs_bits(out.y);
         nb = a0 > a1 ? a0 : a1;
@@ -1480,8 +1493,18 @@ int launch_newton_F(const LevelGeo& L, const double2* W, const double2* G, doubl
                     const FConst& fc, unsigned long long* norm, cudaStream_t s) {
     Lists ls = make_lists(L);
     int tot = ls.n0 + ls.n1 + ls.ng;
-    launch_k(k_newton_F<D>, grid_for(tot), block_for(tot), 0, s, ls, stages::ghost_tab<double>(L), W, G, F, Fc,
-             make_offs<D>(L.st[1], L.st[2]), L.st[1], L.st[2], fc, norm);
+    launch_k(k_newton_F<D, false>, grid_for(tot), block_for(tot), 0, s, ls, stages::ghost_tab<double>(L), W,
+             const_cast<double2*>(G), F, Fc, make_offs<D>(L.st[1], L.st[2]), fc, norm);
+    return 1;
+}
+
+template <int D>
+int launch_newton_start(const LevelGeo& L, const double2* W, double2* G, double2* F, double2* Fc, const FConst& fc,
+                        unsigned long long* norm, cudaStream_t s) {
+    Lists ls = make_lists(L);
+    int tot = ls.n0 + ls.n1 + ls.ng;
+    launch_k(k_newton_F<D, true>, grid_for(tot), block_for(tot), 0, s, ls, stages::ghost_tab<double>(L), W, G, F, Fc,
+             make_offs<D>(L.st[1], L.st[2]), fc, norm);
     return 1;
 }
 
@@ -1584,6 +1607,10 @@ SULF_INST(3, float)
 
 template int launch_old_time<2>(const LevelGeo&, const double2*, double2*, const FConst&, cudaStream_t);
 template int launch_old_time<3>(const LevelGeo&, const double2*, double2*, const FConst&, cudaStream_t);
+template int launch_newton_start<2>(const LevelGeo&, const double2*, double2*, double2*, double2*, const FConst&,
+                                    unsigned long long*, cudaStream_t);
+template int launch_newton_start<3>(const LevelGeo&, const double2*, double2*, double2*, double2*, const FConst&,
+                                    unsigned long long*, cudaStream_t);
 template int launch_newton_F<2>(const LevelGeo&, const double2*, const double2*, double2*, double2*, const FConst&,
                                 unsigned long long*, cudaStream_t);
 template int launch_newton_F<3>(const LevelGeo&, const double2*, const double2*, double2*, double2*, const FConst&,

@@ -80,7 +80,8 @@ __device__ __forceinline__ void c_row(const Coef<T>& c, T s, T cp, T& ph, T& pcs
 // level of mixed precision (MIXED)
 template <int D, typename T, bool FINE, bool MIXED>
 __global__ void __launch_bounds__(kT) k_s_rho(SLev<D, T> L, SLev<D, float> U, const typename V2<T>::t* __restrict__ Wc,
-                                               Coef<T> c, const double2* __restrict__ F, double* __restrict__ tt) {
+                                               Coef<T> c, const double2* __restrict__ F, double* __restrict__ tt,
+                                               double* __restrict__ uu) {
     pdl_enter();
     const int t = blockIdx.x * blockDim.x + threadIdx.x;
     const int nin = L.n0 + L.n1;
@@ -103,6 +104,7 @@ __global__ void __launch_bounds__(kT) k_s_rho(SLev<D, T> L, SLev<D, float> U, co
         const double2 f = F[p];
         const double t0 = f.y * (double)inv;
         tt[sl] = t0;
+        uu[sl] = (double)(c.kap * ph);
         if (MIXED) {
             U.rho[sl] = (float)rho;
             U.cs[sl] = (float)C;
@@ -125,10 +127,8 @@ __global__ void __launch_bounds__(kT) k_s_rho(SLev<D, T> L, SLev<D, float> U, co
     }
 }
 
-template <int D, typename T, bool FINE, bool MIXED>
-__global__ void __launch_bounds__(kT) k_s_coefs(SLev<D, T> L, SLev<D, float> U,
-                                                 const typename V2<T>::t* __restrict__ Wc, Coef<T> c,
-                                                 const double2* __restrict__ F, const double* __restrict__ tt) {
+template <int D, typename T>
+__global__ void __launch_bounds__(kT) k_s_coefs(SLev<D, T> L, const typename V2<T>::t* __restrict__ Wc, Coef<T> c) {
     pdl_enter();
     typedef typename V2<T>::t T2;
     const int t = blockIdx.x * blockDim.x + threadIdx.x;
@@ -145,15 +145,13 @@ __global__ void __launch_bounds__(kT) k_s_coefs(SLev<D, T> L, SLev<D, float> U,
     const T s = w.x, cp = w.y;
     T ph, pcs, pcc;
     c_row<T>(c, s, cp, ph, pcs, pcc);
-    T sg = 0, se = 0, et = 0;
+    T sg = 0, se = 0;
     T2 wq[2 * D];
     T rq[2 * D];
-    double tq[2 * D];
 #pragma unroll
     for (int q = 0; q < 2 * D; q++) {
         wq[q] = Wc[(q & 1) ? p - st[q >> 1] : p + st[q >> 1]];
         rq[q] = L.rho[so + o[q]];
-        if (FINE) tq[q] = tt[so + o[q]];
     }
     T g[2 * D];
 #pragma unroll
@@ -163,7 +161,6 @@ __global__ void __launch_bounds__(kT) k_s_coefs(SLev<D, T> L, SLev<D, float> U,
         sg += gq;
         se += eq;
         g[q] = fmadd(eq, rq[q], gq);
-        if (FINE) et = fmadd(eq, (T)tq[q], et);
         L.gt[q * L.gs + t] = g[q];
     }
     const T Pss = ph * c.idt + c.a2mc * ph * cp + sg;
@@ -172,29 +169,75 @@ __global__ void __launch_bounds__(kT) k_s_coefs(SLev<D, T> L, SLev<D, float> U,
     const T di = (T)1 / dd;
     L.dd[t] = dd;
     L.di[t] = di;
-    if (!FINE && L.perm) {
+    if (L.perm) {
         const CPerm q = L.perm[t];
 #pragma unroll
         for (int a = 0; a < 2 * D; a++) L.cf[q.off + a * q.stride] = g[a];
         L.cf[q.off + 2 * D * q.stride] = dd;
         L.cf[q.off + (2 * D + 1) * q.stride] = di;
     }
-    if (FINE) {
-        const T bs = (T)F[p].x - Psc * (T)tt[sl];
-        const T b = bs - et;
-        L.b[t] = b;
-        if (MIXED) {
+}
+
+// The finest level's rows in FP64, with the right-hand side b~ and the start
+// of the first sweep, and in mixed precision the FP32 copies.  The FP64 pipe
+// bounds it, so what a node gives its neighbours (u = kappa phi, C, rho, t)
+// comes from k_s_rho: six FP64 instructions per neighbour (g = u_q + u_p, e =
+// C_p - C_q, gt = g + e rho_q, the sums of u_q, C_q and e t_q).
+template <int D, bool MIXED>
+__global__ void __launch_bounds__(kT) k_s_coefs_fine(const __grid_constant__ SLev<D, double> L,
+                                                      const __grid_constant__ SLev<D, float> U,
+                                                      const double2* __restrict__ Wc, Coef<double> c,
+                                                      const double2* __restrict__ F, const double* __restrict__ tt,
+                                                      const double* __restrict__ uu) {
+    pdl_enter();
+    const int t = blockIdx.x * blockDim.x + threadIdx.x;
+    if (t >= L.n0 + L.n1) return;
+    const int colour = t >= L.n0;
+    const int e = L.hl[t], h = e >> kEntHalf;
+    int ii[3], o[2 * D];
+    half_coords<D>(h, e & 1, L.H, L.n, ii);
+    nbr_offsets<D, double>(L, e & 1, o);
+    const int p = ii[0] + L.n * (ii[1] + (D == 3 ? L.n * ii[2] : 0));
+    const int sl = colour * L.Hn + h, so = (1 - colour) * L.Hn + h;
+    const double2 w = Wc[p], f = F[p];
+    const double up = uu[sl], Cp = L.cs[sl], rho = L.rho[sl], tp = tt[sl];
+    double uq[2 * D], cq[2 * D], rq[2 * D], tq[2 * D];
 #pragma unroll
-            for (int q = 0; q < 2 * D; q++) U.gt[q * U.gs + t] = (float)g[q];
-            const float bf = (float)b, df = (float)di;
-            U.dd[t] = (float)dd;
-            U.di[t] = df;
-            U.b[t] = bf;
-            // the first red half-sweep from zero, the neighbours' x^c = 0 off their c rows
-            if (!colour) U.X[sl] = (float)bs * df;
-        } else if (!colour) {
-            L.X[sl] = bs * di;
-        }
+    for (int q = 0; q < 2 * D; q++) {
+        uq[q] = uu[so + o[q]];
+        cq[q] = L.cs[so + o[q]];
+        rq[q] = L.rho[so + o[q]];
+        tq[q] = tt[so + o[q]];
+    }
+    double su = 0, sc = 0, et = 0, g[2 * D];
+#pragma unroll
+    for (int q = 0; q < 2 * D; q++) {
+        const double eq = Cp - cq[q];
+        su += uq[q];
+        sc += eq;
+        g[q] = fma(eq, rq[q], uq[q] + up);
+        et = fma(eq, tq[q], et);
+        L.gt[q * L.gs + t] = g[q];
+    }
+    const double ph = fma(c.alpha, w.y, c.beta), as = c.alpha * w.x;
+    const double Pss = fma(ph, fma(c.a2mc, w.y, c.idt), fma(2.0 * D, up, su));
+    const double Psc = fma(as, c.idt, fma(c.a2mc, fma(as, w.y, ph * w.x), sc));
+    const double dd = fma(-Psc, rho, Pss), di = 1.0 / dd;
+    const double bs = fma(-Psc, tp, f.x), b = bs - et;
+    L.dd[t] = dd;
+    L.di[t] = di;
+    L.b[t] = b;
+    if (MIXED) {
+#pragma unroll
+        for (int q = 0; q < 2 * D; q++) U.gt[q * U.gs + t] = (float)g[q];
+        const float df = (float)di;
+        U.dd[t] = (float)dd;
+        U.di[t] = df;
+        U.b[t] = (float)b;
+        // the first red half-sweep from zero, the neighbours' x^c = 0 off their c rows
+        if (!colour) U.X[sl] = (float)bs * df;
+    } else if (!colour) {
+        L.X[sl] = bs * di;
     }
 }
 
@@ -665,20 +708,31 @@ __global__ void __launch_bounds__(kT) k_inject_to(stages::Lists ls, int cn, cons
         cW[I] = out;
         return;
     }
-    TF ss = 0, sc = 0;
-    int cnt = 0;
-    for (int kk = 0; kk < (D == 2 ? 9 : 27); kk++) {
+    constexpr int K = D == 2 ? 9 : 27;
+    int8_t ty[K];
+    typename V2<TF>::t v[K];
+    int q[K];
+#pragma unroll
+    for (int kk = 0; kk < K; kk++) {
         const int k[3] = {kk % 3 - 1, (kk / 3) % 3 - 1, D == 3 ? kk / 9 - 1 : 0};
         bool ok = true;
+#pragma unroll
         for (int a = 0; a < D; a++) ok = ok && 2 * ii[a] + k[a] >= 0 && 2 * ii[a] + k[a] < fn;
-        if (!ok) continue;
-        const int q = f + k[0] + fn * (k[1] + (D == 3 ? fn * k[2] : 0));
-        if (ftype[q] != T_IN && ftype[q] != T_GHOST) continue;
-        const typename V2<TF>::t v = fW[q];
-        ss += v.x;
-        sc += v.y;
-        cnt++;
+        q[kk] = f + k[0] + fn * (k[1] + (D == 3 ? fn * k[2] : 0));
+        ty[kk] = ok ? ftype[q[kk]] : (int8_t)T_OUT;
     }
+    TF ss = 0, sc = 0;
+    int cnt = 0;
+#pragma unroll
+    for (int kk = 0; kk < K; kk++)
+        if (ty[kk] == T_IN || ty[kk] == T_GHOST) v[kk] = fW[q[kk]];
+#pragma unroll
+    for (int kk = 0; kk < K; kk++)
+        if (ty[kk] == T_IN || ty[kk] == T_GHOST) {
+            ss += v[kk].x;
+            sc += v[kk].y;
+            cnt++;
+        }
     out.x = (T)(cnt ? ss / (TF)cnt : (TF)0);
     out.y = (T)(cnt ? sc / (TF)cnt : (TF)0);
     cW[I] = out;
@@ -741,25 +795,37 @@ __global__ void __launch_bounds__(kFacThreads) k_s_factor(SLev<D, T> L, const in
     }
     __syncthreads();
     __shared__ int s_piv;
-    __shared__ T s_inv;
+    // a thread's elements (row, local column) of the elimination, packed: a
+    // half-empty FP64 instruction costs as much as a full one
+    constexpr int kEl = 4;
+    const int nel = m * mc, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    int er[kEl], ec[kEl];
+#pragma unroll
+    for (int q = 0; q < kEl; q++) {
+        const int t = threadIdx.x + q * kFacThreads;
+        er[q] = t / mc;
+        ec[q] = t % mc;
+    }
     for (int k = 0; k < m; k++) {
         T* fb = fac + (size_t)(k & 1) * (m + 1);
         if (k % C == me) {
             const int kl = k / C;
             __syncthreads();  // this CTA's updates of column k in the previous step
-            if (threadIdx.x < 32) {
-                const int lane = threadIdx.x;
-                T bv = -1;
+            if (warp == 0) {
+                // magnitudes compared as integers (an FP64 compare takes the
+                // FP64 pipe); a NaN is no pivot
+                unsigned long long bv = 0;
                 int bi = k;
                 for (int i = k + lane; i < m; i += 32) {
-                    const T v = fabs(A[(size_t)i * mc + kl]);
+                    unsigned long long v = abs_bits(A[(size_t)i * mc + kl]);
+                    if (v > 0x7ff0000000000000ULL) v = 0;
                     if (v > bv) {
                         bv = v;
                         bi = i;
                     }
                 }
                 for (int o = 16; o > 0; o >>= 1) {
-                    const T ov = __shfl_down_sync(0xffffffffu, bv, o);
+                    const unsigned long long ov = __shfl_down_sync(0xffffffffu, bv, o);
                     const int oi = __shfl_down_sync(0xffffffffu, bi, o);
                     if (ov > bv || (ov == bv && oi < bi)) {
                         bv = ov;
@@ -768,46 +834,56 @@ __global__ void __launch_bounds__(kFacThreads) k_s_factor(SLev<D, T> L, const in
                 }
                 if (lane == 0) {
                     s_piv = bi;
-                    s_inv = (T)1 / A[(size_t)bi * mc + kl];
-                    if (!(bv > (T)0)) *singular = 1;
+                    if (bv == 0) *singular = 1;
                 }
             }
             __syncthreads();
             const int pr = s_piv;
-            for (int t = threadIdx.x; t < m * C; t += blockDim.x) {
-                const int rk = t / m, i = t % m;
-                const int src = i == k ? pr : (i == pr ? k : i);
-                T* dst = cl.map_shared_rank(fb, rk);
-                dst[i] = A[(size_t)src * mc + kl];
-                if (i == 0) {
-                    dst[m] = s_inv;
-                    cl.map_shared_rank(piv, rk)[k] = pr;
+            if (warp < C) {
+                T* dst = cl.map_shared_rank(fb, warp);
+                for (int i = lane; i < m; i += 32) {
+                    const int src = i == k ? pr : (i == pr ? k : i);
+                    dst[i] = A[(size_t)src * mc + kl];
                 }
+            } else if (warp == C && lane < C) {
+                cl.map_shared_rank(fb, lane)[m] = (T)1 / A[(size_t)pr * mc + kl];
+                cl.map_shared_rank(piv, lane)[k] = pr;
             }
         }
         cl.sync();
+        // rows k and pr change places, row k is scaled by the reciprocal pivot,
+        // column k eliminated from the others: all reads, then all writes
         const int pr = piv[k];
         const T inv = fb[m];
-        for (int jl = threadIdx.x; jl < mc; jl += blockDim.x) {
-            const int j = jl * C + me;
-            if (j >= m) continue;
-            T rowk = A[(size_t)k * mc + jl];
-            if (pr != k) {
-                const T rowp = A[(size_t)pr * mc + jl];
-                A[(size_t)pr * mc + jl] = rowk;
-                rowk = rowp;
+        auto value = [&](int i, int jl) -> T {
+            const T top = A[(size_t)pr * mc + jl] * inv;
+            const bool own = jl * C + me == k;
+            if (i == k) return own ? inv : top;
+            if (own) return -fb[i] * inv;
+            const T v = i == pr ? A[(size_t)k * mc + jl] : A[(size_t)i * mc + jl];
+            return fmadd(-fb[i], top, v);
+        };
+        if (nel <= kEl * kFacThreads) {
+            T v[kEl];
+#pragma unroll
+            for (int q = 0; q < kEl; q++)
+                if ((int)threadIdx.x + q * kFacThreads < nel) v[q] = value(er[q], ec[q]);
+            __syncthreads();
+#pragma unroll
+            for (int q = 0; q < kEl; q++)
+                if ((int)threadIdx.x + q * kFacThreads < nel) A[(size_t)er[q] * mc + ec[q]] = v[q];
+        } else {
+            // larger matrices: a column at a time per thread group
+            for (int jl = warp; jl < mc; jl += kFacThreads / 32) {
+                const T rowk = A[(size_t)k * mc + jl], top = A[(size_t)pr * mc + jl] * inv;
+                const bool own = jl * C + me == k;
+                __syncwarp();
+                for (int i = lane; i < m; i += 32) {
+                    const T v = i == pr ? rowk : A[(size_t)i * mc + jl];
+                    A[(size_t)i * mc + jl] =
+                        i == k ? (own ? inv : top) : (own ? -fb[i] * inv : fmadd(-fb[i], top, v));
+                }
             }
-            A[(size_t)k * mc + jl] = j == k ? inv : rowk * inv;
-        }
-        __syncthreads();
-        for (int t = threadIdx.x; t < m * mc; t += blockDim.x) {
-            const int i = t / mc, jl = t % mc;
-            const int j = jl * C + me;
-            if (i == k || j >= m) continue;
-            if (j == k)
-                A[(size_t)i * mc + jl] = -fb[i] * inv;
-            else
-                A[(size_t)i * mc + jl] -= fb[i] * A[(size_t)k * mc + jl];
         }
     }
     __syncthreads();
@@ -1394,39 +1470,37 @@ template <int D, typename T>
 int launch_s_rho(const SLev<D, T>& L, const typename V2<T>::t* Wc, const Coef<T>& c, cudaStream_t s) {
     const int tot = L.n0 + L.n1 + L.ng;
     launch_k(k_s_rho<D, T, false, false>, grid_for(tot), block_for(tot), 0, s, L, SLev<D, float>{}, Wc, c,
-             (const double2*)nullptr, (double*)nullptr);
+             (const double2*)nullptr, (double*)nullptr, (double*)nullptr);
     return 1;
 }
 
 template <int D>
 int launch_s_rho_fine(const SLev<D, double>& L, const double2* Wc, const Coef<double>& c, const double2* F, double* tt,
-                      const SLev<D, float>* U, cudaStream_t s) {
+                      double* uu, const SLev<D, float>* U, cudaStream_t s) {
     const int tot = L.n0 + L.n1 + L.ng;
     if (U)
-        launch_k(k_s_rho<D, double, true, true>, grid_for(tot), block_for(tot), 0, s, L, *U, Wc, c, F, tt);
+        launch_k(k_s_rho<D, double, true, true>, grid_for(tot), block_for(tot), 0, s, L, *U, Wc, c, F, tt, uu);
     else
         launch_k(k_s_rho<D, double, true, false>, grid_for(tot), block_for(tot), 0, s, L, SLev<D, float>{}, Wc, c, F,
-                 tt);
+                 tt, uu);
     return 1;
 }
 
 template <int D, typename T>
 int launch_s_coefs(const SLev<D, T>& L, const typename V2<T>::t* Wc, const Coef<T>& c, cudaStream_t s) {
     const int tot = L.n0 + L.n1;
-    launch_k(k_s_coefs<D, T, false, false>, grid_for(tot), block_for(tot), 0, s, L, SLev<D, float>{}, Wc, c,
-             (const double2*)nullptr, (const double*)nullptr);
+    launch_k(k_s_coefs<D, T>, grid_for(tot), block_for(tot), 0, s, L, Wc, c);
     return 1;
 }
 
 template <int D>
 int launch_s_coefs_fine(const SLev<D, double>& L, const double2* Wc, const Coef<double>& c, const double2* F,
-                        const double* tt, const SLev<D, float>* U, cudaStream_t s) {
+                        const double* tt, const double* uu, const SLev<D, float>* U, cudaStream_t s) {
     const int tot = L.n0 + L.n1;
     if (U)
-        launch_k(k_s_coefs<D, double, true, true>, grid_for(tot), block_for(tot), 0, s, L, *U, Wc, c, F, tt);
+        launch_k(k_s_coefs_fine<D, true>, grid_for(tot), block_for(tot), 0, s, L, *U, Wc, c, F, tt, uu);
     else
-        launch_k(k_s_coefs<D, double, true, false>, grid_for(tot), block_for(tot), 0, s, L, SLev<D, float>{}, Wc, c, F,
-                 tt);
+        launch_k(k_s_coefs_fine<D, false>, grid_for(tot), block_for(tot), 0, s, L, SLev<D, float>{}, Wc, c, F, tt, uu);
     return 1;
 }
 
@@ -1633,9 +1707,10 @@ SULF_INST_S(3, double)
 SULF_INST_S(3, float)
 #define SULF_INST_SD(D)                                                                                            \
     template int launch_s_rho_fine<D>(const SLev<D, double>&, const double2*, const Coef<double>&, const double2*, \
-                                      double*, const SLev<D, float>*, cudaStream_t);                               \
+                                      double*, double*, const SLev<D, float>*, cudaStream_t);                      \
     template int launch_s_coefs_fine<D>(const SLev<D, double>&, const double2*, const Coef<double>&,               \
-                                        const double2*, const double*, const SLev<D, float>*, cudaStream_t);       \
+                                        const double2*, const double*, const double*, const SLev<D, float>*,       \
+                                        cudaStream_t);                                                             \
     template int launch_s_outer<D>(const SLev<D, double>&, const SLev<D, float>&, unsigned long long*,             \
                                    cudaStream_t);                                                                  \
     template int launch_s_batched_outer<D>(const SLev<D, double>*, const SLev<D, float>*, const int*, int, int,    \

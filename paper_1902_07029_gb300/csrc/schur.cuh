@@ -145,7 +145,7 @@ struct SVec {
     T2* D2 = nullptr;
     T *gt = nullptr, *dd = nullptr, *di = nullptr, *b = nullptr, *snap = nullptr;
     T *A = nullptr, *Ainv = nullptr;  // coarsest level: work matrix (where it does not fit on chip) and inverse
-    T* tt = nullptr;                  // finest level, FP64: t by slot
+    T *tt = nullptr, *uu = nullptr;   // finest level, FP64: t and u = kappa phi by slot
 };
 
 template <int D, typename T>
@@ -218,14 +218,14 @@ template <int D, typename T>
 int launch_s_rho(const SLev<D, T>& L, const typename V2<T>::t* Wc, const Coef<T>& c, cudaStream_t s);
 template <int D>
 int launch_s_rho_fine(const SLev<D, double>& L, const double2* Wc, const Coef<double>& c, const double2* F, double* tt,
-                      const SLev<D, float>* U, cudaStream_t s);
+                      double* uu, const SLev<D, float>* U, cudaStream_t s);
 // the rows gt, dd, 1/dd of the inside nodes (and on the finest level b~ and
 // the start of the first sweep)
 template <int D, typename T>
 int launch_s_coefs(const SLev<D, T>& L, const typename V2<T>::t* Wc, const Coef<T>& c, cudaStream_t s);
 template <int D>
 int launch_s_coefs_fine(const SLev<D, double>& L, const double2* Wc, const Coef<double>& c, const double2* F,
-                        const double* tt, const SLev<D, float>* U, cudaStream_t s);
+                        const double* tt, const double* uu, const SLev<D, float>* U, cudaStream_t s);
 // threads of a phase
 template <int D, typename T>
 long long s_threads(SPhase ph, const SLev<D, T>& L, const SLev<D, T>* C);

@@ -155,6 +155,21 @@ struct sulf_domain {
         int max_cycles = 0;
         long long kernels = 0;  // per cycle
     } loop[2];
+    // The phases of a Newton iteration around the cycles as graphs: the set-up
+    // of the linear solve, per precision, and the update with the new residual.
+    // Captured at their second use; recaptured when anything baked into them
+    // changes.
+    struct StepGraph {
+        cudaGraphExec_t exec = nullptr;
+        int uses = 0;
+        double dt = 0;
+        sulf_solver sv{};
+        sulf_model model{};
+        const void *src = nullptr, *sbg = nullptr, *rhsc = nullptr;
+        long long kernels = 0;
+    } prep[2], upd;
+    cudaStream_t aux = nullptr;  // branch of the set-up: the coarse levels
+    cudaEvent_t ev_fork = nullptr, ev_join = nullptr;
     bool loop_off = false;
     bool loop_used = false;  // the last linear solve ran as one loop-graph launch
     int* dcyc = nullptr;      // cycles run by the device loop
@@ -269,6 +284,11 @@ void drop_graphs(sulf_domain* d) {
         if (g.exec) {
             cudaGraphExecDestroy(g.exec);
             g.exec = nullptr;
+        }
+    for (auto* g : {&d->prep[0], &d->prep[1], &d->upd})
+        if (g->exec) {
+            cudaGraphExecDestroy(g->exec);
+            g->exec = nullptr;
         }
 }
 
@@ -395,7 +415,10 @@ int alloc_schur(sulf_domain* d, SVec<T>* V, int nl, bool outer) {
         get(v.dd, nin, false);
         get(v.di, nin, false);
         get(v.b, nin + G.ng, false);
-        if (!f32 && l == 0) get(v.tt, ns, false);
+        if (!f32 && l == 0) {
+            get(v.tt, ns, false);
+            get(v.uu, ns, false);
+        }
         if (outer) continue;
         get(v.snap, (size_t)G.ng, false);
         // zero where never written: defects of the black nodes away from the
@@ -803,26 +826,42 @@ SLev<D, double> fine_slev(sulf_domain* d) {
 // set-up of a linear solve J dW = F in this form: the rows of every level, the
 // coarsest inverse, and the first sweep of the first cycle, which runs from a
 // zero that is off the c rows
+// (fork: the coarse levels on a branch of their own, inside a capture)
 template <int D>
-int schur_prepare(sulf_domain* d) {
+int schur_prepare(sulf_domain* d, bool fork = false) {
     const SLev<D, double> L0 = fine_slev<D>(d);
     const Coef<double> c0 = make_coef<double>(d, 0);
     const double2* F = d->v64[0].rhs;
-    double* tt = d->s64[0].tt;
-    if (d->solver.precision == 1) {
-        const SLev<D, float> U = make_slev<D, float>(d->geo[0], d->sgeo[0], d->s32[0]);
-        d->launches += launch_s_rho_fine<D>(L0, d->W, c0, F, tt, &U, d->stream);
-        d->launches += launch_s_coefs_fine<D>(L0, d->W, c0, F, tt, &U, d->stream);
-        if (int rc = SMG<D, float>{d, d->s32}.prepare_coarse()) return rc;
-        d->launches += launch_s_relax<D, float>(U, 1, true, true, false, false, d->stream);
-        d->launches += launch_s_ghosts<D, float>(U, false, false, d->stream);
-    } else {
-        d->launches += launch_s_rho_fine<D>(L0, d->W, c0, F, tt, nullptr, d->stream);
-        d->launches += launch_s_coefs_fine<D>(L0, d->W, c0, F, tt, nullptr, d->stream);
-        if (int rc = SMG<D, double>{d, d->s64}.prepare_coarse()) return rc;
-        d->launches += launch_s_relax<D, double>(L0, 1, true, true, false, false, d->stream);
-        d->launches += launch_s_ghosts<D, double>(L0, false, false, d->stream);
+    double *tt = d->s64[0].tt, *uu = d->s64[0].uu;
+    const bool mixed = d->solver.precision == 1;
+    const cudaStream_t s = d->stream;
+    auto coarse = [&] {
+        return mixed ? SMG<D, float>{d, d->s32}.prepare_coarse() : SMG<D, double>{d, d->s64}.prepare_coarse();
+    };
+    if (fork) {
+        SULF_CUDA_TRY(cudaEventRecord(d->ev_fork, s));
+        SULF_CUDA_TRY(cudaStreamWaitEvent(d->aux, d->ev_fork, 0));
+        d->stream = d->aux;
+        const int rc = coarse();
+        d->stream = s;
+        if (rc) return rc;
+        SULF_CUDA_TRY(cudaEventRecord(d->ev_join, d->aux));
     }
+    SLev<D, float> U{};
+    if (mixed) U = SMG<D, float>{d, d->s32}.lev(0);
+    d->launches += launch_s_rho_fine<D>(L0, d->W, c0, F, tt, uu, mixed ? &U : nullptr, s);
+    d->launches += launch_s_coefs_fine<D>(L0, d->W, c0, F, tt, uu, mixed ? &U : nullptr, s);
+    if (!fork)
+        if (int rc = coarse()) return rc;
+    // this relaxation reads rows that the kernel just before may have written,
+    // ahead of a dependent launch's wait: not launched as one
+    const bool pdl = launch_pdl();
+    set_launch_pdl(false);
+    d->launches += mixed ? launch_s_relax<D, float>(U, 1, true, true, false, false, s)
+                         : launch_s_relax<D, double>(L0, 1, true, true, false, false, s);
+    set_launch_pdl(pdl);
+    d->launches += mixed ? launch_s_ghosts<D, float>(U, false, false, s) : launch_s_ghosts<D, double>(L0, false, false, s);
+    if (fork) SULF_CUDA_TRY(cudaStreamWaitEvent(s, d->ev_join, 0));
     SULF_CUDA_TRY(cudaMemsetAsync(d->dskip, 1, sizeof(int), d->stream));
     SULF_CUDA_TRY(cudaMemsetAsync(d->dnorm, 0, sizeof(unsigned long long) * 2, d->stream));
     return SULF_OK;
@@ -1030,6 +1069,58 @@ struct PdlScope {
     }
 };
 
+// run fn (work on the handle's stream, the same at every call): directly the
+// first time, then from its graph
+template <class F>
+int run_captured(sulf_domain* d, sulf_domain::StepGraph& g, F&& fn) {
+    if (!d->solver.graphs || d->capturing) return fn(false);
+    const void *src = d->src_on ? d->src : nullptr, *sbg = d->sbg_on ? d->sbg : nullptr, *rhsc = d->v64[0].rhsc;
+    const bool same = g.uses > 0 && g.dt == d->dt && same_solver(g.sv, d->solver) &&
+                      memcmp(&g.model, &d->model, sizeof g.model) == 0 && g.src == src && g.sbg == sbg && g.rhsc == rhsc;
+    if (!same) {
+        if (g.exec) cudaGraphExecDestroy(g.exec);
+        g.exec = nullptr;
+        g.uses = 0;
+        g.dt = d->dt;
+        g.sv = d->solver;
+        g.model = d->model;
+        g.src = src;
+        g.sbg = sbg;
+        g.rhsc = rhsc;
+    }
+    if (g.uses++ == 0) return fn(false);
+    if (!g.exec) {
+        if (!d->aux) {
+            SULF_CUDA_TRY(cudaStreamCreateWithFlags(&d->aux, cudaStreamNonBlocking));
+            SULF_CUDA_TRY(cudaEventCreateWithFlags(&d->ev_fork, cudaEventDisableTiming));
+            SULF_CUDA_TRY(cudaEventCreateWithFlags(&d->ev_join, cudaEventDisableTiming));
+        }
+        const long long l0 = d->launches;
+        SULF_CUDA_TRY(cudaStreamBeginCapture(d->stream, cudaStreamCaptureModeThreadLocal));
+        d->capturing = true;
+        const int rc = fn(true);
+        cudaGraph_t graph = nullptr;
+        const cudaError_t e = cudaStreamEndCapture(d->stream, &graph);
+        d->capturing = false;
+        g.kernels = d->launches - l0;
+        d->launches = l0;
+        if (rc) {
+            if (graph) cudaGraphDestroy(graph);
+            return rc;
+        }
+        if (e != cudaSuccess) return sulf_fail_cuda(e, "cudaStreamEndCapture");
+        const cudaError_t ei = cudaGraphInstantiate(&g.exec, graph, 0);
+        cudaGraphDestroy(graph);
+        if (ei != cudaSuccess) {
+            g.exec = nullptr;
+            return sulf_fail_cuda(ei, "cudaGraphInstantiate");
+        }
+    }
+    SULF_CUDA_TRY(cudaGraphLaunch(g.exec, d->stream));
+    d->launches += g.kernels;
+    return SULF_OK;
+}
+
 // run one cycle: replay the captured graph (capturing it first if needed), or
 // launch the kernels directly
 template <int D>
@@ -1092,7 +1183,7 @@ int linear_solve(sulf_domain* d, double fnorm, int max_cycles, double rtol, doub
     if (rc) return rc;
     if (!d->s_on) SULF_CUDA_TRY(cudaMemsetAsync(d->v64[0].x, 0, sizeof(double2) * G0.nn, d->stream));
     if (d->s_on) {
-        rc = schur_prepare<D>(d);
+        rc = run_captured(d, d->prep[d->solver.precision], [&](bool fork) { return schur_prepare<D>(d, fork); });
     } else if (d->solver.precision == 0) {
         rc = ensure_tail<D, double>(d, d->v64);
         if (rc) return rc;
@@ -1147,10 +1238,8 @@ int cn_step(sulf_domain* d) {
     const LevelGeo& G0 = d->geo[0];
     LevelVec<double>& V0 = d->v64[0];
     FConst fc = make_fconst(d);
-    SULF_CUDA_TRY(cudaMemcpyAsync(d->Wn, d->W, sizeof(double2) * G0.nn, cudaMemcpyDeviceToDevice, d->stream));
-    d->launches += launch_old_time<D>(G0, d->Wn, d->G, fc, d->stream);
     SULF_CUDA_TRY(cudaMemsetAsync(d->dnorm, 0, sizeof(unsigned long long) * 4, d->stream));
-    d->launches += launch_newton_F<D>(G0, d->W, d->G, V0.rhs, V0.rhsc, fc, d->dnorm, d->stream);
+    d->launches += launch_newton_start<D>(G0, d->W, d->G, V0.rhs, V0.rhsc, fc, d->dnorm, d->stream);
     int rc = read_norms(d, 1);
     if (rc) return rc;
     double fn = bits_to_double(d->hnorm[0]);
@@ -1167,12 +1256,17 @@ int cn_step(sulf_domain* d) {
         if (nc < 0) return nc;
         d->cycles_last += nc;
         d->cycles_total += nc;
-        SULF_CUDA_TRY(cudaMemsetAsync(d->dnorm, 0, sizeof(unsigned long long) * 4, d->stream));
-        if (d->s_on)
-            d->launches += launch_s_update<D>(fine_slev<D>(d), d->s64[0].tt, d->W, d->dnorm, nullptr, d->stream);
-        else
-            d->launches += launch_newton_update(G0, d->W, V0.x, d->dnorm, d->stream);
-        d->launches += launch_newton_F<D>(G0, d->W, d->G, V0.rhs, V0.rhsc, fc, d->dnorm + 2, d->stream);
+        auto update = [&](bool) {
+            SULF_CUDA_TRY(cudaMemsetAsync(d->dnorm, 0, sizeof(unsigned long long) * 4, d->stream));
+            if (d->s_on)
+                d->launches += launch_s_update<D>(fine_slev<D>(d), d->s64[0].tt, d->W, d->dnorm, nullptr, d->stream);
+            else
+                d->launches += launch_newton_update(G0, d->W, V0.x, d->dnorm, d->stream);
+            d->launches += launch_newton_F<D>(G0, d->W, d->G, V0.rhs, V0.rhsc, fc, d->dnorm + 2, d->stream);
+            return SULF_OK;
+        };
+        rc = d->s_on ? run_captured(d, d->upd, update) : update(false);
+        if (rc) return rc;
         rc = read_norms(d, 3);
         if (rc) return rc;
         double dn = bits_to_double(d->hnorm[0]), wn = bits_to_double(d->hnorm[1]);
@@ -1294,6 +1388,11 @@ void sulf_destroy(sulf_handle h) {
     if (h->stream) cudaStreamSynchronize(h->stream);
     for (auto& g : h->graph)
         if (g.exec) cudaGraphExecDestroy(g.exec);
+    for (auto* g : {&h->prep[0], &h->prep[1], &h->upd})
+        if (g->exec) cudaGraphExecDestroy(g->exec);
+    if (h->aux) cudaStreamDestroy(h->aux);
+    if (h->ev_fork) cudaEventDestroy(h->ev_fork);
+    if (h->ev_join) cudaEventDestroy(h->ev_join);
     for (cudaEvent_t e : h->evpool) cudaEventDestroy(e);
     h->mem.release();
     if (h->hnorm) cudaFreeHost(h->hnorm);
@@ -2364,10 +2463,8 @@ int lockstep_step(LockClass<D>& C, LockGraphs<D>& P, int* status, std::vector<st
             sulf_domain* d = C.h[i];
             const LevelGeo& G0 = d->geo[0];
             FConst fc = make_fconst(d);
-            SULF_CUDA_TRY(cudaMemcpyAsync(d->Wn, d->W, sizeof(double2) * G0.nn, cudaMemcpyDeviceToDevice, b));
-            d->launches += launch_old_time<D>(G0, d->Wn, d->G, fc, b);
             SULF_CUDA_TRY(cudaMemsetAsync(d->dnorm, 0, sizeof(unsigned long long) * 4, b));
-            d->launches += launch_newton_F<D>(G0, d->W, d->G, d->v64[0].rhs, d->v64[0].rhsc, fc, d->dnorm, b);
+            d->launches += launch_newton_start<D>(G0, d->W, d->G, d->v64[0].rhs, d->v64[0].rhsc, fc, d->dnorm, b);
             SULF_CUDA_TRY(cudaMemcpyAsync(d->hnorm, d->dnorm, sizeof(unsigned long long), cudaMemcpyDeviceToHost, b));
             return SULF_OK;
         });
@@ -2627,10 +2724,8 @@ int autotune(sulf_domain* d, double dt, sulf_tune_result* out) {
     const LevelGeo& G0 = d->geo[0];
     d->dt = dt;
     FConst fc = make_fconst(d);
-    SULF_CUDA_TRY(cudaMemcpyAsync(d->Wn, d->W, sizeof(double2) * G0.nn, cudaMemcpyDeviceToDevice, d->stream));
-    d->launches += launch_old_time<D>(G0, d->Wn, d->G, fc, d->stream);
     SULF_CUDA_TRY(cudaMemsetAsync(d->dnorm, 0, sizeof(unsigned long long) * 4, d->stream));
-    d->launches += launch_newton_F<D>(G0, d->W, d->G, d->v64[0].rhs, d->v64[0].rhsc, fc, d->dnorm, d->stream);
+    d->launches += launch_newton_start<D>(G0, d->W, d->G, d->v64[0].rhs, d->v64[0].rhsc, fc, d->dnorm, d->stream);
     if (int rc = read_norms(d, 1)) return rc;
     double fn = bits_to_double(d->hnorm[0]);
     if (!(fn > 0)) fn = 1.0;

@@ -263,6 +263,10 @@ int launch_gather_list(const LevelGeo& L, const double2* box, double2* list, cud
 template <int D>
 int launch_newton_F(const LevelGeo& L, const double2* W, const double2* G, double2* F, double2* Fc,
                     const FConst& fc, unsigned long long* norm, cudaStream_t s);
+// the old-time part and the first residual of a step, both at W = W^n
+template <int D>
+int launch_newton_start(const LevelGeo& L, const double2* W, double2* G, double2* F, double2* Fc, const FConst& fc,
+                        unsigned long long* norm, cudaStream_t s);
 int launch_newton_update(const LevelGeo& L, double2* W, const double2* x, unsigned long long* norms,
                          cudaStream_t s);
 int launch_norm_active(const LevelGeo& L, const double2* v, unsigned long long* norm, cudaStream_t s);
