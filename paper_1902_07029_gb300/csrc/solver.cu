@@ -52,19 +52,36 @@ void retain_pool_memory() {
 }
 }  // namespace
 
+// Blocks of up to half a chunk come from a chunk shared with others: a domain
+// has some two hundred arrays, and an allocation with its synchronisation for
+// each was most of the first step of a small one
+constexpr size_t kChunkBytes = 2 << 20;
+
 void* DevMem::get(size_t n) {
-    void* p = nullptr;
     size_t sz = (n + 255) & ~size_t(255);
     if (sz == 0) sz = 256;
+    const bool shared = sz <= kChunkBytes / 2;
+    if (shared && sz <= left) {
+        void* p = chunk;
+        chunk += sz;
+        left -= sz;
+        return p;
+    }
+    const size_t want = shared ? kChunkBytes : sz;
+    void* p = nullptr;
     retain_pool_memory();
-    if (cudaMallocAsync(&p, sz, stream) != cudaSuccess) {
+    if (cudaMallocAsync(&p, want, stream) != cudaSuccess) {
         cudaGetLastError();
         return nullptr;
     }
     // set-up only: make the block usable from any stream right away
     if (cudaStreamSynchronize(stream) != cudaSuccess) return nullptr;
     ptrs.push_back(p);
-    bytes += sz;
+    bytes += want;
+    if (shared) {
+        chunk = (char*)p + sz;
+        left = want - sz;
+    }
     return p;
 }
 
@@ -73,6 +90,8 @@ void DevMem::release() {
     if (stream) cudaStreamSynchronize(stream);
     ptrs.clear();
     bytes = 0;
+    chunk = nullptr;
+    left = 0;
 }
 
 }  // namespace sulf

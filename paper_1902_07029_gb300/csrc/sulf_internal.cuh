@@ -175,6 +175,8 @@ struct FConst {
 struct DevMem {
     std::vector<void*> ptrs;
     size_t bytes = 0;
+    char* chunk = nullptr;  // free part of the current chunk of small blocks
+    size_t left = 0;
     cudaStream_t stream = nullptr;
     void* get(size_t n);
     void release();
