@@ -22,9 +22,21 @@ constexpr size_t kCoarseSmem = 224 * 1024;
 enum { kOpNone = 0, kOpRed, kOpBlack, kOpGhosts, kOpDefect, kOpRestrict, kOpSolve, kOpProlong, kOpVisit };
 constexpr unsigned kOpDelta = 1u << 16, kOpLast = 1u << 17, kOpAll = 1u << 18, kOpFar = 1u << 19, kOpWide = 1u << 20;
 constexpr unsigned kOpSkipRed = 1u << 21, kOpDown = 1u << 22;  // of a visit: first red half-sweep done; defect after
-constexpr int kCoarseLog = 2;
-constexpr int kCoarseLanes = 1 << kCoarseLog;                // lanes of a row of more than kShortRow entries
-constexpr int kShortRow = 6, kLongRow = 64;    // and of more than kLongRow: a warp
+constexpr unsigned kOpTop = 1u << 23;                           // the cycle's first visit of the finest level
+// a table entry that names a value of any array: owner << kAddrBits | byte
+// offset in the owner's shared memory
+constexpr int kAddrBits = 20;
+constexpr unsigned kAddrMask = (1u << kAddrBits) - 1;
+// entries a lane of a table's row has, up to 32 lanes a row: with four the
+// longest row is one round of loads, while an SM's two FP64 lanes make the
+// partial sums dear (33^3 box, rows of 1 to 90 entries, four lanes a row and a
+// warp above 64: 6000 cycles a phase)
+template <typename T>
+constexpr int kRowEntries = sizeof(T) == 4 ? 4 : 8;
+// a table's warp: its first row | log2 lanes per row << 16 | rows << 20
+__host__ __device__ constexpr unsigned row_job(int row, int lg, int cnt) {
+    return (unsigned)row | (unsigned)lg << 16 | (unsigned)cnt << 20;
+}
 
 __device__ __forceinline__ unsigned cta_rank() {
     unsigned r;
@@ -129,11 +141,21 @@ struct Coarse {
         }
     }
 
-    // entries beg, beg + step, ... < end of a CSR table times the values they
-    // name; `composed`: an entry's upper half selects the array (x, snap, b)
+    // address of a table entry's value (an array at byte offset off, or by kAddrBits)
     template <class R>
-    __device__ __forceinline__ T entries(bool w, int beg, int end, int step, const R* ref, const T* val, int off,
-                                         int off1, int off2) const {
+    __device__ __forceinline__ unsigned where(bool w, int off, R u) const {
+        if (sizeof(R) == 4) {
+            const unsigned a = sa + (u & kAddrMask);
+            return w ? map_rank(a, u >> kAddrBits) : a;
+        }
+        const unsigned a = sa + off + (u & kRefMask) * (unsigned)sizeof(T);
+        return w ? map_rank(a, u >> kRefBits) : a;
+    }
+
+    // entries beg, beg + step, ... < end of a CSR table times the values they name
+    template <class R>
+    __device__ __forceinline__ T entries(bool w, int beg, int end, int step, const R* ref, const T* val,
+                                         int off) const {
         T v = 0;
         for (int j0 = beg; j0 < end; j0 += 4 * step) {
             unsigned u[4];
@@ -141,17 +163,15 @@ struct Coarse {
 #pragma unroll
             for (int q = 0; q < 4; q++) {
                 const int j = j0 + q * step < end ? j0 + q * step : j0;
-                u[q] = ref[j];
+                u[q] = where<R>(w, off, ref[j]);
                 c[q] = val[j];
             }
-            if (sizeof(R) == 2) {
-                get<4, T>(w, off, u, x);
+            if (w) {
+#pragma unroll
+                for (int q = 0; q < 4; q++) ld_at<true>(u[q], x[q]);
             } else {
 #pragma unroll
-                for (int q = 0; q < 4; q++) {
-                    const unsigned kind = u[q] >> 16, r = u[q] & 0xffffu;
-                    get<1, T>(w, kind == 0 ? off : (kind == 1 ? off1 : off2), &r, x + q);
-                }
+                for (int q = 0; q < 4; q++) ld_at<false>(u[q], x[q]);
             }
 #pragma unroll
             for (int q = 0; q < 4; q++)
@@ -160,34 +180,31 @@ struct Coarse {
         return v;
     }
 
-    // the rows of a table after the `skip` first threads' own work first(t) (a
-    // multiple of 32); done(ghost, sum)
+    // the rows of a table, by `stride` threads, after the `skip` first threads'
+    // own work first(t) (a multiple of 32); done(ghost, sum)
     template <class R, class First, class Done>
-    __device__ __forceinline__ void rows(bool w, int skip, const CTab& tab, int off, int off1, int off2,
-                                         const First& first, const Done& done) const {
-        const int nx = tab.nx, nl = tab.nl, ns = tab.ns;
-        const int tl = skip + 32 * nx, ts = tl + (nl * kCoarseLanes + 31) / 32 * 32, tot = ts + (ns + 31) / 32 * 32;
-        for (int t = tid; t < tot; t += nthr) {
+    __device__ __forceinline__ void rows(bool w, int stride, int skip, const CTab& tab, int off, const First& first,
+                                         const Done& done) const {
+        const int tot = skip + 32 * tab.nw;
+        const int* ptr = at<const int>(tab.ptr);
+        for (int t = tid; t < tot; t += stride) {
             if (t < skip) {
                 first(t);
                 continue;
             }
-            const int lanes = t >= ts ? 1 : (t >= tl ? kCoarseLanes : 32), lg = t >= ts ? 0 : (t >= tl ? kCoarseLog : 5);
-            const int q = (t - (t >= ts ? ts : (t >= tl ? tl : skip))), i = q >> lg, ln = q & (lanes - 1);
-            const bool on = i < (t >= ts ? ns : (t >= tl ? nl : nx));
-            const int r = i + (t >= ts ? nx + nl : (t >= tl ? nx : 0));
+            const unsigned job = at<const unsigned>(tab.job)[(t - skip) >> 5];
+            const int lg = job >> 16 & 15, lane = t & 31, i = lane >> lg, ln = lane & ((1 << lg) - 1);
+            const bool on = i < (int)(job >> 20);
+            const int r = (int)(job & 0xffff) + i;
             T v = 0;
-            if (on) {
-                const int* ptr = at<const int>(tab.ptr);
-                v = entries<R>(w, ptr[r] + ln, ptr[r + 1], lanes, at<const R>(tab.ref), at<const T>(tab.val), off, off1,
-                               off2);
-            }
-            for (int o = lanes >> 1; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+            if (on)
+                v = entries<R>(w, ptr[r] + ln, ptr[r + 1], 1 << lg, at<const R>(tab.ref), at<const T>(tab.val), off);
+            for (int o = 1 << lg >> 1; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
             if (on && ln == 0) done(at<const uint16_t>(tab.idx)[r], v);
         }
     }
 
-    // a row's neighbour sum: gt . x over the axis neighbours added to r
+    // a row's neighbour sum: gt/dd . x over the axis neighbours added to r
     __device__ __forceinline__ T couple(bool w, const T* coef, int nr, int i, int x, const unsigned* u, T r) const {
         T xv[2 * D];
         get<2 * D, T>(w, x, u, xv);
@@ -220,7 +237,7 @@ struct Coarse {
                 }
                 r = fmadd(-coef[(2 * D + 2) * nr + nx + i], sd, r + sc);
             }
-            r = couple(w, coef, nr, i, xo, u, r) * coef[(2 * D + 1) * nr + i];
+            r = couple(w, coef, nr, i, xo, u, r * coef[(2 * D + 1) * nr + i]);
             x[i] = r;
             if (last) y[i] = coef[(2 * D + 2) * nr + i] * r;
         }
@@ -233,7 +250,7 @@ struct Coarse {
         T* x = at<T>(L.x) + L.nr;
         T* y = at<T>(L.y) + L.nr;
         rows<unsigned>(
-            w, 0, L.g, L.x, L.snap, L.b, [](int) {},
+            w, nthr, 0, L.g, 0, [](int) {},
             [&](int g, T v) {
                 x[g] = v;
                 if (last) y[g] = rho[g] * v;
@@ -249,14 +266,14 @@ struct Coarse {
         const T* b = at<const T>(L.b);
         T* R = at<T>(L.y);
         rows<uint16_t>(
-            w, (own + 31) / 32 * 32, L.r, xo, 0, 0,
+            w, nthr, (own + 31) / 32 * 32, L.r, xo,
             [&](int t) {
                 if (t >= own) return;
                 const int i = t < cr ? t : cbn + t;
                 unsigned u[2 * D];
 #pragma unroll
                 for (int q = 0; q < 2 * D; q++) u[q] = nbr[q * nr + i];
-                R[i] = couple(w, coef, nr, i, xo, u, fmadd(-coef[2 * D * nr + i], x[i], b[i]));
+                R[i] = coef[2 * D * nr + i] * couple(w, coef, nr, i, xo, u, fmadd(b[i], coef[(2 * D + 1) * nr + i], -x[i]));
             },
             [&](int g, T v) { R[nr + g] = b[nr + g] - v; });
     }
@@ -271,11 +288,17 @@ struct Coarse {
         const T* di = at<const T>(C.coef) + (2 * D + 1) * nr;
         T* b = at<T>(C.b);
         T* x = at<T>(C.x);
+        // a row's entries are a chain of loads and multiply-adds: up to four
+        // lanes share it where the threads suffice
+        const int lg = 4 * nr <= nthr ? 2 : (2 * nr <= nthr ? 1 : 0);
         rows<uint16_t>(
-            w, (nr + 31) / 32 * 32, C.c, yo, 0, 0,
-            [&](int i) {
-                if (i >= nr) return;
-                const T v = entries<uint16_t>(w, ptr[i], ptr[i + 1], 1, ref, val, yo, 0, 0);
+            w, nthr, ((nr << lg) + 31) / 32 * 32, C.c, yo,
+            [&](int t) {
+                const int i = t >> lg, ln = t & ((1 << lg) - 1);
+                T v = 0;
+                if (i < nr) v = entries<uint16_t>(w, ptr[i] + ln, ptr[i + 1], 1 << lg, ref, val, yo);
+                for (int o = 1 << lg >> 1; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+                if (i >= nr || ln) return;
                 b[i] = v;
                 x[i] = i < cr ? v * di[i] : (T)0;
             },
@@ -334,8 +357,8 @@ struct Coarse {
     }
 
     // The sweeps of one visit of a level whose rows fit the threads, and after
-    // the down sweeps the defect: a thread has a red row, a black row or four
-    // lanes share a ghost's row, kept in registers (coefficients and
+    // the down sweeps the defect: a thread has a red row, a black row and a
+    // lane of a ghost's row, kept in registers (coefficients and
     // addresses) over the visit, so a phase is a handful of loads and
     // multiply-adds between two barriers.  What a warp executes between two
     // barriers is its latency and what all warps execute the CTA's, so nothing
@@ -345,15 +368,16 @@ struct Coarse {
     template <bool W>
     __device__ __forceinline__ void visit(const CLev& L, int nsw, bool skip_red, bool delta, bool last,
                                           bool dft) const {
-        const int nr = L.nr, cr = L.cr, cg = L.cg;
-        const int tb = (cr + 31) & ~31, tg = tb + ((L.cb + 31) & ~31), nact = tg + ((4 * cg + 31) & ~31);
+        const int nr = L.nr, cr = L.cr;
+        const int nact = max((max(cr, L.cb) + 31) & ~31, 32 * L.g.nw);
         auto barrier = [&] {
             if (W)
                 cluster_barrier();
             else
                 asm volatile("bar.sync 1, %0;" ::"r"(nact) : "memory");
         };
-        const int nbar = 3 * nsw - (skip_red ? 1 : 0) - (dft ? 0 : 1);  // (before the defect: one more)
+        const int nph = 3 * nsw - (skip_red ? 1 : 0);
+        const int nbar = nph - (dft ? 0 : 1);  // (before the defect: one more)
         if (tid >= nact) {
             if (W)
                 for (int q = 0; q < nbar; q++) cluster_barrier();
@@ -361,148 +385,131 @@ struct Coarse {
         }
         const T* coef = at<const T>(L.coef);
         const int xo = L.x;
+        const T* bs = at<const T>(L.b);
         T* xs = at<T>(xo);
         T* y = at<T>(L.y);
-        if (tid < tg) {
-            const bool black = tid >= tb;
-            const int i = black ? cr + tid - tb : tid;
-            const bool on = black ? i < nr : i < cr;
-            const bool near = on && black && i >= cr + L.cbn, own = on && (!black || near);
-            unsigned u[2 * D];
-            T g[2 * D], di = 0, b = 0, dsum = 0, rho = 0;
+        const bool gwarp = tid >> 5 < L.g.nw;
+        const unsigned job = gwarp ? at<const unsigned>(L.g.job)[tid >> 5] : 0;
+        const int lg = job >> 16 & 15, ln = tid & ((1 << lg) - 1), gr = (int)(job & 0xffff) + ((tid & 31) >> lg);
+        const bool rowg = (tid & 31) >> lg < (int)(job >> 20);
+        int gi = 0;
+        constexpr bool kRegs = sizeof(T) == 4;  // FP64 coefficients stay in shared memory (registers)
+        unsigned u[2][2 * D], a[4];
+        T g[2][2 * D], bb[2], c[4];  // bb: b/dd, at first with what the neighbours are off their c rows by
+        bool on[2], own[2];
+        {
             const uint16_t* nbr = at<const uint16_t>(L.nbr);
-            if (on) {
+#pragma unroll
+            for (int k = 0; k < 2; k++) {
+                const int i = k ? cr + tid : tid;
+                on[k] = tid < (k ? L.cb : cr);
+                own[k] = on[k] && (k == 0 || tid >= L.cbn);  // has a defect, sees values off their c rows
+                if (!on[k]) continue;
+                T r = bs[i];
 #pragma unroll
                 for (int q = 0; q < 2 * D; q++) {
-                    u[q] = nbr[q * nr + i];
-                    g[q] = coef[q * nr + i];
+                    u[k][q] = nbr[q * nr + i];
+                    if (kRegs) g[k][q] = coef[q * nr + i];
                 }
-                di = coef[(2 * D + 1) * nr + i];
-                b = at<const T>(L.b)[i];
-                if (last) rho = coef[(2 * D + 2) * nr + i];
-                if (delta && own) {
+                if (delta && own[k]) {
                     // what the neighbours are off their c rows by
                     T2 d[2 * D];
 #pragma unroll
-                    for (int q = 0; q < 2 * D; q++) ld_at<W>(addr<W, T2>(L.d2, u[q]), d[q]);
+                    for (int q = 0; q < 2 * D; q++) ld_at<W>(addr<W, T2>(L.d2, u[k][q]), d[q]);
                     T sd = 0, sc = 0;
 #pragma unroll
                     for (int q = 0; q < 2 * D; q++) {
                         sd += d[q].x;
                         sc += d[q].y;
                     }
-                    dsum = fmadd(-coef[(2 * D + 2) * nr + L.nx + i], sd, sc);
+                    r = fmadd(-coef[(2 * D + 2) * nr + L.nx + i], sd, r + sc);
                 }
+                bb[k] = r * coef[(2 * D + 1) * nr + i];
 #pragma unroll
-                for (int q = 0; q < 2 * D; q++) u[q] = addr<W, T>(xo, u[q]);
+                for (int q = 0; q < 2 * D; q++) u[k][q] = addr<W, T>(xo, u[k][q]);
             }
-            // phases: red, black, ghosts, red, ...; one copy of the code
-            int kind = skip_red ? 1 : 0;
-            const int mine = black ? 1 : 0;
+        }
+        const unsigned* ref = at<const unsigned>(L.g.ref);
+        const T* val = at<const T>(L.g.val);
+        int beg = 0, end = 0;
+        // address of entry k of the ghost's row (past the end: its last one's, times 0)
+        auto entry = [&](int k) { return where<unsigned>(W, 0, ref[min(k, end - 1)]); };
+        if (rowg) {
+            const int* ptr = at<const int>(L.g.ptr);
+            gi = at<const uint16_t>(L.g.idx)[gr];
+            beg = ptr[gr] + ln;
+            end = ptr[gr + 1];
+#pragma unroll
+            for (int q = 0; q < 4; q++) {
+                const int k = beg + (q << lg);
+                a[q] = entry(k);
+                c[q] = k < end ? val[k] : (T)0;
+            }
+        }
+        const int plast = last ? nph - 3 : nph;  // from here on y = rho s is kept
+        auto row = [&](int k, int p) {
+            const int i = k ? cr + tid : tid;
+            T v[2 * D], r = bb[k];
+#pragma unroll
+            for (int e = 0; e < 2 * D; e++) ld_at<W>(u[k][e], v[e]);
+#pragma unroll
+            for (int e = 0; e < 2 * D; e++) r = fmadd(kRegs ? g[k][e] : coef[e * nr + i], v[e], r);
+            xs[i] = r;
+            if (p >= plast) y[i] = coef[(2 * D + 2) * nr + i] * r;
+            if (p < 3 && delta) bb[k] = bs[i] * coef[(2 * D + 1) * nr + i];
+        };
+        // phases: red, black, ghosts, red, ...; one copy of each phase's code
+        int kind = skip_red ? 1 : 0;
 #pragma unroll 1
-            for (int q = 0; q < 3 * nsw - (skip_red ? 1 : 0); q++) {
-                if (on && kind == mine) {
-                    T v[2 * D], r = b + dsum;
+        for (int p = 0; p < nph; p++) {
+            if (kind == 0) {
+                if (on[0]) row(0, p);
+            } else if (kind == 1) {
+                if (rowg && ln == 0) at<T>(L.snap)[gi] = xs[nr + gi];
+                if (on[1]) row(1, p);
+            } else if (gwarp) {
+                T v = 0;
+                if (rowg) {
+                    T w[4];
 #pragma unroll
-                    for (int e = 0; e < 2 * D; e++) ld_at<W>(u[e], v[e]);
+                    for (int q = 0; q < 4; q++) ld_at<W>(a[q], w[q]);
 #pragma unroll
-                    for (int e = 0; e < 2 * D; e++) r = fmadd(g[e], v[e], r);
-                    r *= di;
-                    xs[i] = r;
-                    if (last) y[i] = rho * r;  // the last sweep's stays
-                    dsum = 0;
-                }
-                kind = kind == 2 ? 0 : kind + 1;
-                if (q < nbar) barrier();
-            }
-            if (dft && own) {
-                T v[2 * D];
-#pragma unroll
-                for (int q = 0; q < 2 * D; q++) ld_at<W>(u[q], v[q]);
-                T r = fmadd(-coef[2 * D * nr + i], xs[i], b);
-#pragma unroll
-                for (int q = 0; q < 2 * D; q++) r = fmadd(g[q], v[q], r);
-                y[i] = r;
-            }
-        } else {
-            const int t = tid - tg, gi = t >> 2, ln = t & 3;
-            const bool on = gi < cg;
-            const unsigned* ref = at<const unsigned>(L.g.ref);
-            const T* val = at<const T>(L.g.val);
-            T* snap = at<T>(L.snap);
-            const int so = L.snap, bo = L.b;
-            int beg = 0, end = 0;
-            unsigned a[4];
-            T c[4], rho = 0;
-            auto fetch = [&](int j) {
-#pragma unroll
-                for (int q = 0; q < 4; q++) {
-                    const int k = j + 4 * q;
-                    const unsigned e = ref[k < end ? k : beg], kind = e >> 16;
-                    a[q] = addr<W, T>(kind == 0 ? xo : (kind == 1 ? so : bo), e & 0xffffu);
-                    c[q] = k < end ? val[k] : (T)0;
-                }
-            };
-            if (on) {
-                const int* ptr = at<const int>(L.g.ptr);
-                beg = ptr[gi] + ln;
-                end = ptr[gi + 1];
-                if (beg >= end) beg = end - 1;  // (a lane without an entry reads one and drops it)
-                fetch(ptr[gi] + ln);
-                if (last) rho = coef[(2 * D + 3) * nr + gi];
-            }
-            const bool more = on && beg + 16 < end;
-            int kind = skip_red ? 1 : 0;
+                    for (int q = 0; q < 4; q++) v = fmadd(c[q], w[q], v);
 #pragma unroll 1
-            for (int p = 0; p < 3 * nsw - (skip_red ? 1 : 0); p++) {
-                if (kind == 1) {
-                    if (on && ln == 0) snap[gi] = xs[nr + gi];
-                } else if (kind == 2) {
-                    T v = 0;
-                    if (on) {
-                        T w[4];
+                    for (int j = beg + (4 << lg); j < end; j += 4 << lg) {
 #pragma unroll
-                        for (int q = 0; q < 4; q++) ld_at<W>(a[q], w[q]);
+                        for (int q = 0; q < 4; q++) ld_at<W>(entry(j + (q << lg)), w[q]);
 #pragma unroll
-                        for (int q = 0; q < 4; q++) v = fmadd(c[q], w[q], v);
-                        if (more) {
-#pragma unroll 1
-                            for (int j = beg + 16; j < end; j += 16) {
-#pragma unroll
-                                for (int q = 0; q < 4; q++) {
-                                    const int k = j + 4 * q;
-                                    const unsigned e = ref[k < end ? k : beg], kd = e >> 16;
-                                    ld_at<W>(addr<W, T>(kd == 0 ? xo : (kd == 1 ? so : bo), e & 0xffffu), w[q]);
-                                }
-#pragma unroll
-                                for (int q = 0; q < 4; q++) {
-                                    const int k = j + 4 * q;
-                                    v = fmadd(k < end ? val[k] : (T)0, w[q], v);
-                                }
-                            }
+                        for (int q = 0; q < 4; q++) {
+                            const int k = j + (q << lg);
+                            v = fmadd(k < end ? val[k] : (T)0, w[q], v);
                         }
                     }
-                    v += __shfl_xor_sync(0xffffffffu, v, 2);
-                    v += __shfl_xor_sync(0xffffffffu, v, 1);
-                    if (on && ln == 0) {
-                        xs[nr + gi] = v;
-                        if (last) y[nr + gi] = rho * v;
-                    }
                 }
-                kind = kind == 2 ? 0 : kind + 1;
-                if (p < nbar) barrier();
-            }
-            if (dft) {
-                T v = 0;
-                if (on) {
-                    const int* ptr = at<const int>(L.r.ptr);
-                    v = entries<uint16_t>(W, ptr[gi] + ln, ptr[gi + 1], 4, at<const uint16_t>(L.r.ref),
-                                          at<const T>(L.r.val), xo, 0, 0);
+                for (int o = 1 << lg >> 1; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+                if (rowg && ln == 0) {
+                    xs[nr + gi] = v;
+                    if (p >= plast) y[nr + gi] = coef[(2 * D + 3) * nr + gi] * v;
                 }
-                v += __shfl_xor_sync(0xffffffffu, v, 2);
-                v += __shfl_xor_sync(0xffffffffu, v, 1);
-                if (on && ln == 0) y[nr + gi] = at<const T>(L.b)[nr + gi] - v;
             }
+            kind = kind == 2 ? 0 : kind + 1;
+            if (p < nbar) barrier();
+        }
+        if (dft) {
+#pragma unroll
+            for (int k = 0; k < 2; k++) {
+                if (!own[k]) continue;
+                const int i = k ? cr + tid : tid;
+                T v[2 * D];
+#pragma unroll
+                for (int q = 0; q < 2 * D; q++) ld_at<W>(u[k][q], v[q]);
+                T r = bb[k] - xs[i];
+#pragma unroll
+                for (int q = 0; q < 2 * D; q++) r = fmadd(kRegs ? g[k][q] : coef[q * nr + i], v[q], r);
+                y[i] = r * coef[2 * D * nr + i];
+            }
+            rows<uint16_t>(
+                W, nact, 0, L.r, xo, [](int) {}, [&](int g, T v) { y[nr + g] = bs[nr + g] - v; });
         }
         // (the caller's barrier follows)
     }
@@ -582,6 +589,7 @@ __global__ void __launch_bounds__(kCoarseThreads, 1) k_s_coarse(const CDesc<T>* 
         for (int i = threadIdx.x; i < 2 * lev[l].cr; i += blockDim.x) k.template at<T>(lev[l].d2)[i] = 0;
     const int nx = lev[0].nx;
     pdl_enter();
+    const bool done = d.skip && *(const volatile int*)d.skip;  // the finest level's first sweep
     {
         // the first level's right-hand side, and its red half-sweep from zero
         const CLev& L = lev[0];
@@ -590,7 +598,7 @@ __global__ void __launch_bounds__(kCoarseThreads, 1) k_s_coarse(const CDesc<T>* 
         for (int i = threadIdx.x; i < nx; i += blockDim.x) {
             const T v = __ldcg(bg + i);
             k.template at<T>(L.b)[i] = v;
-            k.template at<T>(L.x)[i] = i < cr ? v * di[i] : (T)0;
+            k.template at<T>(L.x)[i] = d.skip ? __ldcg(X + slot[i]) : (i < cr ? v * di[i] : (T)0);
         }
     }
     for (int pc = 0; pc < nop; pc++) {
@@ -606,12 +614,16 @@ __global__ void __launch_bounds__(kCoarseThreads, 1) k_s_coarse(const CDesc<T>* 
                 case kOpRestrict: k.restrict_to(*(&L - 1), L, w); break;
                 case kOpSolve: k.solve(L, w, d, ag); break;
                 case kOpProlong: k.prolong(L, *(&L + 1), w); break;
-                case kOpVisit:
+                case kOpVisit: {
+                    const bool first = done && (o & kOpTop);
+                    const int nsw = (int)(o >> 24) - (first ? 1 : 0);
+                    const bool skip_red = (o & kOpSkipRed) && !first;
                     if (w)
-                        k.template visit<true>(L, o >> 24, o & kOpSkipRed, delta, last, o & kOpDown);
+                        k.template visit<true>(L, nsw, skip_red, delta, last, o & kOpDown);
                     else
-                        k.template visit<false>(L, o >> 24, o & kOpSkipRed, delta, last, o & kOpDown);
+                        k.template visit<false>(L, nsw, skip_red, delta, last, o & kOpDown);
                     break;
+                }
                 default: break;
             }
         }
@@ -675,6 +687,20 @@ bool cluster_fits(int C, size_t smem) {
 
 inline size_t up16(size_t n) { return (n + 15) & ~size_t(15); }
 
+// the warps of a table's rows, given their lengths, longest first
+template <typename T>
+std::vector<unsigned> row_jobs(const std::vector<int>& len) {
+    std::vector<unsigned> jobs;
+    for (int i = 0, n = (int)len.size(); i < n;) {
+        int lg = 0;
+        while (lg < 5 && kRowEntries<T> << lg < len[i]) lg++;
+        const int cnt = std::min(32 >> lg, n - i);
+        jobs.push_back(row_job(i, lg, cnt));
+        i += cnt;
+    }
+    return jobs;
+}
+
 template <typename T>
 struct Download {
     std::vector<T> v;
@@ -699,7 +725,7 @@ struct HostLevel {
 
 template <int D, typename T>
 int build_coarse(CoarseSet<T>& S, const LevelGeo* G, const SGeo* SG, const SVec<T>* V, int L, int want, int nu1,
-                 int nu2, int max_cta, double* acc, DevMem& mem, cudaStream_t s, std::string& err) {
+                 int nu2, int max_cta, double* acc, const int* skip, DevMem& mem, cudaStream_t s, std::string& err) {
     S.l0 = -1;
     S.want = want;
     S.nu1 = nu1;
@@ -708,16 +734,23 @@ int build_coarse(CoarseSet<T>& S, const LevelGeo* G, const SGeo* SG, const SVec<
     S.rows = true;
     if (want < 0 || want > L - 1) return SULF_OK;
     const bool f32 = std::is_same<T, float>::value;
-    // levels of up to this many nodes run on CTA 0: FP32 phases are short
-    // there; an SM's two FP64 lanes make it slow sooner
-    const int narrow = f32 ? 1200 : 600;
-    constexpr size_t kNodeBytes = sizeof(T) * (2 * D + 9);
+    // Levels of up to this many nodes run on CTA 0, whose phases are short: 120
+    // cycles against the 770 of a cluster's, while an SM's two FP64 lanes or
+    // the ghosts of 3-D levels make them long sooner.  Two CN steps with 300 /
+    // 600 / 1200: 257^2 star, mixed 7.49 / 7.47 / 7.77 and 5.81 / 5.81 / 5.70 ms;
+    // 1025^2 star, FP64 8.77 / 8.62 / 8.63, mixed 5.92 / 5.79 / 5.80; 321^2 star
+    // (Neumann), FP64 8.33 / 7.87 / 7.89; 65^3 box, mixed 17.2 / 18.4 / 18.4;
+    // 129^3 box, FP64 28.0 / 28.7 / 28.7.
+    const int narrow = D == 3 ? 300 : (f32 ? 1200 : 600);
+    // The finest level joins where its rows fit the threads (a visit, else its
+    // phases are no shorter there than as kernels of their own).
+    auto top_fits = [&](int C) { return std::max(SG[0].n0, SG[0].n1) <= kCoarseThreads * C; };
     // the first level that fits, with the smallest cluster
     int l0 = want, ncta = 0;
     for (; l0 < L; l0++) {
         size_t nodes = 0;
         for (int l = l0; l < L; l++) nodes += (size_t)G[l].nin[0] + G[l].nin[1] + G[l].ng;
-        if (nodes > 40000) continue;
+        if (nodes > 40000 || (l0 == 0 && !top_fits(std::min(max_cta, kCoarseMaxCta)))) continue;
         break;
     }
     if (l0 >= L) return SULF_OK;
@@ -766,6 +799,7 @@ int build_coarse(CoarseSet<T>& S, const LevelGeo* G, const SGeo* SG, const SVec<
     for (; l0 < L && !fit; l0++) {
         for (int C : {8, 16}) {
             if (C > max_cta) break;
+            if (l0 == 0 && !top_fits(C)) continue;
             const int n = L - l0;
             ncta = C;
             // deal the nodes: bands of the box order (slots are box order up to
@@ -820,13 +854,22 @@ int build_coarse(CoarseSet<T>& S, const LevelGeo* G, const SGeo* SG, const SVec<
             // levels whose rows fit the threads are swept a visit at a time
             auto fits = [&](int l) {
                 const HostLevel& h = H[l0 + l];
-                for (int r = 0; r < C; r++)
-                    if (((h.cr[r] + 31) & ~31) + ((h.cb[r] + 31) & ~31) + ((4 * h.cg[r] + 31) & ~31) > kCoarseThreads)
+                const int nin = SG[l0 + l].n0 + SG[l0 + l].n1;
+                for (int r = 0; r < C; r++) {
+                    std::vector<int> len;
+                    for (int q = 0; q < h.cg[r]; q++) {
+                        const int gi = h.own[r][h.cr[r] + h.cb[r] + q] - nin;
+                        len.push_back(h.gptr.v[gi + 1] - h.gptr.v[gi]);
+                        if (!len.back()) return false;
+                    }
+                    std::sort(len.begin(), len.end(), std::greater<int>());
+                    if (std::max(h.cr[r], h.cb[r]) > kCoarseThreads ||
+                        32 * row_jobs<T>(len).size() > (size_t)kCoarseThreads)
                         return false;
-                for (int q = 0; q < G[l0 + l].ng; q++)
-                    if (h.gptr.v[q + 1] - h.gptr.v[q] > kLongRow || h.gptr.v[q + 1] == h.gptr.v[q]) return false;
+                }
                 return nu1 < 256 && nu2 < 256;
             };
+            if (l0 == 0 && !fits(0)) continue;
             // the program
             prog.clear();
             {
@@ -846,7 +889,8 @@ int build_coarse(CoarseSet<T>& S, const LevelGeo* G, const SGeo* SG, const SVec<
                 for (int l = 0; l + 1 < n; l++) {
                     const bool both = wide(l) || wide(l + 1);
                     if (fits(l)) {
-                        op(kOpVisit, l, l, l, (unsigned)nu1 << 24 | kOpSkipRed | kOpDown, both);
+                        const unsigned top = l0 + l > 0 ? kOpSkipRed : (f32 ? kOpSkipRed | kOpTop : kOpTop);
+                        op(kOpVisit, l, l, l, (unsigned)nu1 << 24 | top | kOpDown, both);
                     } else {
                         for (int q = 0; q < nu1; q++) sweep(l, q > 0, 0, false);
                         op(kOpDefect, l, l, l, 0, both);
@@ -926,28 +970,29 @@ int build_coarse(CoarseSet<T>& S, const LevelGeo* G, const SGeo* SG, const SVec<
                     return d.tab_at + (int)(o - t0);
                 };
                 // rows given in ghost order, stored longest first
-                auto put_tab = [&](CTab& tb, const std::vector<int>& rp, const auto& ref, const std::vector<T>& val,
-                                   bool sorted) {
+                auto put_tab = [&](CTab& tb, const std::vector<int>& rp, const auto& ref, const std::vector<T>& val) {
                     const int cnt = (int)rp.size() - 1;
                     std::vector<uint16_t> idx(cnt);
                     for (int i = 0; i < cnt; i++) idx[i] = (uint16_t)i;
                     auto len = [&](int i) { return rp[i + 1] - rp[i]; };
-                    if (sorted) std::stable_sort(idx.begin(), idx.end(), [&](int a, int b) { return len(a) > len(b); });
-                    std::vector<int> p(1, 0);
+                    std::stable_sort(idx.begin(), idx.end(), [&](int a, int b) { return len(a) > len(b); });
+                    std::vector<int> p(1, 0), ln;
                     auto rf = ref;
                     std::vector<T> vl;
                     rf.clear();
-                    tb.nx = tb.nl = tb.ns = 0;
                     for (int i : idx) {
                         rf.insert(rf.end(), ref.begin() + rp[i], ref.begin() + rp[i + 1]);
                         vl.insert(vl.end(), val.begin() + rp[i], val.begin() + rp[i + 1]);
                         p.push_back((int)rf.size());
-                        (len(i) > kLongRow ? tb.nx : (len(i) > kShortRow ? tb.nl : tb.ns))++;
+                        ln.push_back(len(i));
                     }
                     tb.ptr = put(p.data(), 4 * p.size());
                     tb.ref = put(rf.data(), sizeof(rf[0]) * rf.size());
                     tb.val = put(vl.data(), sizeof(T) * vl.size());
                     tb.idx = put(idx.data(), 2 * idx.size());
+                    const std::vector<unsigned> jobs = row_jobs<T>(ln);
+                    tb.nw = (int)jobs.size();
+                    tb.job = put(jobs.data(), 4 * jobs.size());
                 };
                 for (int l = l0; l < L; l++) {
                     CLev& c = lev[(size_t)r * n + l - l0];
@@ -977,19 +1022,22 @@ int build_coarse(CoarseSet<T>& S, const LevelGeo* G, const SGeo* SG, const SVec<
                         const int gi = h.own[r][c.nr + q] - nin;
                         for (int j = h.gptr.v[gi]; j < h.gptr.v[gi + 1]; j++) {
                             const int code = h.gcode.v[j];
-                            unsigned kind = 0, ref;
+                            unsigned ref;
+                            int base = c.x;
                             if (code >= 0) {
                                 ref = h.ref[code];
                             } else {
                                 const unsigned w = ~(unsigned)code;
                                 ref = h.ref[h.gslot.v[w >> 1]];
-                                kind = (w & 1u) ? 2 : 1;
-                                if (kind == 1) {  // snap holds the ghosts only
+                                base = c.b;
+                                if (!(w & 1u)) {  // snap holds the ghosts only
                                     const int o = (int)(ref >> kRefBits);
                                     ref -= (unsigned)(h.cr[o] + h.cb[o]);
+                                    base = c.snap;
                                 }
                             }
-                            gr.push_back(kind << 16 | ref);
+                            gr.push_back((ref >> kRefBits) << kAddrBits |
+                                         (unsigned)(base + (int)(ref & kRefMask) * (int)sizeof(T)));
                             val.push_back((T)h.gval.v[j]);
                         }
                         ptr.push_back((int)gr.size());
@@ -999,8 +1047,8 @@ int build_coarse(CoarseSet<T>& S, const LevelGeo* G, const SGeo* SG, const SVec<
                         }
                         rp.push_back((int)rr.size());
                     }
-                    put_tab(c.g, ptr, gr, val, !fits(l - l0));
-                    put_tab(c.r, rp, rr, rv, !fits(l - l0));
+                    put_tab(c.g, ptr, gr, val);
+                    put_tab(c.r, rp, rr, rv);
                     // coarse corners of the black nodes and the ghosts
                     auto coords = [&](int t, int* ii) {
                         int sl = t >= nin ? h.gslot.v[t - nin] : (t >= g.n0 ? g.Hn : 0) + (h.hl.v[t] >> kEntHalf);
@@ -1092,7 +1140,7 @@ int build_coarse(CoarseSet<T>& S, const LevelGeo* G, const SGeo* SG, const SVec<
                             }
                             ptr.push_back((int)rr.size());
                         }
-                        put_tab(c.c, ptr, rr, rv, true);
+                        put_tab(c.c, ptr, rr, rv);
                     }
                 }
                 d.tab_len[r] = (int)(tab.size() - t0);
@@ -1130,7 +1178,6 @@ int build_coarse(CoarseSet<T>& S, const LevelGeo* G, const SGeo* SG, const SVec<
         }
         if (fit) break;
     }
-    (void)kNodeBytes;
     if (!fit) return SULF_OK;
     const int n = L - l0, C = ncta;
     // device copies
@@ -1180,14 +1227,19 @@ int build_coarse(CoarseSet<T>& S, const LevelGeo* G, const SGeo* SG, const SVec<
                 perm[l][H[l].own[r][i]] = CPerm{base + i, c.nr, base + (2 * D + 2) * c.nr + i, c.nx};
         }
     }
-    // (the first level and its lists may change with the threshold: new
-    // arrays, the old ones stay with the handle)
+    // (rebuilt for another threshold or cluster size: the old set's arrays,
+    // which nothing in flight reads, where they are large enough)
+    size_t used = 0;
     auto upload = [&](auto*& dst, const auto& v) {
-        dst = (std::remove_reference_t<decltype(dst)>)mem.get(sizeof(v[0]) * v.size() + 64);
-        return dst && cudaMemcpyAsync(dst, v.data(), sizeof(v[0]) * v.size(), cudaMemcpyHostToDevice, s) == cudaSuccess;
+        const size_t nb = sizeof(v[0]) * v.size();
+        if (used == S.kept.size()) S.kept.push_back({nullptr, 0});
+        auto& k = S.kept[used++];
+        if (!k.first || k.second < nb) k = {mem.get(nb + 64), nb};
+        dst = (std::remove_reference_t<decltype(dst)>)k.first;
+        return dst && cudaMemcpyAsync(dst, v.data(), nb, cudaMemcpyHostToDevice, s) == cudaSuccess;
     };
     for (int l = 0; l < SULF_MAXLEV; l++) S.perm[l] = nullptr;
-    for (int l = l0; l < L; l++)
+    for (int l = L - 1; l >= l0; l--)
         if (!upload(S.perm[l], perm[l])) return oom();
     std::vector<char> head((size_t)C * d.head_len, 0);
     for (int r = 0; r < C; r++) {
@@ -1205,6 +1257,7 @@ int build_coarse(CoarseSet<T>& S, const LevelGeo* G, const SGeo* SG, const SVec<
     d.slot = S.slot;
     d.X = V[l0].X;
     d.acc = l0 == 0 ? acc : nullptr;
+    d.skip = l0 == 0 ? skip : nullptr;
     d.cnt_m = S.cnt_m;
     d.nlev = n;
     d.ncta = C;
@@ -1259,7 +1312,7 @@ int launch_coarse_batched(const CDesc<T>* const* descs, int K, const int* active
 
 #define SULF_INST_COARSE(D, T)                                                                                      \
     template int build_coarse<D, T>(CoarseSet<T>&, const LevelGeo*, const SGeo*, const SVec<T>*, int, int, int, int, \
-                                    int, double*, DevMem&, cudaStream_t, std::string&);                                            \
+                                    int, double*, const int*, DevMem&, cudaStream_t, std::string&);                                            \
     template int launch_coarse<D, T>(const CoarseSet<T>&, cudaStream_t);                                          \
     template int launch_coarse_batched<D, T>(const CDesc<T>* const*, int, const int*, int, size_t, cudaStream_t);
 SULF_INST_COARSE(2, double)

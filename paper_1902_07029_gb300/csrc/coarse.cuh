@@ -20,11 +20,11 @@ namespace sulf {
 constexpr int kCoarseThreads = 512;
 constexpr int kCoarseMaxCta = 16;
 
-// rows of one table, longest first: `nx` rows by whole warps, `nl` by kRowLanes
-// lanes each, `ns` by one thread each; idx (u16): the ghost of a row
+// rows of one table, longest first, dealt to `nw` warps: job (u32) says a
+// warp's rows and the lanes of each; idx (u16): the ghost of a row
 struct CTab {
-    int ptr, ref, val, idx;  // byte offsets
-    int nx, nl, ns;
+    int ptr, ref, val, idx, job;  // byte offsets
+    int nw;
 };
 
 // one level as one CTA sees it: counts, byte offsets into its shared memory
@@ -34,9 +34,9 @@ struct CLev {
     int nr, nx;           // rows (cr + cb), nodes (nr + cg)
     int wide;             // dealt to all CTAs (else to CTA 0)
     int x, y, d2, b, snap;
-    int coef;             // gt[2D][nr], dd[nr], 1/dd[nr], rho[nx], C[nx]
+    int coef;             // gt/dd[2D][nr], dd[nr], 1/dd[nr], rho[nx], C[nx]
     int nbr;              // u16 [2D][nr]
-    CTab g;               // composed ghost rows: kind << 16 | ref (0 x, 1 snap, 2 b)
+    CTab g;               // composed ghost rows: owner << kAddrBits | byte offset of the value
     CTab r;               // ghost rows of the defect
     int pro;              // u16 [2^D][cb + cg]: coarse corners
     int cptr, cref, cval;  // rows of the restriction onto the own inside nodes
@@ -56,6 +56,7 @@ struct CDesc {
     const int* slot;        // slots of the first level's nodes, same order
     T* X;                   // the first level's x by slot
     double* acc;            // finest level of mixed precision: X is added to it (else null)
+    const int* skip;        // the first level is the finest: X is its start, set: its first sweep is done (else null)
     const int* cnt_m;       // coarsest level: own nodes of each CTA
     int nlev;
     int ncta;
@@ -85,13 +86,14 @@ struct CoarseSet {
     int* slot = nullptr;
     char* head = nullptr;
     int* cnt_m = nullptr;
+    std::vector<std::pair<void*, size_t>> kept;  // the uploaded arrays and their sizes
 };
 
 // (re)builds the set for levels l0 .. L-1 (the smallest l0 >= want that fits);
 // l0 = -1 where none does
 template <int D, typename T>
 int build_coarse(CoarseSet<T>& S, const LevelGeo* G, const SGeo* SG, const SVec<T>* V, int L, int want, int nu1,
-                 int nu2, int max_cta, double* acc, DevMem& mem, cudaStream_t s, std::string& err);
+                 int nu2, int max_cta, double* acc, const int* skip, DevMem& mem, cudaStream_t s, std::string& err);
 template <int D, typename T>
 int launch_coarse(const CoarseSet<T>& S, cudaStream_t s);
 // the fused levels of K domains (device array of their descriptors), a cluster

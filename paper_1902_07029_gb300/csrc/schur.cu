@@ -95,7 +95,7 @@ __global__ void __launch_bounds__(kT) k_s_rho(SLev<D, T> L, SLev<D, float> U, co
     const T rho = pcs * inv, C = c.kap * c.alpha * w.x;
     L.rho[sl] = rho;
     L.cs[sl] = C;
-    if (!FINE && L.perm) {
+    if (!MIXED && L.perm) {
         const CPerm q = L.perm[t];
         L.cf[q.roff] = rho;
         L.cf[q.roff + q.nx] = C;
@@ -108,10 +108,16 @@ __global__ void __launch_bounds__(kT) k_s_rho(SLev<D, T> L, SLev<D, float> U, co
         if (MIXED) {
             U.rho[sl] = (float)rho;
             U.cs[sl] = (float)C;
+            if (U.perm) {
+                const CPerm q = U.perm[t];
+                U.cf[q.roff] = (float)rho;
+                U.cf[q.roff + q.nx] = (float)C;
+            }
             L.X[sl] = 0;
             if (t >= nin) {
                 L.b[t] = (T)f.x;
                 U.b[t] = (float)f.x;
+                if (U.bpos) U.bf[U.bpos[t]] = (float)f.x;
                 U.X[sl] = 0.f;
                 U.D2[sl] = make_float2((float)-t0, (float)(-(double)C * t0));
             }
@@ -123,6 +129,7 @@ __global__ void __launch_bounds__(kT) k_s_rho(SLev<D, T> L, SLev<D, float> U, co
             L.D2[sl] = d;
             L.X[sl] = 0;
             L.b[t] = (T)f.x;
+            if (L.bpos) L.bf[L.bpos[t]] = (T)f.x;
         }
     }
 }
@@ -172,7 +179,7 @@ __global__ void __launch_bounds__(kT) k_s_coefs(SLev<D, T> L, const typename V2<
     if (L.perm) {
         const CPerm q = L.perm[t];
 #pragma unroll
-        for (int a = 0; a < 2 * D; a++) L.cf[q.off + a * q.stride] = g[a];
+        for (int a = 0; a < 2 * D; a++) L.cf[q.off + a * q.stride] = g[a] * di;
         L.cf[q.off + 2 * D * q.stride] = dd;
         L.cf[q.off + (2 * D + 1) * q.stride] = di;
     }
@@ -234,10 +241,26 @@ __global__ void __launch_bounds__(kT) k_s_coefs_fine(const __grid_constant__ SLe
         U.dd[t] = (float)dd;
         U.di[t] = df;
         U.b[t] = (float)b;
+        if (U.perm) {
+            const CPerm q = U.perm[t];
+#pragma unroll
+            for (int a = 0; a < 2 * D; a++) U.cf[q.off + a * q.stride] = (float)g[a] * df;
+            U.cf[q.off + 2 * D * q.stride] = (float)dd;
+            U.cf[q.off + (2 * D + 1) * q.stride] = df;
+            U.bf[U.bpos[t]] = (float)b;
+        }
         // the first red half-sweep from zero, the neighbours' x^c = 0 off their c rows
         if (!colour) U.X[sl] = (float)bs * df;
-    } else if (!colour) {
-        L.X[sl] = bs * di;
+    } else {
+        if (L.perm) {
+            const CPerm q = L.perm[t];
+#pragma unroll
+            for (int a = 0; a < 2 * D; a++) L.cf[q.off + a * q.stride] = g[a] * di;
+            L.cf[q.off + 2 * D * q.stride] = dd;
+            L.cf[q.off + (2 * D + 1) * q.stride] = di;
+            L.bf[L.bpos[t]] = b;
+        }
+        if (!colour) L.X[sl] = bs * di;
     }
 }
 
@@ -478,6 +501,7 @@ __device__ __forceinline__ void s_outer(const SLev<D, double>& L, const SLev<D, 
             const int h = e >> kEntHalf;
             r = inside_defect<D, double>(L, t, colour, h, e & 1, g, dd);
             U.b[t] = (float)r;
+            if (U.bpos) U.bf[U.bpos[t]] = (float)r;
             if (!colour) U.X[h] = (float)r * df;
         }
     } else {
@@ -485,6 +509,7 @@ __device__ __forceinline__ void s_outer(const SLev<D, double>& L, const SLev<D, 
         r = ghost_defect<D, double>(L, p);
         if (p.on && p.lane == 0) {
             U.b[nin + p.g] = (float)r;
+            if (U.bpos) U.bf[U.bpos[nin + p.g]] = (float)r;
             U.X[L.gslot[p.g]] = 0.f;
         }
     }

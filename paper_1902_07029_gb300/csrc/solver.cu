@@ -396,20 +396,18 @@ int ensure32(sulf_domain* d) {
 
 // whether the solver controls allow it: collective red-black V- or W-cycles
 // with pre- and post-relaxation and the composed ghost relaxation (and in
-// mixed precision not the stored-coefficient or tiled FP32 sweeps).  Small
-// mixed-precision domains stay with the two-unknown kernels, whose coarse
-// levels run as one single-CTA launch (13 k active nodes, 257^2 star: 9.8 ms
-// for two CN steps against 10.9; 104 k nodes, 65^3 box: 26.7 against 28.2 the
-// other way)
-constexpr long long kSchurMinMixed = 0;
-// automatic fused-level threshold: nodes of the first level of the cluster kernel
-constexpr int kCoarseAuto = 40000;
+// mixed precision not the stored-coefficient or tiled FP32 sweeps)
 bool schur_wanted(const sulf_domain* d) {
     const sulf_solver& v = d->solver;
-    if (v.precision == 1 && (long long)d->geo[0].nin[0] + d->geo[0].nin[1] < kSchurMinMixed) return false;
     return d->L >= 2 && v.smoother == 0 && v.cycle != 3 && v.nu1 >= 1 && v.nu2 >= 1 && v.ghost_compose &&
            (v.precision == 0 || v.relax_matrix_free == 1);
 }
+
+// Automatic fused-level threshold: nodes of the first level of the cluster
+// kernel.  Its FP64 lanes and its ghost rows (3-D) bound it sooner: two CN steps
+// with the first level at 5.5 k / 21 k nodes: 1025^2 star, mixed 5.87 / 5.72 ms,
+// FP64 8.64 / 8.66; 65^3 box, mixed 15.0 (2.7 k) / 15.6 (17 k).
+int coarse_auto(int dim, bool f32) { return dim == 2 && f32 ? 40000 : 10000; }
 
 // levels 0 .. nl-1; outer: only what the FP64 defect of mixed precision uses
 template <typename T>
@@ -457,9 +455,12 @@ int alloc_schur(sulf_domain* d, SVec<T>* V, int nl, bool outer) {
 // the fused coarse levels of the current threshold (sulf_solver::fuse_below);
 // at_least: the first of them no finer than this level; max_cta: cluster size
 template <typename T>
-int ensure_coarse(sulf_domain* d, CoarseSet<T>& S, const SVec<T>* V, int at_least = 1, int max_cta = kCoarseMaxCta) {
+int ensure_coarse(sulf_domain* d, CoarseSet<T>& S, const SVec<T>* V, int at_least = 0, int max_cta = kCoarseMaxCta) {
     int want = -1;
-    const int fb = d->solver.fuse_below >= 0 ? d->solver.fuse_below : kCoarseAuto;
+    if (d->prof) at_least = std::max(at_least, 1);  // the finest level's launches are timed
+    double* acc = std::is_same<T, float>::value ? d->s64[0].X : nullptr;
+    const int fb = d->solver.fuse_below >= 0 ? d->solver.fuse_below
+                                               : coarse_auto(d->dim, std::is_same<T, float>::value);
     if (fb > 0 && d->solver.cycle == 1)
         for (int l = at_least; l < d->L && want < 0; l++)
             if ((long long)d->geo[l].nin[0] + d->geo[l].nin[1] + d->geo[l].ng <= fb) want = l;
@@ -468,10 +469,10 @@ int ensure_coarse(sulf_domain* d, CoarseSet<T>& S, const SVec<T>* V, int at_leas
     SULF_CUDA_TRY(cudaStreamSynchronize(d->stream));
     drop_graphs(d);
     std::string err;
-    int rc = d->dim == 2 ? build_coarse<2, T>(S, d->geo, d->sgeo, V, d->L, want, nu1, nu2, max_cta, nullptr, d->mem,
-                                              d->stream, err)
-                         : build_coarse<3, T>(S, d->geo, d->sgeo, V, d->L, want, nu1, nu2, max_cta, nullptr, d->mem,
-                                              d->stream, err);
+    int rc = d->dim == 2 ? build_coarse<2, T>(S, d->geo, d->sgeo, V, d->L, want, nu1, nu2, max_cta, acc, d->dskip,
+                                              d->mem, d->stream, err)
+                         : build_coarse<3, T>(S, d->geo, d->sgeo, V, d->L, want, nu1, nu2, max_cta, acc, d->dskip,
+                                              d->mem, d->stream, err);
     return rc ? sulf_fail(rc, err) : SULF_OK;
 }
 
