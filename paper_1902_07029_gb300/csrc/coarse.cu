@@ -852,7 +852,7 @@ int build_coarse(CoarseSet<T>& S, const LevelGeo* G, const SGeo* SG, const SVec<
             // uniform offsets of the values
             std::vector<CLev> base(n);
             // levels whose rows fit the threads are swept a visit at a time
-            auto fits = [&](int l) {
+            auto visit_fits = [&](int l) {
                 const HostLevel& h = H[l0 + l];
                 const int nin = SG[l0 + l].n0 + SG[l0 + l].n1;
                 for (int r = 0; r < C; r++) {
@@ -869,6 +869,9 @@ int build_coarse(CoarseSet<T>& S, const LevelGeo* G, const SGeo* SG, const SVec<
                 }
                 return nu1 < 256 && nu2 < 256;
             };
+            std::vector<char> fits_(n);
+            for (int l = 0; l < n; l++) fits_[l] = visit_fits(l);
+            auto fits = [&](int l) { return fits_[l] != 0; };
             if (l0 == 0 && !fits(0)) continue;
             // the program
             prog.clear();
@@ -935,10 +938,10 @@ int build_coarse(CoarseSet<T>& S, const LevelGeo* G, const SGeo* SG, const SVec<
             d.coef_at = (int)off;
             // coefficients: own offsets, the tables after the largest of them
             lev.assign((size_t)C * n, CLev{});
-            size_t coef_max = 0;
+            size_t coef_max = 0, lists_max = 0;
             coef_tot = 0;
             for (int r = 0; r < C; r++) {
-                size_t e = 0;
+                size_t e = 0, lists = 0;
                 d.coef_off[r] = (int)coef_tot;
                 for (int l = l0; l < L; l++) {
                     CLev& c = lev[(size_t)r * n + l - l0];
@@ -951,14 +954,18 @@ int build_coarse(CoarseSet<T>& S, const LevelGeo* G, const SGeo* SG, const SVec<
                     c.nr = c.cr + c.cb;
                     c.nx = c.nr + c.cg;
                     c.coef = d.coef_at + (int)(sizeof(T) * e);
+                    lists += 4 * D * (size_t)c.nr + (l + 1 < L ? 2 * (size_t)(c.cb + c.cg) << D : 0);
                     e += up16(sizeof(T) * ((size_t)(2 * D + 2) * c.nr + 2 * (size_t)c.nx)) / sizeof(T);
                 }
                 d.coef_len[r] = (int)e;
                 coef_tot += e;
                 coef_max = std::max(coef_max, e);
+                lists_max = std::max(lists_max, lists);
             }
             d.tab_at = d.coef_at + (int)up16(sizeof(T) * coef_max);
+            if (d.tab_at + lists_max > kCoarseSmem) continue;  // (before the tables are built)
             tab.clear();
+            tab.reserve((size_t)C * (kCoarseSmem - d.tab_at));
             size_t tab_max = 0;
             for (int r = 0; r < C; r++) {
                 const size_t t0 = tab.size();
