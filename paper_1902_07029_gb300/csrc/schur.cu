@@ -320,6 +320,23 @@ __device__ __forceinline__ void s_relax(const SLev<D, T>& L, int t, int colour, 
     if (use_acc) L.acc[sl] += (double)r;
 }
 
+// The red half-sweep that opens an FP64 cycle, from the defects that the norm
+// of the cycle before left in R: x + r / dd is what the row gives, and takes 36
+// instead of 84 bytes a node (3-D) and one FP64 instruction instead of seven
+// (257^3 box, two CN steps: 77.4 -> 76.2 and 80.6 -> 79.6 ms).
+template <int D, typename T>
+__device__ __forceinline__ void s_correct(const SLev<D, T>& L, int t) {
+    int h = 0;
+    T di = 0;
+    if (t < L.n0) {
+        h = L.hl[t] >> kEntHalf;
+        di = L.di[t];
+    }
+    pdl_enter();
+    if (*L.skip || t >= L.n0) return;
+    L.X[h] = fmadd(L.R[h], di, L.X[h]);
+}
+
 template <int D, typename T>
 __device__ __forceinline__ T ghost_input(const SLev<D, T>& L, int code) {
     if (code >= 0) return L.X[code];
@@ -466,7 +483,8 @@ __device__ __forceinline__ void s_residual(const SLev<D, T>& L, int t, unsigned 
     if (t < nrow) {
         if (t < nin) {
             r = inside_defect<D, T>(L, pos, colour, e >> kEntHalf, e & 1, g, dd);
-            if (!NORM) L.R[colour * L.Hn + (e >> kEntHalf)] = r;
+            // (with the norm: the red ones for the next cycle, s_correct)
+            if (!NORM || !colour) L.R[colour * L.Hn + (e >> kEntHalf)] = r;
         }
     } else {
         const GhostPart p = ghost_part<D, T>(L, t - nrow, kGopLanes, kGopLanes);
@@ -951,13 +969,14 @@ __device__ __forceinline__ void s_solve(const SLev<D, T>& L, int t) {
 // ---------------------------------------------------------------------------
 // the phases as kernels, of one domain and of many
 
-enum { kPhRelax = 0, kPhDelta, kPhGhosts, kPhResidual, kPhNorm, kPhRestrict, kPhProlong, kPhSolve };
+enum { kPhRelax = 0, kPhCorrect, kPhDelta, kPhGhosts, kPhResidual, kPhNorm, kPhRestrict, kPhProlong, kPhSolve };
 
 // flags: 1 black colour, 2 snap, 4 skip on the flag, 8 accumulate
 template <int D, typename T, int PH>
 __device__ __forceinline__ void s_phase(const SLev<D, T>& L, const SLev<D, T>& C, int t, int flags,
                                         unsigned long long* norm) {
     if (PH == kPhRelax) s_relax<D, T, false>(L, t, flags & 1, flags & 2, flags & 4, flags & 8);
+    if (PH == kPhCorrect) s_correct<D, T>(L, t);
     if (PH == kPhDelta) s_relax<D, T, true>(L, t, flags & 1, flags & 2, flags & 4, flags & 8);
     if (PH == kPhGhosts) s_ghosts<D, T>(L, t, flags & 4, flags & 8);
     if (PH == kPhResidual) s_residual<D, T, false>(L, t, norm);
@@ -1544,6 +1563,7 @@ inline int relax_flags(int colour, bool snap, bool skip, bool acc) {
 template <int D, typename T>
 long long s_threads(SPhase ph, const SLev<D, T>& L, const SLev<D, T>* C) {
     switch (ph) {
+        case SPhase::correct:
         case SPhase::red: return L.n0;
         case SPhase::black: return L.n1 > L.ng ? L.n1 : L.ng;
         case SPhase::ghosts: return ghost_threads<D, T>(L, kGopLanes, 32);
@@ -1568,6 +1588,11 @@ template <int D, typename T>
 int launch_s_ghosts(const SLev<D, T>& L, bool skip, bool acc, cudaStream_t s) {
     return launch_one<D, T, kPhGhosts>(L, s_threads<D, T>(SPhase::ghosts, L, nullptr), relax_flags(0, false, skip, acc),
                                        nullptr, s);
+}
+
+template <int D, typename T>
+int launch_s_correct(const SLev<D, T>& L, cudaStream_t s) {
+    return launch_one<D, T, kPhCorrect>(L, L.n0, 0, nullptr, s);
 }
 
 template <int D, typename T>
@@ -1611,6 +1636,9 @@ int launch_s_batched(SPhase ph, bool delta, const SLev<D, T>* lv, const SLev<D, 
     if (!lc) lc = lv;
     const int fl = relax_flags(ph == SPhase::black, ph == SPhase::black, skip, acc);
     switch (ph) {
+        case SPhase::correct:
+            launch_k(kb_s_phase<D, T, kPhCorrect>, nb, kT, 0, s, lv, lc, pre, K, active, fl, norms);
+            break;
         case SPhase::red:
         case SPhase::black:
             if (delta)
@@ -1719,6 +1747,7 @@ int launch_inject_to(const LevelGeo& F, const typename V2<TF>::t* fW, const Leve
     template long long s_threads<D, T>(SPhase, const SLev<D, T>&, const SLev<D, T>*);                              \
     template int launch_s_relax<D, T>(const SLev<D, T>&, int, bool, bool, bool, bool, cudaStream_t);               \
     template int launch_s_ghosts<D, T>(const SLev<D, T>&, bool, bool, cudaStream_t);                               \
+    template int launch_s_correct<D, T>(const SLev<D, T>&, cudaStream_t);                                          \
     template int launch_s_residual<D, T>(const SLev<D, T>&, unsigned long long*, cudaStream_t);                    \
     template int launch_s_restrict<D, T>(const SLev<D, T>&, const SLev<D, T>&, cudaStream_t);                      \
     template int launch_s_prolong<D, T>(const SLev<D, T>&, const SLev<D, T>&, cudaStream_t);                       \

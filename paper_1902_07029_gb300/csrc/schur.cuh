@@ -113,7 +113,7 @@ struct SLev {
 
 // phases of the cycle over a level (restriction and prolongation: a level and
 // the next coarser one)
-enum class SPhase { red, black, ghosts, residual, outer, restrict_to, prolong_from, solve };
+enum class SPhase { correct, red, black, ghosts, residual, outer, restrict_to, prolong_from, solve };
 
 // geometry of a level in these terms (precision independent)
 struct SGeo {
@@ -237,6 +237,8 @@ template <int D, typename T>
 int launch_s_ghosts(const SLev<D, T>& L, bool skip, bool acc, cudaStream_t s);
 // defect of the red nodes, of the black ones next to a ghost and of the
 // ghosts into R (norm null), or its max-norm only (and *L.skip set to 0)
+template <int D, typename T>
+int launch_s_correct(const SLev<D, T>& L, cudaStream_t s);
 template <int D, typename T>
 int launch_s_residual(const SLev<D, T>& L, unsigned long long* norm, cudaStream_t s);
 // mixed precision: the FP64 defect of every row with its max-norm, stored as

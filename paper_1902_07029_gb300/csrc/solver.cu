@@ -783,7 +783,10 @@ struct SMG {
         if (whole) fine_sweeps++;
         const unsigned fl = d->capturing ? cudaEventRecordExternal : cudaEventRecordDefault;
         if (timed) cudaEventRecordWithFlags(next_event(d), d->stream, fl);
-        if (!skip_red) d->launches += launch_s_relax<D, T>(L, 0, delta, false, skip, add, d->stream);
+        // (an FP64 cycle's first red half-sweep: from the defects of the last norm)
+        if (!skip_red)
+            d->launches += skip ? launch_s_correct<D, T>(L, d->stream)
+                                : launch_s_relax<D, T>(L, 0, delta, false, skip, add, d->stream);
         d->launches += launch_s_relax<D, T>(L, 1, delta, true, skip, add, d->stream);
         if (timed) cudaEventRecordWithFlags(next_event(d), d->stream, fl);
         d->launches += launch_s_ghosts<D, T>(L, skip, add, d->stream);
@@ -2061,7 +2064,7 @@ struct LockClass {
     bool schur = false;
     const SLev<D, double>* s64[SULF_MAXLEV] = {};
     const SLev<D, float>* s32[SULF_MAXLEV] = {};
-    Blocks sb[SULF_MAXLEV][8];
+    Blocks sb[SULF_MAXLEV][9];
     int scoarse = -1, sncta = 0;
     size_t ssmem = 0;
     const void* sdesc = nullptr;
@@ -2227,7 +2230,7 @@ struct LockClass {
         }
         if (int rc = upload_slevels<T>(L, out)) return rc;
         for (int l = 0; l < L; l++)
-            for (int p = 0; p < 8; p++) {
+            for (int p = 0; p < 9; p++) {
                 const SPhase ph = (SPhase)p;
                 const bool pair = ph == SPhase::restrict_to || ph == SPhase::prolong_from;
                 if ((pair && l + 1 >= L) || (scoarse >= 0 && l >= scoarse)) continue;
@@ -2272,7 +2275,7 @@ struct LockClass {
             return;
         }
         auto sweep = [&](bool skip_red, bool delta, bool skip, bool add) {
-            if (!skip_red) srun<T>(lv, SPhase::red, l, delta, skip, add);
+            if (!skip_red) srun<T>(lv, skip ? SPhase::correct : SPhase::red, l, delta, skip, add);
             srun<T>(lv, SPhase::black, l, delta, skip, add);
             srun<T>(lv, SPhase::ghosts, l, false, skip, add);
         };
