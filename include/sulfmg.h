@@ -81,10 +81,13 @@ typedef struct {
    graphs        1 = each multigrid cycle is captured once as a CUDA graph and
                  replayed; 0 = kernels launched one by one               default 1
    fuse_below    the first level with at most this many active nodes and all
-                 coarser ones run as one single-CTA kernel per V-cycle;
+                 coarser ones run as one kernel per V-cycle: on a thread-block
+                 cluster for the cycle on the equation for s (the default
+                 controls; the first such level that fits its shared memory),
+                 on one CTA for the two-unknown cycle;
                  0 = every level as separate kernels (W-cycles always are);
-                 -1 = automatic: 150 for FP64, 1000 for mixed precision
-                 (the fused kernel runs on one SM)                       default -1
+                 -1 = automatic: 40000 (2-D, mixed precision) or 10000, and
+                 150 / 1000 (FP64 / mixed) on one CTA                     default -1
    pdl           1 = kernels of a step are launched as programmatic dependent
                  launches (each may be scheduled while its predecessor runs and
                  waits on the device for its completion); 0 = plain stream
@@ -100,7 +103,8 @@ typedef struct {
                  after the dependent-launch wait instead of prefetching them
                  across it, and is compiled for six resident CTAs per SM
                  instead of four: more warps hide the load latency; no effect
-                 in FP32.  Same results either way.                default 0
+                 in FP32 nor on the cycle on the equation for s.  Same results
+                 either way.                                       default 0
    relax_matrix_free 1 = the FP32 red-black collective relaxation of the
                  mixed form recomputes each node's stencil coefficients from
                  (s, c) instead of reading the stored ones (same expressions:
