@@ -50,18 +50,15 @@ PEAKS_FILE = os.path.join(ROOT, "MEASURED_PEAKS.json")
 # One colour launch updates half of the inside nodes; per updated node it is
 # charged these bytes.
 SWEEP_BYTES = {"fp64": 64, "mixed": 32}
-# Compulsory bytes of one colour update as this library streams it.  FP64:
-# the stencil coefficients precomputed once per Newton iteration -- rhs, the
-# rows of the inverse 2x2 block, the own and the other colour's edge
-# coefficients and the unknown read and written: 2-D 16 + 32 + 2*16 + 2*16 +
-# 32 = 144 B, 3-D 16 + 32 + 3*16 + 3*16 + 32 = 176 B.  FP32 (coefficients
-# recomputed from (s, c)): (s, c) of the node and of one node of the other
-# colour, x of the other colour, rhs, x written: 5 * 8 = 40 B.
-STREAM_BYTES = {2: {"fp64": 144, "mixed": 40}, 3: {"fp64": 176, "mixed": 40}}
-# FP64/FP32 arithmetic of one update: per axis four fused multiply-adds for
-# the off-diagonal part, then two fused multiply-adds and two multiplies for
-# the 2x2 block solve: 2-D 10 FMA + 2 MUL = 22 flop, 3-D 14 FMA + 2 MUL = 30.
-RELAX_FLOPS = {2: 22, 3: 30}
+# Compulsory bytes of one colour update as this library streams it: the cycle
+# runs on the equation for s alone, whose rows are stored once per Newton
+# iteration -- the edge terms (2 per axis), 1/dd, the right-hand side, one value
+# of the other colour, the value written and a 4-byte list entry: FP64 3-D
+# 6 * 8 + 4 * 8 + 4 = 84 B, 2-D 68 B; FP32 44 and 36 B.
+STREAM_BYTES = {2: {"fp64": 68, "mixed": 36}, 3: {"fp64": 84, "mixed": 44}}
+# Arithmetic of one update: a fused multiply-add per neighbour and the
+# multiply with 1/dd: 2-D 4 FMA + 1 MUL = 9 flop, 3-D 6 FMA + 1 MUL = 13.
+RELAX_FLOPS = {2: 9, 3: 13}
 # FP64 peak from the unit counts and clock: 152 SMs x 2 FP64 FMA lanes per
 # clock x 2 flop x 2.07 GHz
 FP64_PEAK_TFLOPS = 152 * 2 * 2 * 2.070e9 / 1e12
@@ -73,16 +70,14 @@ CYCLE_BYTES = {2: 344.0 * 4 / 3, 3: 344.0 * 8 / 7}
 # DRAM bytes (read + write) of one finest-level relaxation launch from an ncu
 # capture of the current kernel (cold cache), per workload and precision
 RELAX_TRAFFIC = {
-    # 129^3 capture (profiles/relax_inside_fp64_rbox129.md): 103.9 MB per
-    # 521 488 updates = 199.2 B per update, scaled to the 257^3 launch
-    ("rbox257", "fp64"): (199.2 * 4142122, "profiles/relax_inside_fp64_rbox129.md (199.2 B per update measured at "
-                                           "129^3, scaled to the 4 142 122 updates of a 257^3 launch)"),
-    ("star1025", "fp64"): (23.52e6 + 2.0e3, "profiles/relax_inside_fp64_star1025.md"),
-    # 129^3 capture of the matrix-free FP32 kernel (profiles/relax_mf_fp32_rbox129.md): 31.6 MB per
-    # 521 488 updates = 60.6 B per update, scaled to the 257^3 launch
-    ("rbox257", "mixed"): (60.6 * 4142122, "profiles/relax_mf_fp32_rbox129.md (60.6 B per update measured at "
-                                          "129^3, scaled to the 4 142 122 updates of a 257^3 launch)"),
+    # 129^3 captures (profiles/scalar_cycle_rbox129.md): 41.9 and 22.4 MB per
+    # 521 488 updates, scaled to the 257^3 launch
+    ("rbox257", "fp64"): (80.4 * 4142122, "profiles/scalar_cycle_rbox129.md (80.4 B per update measured at 129^3, "
+                                          "scaled to the 4 142 122 updates of a 257^3 launch)"),
+    ("rbox257", "mixed"): (43.0 * 4142122, "profiles/scalar_cycle_rbox129.md (43.0 B per update measured at 129^3, "
+                                           "scaled to the 4 142 122 updates of a 257^3 launch)"),
 }
+
 
 
 def whole_job_value(elapsed_ms_local: float, units_local: int, device=None) -> tuple[float, float]:
@@ -383,9 +378,9 @@ def _measure(pkg, args, name, precision, dev, rank, world, e2e_steps):
 
 
 def _roofline(m, name, prec_name, peaks):
-    """The dominant kernel (finest-level inside relaxation, one colour launch)
-    against its binding roof: the FP64 pipe for the FP64 form, HBM for the FP32
-    relaxation of the mixed form; both byte models are reported."""
+    """The finest-level relaxation (one colour launch) against HBM, the binding
+    roof in both precisions: at the measured copy bandwidth the 84 streamed
+    bytes of a 3-D FP64 update take 12.4 ps, its 7 FP64 instructions 11.1 ps."""
     dim = m["dim"]
     avg_us = 1e3 * m["relax_ms"] / max(m["relax_n"], 1)
     n = m["n_inside"] / 2.0
@@ -395,34 +390,26 @@ def _roofline(m, name, prec_name, peaks):
     ach_stream = STREAM_BYTES[dim][prec_name] * n / sec / 1e9 if sec else None
     ach_flops = RELAX_FLOPS[dim] * n / sec / 1e12 if sec else None
     traffic = RELAX_TRAFFIC.get((name, prec_name), (None, None))
-    hbm_part = {"achieved": ach_sweep, "peak": hbm, "unit": "GB/s",
-                "frac": (ach_sweep / hbm) if (ach_sweep and hbm) else None,
-                "algorithmic": f"{SWEEP_BYTES[prec_name]} B per updated node (Sec. 8 sweep bytes, coefficients "
-                               f"recomputed); {n:.0f} nodes per launch",
-                "achieved_stream_bytes": ach_stream,
-                "frac_stream_bytes": (ach_stream / hbm) if (ach_stream and hbm) else None,
-                "stream_bytes": f"{STREAM_BYTES[dim][prec_name]} B per update as streamed ("
-                                + ("precomputed coefficients)" if prec_name == "fp64" else
-                                   "coefficients recomputed from (s, c))"),
-                "traffic": traffic[0], "traffic_source": traffic[1]}
-    kname = "k_relax_inside" if prec_name == "fp64" else "k_relax_mf (coefficients from (s, c))"
-    common = {"kernel": f"{kname} (finest level, one colour)", "avg_launch_us": avg_us,
-              "launches": m["relax_n"], "sample": "one event bracket around the two back-to-back colour launches of "
-              "the first finest-level sweep of every cycle of the last timed step (library stream)"}
+    out = {"kernel": f"s_relax ({'FP64' if prec_name == 'fp64' else 'FP32'}, finest level, one colour)",
+           "avg_launch_us": avg_us, "launches": m["relax_n"],
+           "sample": "one event bracket around the two back-to-back colour launches of the first finest-level sweep "
+           "of every cycle that both colours run in full, on the last timed step (library stream)",
+           "bound": "hbm", "achieved": ach_stream, "peak": hbm, "unit": "GB/s",
+           "frac": (ach_stream / hbm) if (ach_stream and hbm) else None,
+           "algorithmic": f"{STREAM_BYTES[dim][prec_name]} B per update as streamed (rows of the equation for s); "
+                          f"{n:.0f} updates per launch",
+           "achieved_sweep_bytes": ach_sweep,
+           "sweep_bytes": f"{SWEEP_BYTES[prec_name]} B per updated node (Sec. 8 sweep bytes of both unknowns)",
+           "traffic": traffic[0], "traffic_source": traffic[1],
+           "peak_note": "measured HBM copy bandwidth (MEASURED_PEAKS.json)"}
     if prec_name == "fp64":
-        # the FP64 pipe binds: 16 FP64 instructions per 3-D update at two
-        # lanes per SM per clock take longer than the update's bytes at HBM speed
-        return {**common, "bound": "alu", "achieved": ach_flops, "peak": FP64_PEAK_TFLOPS, "unit": "TFLOP/s",
-                "frac": (ach_flops / FP64_PEAK_TFLOPS) if ach_flops else None,
-                "peak_note": "FP64 peak derived from 152 SMs x 2 FP64 FMA lanes/clock x 2 flop x 2.07 GHz",
-                "algorithmic": f"{RELAX_FLOPS[dim]} flop per update; {n:.0f} updates per launch",
-                "traffic": traffic[0], "hbm": hbm_part}
-    return {**common, "bound": "hbm", **{k: hbm_part[k] for k in ("achieved", "peak", "unit", "frac", "algorithmic",
-                                                                    "traffic")},
-            "achieved_stream_bytes": ach_stream, "frac_stream_bytes": hbm_part["frac_stream_bytes"],
-            "stream_bytes": hbm_part["stream_bytes"], "traffic_source": traffic[1],
-            "peak_note": "measured HBM copy bandwidth (MEASURED_PEAKS.json)",
-            "kind": "fp32 relaxation inside fp64 defect correction"}
+        out["alu"] = {"achieved": ach_flops, "peak": FP64_PEAK_TFLOPS, "unit": "TFLOP/s",
+                      "frac": (ach_flops / FP64_PEAK_TFLOPS) if ach_flops else None,
+                      "peak_note": "FP64 peak derived from 152 SMs x 2 FP64 FMA lanes/clock x 2 flop x 2.07 GHz",
+                      "algorithmic": f"{RELAX_FLOPS[dim]} flop per update"}
+    else:
+        out["kind"] = "fp32 relaxation inside fp64 defect correction"
+    return out
 
 
 def _step_bandwidth(m, prec_name, peaks):
