@@ -918,7 +918,9 @@ __global__ void __launch_bounds__(kFacThreads) k_coarsest_factor_cluster(
         add(2 * r + 1, 2 * r, c.a2ms * ph * cp);
         add(2 * r + 1, 2 * r + 1, c.idt + c.a2ms * (c.alpha * s * cp + ph * s));
     }
-    __syncthreads();
+    // (all of the cluster: another CTA's shared memory may be written only once
+    // that CTA is known to run)
+    cl.sync();
     __shared__ int s_piv;
     __shared__ T s_inv;
     for (int k = 0; k < m; k++) {

@@ -836,7 +836,9 @@ __global__ void __launch_bounds__(kFacThreads) k_s_factor(SLev<D, T> L, const in
             for (int j = L.rptr[r - nin]; j < L.rptr[r - nin + 1]; j++) add(r, spos[L.rslot[j]], L.rval[j]);
         }
     }
-    __syncthreads();
+    // (all of the cluster: another CTA's shared memory may be written only once
+    // that CTA is known to run)
+    cl.sync();
     __shared__ int s_piv;
     // a thread's elements (row, local column) of the elimination, packed: a
     // half-empty FP64 instruction costs as much as a full one
