@@ -561,7 +561,7 @@ __global__ void __launch_bounds__(kCoarseThreads, 1) k_s_coarse(const CDesc<T>* 
     extern __shared__ __align__(16) char coarse_smem[];
     // many domains (lock-step batching): a cluster each, masked ones skipped
     const int inst = many ? (int)(blockIdx.x / cluster_size()) : 0;
-    if (many && !active[inst]) return;
+    if (many && masked(active, inst)) return;
     const CDesc<T>& d = many ? *many[inst] : *one;
     Coarse<D, T> k;
     k.sm = coarse_smem;

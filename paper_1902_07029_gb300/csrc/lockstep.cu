@@ -51,7 +51,7 @@ template <int D, typename T>
 __global__ void __launch_bounds__(kBT) kb_relax(const BLev<D, T>* __restrict__ lv, const int* __restrict__ pre, int K,
                                                  const int* __restrict__ active, int colour) {
     const int i = find_instance(pre, K, blockIdx.x);
-    if (!active[i]) return;
+    if (masked(active, i)) return;
     const BLev<D, T>& L = lv[i];
     const int t = (blockIdx.x - pre[i]) * kBT + threadIdx.x;
     const long long st[3] = {1, L.st1, L.st2};
@@ -73,7 +73,7 @@ template <int D>
 __global__ void __launch_bounds__(kBT) kb_relax_mf(const BLev<D, float>* __restrict__ lv, const int* __restrict__ pre,
                                                     int K, const int* __restrict__ active, int colour) {
     const int i = find_instance(pre, K, blockIdx.x);
-    if (!active[i]) return;
+    if (masked(active, i)) return;
     const BLev<D, float>& L = lv[i];
     const int t = (blockIdx.x - pre[i]) * kBT + threadIdx.x;
     const long long st[3] = {1, L.st1, L.st2};
@@ -95,7 +95,7 @@ template <int D, typename T>
 __global__ void __launch_bounds__(kBT) kb_ghost_op(const BLev<D, T>* __restrict__ lv, const int* __restrict__ pre,
                                                     int K, const int* __restrict__ active) {
     const int i = find_instance(pre, K, blockIdx.x);
-    if (!active[i]) return;
+    if (masked(active, i)) return;
     const BLev<D, T>& L = lv[i];
     const int t = (blockIdx.x - pre[i]) * kBT + threadIdx.x;
     const int gi = t / stages::kGopLanes, ln = t % stages::kGopLanes;
@@ -110,7 +110,7 @@ __global__ void __launch_bounds__(kBT) kb_residual(const BLev<D, T>* __restrict_
                                                     int K, const int* __restrict__ active,
                                                     unsigned long long* norms) {
     const int i = find_instance(pre, K, blockIdx.x);
-    if (!active[i]) return;
+    if (masked(active, i)) return;
     const BLev<D, T>& L = lv[i];
     const int t = (blockIdx.x - pre[i]) * kBT + threadIdx.x;
     pdl_enter();
@@ -125,7 +125,7 @@ template <int D, typename T>
 __global__ void __launch_bounds__(kBT) kb_extend(const BLev<D, T>* __restrict__ lv, const int* __restrict__ pre,
                                                   int K, const int* __restrict__ active) {
     const int i = find_instance(pre, K, blockIdx.x);
-    if (!active[i]) return;
+    if (masked(active, i)) return;
     const BLev<D, T>& L = lv[i];
     const int b = (blockIdx.x - pre[i]) * kBT + threadIdx.x;
     pdl_enter();
@@ -139,7 +139,7 @@ __global__ void __launch_bounds__(kBT) kb_restrict(const BLev<D, T>* __restrict_
                                                     const int* __restrict__ pre, int K,
                                                     const int* __restrict__ active) {
     const int i = find_instance(pre, K, blockIdx.x);
-    if (!active[i]) return;
+    if (masked(active, i)) return;
     const BLev<D, T>& F = fl[i];
     const BLev<D, T>& C = cl[i];
     const int t = (blockIdx.x - pre[i]) * kBT + threadIdx.x;
@@ -154,7 +154,7 @@ __global__ void __launch_bounds__(kBT) kb_prolong(const BLev<D, T>* __restrict__
                                                    const int* __restrict__ pre, int K,
                                                    const int* __restrict__ active) {
     const int i = find_instance(pre, K, blockIdx.x);
-    if (!active[i]) return;
+    if (masked(active, i)) return;
     const BLev<D, T>& F = fl[i];
     const BLev<D, T>& C = cl[i];
     const int t = (blockIdx.x - pre[i]) * kBT + threadIdx.x;
@@ -168,7 +168,7 @@ template <int D, typename T>
 __global__ void __launch_bounds__(kBT) kb_coarsest(const BLev<D, T>* __restrict__ lv, const int* __restrict__ pre,
                                                     int K, const int* __restrict__ active) {
     const int i = find_instance(pre, K, blockIdx.x);
-    if (!active[i]) return;
+    if (masked(active, i)) return;
     const BLev<D, T>& L = lv[i];
     extern __shared__ __align__(16) unsigned char kb_smem[];
     T* b = reinterpret_cast<T*>(kb_smem);
@@ -197,7 +197,7 @@ template <int D>
 __global__ void __launch_bounds__(kBT) kb_zero32(const BLev<D, float>* __restrict__ l32, const int* __restrict__ pre,
                                                   int K, const int* __restrict__ active) {
     const int i = find_instance(pre, K, blockIdx.x);
-    if (!active[i]) return;
+    if (masked(active, i)) return;
     const BLev<D, float>& U = l32[i];
     const int t = (blockIdx.x - pre[i]) * kBT + threadIdx.x;
     pdl_enter();
@@ -211,7 +211,7 @@ __global__ void __launch_bounds__(kBT) kb_accumulate(const BLev<D, double>* __re
                                                       const int* __restrict__ pre, int K,
                                                       const int* __restrict__ active) {
     const int i = find_instance(pre, K, blockIdx.x);
-    if (!active[i]) return;
+    if (masked(active, i)) return;
     const BLev<D, double>& V = l64[i];
     const BLev<D, float>& U = l32[i];
     const int t = (blockIdx.x - pre[i]) * kBT + threadIdx.x;
@@ -235,7 +235,7 @@ __global__ void __launch_bounds__(kBT) kb_residual_to32(const BLev<D, double>* _
                                                          const int* __restrict__ pre, int K,
                                                          const int* __restrict__ active, unsigned long long* norms) {
     const int i = find_instance(pre, K, blockIdx.x);
-    if (!active[i]) return;
+    if (masked(active, i)) return;
     const BLev<D, double>& V = l64[i];
     const int t = (blockIdx.x - pre[i]) * kBT + threadIdx.x;
     pdl_enter();
@@ -252,7 +252,7 @@ __global__ void __launch_bounds__(kBT) kb_to_float(const BLev<D, double>* __rest
                                                     const int* __restrict__ pre, int K,
                                                     const int* __restrict__ active) {
     const int i = find_instance(pre, K, blockIdx.x);
-    if (!active[i]) return;
+    if (masked(active, i)) return;
     const BLev<D, double>& V = l64[i];
     const BLev<D, float>& U = l32[i];
     const int t = (blockIdx.x - pre[i]) * kBT + threadIdx.x;

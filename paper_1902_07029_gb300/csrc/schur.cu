@@ -1025,7 +1025,7 @@ __global__ void __launch_bounds__(kT) kb_s_phase(const SLev<D, T>* __restrict__ 
                                                   const int* __restrict__ pre, int K, const int* __restrict__ active,
                                                   int flags, unsigned long long* norms) {
     const int i = find_instance(pre, K, blockIdx.x);
-    if (!active[i]) return;
+    if (masked(active, i)) return;
     s_phase<D, T, PH>(lv[i], lc[i], (blockIdx.x - pre[i]) * kT + threadIdx.x, flags, norms + i);
 }
 
@@ -1034,7 +1034,7 @@ __global__ void __launch_bounds__(kT) kb_s_outer(const SLev<D, double>* __restri
                                                   const SLev<D, float>* __restrict__ l32, const int* __restrict__ pre,
                                                   int K, const int* __restrict__ active, unsigned long long* norms) {
     const int i = find_instance(pre, K, blockIdx.x);
-    if (!active[i]) return;
+    if (masked(active, i)) return;
     s_outer<D>(l64[i], l32[i], (blockIdx.x - pre[i]) * kT + threadIdx.x, norms + i);
 }
 

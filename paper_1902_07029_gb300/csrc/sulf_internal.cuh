@@ -330,6 +330,16 @@ __device__ __forceinline__ void pdl_enter() {
     asm volatile("griddepcontrol.wait;" ::: "memory");
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 }
+// whether a CTA's instance of a lock-step launch is masked (active is written
+// between launches only).  A masked CTA passes the wait as well: a grid whose
+// CTAs had all left without it (the running instances have no node of this
+// phase) would complete before its predecessor, and the next grid, which waits
+// for this one, would run beside that predecessor.
+__device__ __forceinline__ bool masked(const int* __restrict__ active, int i) {
+    if (active[i]) return false;
+    pdl_enter();
+    return true;
+}
 
 // launch shape of a one-thread-per-node kernel (kernels.cu)
 constexpr int kNodeThreads = 256;

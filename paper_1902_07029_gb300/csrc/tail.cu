@@ -283,7 +283,7 @@ __global__ void __launch_bounds__(kTailThreads, 1) k_tail(const TailLevel<T>* __
 template <int D, typename T>
 __global__ void __launch_bounds__(kTailThreads, 1)
     k_tail_batched(const TailLevel<T>* const* __restrict__ lvs, const int* __restrict__ active, TailParams pr) {
-    if (!active[blockIdx.x]) return;
+    if (masked(active, blockIdx.x)) return;
     pdl_enter();
     tail_cycle<D, T>(lvs[blockIdx.x], pr);
 }

@@ -54,3 +54,32 @@ def test_cluster_meets_before_remote_shared_memory(name):
     first = body.index("map_shared_rank(")
     assert 0 <= body.find("cl.sync()") < first
     assert body.rindex("cl.sync()") > body.rindex("map_shared_rank(")
+
+
+def _functions():
+    """(file, name, body) of the kernels and of the device functions that pass
+    the dependent-launch wait themselves"""
+    out = [k for k in KERNELS if any(w in k[2] for w in ("pdl_enter(", "masked(", "s_phase<", "s_outer<"))]
+    for f in ("schur.cu",):
+        src = _code(f)
+        for m in re.finditer(r"__device__\s+__forceinline__\s+void\s+(s_\w+)\s*\(", src):
+            body = _block(src, m.end())
+            if "pdl_enter(" in body:
+                out.append((f, m.group(1), body))
+    return out
+
+
+@pytest.mark.parametrize("f,name,body", _functions(), ids=[n for _, n, _ in _functions()])
+def test_no_thread_leaves_before_the_dependent_launch_wait(f, name, body):
+    """a grid completes when its CTAs have left; if they can leave without the
+    wait it may complete before the grid it depends on, and the grid after it
+    then runs beside that one"""
+    waits = [body.index(w) for w in ("pdl_enter(", "masked(", "s_phase<", "s_outer<") if w in body]
+    head = re.sub(r"if \([^;]*masked\(active, [\w.]+\)\) return;", "", body[:body.find(";", min(waits)) + 1])
+    tail = body[len(body[:body.find(";", min(waits)) + 1]):]
+    assert "return" not in head
+    # a masked instance's CTAs leave in masked(); the others go on to a wait
+    if "masked(" in body:
+        assert any(w in tail for w in ("pdl_enter(", "s_phase<", "s_outer<"))
+        if "pdl_enter(" in tail:
+            assert "return" not in tail[:tail.index("pdl_enter(")]
