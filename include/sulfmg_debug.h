@@ -73,6 +73,11 @@ int sulf_dbg_coarsest_solve(sulf_handle h, double dt, const double* Wc0, const d
 int sulf_dbg_cycles(sulf_handle h, double dt, const double* Wc0, const double* rhs, double* x, int ncycles,
                     double* rnorms);
 
+/* The device allocation after the handle's next `after` ones is refused once, as
+   if the device were out of memory (after < 0: none).  pending (may be NULL)
+   receives whether an earlier request has not been reached yet. */
+int sulf_dbg_fail_alloc(sulf_handle h, long long after, int* pending);
+
 #ifdef __cplusplus
 }
 #endif

@@ -120,6 +120,7 @@ _SIGS = {
     "sulf_dbg_prolong": (ctypes.c_int, [P, ctypes.c_int, _dp, _dp]),
     "sulf_dbg_inject": (ctypes.c_int, [P, _dp, ctypes.c_int, _dp]),
     "sulf_dbg_cycles": (ctypes.c_int, [P, ctypes.c_double, _dp, _dp, _dp, ctypes.c_int, _dp]),
+    "sulf_dbg_fail_alloc": (ctypes.c_int, [P, ctypes.c_longlong, ctypes.POINTER(ctypes.c_int)]),
     "sulf_dbg_coarsest_solve": (ctypes.c_int, [P, ctypes.c_double, _dp, _dp, _dp]),
 }
 
@@ -386,6 +387,13 @@ class Domain:
         out = np.zeros(2 * self.level_info(l)["n"] ** self.dim)
         _chk(self.lib, self.lib.sulf_dbg_inject(self.h, _d(Wc0), l, _d(out)))
         return out
+
+    def fail_alloc(self, after):
+        """refuse the device allocation after the next `after` ones (None: none);
+        returns whether an earlier request is still pending"""
+        p = ctypes.c_int(0)
+        _chk(self.lib, self.lib.sulf_dbg_fail_alloc(self.h, -1 if after is None else int(after), ctypes.byref(p)))
+        return bool(p.value)
 
     def coarsest_solve(self, dt, Wc0, rhs_c):
         Wc0 = np.ascontiguousarray(Wc0, dtype=np.float64)

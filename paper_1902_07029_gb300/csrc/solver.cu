@@ -58,6 +58,7 @@ void retain_pool_memory() {
 constexpr size_t kChunkBytes = 2 << 20;
 
 void* DevMem::get(size_t n) {
+    if (fail_in && *fail_in >= 0 && (*fail_in)-- == 0) return nullptr;
     size_t sz = (n + 255) & ~size_t(255);
     if (sz == 0) sz = 256;
     const bool shared = sz <= kChunkBytes / 2;
@@ -138,6 +139,7 @@ struct sulf_domain {
     void* noalloc_scratch = nullptr;   // device address of noalloc.cu's static scratch, looked up on
                                        // this handle's first sulf_newton_residual_noalloc call
     DevMem mem;
+    long long fail_in = -1;            // sulf_dbg_fail_alloc
     double t = 0, dt = 0;
     // statistics
     int newton_last = 0, cycles_last = 0;
@@ -978,12 +980,10 @@ bool build_loop(sulf_domain* d, int max_cycles) {
     sulf_domain::LoopGraph& g = d->loop[p];
     if (g.exec) cudaGraphExecDestroy(g.exec);
     g.exec = nullptr;
-    if (!d->dcyc) {
-        d->dcyc = (int*)d->mem.get(sizeof(int) * 4);
-        d->drn = (double*)d->mem.get(sizeof(double) * kLoopMaxCycles);
-        d->dthr = (double*)d->mem.get(sizeof(double) * 2);
-        if (!d->dcyc || !d->drn || !d->dthr) return false;
-    }
+    if (!d->dcyc) d->dcyc = (int*)d->mem.get(sizeof(int) * 4);
+    if (!d->drn) d->drn = (double*)d->mem.get(sizeof(double) * kLoopMaxCycles);
+    if (!d->dthr) d->dthr = (double*)d->mem.get(sizeof(double) * 2);
+    if (!d->dcyc || !d->drn || !d->dthr) return false;
     if (!d->hloop && cudaMallocHost(&d->hloop, sizeof(double) * (4 + kLoopMaxCycles)) != cudaSuccess) {
         d->hloop = nullptr;
         cudaGetLastError();
@@ -1457,6 +1457,7 @@ int sulf_create_domain(const double* levelset, int dim, const double* box, int N
     }
     d->stream = d->own_stream;
     d->mem.stream = d->own_stream;
+    d->mem.fail_in = &d->fail_in;
     std::string err;
     int rc = SULF_OK;
     for (int l = 0; l < nl && rc == SULF_OK; l++) {
@@ -1730,6 +1731,13 @@ int sulf_kernel_time(sulf_handle h, double* ms, long long* launches) {
 
 // ---------------------------------------------------------------------------
 // stage-level entry points (sulfmg_debug.h)
+
+int sulf_dbg_fail_alloc(sulf_handle h, long long after, int* pending) {
+    if (!valid(h)) return sulf_fail(SULF_EINVAL, "invalid handle");
+    if (pending) *pending = h->fail_in >= 0;
+    h->fail_in = after < 0 ? -1 : after;
+    return SULF_OK;
+}
 
 static int dbg_level_ok(sulf_handle h, int l) { return valid(h) && l >= 0 && l < h->L; }
 

@@ -178,6 +178,7 @@ struct DevMem {
     char* chunk = nullptr;  // free part of the current chunk of small blocks
     size_t left = 0;
     cudaStream_t stream = nullptr;
+    long long* fail_in = nullptr;  // tests: >= 0, the requests until one is refused (once)
     void* get(size_t n);
     void release();
 };

@@ -1,0 +1,73 @@
+"""A step that finds no device memory fails with ENOMEM and leaves the handle
+usable: the next step gives, bit for bit, what it gives on a handle that never
+failed, by the same number of kernel launches.  Each allocation of a first step
+is refused in turn (on the host: the request is answered as if the device were
+full)."""
+import numpy as np
+import pytest
+
+import workloads
+
+pytestmark = pytest.mark.gpu
+
+GEOMS = {
+    "disk64": lambda: (workloads.disk(64), 2, 64, 8),
+    "rbox32": lambda: (workloads.rounded_box(32), 3, 32, 8),
+}
+
+
+def _domain(sulfmg, name, **solver):
+    phi, dim, N, cN = GEOMS[name]()
+    d = sulfmg.Domain(phi, dim, (-1.0, 1.0), N, cN)
+    d.set_model(workloads.PAPER_MODEL)
+    d.set_solver(**solver)
+    return d, 0.25 * 2.0 / N
+
+
+def _two_steps(d, dt):
+    """the state after two steps and the second one's launches (the first one's
+    include set-up)"""
+    d.step(dt, 1)
+    n = d.stats()["kernel_launches"]
+    d.step(dt, 1)
+    return d.get_state()[:2], d.stats()["kernel_launches"] - n, d.stats()["loop_graph"]
+
+
+def _sweep(sulfmg, name, **solver):
+    d, dt = _domain(sulfmg, name, **solver)
+    (s0, c0), launches, loop = _two_steps(d, dt)
+    d.close()
+    failed = 0
+    for k in range(2000):
+        d, dt = _domain(sulfmg, name, **solver)
+        d.fail_alloc(k)
+        init = d.get_state()[:2]
+        try:
+            d.step(dt, 1)
+        except sulfmg.SulfError as e:
+            assert e.code == sulfmg.ENOMEM
+            failed += 1
+            for a, b in zip(init, d.get_state()[:2]):
+                np.testing.assert_array_equal(a, b)
+            assert not d.fail_alloc(None)
+        else:
+            if d.fail_alloc(None):  # never reached: every allocation has been refused once
+                d.close()
+                return failed, k
+            # (a refused buffer of the device-side cycle loop only: this step ran without it)
+            d.set_model(workloads.PAPER_MODEL)
+        (s, c), n, lp = _two_steps(d, dt)
+        np.testing.assert_array_equal(s, s0)
+        np.testing.assert_array_equal(c, c0)
+        assert (n, lp) == (launches, loop), f"allocation {k}"
+        d.close()
+    raise AssertionError("a first step of 2000 allocations")
+
+
+@pytest.mark.parametrize("precision", [0, 1], ids=["fp64", "mixed"])
+@pytest.mark.parametrize("name", list(GEOMS))
+def test_two_unknown_path(sulfmg, name, precision):
+    """the vectors of the two-unknown kernels, the fused levels' descriptors and
+    the buffers of the device-side cycle loop"""
+    failed, total = _sweep(sulfmg, name, precision=precision, ghost_compose=0)
+    assert 0 < failed < total
