@@ -1447,10 +1447,15 @@ int build_sgeo_rows(SGeo& S, const LevelGeo& L, DevMem& mem, cudaStream_t s, std
         err = "out of device memory";
         return SULF_ENOMEM;
     };
-    S.bc = L.gop_bc;
-    S.passes = L.gop_passes;
-    S.tau = L.gop_tau;
-    if (L.ng == 0) return SULF_OK;
+    // what the rows are built for: known once they are there
+    S.bc = -1;
+    auto built = [&] {
+        S.bc = L.gop_bc;
+        S.passes = L.gop_passes;
+        S.tau = L.gop_tau;
+        return SULF_OK;
+    };
+    if (L.ng == 0) return built();
     if (L.gop_nnz > S.gcap) {
         S.gcode = (int*)mem.get(sizeof(int) * (L.gop_nnz + 1));
         if (!S.gcode) return oom();
@@ -1506,7 +1511,7 @@ int build_sgeo_rows(SGeo& S, const LevelGeo& L, DevMem& mem, cudaStream_t s, std
         err = "ghost rows failed";
         return SULF_EDEVICE;
     }
-    return SULF_OK;
+    return built();
 }
 
 // ---------------------------------------------------------------------------

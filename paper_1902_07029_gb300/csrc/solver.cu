@@ -139,6 +139,7 @@ struct sulf_domain {
     void* noalloc_scratch = nullptr;   // device address of noalloc.cu's static scratch, looked up on
                                        // this handle's first sulf_newton_residual_noalloc call
     DevMem mem;
+    DevMem mem_s;                      // what the cycle on the equation for s holds
     long long fail_in = -1;            // sulf_dbg_fail_alloc
     double t = 0, dt = 0;
     // statistics
@@ -419,7 +420,7 @@ int alloc_schur(sulf_domain* d, SVec<T>* V, int nl, bool outer) {
     auto get = [&](auto*& p, size_t n, bool zero) {
         if (p || !ok) return;
         const size_t nb = sizeof(*p) * (n + 1);
-        p = (std::remove_reference_t<decltype(p)>)d->mem.get(nb);
+        p = (std::remove_reference_t<decltype(p)>)d->mem_s.get(nb);
         ok = p && (!zero || cudaMemsetAsync(p, 0, nb, d->stream) == cudaSuccess);
     };
     for (int l = 0; l < nl; l++) {
@@ -472,9 +473,9 @@ int ensure_coarse(sulf_domain* d, CoarseSet<T>& S, const SVec<T>* V, int at_leas
     drop_graphs(d);
     std::string err;
     int rc = d->dim == 2 ? build_coarse<2, T>(S, d->geo, d->sgeo, V, d->L, want, nu1, nu2, max_cta, acc, d->dskip,
-                                              d->mem, d->stream, err)
+                                              d->mem_s, d->stream, err)
                          : build_coarse<3, T>(S, d->geo, d->sgeo, V, d->L, want, nu1, nu2, max_cta, acc, d->dskip,
-                                              d->mem, d->stream, err);
+                                              d->mem_s, d->stream, err);
     return rc ? sulf_fail(rc, err) : SULF_OK;
 }
 
@@ -488,7 +489,24 @@ int ensure_path(sulf_domain* d) {
     return d->solver.precision == 1 ? ensure32(d) : SULF_OK;
 }
 
-int ensure_schur(sulf_domain* d, bool coarse) {
+// gives back what that cycle holds; its next use builds it anew
+void release_schur(sulf_domain* d) {
+    drop_graphs(d);
+    cudaStreamSynchronize(d->stream);
+    d->mem_s.release();
+    for (int l = 0; l < d->L; l++) {
+        d->sgeo[l] = SGeo();
+        d->s64[l] = SVec<double>();
+        d->s32[l] = SVec<float>();
+    }
+    d->cs64 = CoarseSet<double>();
+    d->cs32 = CoarseSet<float>();
+    d->dskip = nullptr;
+    d->s_geo = 0;
+    d->s_on = false;
+}
+
+int build_schur(sulf_domain* d, bool coarse) {
     d->s_on = false;
     if (!schur_wanted(d) || d->s_geo < 0) return SULF_OK;
     for (int l = 0; l < d->L; l++) {
@@ -502,14 +520,14 @@ int ensure_schur(sulf_domain* d, bool coarse) {
         for (int l = 0; l < d->L; l++) {
             bool ok = false;
             int rc = build_sgeo(d->sgeo[l], d->geo[l], l ? &d->geo[l - 1] : nullptr, l ? &d->sgeo[l - 1] : nullptr,
-                                l + 1 < d->L ? &d->geo[l + 1] : nullptr, d->mem, d->stream, err, d->launches, ok);
+                                l + 1 < d->L ? &d->geo[l + 1] : nullptr, d->mem_s, d->stream, err, d->launches, ok);
             if (rc) return sulf_fail(rc, err);
             if (!ok) {
                 d->s_geo = -1;
                 return SULF_OK;
             }
         }
-        d->dskip = (int*)d->mem.get(sizeof(int));
+        d->dskip = (int*)d->mem_s.get(sizeof(int));
         if (!d->dskip) return sulf_fail(SULF_ENOMEM, "out of device memory");
         d->s_geo = 1;
     }
@@ -518,7 +536,7 @@ int ensure_schur(sulf_domain* d, bool coarse) {
         SGeo& S = d->sgeo[l];
         const LevelGeo& G = d->geo[l];
         if (S.bc == G.gop_bc && S.passes == G.gop_passes && S.tau == G.gop_tau) continue;
-        int rc = build_sgeo_rows(S, G, d->mem, d->stream, err, d->launches);
+        int rc = build_sgeo_rows(S, G, d->mem_s, d->stream, err, d->launches);
         if (rc) return sulf_fail(rc, err);
         changed = true;
     }
@@ -538,6 +556,14 @@ int ensure_schur(sulf_domain* d, bool coarse) {
     }
     d->s_on = true;
     return SULF_OK;
+}
+
+// (a set-up that failed half-way leaves nothing: neither lists that a later
+// call would take for complete nor memory that it would ask for again)
+int ensure_schur(sulf_domain* d, bool coarse) {
+    const int rc = build_schur(d, coarse);
+    if (rc) release_schur(d);
+    return rc;
 }
 
 // ---- profiling events around the finest-level inside relaxation ----
@@ -1418,6 +1444,7 @@ void sulf_destroy(sulf_handle h) {
     if (h->ev_join) cudaEventDestroy(h->ev_join);
     for (cudaEvent_t e : h->evpool) cudaEventDestroy(e);
     h->mem.release();
+    h->mem_s.release();
     if (h->hnorm) cudaFreeHost(h->hnorm);
     if (h->hloop) cudaFreeHost(h->hloop);
     for (auto& g : h->loop)
@@ -1457,7 +1484,8 @@ int sulf_create_domain(const double* levelset, int dim, const double* box, int N
     }
     d->stream = d->own_stream;
     d->mem.stream = d->own_stream;
-    d->mem.fail_in = &d->fail_in;
+    d->mem_s.stream = d->own_stream;
+    d->mem.fail_in = d->mem_s.fail_in = &d->fail_in;
     std::string err;
     int rc = SULF_OK;
     for (int l = 0; l < nl && rc == SULF_OK; l++) {
@@ -1704,7 +1732,7 @@ int sulf_get_stats(sulf_handle h, sulf_stats* o) {
     o->n_inside = h->geo[0].nin[0] + (long long)h->geo[0].nin[1];
     o->n_ghost = h->geo[0].ng;
     for (int k = 0; k < 3; k++) o->ghost_rows[k] = h->geo[0].kinds[k];
-    o->device_bytes = h->mem.bytes;
+    o->device_bytes = h->mem.bytes + h->mem_s.bytes;
     o->loop_graph = h->loop_used ? 1 : 0;
     return SULF_OK;
 }

@@ -71,3 +71,47 @@ def test_two_unknown_path(sulfmg, name, precision):
     the buffers of the device-side cycle loop"""
     failed, total = _sweep(sulfmg, name, precision=precision, ghost_compose=0)
     assert 0 < failed < total
+
+
+@pytest.mark.parametrize("precision", [0, 1], ids=["fp64", "mixed"])
+@pytest.mark.parametrize("name", list(GEOMS))
+def test_cycle_on_the_equation_for_s(sulfmg, name, precision):
+    """its lists, rows, vectors and cluster tables: a level whose rows were not
+    built is not taken for built by the next step"""
+    failed, total = _sweep(sulfmg, name, precision=precision)
+    assert 0 < failed < total
+
+
+@pytest.mark.parametrize("precision", [0, 1], ids=["fp64", "mixed"])
+def test_rebuild_for_another_boundary_condition(sulfmg, precision):
+    """the rows of a handle that has stepped, rebuilt for the Neumann condition:
+    a refused allocation leaves none of the Dirichlet rows in use"""
+
+    def start():
+        d, dt = _domain(sulfmg, "disk64", precision=precision)
+        d.step(dt, 1)
+        d.set_bc(1)
+        d.set_model(workloads.PAPER_MODEL)
+        return d, dt
+
+    d, dt = start()
+    (s0, c0), launches, _ = _two_steps(d, dt)
+    d.close()
+    for k in range(100):
+        d, dt = start()
+        d.fail_alloc(k)
+        try:
+            d.step(dt, 1)
+            done = d.fail_alloc(None)
+            d.set_model(workloads.PAPER_MODEL)
+        except sulfmg.SulfError as e:
+            assert e.code == sulfmg.ENOMEM
+            done = False
+        (s, c), n, _ = _two_steps(d, dt)
+        np.testing.assert_array_equal(s, s0)
+        np.testing.assert_array_equal(c, c0)
+        assert n == launches
+        d.close()
+        if done:
+            return
+    raise AssertionError("a rebuild of 100 allocations")
