@@ -731,7 +731,7 @@ int build_coarse(CoarseSet<T>& S, const LevelGeo* G, const SGeo* SG, const SVec<
     S.nu1 = nu1;
     S.nu2 = nu2;
     S.max_cta = max_cta;
-    S.rows = true;
+    S.rows = false;  // (the caller's note of success)
     if (want < 0 || want > L - 1) return SULF_OK;
     const bool f32 = std::is_same<T, float>::value;
     // Levels of up to this many nodes run on CTA 0, whose phases are short: 120

@@ -72,7 +72,7 @@ template <typename T>
 struct CoarseSet {
     int l0 = -1;
     int want = -2, nu1 = 0, nu2 = 0, max_cta = 0;  // what it was built for
-    bool rows = false;      // built for the current boundary rows
+    bool rows = false;      // built, and for the current boundary rows
     size_t smem = 0;
     int ncta = 0;
     CDesc<T>* dev = nullptr;

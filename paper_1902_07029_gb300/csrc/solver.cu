@@ -476,7 +476,9 @@ int ensure_coarse(sulf_domain* d, CoarseSet<T>& S, const SVec<T>* V, int at_leas
                                               d->mem_s, d->stream, err)
                          : build_coarse<3, T>(S, d->geo, d->sgeo, V, d->L, want, nu1, nu2, max_cta, acc, d->dskip,
                                               d->mem_s, d->stream, err);
-    return rc ? sulf_fail(rc, err) : SULF_OK;
+    if (rc) return sulf_fail(rc, err);
+    S.rows = true;
+    return SULF_OK;
 }
 
 // decides d->s_on for the next linear solve and builds what it needs (coarse:

@@ -115,3 +115,48 @@ def test_rebuild_for_another_boundary_condition(sulfmg, precision):
         if done:
             return
     raise AssertionError("a rebuild of 100 allocations")
+
+
+@pytest.mark.parametrize("precision", [0, 1], ids=["fp64", "mixed"])
+def test_lock_step_set_up(sulfmg, precision):
+    """the same for a lock-step class: the cluster tables of the instance that
+    found no memory are built by the next call"""
+
+    def start():
+        doms = [_domain(sulfmg, "disk64", precision=precision)[0] for _ in range(2)]
+        return doms, sulfmg.Batch(doms, nstreams=1, lockstep=True), 0.25 * 2.0 / 64
+
+    def run(doms, batch, dt):
+        batch.step(dt, 1)
+        n = [d.stats()["kernel_launches"] for d in doms]
+        batch.step(dt, 1)
+        return [d.get_state()[:2] for d in doms], [d.stats()["kernel_launches"] - m for d, m in zip(doms, n)]
+
+    def close(doms, batch):
+        batch.close()
+        for d in doms:
+            d.close()
+
+    doms, batch, dt = start()
+    ref, launches = run(doms, batch, dt)
+    close(doms, batch)
+    for k in range(500):
+        doms, batch, dt = start()
+        doms[1].fail_alloc(k)
+        try:
+            batch.step(dt, 1)
+            done = doms[1].fail_alloc(None)
+            for d in doms:
+                d.set_model(workloads.PAPER_MODEL)
+        except sulfmg.SulfError as e:
+            assert e.code == sulfmg.ENOMEM
+            done = False
+        out, n = run(doms, batch, dt)
+        close(doms, batch)
+        for (s, c), (s0, c0) in zip(out, ref):
+            np.testing.assert_array_equal(s, s0)
+            np.testing.assert_array_equal(c, c0)
+        assert n == launches, f"allocation {k}"
+        if done:
+            return
+    raise AssertionError("a lock-step set-up of 500 allocations")
