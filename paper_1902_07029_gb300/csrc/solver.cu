@@ -2506,9 +2506,11 @@ struct LockGraphs {
 };
 
 // The per-instance phases run for every instance of the class, whatever its
-// state: an instance that left its Newton loop (converged, or failed) gets a
-// zero update (its x is zeroed by the set-up and its cycles are masked), so
-// its state does not change, and its norms are not read.
+// state: an instance that left its Newton loop (converged, or failed) gets no
+// update (two unknowns: a zero one, its x is zeroed by the set-up and its cycles
+// are masked; the equation for s, whose set-up leaves the first sweep in x: none,
+// by its flag in dnewton), so its state does not change, and its norms are not
+// read.
 template <int D>
 int lockstep_step(LockClass<D>& C, LockGraphs<D>& P, int* status, std::vector<std::string>& err) {
     const int K = C.K;
@@ -2550,11 +2552,6 @@ int lockstep_step(LockClass<D>& C, LockGraphs<D>& P, int* status, std::vector<st
         bool any = false;
         for (int i = 0; i < K; i++) any = any || inewton[i];
         if (!any) break;
-        if (C.schur) {
-            // (an instance out of its loop keeps its state: no update)
-            SULF_CUDA_TRY(cudaMemcpyAsync(C.dnewton, inewton.data(), sizeof(int) * K, cudaMemcpyHostToDevice, C.s));
-            SULF_CUDA_TRY(cudaStreamSynchronize(C.s));
-        }
         // per instance: the Jacobian of this Newton iteration on every level
         rc = C.run_phase(P.prepare, [&] {
             return C.per_instance([&](int i, cudaStream_t b) {
@@ -2592,6 +2589,10 @@ int lockstep_step(LockClass<D>& C, LockGraphs<D>& P, int* status, std::vector<st
         // the cycles of the linear solves, in lock step
         std::vector<double> rprev(fn);
         std::vector<int> cyc(K, 0);
+        // whose update is made: not that of an instance out of its loop, nor of
+        // one that the set-up has just found singular
+        if (C.schur)
+            SULF_CUDA_TRY(cudaMemcpyAsync(C.dnewton, inewton.data(), sizeof(int) * K, cudaMemcpyHostToDevice, C.s));
         if (int rc = C.set_active()) return rc;
         for (int c = 1; c <= sv.max_cycles; c++) {
             bool on = false;
