@@ -11,8 +11,8 @@ import workloads
 pytestmark = pytest.mark.gpu
 
 GEOMS = {
-    "disk64": lambda: (workloads.disk(64), 2, 64, 8),
-    "rbox32": lambda: (workloads.rounded_box(32), 3, 32, 8),
+    "disk32": lambda: (workloads.disk(32), 2, 32, 8),
+    "rbox16": lambda: (workloads.rounded_box(16), 3, 16, 4),
 }
 
 
@@ -21,7 +21,7 @@ def _domain(sulfmg, name, **solver):
     d = sulfmg.Domain(phi, dim, (-1.0, 1.0), N, cN)
     d.set_model(workloads.PAPER_MODEL)
     d.set_solver(**solver)
-    return d, 0.25 * 2.0 / N
+    return d, 0.05 * 2.0 / N
 
 
 def _two_steps(d, dt):
@@ -88,7 +88,7 @@ def test_rebuild_for_another_boundary_condition(sulfmg, precision):
     a refused allocation leaves none of the Dirichlet rows in use"""
 
     def start():
-        d, dt = _domain(sulfmg, "disk64", precision=precision)
+        d, dt = _domain(sulfmg, "disk32", precision=precision)
         d.step(dt, 1)
         d.set_bc(1)
         d.set_model(workloads.PAPER_MODEL)
@@ -123,8 +123,8 @@ def test_lock_step_set_up(sulfmg, precision):
     found no memory are built by the next call"""
 
     def start():
-        doms = [_domain(sulfmg, "disk64", precision=precision)[0] for _ in range(2)]
-        return doms, sulfmg.Batch(doms, nstreams=1, lockstep=True), 0.25 * 2.0 / 64
+        doms = [_domain(sulfmg, "disk32", precision=precision)[0] for _ in range(2)]
+        return doms, sulfmg.Batch(doms, nstreams=1, lockstep=True), 0.05 * 2.0 / 32
 
     def run(doms, batch, dt):
         batch.step(dt, 1)
