@@ -291,8 +291,8 @@ int sulf_newton_residual_noalloc(sulf_handle h, double dt, const double* W_dev, 
    for V-cycles with red-black sweeps), ghost_compose, pdl,
    relax_occupancy and relax_matrix_free.  Each candidate
    is timed on this handle's own problem -- the Newton system of a CN step of
-   size dt from the current state -- as a linear solve of 6 cycles (built
-   once, then timed); the fused-level thresholds {0, 60, 150, 400, 1000, 3000,
+   size dt from the current state -- as a linear solve of 6 cycles (run until
+   its graphs exist, then timed); the fused-level thresholds {0, 60, 150, 400, 1000, 3000,
    10000} are tried first, then ghost_compose and pdl at the best one, then
    relax_occupancy (FP64) or relax_matrix_free (mixed precision).  The
    fastest candidate is written into the handle's solver controls (the state

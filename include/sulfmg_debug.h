@@ -78,6 +78,10 @@ int sulf_dbg_cycles(sulf_handle h, double dt, const double* Wc0, const double* r
    receives whether an earlier request has not been reached yet. */
 int sulf_dbg_fail_alloc(sulf_handle h, long long after, int* pending);
 
+/* what the handle has built and runs (2 entries): graphs captured so far, and
+   those of them captured inside a solve that sulf_autotune timed */
+int sulf_dbg_route(sulf_handle h, int64_t* route);
+
 #ifdef __cplusplus
 }
 #endif

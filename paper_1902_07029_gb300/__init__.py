@@ -121,6 +121,7 @@ _SIGS = {
     "sulf_dbg_inject": (ctypes.c_int, [P, _dp, ctypes.c_int, _dp]),
     "sulf_dbg_cycles": (ctypes.c_int, [P, ctypes.c_double, _dp, _dp, _dp, ctypes.c_int, _dp]),
     "sulf_dbg_fail_alloc": (ctypes.c_int, [P, ctypes.c_longlong, ctypes.POINTER(ctypes.c_int)]),
+    "sulf_dbg_route": (ctypes.c_int, [P, _i64p]),
     "sulf_dbg_coarsest_solve": (ctypes.c_int, [P, ctypes.c_double, _dp, _dp, _dp]),
 }
 
@@ -394,6 +395,13 @@ class Domain:
         p = ctypes.c_int(0)
         _chk(self.lib, self.lib.sulf_dbg_fail_alloc(self.h, -1 if after is None else int(after), ctypes.byref(p)))
         return bool(p.value)
+
+    def route(self):
+        """what the handle has built and runs (sulf_dbg_route)"""
+        names = ("captures", "captures_timed")
+        r = np.zeros(len(names), dtype=np.int64)
+        _chk(self.lib, self.lib.sulf_dbg_route(self.h, r.ctypes.data_as(_i64p)))
+        return {n: int(v) for n, v in zip(names, r)}
 
     def coarsest_solve(self, dt, Wc0, rhs_c):
         Wc0 = np.ascontiguousarray(Wc0, dtype=np.float64)

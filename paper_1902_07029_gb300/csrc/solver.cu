@@ -141,6 +141,9 @@ struct sulf_domain {
     DevMem mem;
     DevMem mem_s;                      // what the cycle on the equation for s holds
     long long fail_in = -1;            // sulf_dbg_fail_alloc
+    // graphs captured, and those of them inside a solve that the tuner timed
+    // (sulf_dbg_route)
+    long long captures = 0, captures_timed = 0;
     double t = 0, dt = 0;
     // statistics
     int newton_last = 0, cycles_last = 0;
@@ -1069,6 +1072,7 @@ bool build_loop(sulf_domain* d, int max_cycles) {
     g.sv = d->solver;
     g.s_on = d->s_on;
     g.max_cycles = max_cycles;
+    d->captures++;
     return true;
 }
 
@@ -1166,6 +1170,7 @@ int run_captured(sulf_domain* d, sulf_domain::StepGraph& g, F&& fn) {
             g.exec = nullptr;
             return sulf_fail_cuda(ei, "cudaGraphInstantiate");
         }
+        d->captures++;
     }
     SULF_CUDA_TRY(cudaGraphLaunch(g.exec, d->stream));
     d->launches += g.kernels;
@@ -1209,6 +1214,7 @@ int run_cycle(sulf_domain* d) {
         e = cudaGraphInstantiate(&g.exec, graph, 0);
         cudaGraphDestroy(graph);
         if (e != cudaSuccess) return sulf_fail_cuda(e, "cudaGraphInstantiate");
+        d->captures++;
         g.kernels = d->launches - l0;
         d->launches = l0;
         g.ev1 = d->evused;
@@ -1766,6 +1772,13 @@ int sulf_dbg_fail_alloc(sulf_handle h, long long after, int* pending) {
     if (!valid(h)) return sulf_fail(SULF_EINVAL, "invalid handle");
     if (pending) *pending = h->fail_in >= 0;
     h->fail_in = after < 0 ? -1 : after;
+    return SULF_OK;
+}
+
+int sulf_dbg_route(sulf_handle h, int64_t* r) {
+    if (!valid(h) || !r) return sulf_fail(SULF_EINVAL, "invalid arguments");
+    r[0] = h->captures;
+    r[1] = h->captures_timed;
     return SULF_OK;
 }
 
@@ -2751,7 +2764,7 @@ int lockstep_advance(const sulf_handle* hs, int K, double dt, int nsteps, int* s
 // threshold, the composed ghost relaxation and dependent launch.  A candidate
 // is timed on the handle's own problem -- the Newton system of a CN step of
 // size dt from the current state -- as a linear solve of a fixed number of
-// cycles (the defect test is off), once to build its graphs and once timed.
+// cycles (the defect test is off), untimed until its graphs exist, then timed.
 // The state is not changed.  Results are kept per problem class for the
 // process, so same-size instances of a batch tune once.
 namespace {
@@ -2770,14 +2783,23 @@ TuneKey tune_key(const sulf_domain* d) {
 template <int D>
 int time_solve(sulf_domain* d, double fnorm, int ncycles, double* ms) {
     PdlScope pdl(d->solver.pdl != 0, d->solver.relax_occupancy, d->solver.relax_matrix_free);
-    int c = linear_solve<D>(d, fnorm, ncycles, 0.0, nullptr);  // builds the graphs of this candidate
-    if (c < 0) return c;
+    // untimed until a solve captures nothing: the cycles' graph comes at the
+    // first one, that of the set-up at the second (run_captured)
+    long long before;
+    int c, k = 0;
+    do {
+        before = d->captures;
+        c = linear_solve<D>(d, fnorm, ncycles, 0.0, nullptr);
+        if (c < 0) return c;
+    } while (d->captures != before && ++k < 4);
     SULF_CUDA_TRY(cudaStreamSynchronize(d->stream));
+    before = d->captures;
     const double t0 = host_ms();
     c = linear_solve<D>(d, fnorm, ncycles, 0.0, nullptr);
     if (c < 0) return c;
     SULF_CUDA_TRY(cudaStreamSynchronize(d->stream));
     *ms = (host_ms() - t0) / ncycles;
+    d->captures_timed += d->captures - before;
     return SULF_OK;
 }
 
