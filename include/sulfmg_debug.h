@@ -82,6 +82,10 @@ int sulf_dbg_fail_alloc(sulf_handle h, long long after, int* pending);
    those of them captured inside a solve that sulf_autotune timed */
 int sulf_dbg_route(sulf_handle h, int64_t* route);
 
+/* r as the result that the process cache of sulf_autotune holds for the
+   handle's problem class */
+int sulf_dbg_tune_put(sulf_handle h, const sulf_tune_result* r);
+
 #ifdef __cplusplus
 }
 #endif

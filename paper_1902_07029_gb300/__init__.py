@@ -122,6 +122,7 @@ _SIGS = {
     "sulf_dbg_cycles": (ctypes.c_int, [P, ctypes.c_double, _dp, _dp, _dp, ctypes.c_int, _dp]),
     "sulf_dbg_fail_alloc": (ctypes.c_int, [P, ctypes.c_longlong, ctypes.POINTER(ctypes.c_int)]),
     "sulf_dbg_route": (ctypes.c_int, [P, _i64p]),
+    "sulf_dbg_tune_put": (ctypes.c_int, [P, ctypes.POINTER(SulfTuneResult)]),
     "sulf_dbg_coarsest_solve": (ctypes.c_int, [P, ctypes.c_double, _dp, _dp, _dp]),
 }
 
@@ -402,6 +403,11 @@ class Domain:
         r = np.zeros(len(names), dtype=np.int64)
         _chk(self.lib, self.lib.sulf_dbg_route(self.h, r.ctypes.data_as(_i64p)))
         return {n: int(v) for n, v in zip(names, r)}
+
+    def tune_put(self, **result):
+        """a result for this problem class into the process cache (sulf_dbg_tune_put)"""
+        r = SulfTuneResult(**result)
+        _chk(self.lib, self.lib.sulf_dbg_tune_put(self.h, ctypes.byref(r)))
 
     def coarsest_solve(self, dt, Wc0, rhs_c):
         Wc0 = np.ascontiguousarray(Wc0, dtype=np.float64)

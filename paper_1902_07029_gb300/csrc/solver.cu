@@ -1349,7 +1349,8 @@ bool valid(sulf_handle h) { return h != nullptr; }
 // tile lists of the temporally blocked sweep (tiles holding an inside node)
 // and the second unknown buffer, for the 3-D levels with enough inside nodes
 int ensure_tiles(sulf_domain* d) {
-    if (d->dim != 3 || !d->have32) return SULF_OK;
+    if (d->dim != 3) return SULF_OK;
+    if (int rc = ensure32(d)) return rc;
     for (int l = 0; l < d->L; l++) {
         LevelGeo& G = d->geo[l];
         if (G.tiles || (long long)G.nin[0] + G.nin[1] < kTileMinInside) continue;
@@ -1579,10 +1580,7 @@ int sulf_set_solver(sulf_handle h, const sulf_solver* s) {
     if (int rc = refresh_ghost_ops(h)) return rc;
     if (v.smoother == 2)
         if (int rc = ensure_lex(h)) return rc;
-    if (v.precision == 1 && v.relax_matrix_free == 2) {
-        if (int rc = ensure32(h)) return rc;
-        return ensure_tiles(h);
-    }
+    if (v.precision == 1 && v.relax_matrix_free == 2) return ensure_tiles(h);
     return SULF_OK;
 }
 
@@ -2932,6 +2930,13 @@ int sulf_autotune(sulf_handle h, double dt, int use_cache, sulf_tune_result* out
         g_tune_cache[key] = r;
     }
     if (out) *out = r;
+    return SULF_OK;
+}
+
+int sulf_dbg_tune_put(sulf_handle h, const sulf_tune_result* r) {
+    if (!valid(h) || !r) return sulf_fail(SULF_EINVAL, "invalid arguments");
+    std::lock_guard<std::mutex> lk(g_tune_mu);
+    g_tune_cache[tune_key(h)] = *r;
     return SULF_OK;
 }
 

@@ -1,4 +1,5 @@
 """What the autotuner measures and leaves behind."""
+import numpy as np
 import pytest
 
 import workloads
@@ -23,3 +24,29 @@ def test_no_graph_is_captured_in_a_timed_solve(sulfmg, precision):
     r = d.route()
     assert r["captures"] > 0 and r["captures_timed"] == 0
     d.close()
+
+
+def test_cached_tiled_sweep_is_used(sulfmg):
+    """a fresh domain that takes relax_matrix_free = 2 from the cache runs the
+    tiled sweep, as one that is given the control does"""
+    N, cN, dt = 72, 9, 0.1 * 2.0 / 72
+
+    def two_steps(d):
+        d.step(dt, 1)
+        n = d.stats()["kernel_launches"]
+        d.step(dt, 1)
+        return d.get_state()[:2], d.stats()["kernel_launches"] - n
+
+    a = _domain(sulfmg, 3, N, cN, precision=1, relax_matrix_free=2)
+    assert a.level_info(0)["nin"] > 100000  # tiled
+    (s0, c0), n0 = two_steps(a)
+    a.close()
+    b = _domain(sulfmg, 3, N, cN, precision=1)
+    b.tune_put(fuse_below=-1, ghost_compose=1, pdl=1, relax_matrix_free=2, candidates=1)
+    r = b.autotune(dt)
+    assert r["cached"] == 1 and r["relax_matrix_free"] == 2
+    (s, c), n = two_steps(b)
+    assert n == n0
+    np.testing.assert_array_equal(s, s0)
+    np.testing.assert_array_equal(c, c0)
+    b.close()
