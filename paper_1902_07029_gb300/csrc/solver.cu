@@ -140,6 +140,7 @@ struct sulf_domain {
                                        // this handle's first sulf_newton_residual_noalloc call
     DevMem mem;
     DevMem mem_s;                      // what the cycle on the equation for s holds
+    DevMem mem_two;                    // the two-unknown kernels' vectors
     long long fail_in = -1;            // sulf_dbg_fail_alloc
     // graphs captured, and those of them inside a solve that the tuner timed
     // (sulf_dbg_route)
@@ -342,24 +343,24 @@ int alloc_vectors(sulf_domain* d, LevelVec<T>* V) {
         LevelVec<T>& v = V[l];
         size_t nb2 = sizeof(T2) * G.nn;
         const bool wc = !v.Wc, rhs = !v.rhs;
-        if (wc) v.Wc = (T2*)d->mem.get(nb2);
-        if (rhs) v.rhs = (T2*)d->mem.get(nb2);
-        v.x = (T2*)d->mem.get(nb2);
-        v.res = (T2*)d->mem.get(nb2);
-        for (int k = 0; k < 2; k++) v.gbuf[k] = (T*)d->mem.get(sizeof(T) * (G.ng + 1));
-        for (int a = 0; a < G.dim; a++) v.edge[a] = (T2*)d->mem.get(nb2);
-        v.Pa = (T2*)d->mem.get(nb2);
-        v.Pb = (T2*)d->mem.get(nb2);
-        v.Ia = (T2*)d->mem.get(nb2);
-        v.Ib = (T2*)d->mem.get(nb2);
+        if (wc) v.Wc = (T2*)d->mem_two.get(nb2);
+        if (rhs) v.rhs = (T2*)d->mem_two.get(nb2);
+        v.x = (T2*)d->mem_two.get(nb2);
+        v.res = (T2*)d->mem_two.get(nb2);
+        for (int k = 0; k < 2; k++) v.gbuf[k] = (T*)d->mem_two.get(sizeof(T) * (G.ng + 1));
+        for (int a = 0; a < G.dim; a++) v.edge[a] = (T2*)d->mem_two.get(nb2);
+        v.Pa = (T2*)d->mem_two.get(nb2);
+        v.Pb = (T2*)d->mem_two.get(nb2);
+        v.Ia = (T2*)d->mem_two.get(nb2);
+        v.Ib = (T2*)d->mem_two.get(nb2);
         const size_t nc2 = sizeof(T2) * 2 * ((size_t)G.nin[0] + G.nin[1] + 1);
-        v.Pc = (T2*)d->mem.get(nc2);
-        v.Ic = (T2*)d->mem.get(nc2);
-        v.gc = (T2*)d->mem.get(sizeof(T2) * (G.ng + 1));
-        v.gci = (T*)d->mem.get(sizeof(T) * (G.ng + 1));
+        v.Pc = (T2*)d->mem_two.get(nc2);
+        v.Ic = (T2*)d->mem_two.get(nc2);
+        v.gc = (T2*)d->mem_two.get(sizeof(T2) * (G.ng + 1));
+        v.gci = (T*)d->mem_two.get(sizeof(T) * (G.ng + 1));
         if (std::is_same<T, double>::value) {
             const size_t nl = sizeof(T2) * ((size_t)G.nin[0] + G.nin[1] + G.ng + 1);
-            v.rhsc = (T2*)d->mem.get(nl);
+            v.rhsc = (T2*)d->mem_two.get(nl);
             if (!v.rhsc) return sulf_fail(SULF_ENOMEM, "out of device memory");
             SULF_CUDA_TRY(cudaMemsetAsync(v.rhsc, 0, nl, d->stream));
         }
@@ -372,18 +373,43 @@ int alloc_vectors(sulf_domain* d, LevelVec<T>* V) {
         SULF_CUDA_TRY(cudaMemsetAsync(v.res, 0, nb2, d->stream));
         if (l == d->L - 1) {
             size_t m = 2 * (size_t)G.nact;
-            v.A = (T*)d->mem.get(sizeof(T) * (m * m + 1));
-            v.Ainv = (T*)d->mem.get(sizeof(T) * (m * m + 1));
+            v.A = (T*)d->mem_two.get(sizeof(T) * (m * m + 1));
+            v.Ainv = (T*)d->mem_two.get(sizeof(T) * (m * m + 1));
             if (!v.A || !v.Ainv) return sulf_fail(SULF_ENOMEM, "out of device memory");
         }
     }
     return SULF_OK;
 }
 
+// gives those vectors back; their next use allocates them anew
+void release_two(sulf_domain* d) {
+    drop_graphs(d);
+    cudaStreamSynchronize(d->stream);
+    d->mem_two.release();
+    for (int l = 0; l < d->L; l++) {
+        LevelVec<double> core;  // (alloc_core)
+        core.Wc = d->v64[l].Wc;
+        core.rhs = l == 0 ? d->v64[0].rhs : nullptr;
+        d->v64[l] = core;
+        d->v32[l] = LevelVec<float>();
+        LevelGeo& G = d->geo[l];
+        G.tiles = nullptr;
+        G.ntiles = G.tile_nx = G.tile_ny = 0;
+    }
+    d->have64 = d->have32 = false;
+    for (int p = 0; p < 2; p++) {
+        d->tail_desc[p] = nullptr;
+        d->tail_ready[p] = false;
+    }
+}
+
 int ensure64(sulf_domain* d) {
     if (d->have64) return SULF_OK;
     int rc = alloc_vectors<double>(d, d->v64);
-    if (rc) return rc;
+    if (rc) {
+        release_two(d);
+        return rc;
+    }
     // a residual F computed before has no list-ordered copy yet
     d->launches += launch_gather_list(d->geo[0], d->v64[0].rhs, d->v64[0].rhsc, d->stream);
     d->have64 = true;
@@ -393,7 +419,10 @@ int ensure64(sulf_domain* d) {
 int ensure32(sulf_domain* d) {
     if (d->have32) return SULF_OK;
     int rc = alloc_vectors<float>(d, d->v32);
-    if (rc) return rc;
+    if (rc) {
+        release_two(d);
+        return rc;
+    }
     d->have32 = true;
     return SULF_OK;
 }
@@ -507,19 +536,35 @@ void release_schur(sulf_domain* d) {
     d->cs64 = CoarseSet<double>();
     d->cs32 = CoarseSet<float>();
     d->dskip = nullptr;
-    d->s_geo = 0;
+    if (d->s_geo > 0) d->s_geo = 0;
     d->s_on = false;
 }
 
-int build_schur(sulf_domain* d, bool coarse) {
-    d->s_on = false;
-    if (!schur_wanted(d) || d->s_geo < 0) return SULF_OK;
+// whether the linear solves with the current controls run that cycle (as far as
+// is known before its lists are built)
+bool schur_applies(const sulf_domain* d) {
+    if (!schur_wanted(d) || d->s_geo < 0) return false;
     for (int l = 0; l < d->L; l++) {
         const LevelGeo& G = d->geo[l];
         if (G.ng > 0 && !(G.gop_on && G.gop_bc == d->bc && G.gop_passes == d->solver.ghost_sweeps &&
                           G.gop_tau == level_tau(d, l)))
-            return SULF_OK;
+            return false;
     }
+    return true;
+}
+
+// gives back what the path holds that the current controls do not run
+void release_other_path(sulf_domain* d) {
+    if (schur_applies(d)) {
+        if (d->have64 || d->have32) release_two(d);
+    } else if (d->s_geo > 0) {
+        release_schur(d);
+    }
+}
+
+int build_schur(sulf_domain* d, bool coarse) {
+    d->s_on = false;
+    if (!schur_applies(d)) return SULF_OK;
     std::string err;
     if (!d->s_geo) {
         for (int l = 0; l < d->L; l++) {
@@ -529,6 +574,7 @@ int build_schur(sulf_domain* d, bool coarse) {
             if (rc) return sulf_fail(rc, err);
             if (!ok) {
                 d->s_geo = -1;
+                release_schur(d);
                 return SULF_OK;
             }
         }
@@ -606,7 +652,7 @@ int ensure_tail(sulf_domain* d, const LevelVec<T>* V) {
     int p = std::is_same<T, float>::value ? 1 : 0;
     if (d->tail_ready[p]) return SULF_OK;
     if (!d->tail_desc[p]) {
-        d->tail_desc[p] = d->mem.get(tail_desc_bytes(d->L));
+        d->tail_desc[p] = d->mem_two.get(tail_desc_bytes(d->L));
         if (!d->tail_desc[p]) return sulf_fail(SULF_ENOMEM, "out of device memory");
     }
     int rc = upload_tail_desc<T>(d->geo, V, d->L, d->tail_desc[p], d->stream);
@@ -1368,8 +1414,8 @@ int ensure_tiles(sulf_domain* d) {
         std::vector<int> list;
         for (size_t q = 0; q < has.size(); q++)
             if (has[q]) list.push_back((int)q);
-        int* dl = (int*)d->mem.get(sizeof(int) * (list.size() + 1));
-        float2* x2 = (float2*)d->mem.get(sizeof(float2) * G.nn);
+        int* dl = (int*)d->mem_two.get(sizeof(int) * (list.size() + 1));
+        float2* x2 = (float2*)d->mem_two.get(sizeof(float2) * G.nn);
         if (!dl || !x2) return sulf_fail(SULF_ENOMEM, "out of device memory");
         SULF_CUDA_TRY(cudaMemcpyAsync(dl, list.data(), sizeof(int) * list.size(), cudaMemcpyHostToDevice, d->stream));
         SULF_CUDA_TRY(cudaMemsetAsync(x2, 0, sizeof(float2) * G.nn, d->stream));
@@ -1454,6 +1500,7 @@ void sulf_destroy(sulf_handle h) {
     for (cudaEvent_t e : h->evpool) cudaEventDestroy(e);
     h->mem.release();
     h->mem_s.release();
+    h->mem_two.release();
     if (h->hnorm) cudaFreeHost(h->hnorm);
     if (h->hloop) cudaFreeHost(h->hloop);
     for (auto& g : h->loop)
@@ -1493,8 +1540,8 @@ int sulf_create_domain(const double* levelset, int dim, const double* box, int N
     }
     d->stream = d->own_stream;
     d->mem.stream = d->own_stream;
-    d->mem_s.stream = d->own_stream;
-    d->mem.fail_in = d->mem_s.fail_in = &d->fail_in;
+    d->mem_s.stream = d->mem_two.stream = d->own_stream;
+    d->mem.fail_in = d->mem_s.fail_in = d->mem_two.fail_in = &d->fail_in;
     std::string err;
     int rc = SULF_OK;
     for (int l = 0; l < nl && rc == SULF_OK; l++) {
@@ -1738,7 +1785,7 @@ int sulf_get_stats(sulf_handle h, sulf_stats* o) {
     o->n_inside = h->geo[0].nin[0] + (long long)h->geo[0].nin[1];
     o->n_ghost = h->geo[0].ng;
     for (int k = 0; k < 3; k++) o->ghost_rows[k] = h->geo[0].kinds[k];
-    o->device_bytes = h->mem.bytes + h->mem_s.bytes;
+    o->device_bytes = h->mem.bytes + h->mem_s.bytes + h->mem_two.bytes;
     o->loop_graph = h->loop_used ? 1 : 0;
     return SULF_OK;
 }
@@ -2821,6 +2868,10 @@ int autotune(sulf_domain* d, double dt, sulf_tune_result* out) {
         d->solver.relax_occupancy = occ < 0 ? base.relax_occupancy : occ;
         d->solver.relax_matrix_free = mf < 0 ? base.relax_matrix_free : mf;
         if (int rc = refresh_ghost_ops(d)) return rc;
+        // (a candidate of the other path: never both paths' vectors)
+        release_other_path(d);
+        if (d->solver.precision == 1 && d->solver.relax_matrix_free == 2)
+            if (int rc = ensure_tiles(d)) return rc;
         return time_solve<D>(d, fn, ncyc, ms);
     };
     sulf_tune_result r{};
@@ -2870,8 +2921,6 @@ int autotune(sulf_domain* d, double dt, sulf_tune_result* out) {
     } else if (base.smoother == 0) {
         for (int mf = 0; mf <= (d->dim == 3 ? 2 : 1); mf++) {
             if (mf == base.relax_matrix_free) continue;
-            if (mf == 2)
-                if (int rc = ensure_tiles(d)) return rc;
             double ms = 0;
             if (int rc = trial(r.fuse_below, r.ghost_compose, r.pdl, &ms, -1, mf)) return rc;
             r.candidates++;
@@ -2889,6 +2938,9 @@ int autotune(sulf_domain* d, double dt, sulf_tune_result* out) {
     d->solver.relax_occupancy = r.relax_occupancy;
     d->solver.relax_matrix_free = r.relax_matrix_free;
     if (int rc = refresh_ghost_ops(d)) return rc;
+    release_other_path(d);
+    if (r.relax_matrix_free == 2 && base.precision == 1)
+        if (int rc = ensure_tiles(d)) return rc;
     *out = r;
     return SULF_OK;
 }
@@ -2917,9 +2969,10 @@ int sulf_autotune(sulf_handle h, double dt, int use_cache, sulf_tune_result* out
         h->solver.pdl = r.pdl;
         h->solver.relax_occupancy = r.relax_occupancy;
         h->solver.relax_matrix_free = r.relax_matrix_free;
+        if (int rc = refresh_ghost_ops(h)) return rc;
+        release_other_path(h);
         if (r.relax_matrix_free == 2 && h->solver.precision == 1)
             if (int rc = ensure_tiles(h)) return rc;
-        if (int rc = refresh_ghost_ops(h)) return rc;
     } else {
         const double dt0 = h->dt;
         int rc = h->dim == 2 ? autotune<2>(h, dt, &r) : autotune<3>(h, dt, &r);
