@@ -78,8 +78,9 @@ int sulf_dbg_cycles(sulf_handle h, double dt, const double* Wc0, const double* r
    receives whether an earlier request has not been reached yet. */
 int sulf_dbg_fail_alloc(sulf_handle h, long long after, int* pending);
 
-/* what the handle has built and runs (2 entries): graphs captured so far, and
-   those of them captured inside a solve that sulf_autotune timed */
+/* what the handle has built and runs (3 entries): graphs captured so far, those
+   of them captured inside a solve that sulf_autotune timed, and sets of cluster
+   tables (the fused coarse levels) built so far */
 int sulf_dbg_route(sulf_handle h, int64_t* route);
 
 /* r as the result that the process cache of sulf_autotune holds for the

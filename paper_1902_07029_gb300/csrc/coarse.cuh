@@ -73,6 +73,7 @@ struct CoarseSet {
     int l0 = -1;
     int want = -2, nu1 = 0, nu2 = 0, max_cta = 0;  // what it was built for
     bool rows = false;      // built, and for the current boundary rows
+    int own_want = -2, own = 0;  // lock step: the first level fused with no regard to the class, and what it was found for
     size_t smem = 0;
     int ncta = 0;
     CDesc<T>* dev = nullptr;

@@ -110,9 +110,11 @@ struct sulf_domain {
     SVec<double> s64[SULF_MAXLEV];
     SVec<float> s32[SULF_MAXLEV];
     int s_geo = 0;
-    // the coarse levels fused into one cluster launch, per precision
-    CoarseSet<double> cs64;
-    CoarseSet<float> cs32;
+    // the coarse levels fused into one cluster launch, per precision: of the
+    // handle stepped alone, and of a lock-step class ([1])
+    CoarseSet<double> cs64[2];
+    CoarseSet<float> cs32[2];
+    int in_class = 0;      // 1 while a lock-step class steps the handle
     bool s_on = false;     // the current linear solve runs that cycle
     int* dskip = nullptr;  // device flag: the first sweep of the cycle has been done
     int bc = 0;  // boundary condition for s: 0 Dirichlet (Eq. BCs), 1 Neumann (Eq. BCsN)
@@ -145,6 +147,7 @@ struct sulf_domain {
     // graphs captured, and those of them inside a solve that the tuner timed
     // (sulf_dbg_route)
     long long captures = 0, captures_timed = 0;
+    long long tables = 0;              // cluster tables built (sulf_dbg_route)
     double t = 0, dt = 0;
     // statistics
     int newton_last = 0, cycles_last = 0;
@@ -487,22 +490,38 @@ int alloc_schur(sulf_domain* d, SVec<T>* V, int nl, bool outer) {
     return ok ? SULF_OK : sulf_fail(SULF_ENOMEM, "out of device memory");
 }
 
-// the fused coarse levels of the current threshold (sulf_solver::fuse_below);
-// at_least: the first of them no finer than this level; max_cta: cluster size
+// the set that the handle uses now
 template <typename T>
-int ensure_coarse(sulf_domain* d, CoarseSet<T>& S, const SVec<T>* V, int at_least = 0, int max_cta = kCoarseMaxCta) {
-    int want = -1;
+CoarseSet<T>& coarse_of(sulf_domain* d) {
+    if constexpr (std::is_same<T, double>::value)
+        return d->cs64[d->in_class];
+    else
+        return d->cs32[d->in_class];
+}
+
+// the first level, no finer than at_least, that the current threshold
+// (sulf_solver::fuse_below) fuses (-1: none)
+template <typename T>
+int coarse_want(const sulf_domain* d, int at_least) {
     if (d->prof) at_least = std::max(at_least, 1);  // the finest level's launches are timed
-    double* acc = std::is_same<T, float>::value ? d->s64[0].X : nullptr;
     const int fb = d->solver.fuse_below >= 0 ? d->solver.fuse_below
                                                : coarse_auto(d->dim, std::is_same<T, float>::value);
     if (fb > 0 && d->solver.cycle == 1)
-        for (int l = at_least; l < d->L && want < 0; l++)
-            if ((long long)d->geo[l].nin[0] + d->geo[l].nin[1] + d->geo[l].ng <= fb) want = l;
+        for (int l = at_least; l < d->L; l++)
+            if ((long long)d->geo[l].nin[0] + d->geo[l].nin[1] + d->geo[l].ng <= fb) return l;
+    return -1;
+}
+
+// the fused coarse levels of the current threshold; at_least: the first of them
+// no finer than this level; max_cta: cluster size
+template <typename T>
+int ensure_coarse(sulf_domain* d, CoarseSet<T>& S, const SVec<T>* V, int at_least = 0, int max_cta = kCoarseMaxCta) {
+    const int want = coarse_want<T>(d, at_least);
+    double* acc = std::is_same<T, float>::value ? d->s64[0].X : nullptr;
     const int nu1 = d->solver.nu1, nu2 = d->solver.nu2;
     if (S.rows && S.want == want && S.nu1 == nu1 && S.nu2 == nu2 && S.max_cta == max_cta) return SULF_OK;
     SULF_CUDA_TRY(cudaStreamSynchronize(d->stream));
-    drop_graphs(d);
+    if (!d->in_class) drop_graphs(d);  // (a class captures its graphs anew at every call)
     std::string err;
     int rc = d->dim == 2 ? build_coarse<2, T>(S, d->geo, d->sgeo, V, d->L, want, nu1, nu2, max_cta, acc, d->dskip,
                                               d->mem_s, d->stream, err)
@@ -510,6 +529,7 @@ int ensure_coarse(sulf_domain* d, CoarseSet<T>& S, const SVec<T>* V, int at_leas
                                               d->mem_s, d->stream, err);
     if (rc) return sulf_fail(rc, err);
     S.rows = true;
+    if (S.l0 >= 0) d->tables++;
     return SULF_OK;
 }
 
@@ -533,8 +553,10 @@ void release_schur(sulf_domain* d) {
         d->s64[l] = SVec<double>();
         d->s32[l] = SVec<float>();
     }
-    d->cs64 = CoarseSet<double>();
-    d->cs32 = CoarseSet<float>();
+    for (int k = 0; k < 2; k++) {
+        d->cs64[k] = CoarseSet<double>();
+        d->cs32[k] = CoarseSet<float>();
+    }
     d->dskip = nullptr;
     if (d->s_geo > 0) d->s_geo = 0;
     d->s_on = false;
@@ -593,17 +615,17 @@ int build_schur(sulf_domain* d, bool coarse) {
     }
     if (changed) {
         drop_graphs(d);
-        d->cs64.rows = d->cs32.rows = false;
+        for (int k = 0; k < 2; k++) d->cs64[k].rows = d->cs32[k].rows = false;
     }
     if (d->solver.precision == 0) {
         if (int rc = alloc_schur<double>(d, d->s64, d->L, false)) return rc;
         if (coarse)
-            if (int rc = ensure_coarse<double>(d, d->cs64, d->s64)) return rc;
+            if (int rc = ensure_coarse<double>(d, coarse_of<double>(d), d->s64)) return rc;
     } else {
         if (int rc = alloc_schur<double>(d, d->s64, 1, true)) return rc;
         if (int rc = alloc_schur<float>(d, d->s32, d->L, false)) return rc;
         if (coarse)
-            if (int rc = ensure_coarse<float>(d, d->cs32, d->s32)) return rc;
+            if (int rc = ensure_coarse<float>(d, coarse_of<float>(d), d->s32)) return rc;
     }
     d->s_on = true;
     return SULF_OK;
@@ -828,12 +850,7 @@ struct SMG {
     SVec<T>* V;
     int fine_sweeps = 0;
 
-    const CoarseSet<T>& fused() const {
-        if constexpr (std::is_same<T, double>::value)
-            return d->cs64;
-        else
-            return d->cs32;
-    }
+    const CoarseSet<T>& fused() const { return coarse_of<T>(d); }
 
     SLev<D, T> lev(int l) {
         SLev<D, T> s = make_slev<D, T>(d->geo[l], d->sgeo[l], V[l]);
@@ -1824,6 +1841,7 @@ int sulf_dbg_route(sulf_handle h, int64_t* r) {
     if (!valid(h) || !r) return sulf_fail(SULF_EINVAL, "invalid arguments");
     r[0] = h->captures;
     r[1] = h->captures_timed;
+    r[2] = h->tables;
     return SULF_OK;
 }
 
@@ -2269,13 +2287,6 @@ struct LockClass {
     }
 
     template <typename T>
-    static CoarseSet<T>& coarse_of(sulf_domain* d) {
-        if constexpr (std::is_same<T, double>::value)
-            return d->cs64;
-        else
-            return d->cs32;
-    }
-    template <typename T>
     static SVec<T>* svec_of(sulf_domain* d) {
         if constexpr (std::is_same<T, double>::value)
             return d->s64;
@@ -2300,8 +2311,21 @@ struct LockClass {
     // the levels, lists and coarse clusters of the cycle in precision T
     template <typename T>
     int setup_schur(const SLev<D, T>** out) {
-        // all instances fuse the same levels, on clusters of 8 CTAs
-        for (int first = 1;;) {
+        // All instances fuse the same levels, on clusters of 8 CTAs: from the
+        // first one that each of them can fuse (an instance's own is kept, so a
+        // class that steps again builds no table).
+        int first = 1;
+        for (int i = 0; i < K; i++) {
+            CoarseSet<T>& S = coarse_of<T>(h[i]);
+            const int want = coarse_want<T>(h[i], 1);
+            if (!S.rows || S.nu1 != h[i]->solver.nu1 || S.nu2 != h[i]->solver.nu2 || S.own_want != want) {
+                if (int rc = ensure_coarse<T>(h[i], S, svec_of<T>(h[i]), 1, 8)) return rc;
+                S.own_want = want;
+                S.own = S.l0 < 0 ? L : S.l0;  // (none: L)
+            }
+            first = std::max(first, S.own);
+        }
+        for (;;) {
             int worst = 0, none = 0;
             for (int i = 0; i < K; i++) {
                 CoarseSet<T>& S = coarse_of<T>(h[i]);
@@ -2313,10 +2337,16 @@ struct LockClass {
             if (none == K) break;
             if (none) {
                 first = L;  // one has none: none for all
+                for (int i = 0; i < K; i++)
+                    if (coarse_of<T>(h[i]).l0 < 0) coarse_of<T>(h[i]).own = L;
                 continue;
             }
             bool same = true;
-            for (int i = 0; i < K; i++) same = same && coarse_of<T>(h[i]).l0 == worst;
+            for (int i = 0; i < K; i++) {
+                CoarseSet<T>& S = coarse_of<T>(h[i]);
+                same = same && S.l0 == worst;
+                if (S.l0 > first) S.own = S.l0;  // (more than its own first level needed)
+            }
             if (same) {
                 scoarse = worst;
                 sncta = 8;
@@ -2738,6 +2768,15 @@ int lockstep_run(const std::vector<sulf_domain*>& hs, double dt, int nsteps, int
     C.s = s;
     C.mem = &mem;
     C.schur = true;
+    struct InClass {  // (the handles' own cluster tables and graphs stay as they are)
+        const std::vector<sulf_domain*>& h;
+        explicit InClass(const std::vector<sulf_domain*>& v) : h(v) {
+            for (sulf_domain* d : h) d->in_class = 1;
+        }
+        ~InClass() {
+            for (sulf_domain* d : h) d->in_class = 0;
+        }
+    } in_class(hs);
     for (sulf_domain* d : hs) {
         d->dt = dt;
         if (int rc = refresh_ghost_ops(d)) return rc;
