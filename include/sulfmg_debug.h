@@ -78,9 +78,12 @@ int sulf_dbg_cycles(sulf_handle h, double dt, const double* Wc0, const double* r
    receives whether an earlier request has not been reached yet. */
 int sulf_dbg_fail_alloc(sulf_handle h, long long after, int* pending);
 
-/* what the handle has built and runs (3 entries): graphs captured so far, those
-   of them captured inside a solve that sulf_autotune timed, and sets of cluster
-   tables (the fused coarse levels) built so far */
+/* what the handle has built and runs (7 entries): graphs captured so far; those
+   of them captured inside a solve that sulf_autotune timed; sets of cluster
+   tables (the fused coarse levels) built so far; then of the last linear solve
+   of the handle alone: 1 if it ran the cycle on the equation for s, the first
+   level fused into the cluster kernel (-1: none), the CTAs of its cluster, 1 if
+   that level is dealt to all of them (0: CTA 0 runs it) */
 int sulf_dbg_route(sulf_handle h, int64_t* route);
 
 /* r as the result that the process cache of sulf_autotune holds for the

@@ -399,7 +399,7 @@ class Domain:
 
     def route(self):
         """what the handle has built and runs (sulf_dbg_route)"""
-        names = ("captures", "captures_timed", "tables")
+        names = ("captures", "captures_timed", "tables", "scalar", "first_fused", "ctas", "first_wide")
         r = np.zeros(len(names), dtype=np.int64)
         _chk(self.lib, self.lib.sulf_dbg_route(self.h, r.ctypes.data_as(_i64p)))
         return {n: int(v) for n, v in zip(names, r)}

@@ -1277,6 +1277,7 @@ int build_coarse(CoarseSet<T>& S, const LevelGeo* G, const SGeo* SG, const SVec<
     }
     S.smem = smem;
     S.ncta = C;
+    S.wide = H[l0].wide != 0;
     S.l0 = l0;
     return SULF_OK;
 }

@@ -76,6 +76,7 @@ struct CoarseSet {
     int own_want = -2, own = 0;  // lock step: the first level fused with no regard to the class, and what it was found for
     size_t smem = 0;
     int ncta = 0;
+    bool wide = false;      // the first level is dealt to all CTAs (else CTA 0 runs it)
     CDesc<T>* dev = nullptr;
     CPerm* perm[SULF_MAXLEV] = {};  // device, per level
     T* coef = nullptr;

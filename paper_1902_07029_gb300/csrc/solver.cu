@@ -1842,6 +1842,17 @@ int sulf_dbg_route(sulf_handle h, int64_t* r) {
     r[0] = h->captures;
     r[1] = h->captures_timed;
     r[2] = h->tables;
+    r[3] = h->s_on;
+    auto set = [&](const auto& S) {
+        const bool on = h->s_on && S.l0 >= 0;
+        r[4] = on ? S.l0 : -1;
+        r[5] = on ? S.ncta : 0;
+        r[6] = on && S.wide;
+    };
+    if (h->solver.precision == 0)
+        set(h->cs64[0]);
+    else
+        set(h->cs32[0]);
     return SULF_OK;
 }
 
