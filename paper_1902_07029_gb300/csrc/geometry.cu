@@ -892,6 +892,10 @@ int build_level_geometry(LevelGeo& L, const LevelGeo* finer, bool finest, bool c
     launches += 2;
     if (finest) {
         int* dflag = (int*)mem.get(sizeof(int));
+        if (!dflag) {
+            err = "out of device memory";
+            return SULF_ENOMEM;
+        }
         cudaMemsetAsync(dflag, 0, sizeof(int), s);
         k_check_edge<<<nblk(nn), kThreads, 0, s>>>(L.type, L.n, L.dim, nn, dflag);
         launches++;

@@ -83,3 +83,32 @@ def test_no_thread_leaves_before_the_dependent_launch_wait(f, name, body):
         assert any(w in tail for w in ("pdl_enter(", "s_phase<", "s_outer<"))
         if "pdl_enter(" in tail:
             assert "return" not in tail[:tail.index("pdl_enter(")]
+
+
+def _allocations():
+    """(file, line, pointer, what follows up to the next kernel launch)"""
+    out = []
+    for f in sorted(os.listdir(CSRC)):
+        if not f.endswith(".cu"):
+            continue
+        lines = _code(f).split("\n")
+        for i, l in enumerate(lines):
+            m = re.search(r"([\w.>\[\]-]+) = \([^=]*\)\s*[\w>.-]*get(?:_host)?\(", l)
+            if not m:
+                continue
+            rest = []
+            for r in lines[i:]:
+                if "<<<" in r or "launch_" in r:
+                    break
+                rest.append(r)
+            name = re.sub(r"\[\w+\]", "", m.group(1)).split(".")[-1].split(">")[-1]
+            out.append((f, i + 1, name, "\n".join(rest)))
+    return out
+
+
+def test_allocations_are_checked_before_a_kernel_sees_them():
+    found = _allocations()
+    assert len(found) > 60
+    bad = [(f, i, n) for f, i, n, rest in found
+           if not re.search(rf"![\w.>-]*\b{n}\b|\b{n} (!=|==|&&)", rest)]
+    assert not bad, bad
