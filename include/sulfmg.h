@@ -168,7 +168,9 @@ int sulf_set_stream(sulf_handle h, void* stream);
 /* Advance nsteps Crank-Nicolson steps of size dt (Sec. 3.1), each by Newton
    (Sec. 3.4) with multigrid linear solves (Sec. 3.5).  Blocks until done.
    SULF_ENOTCONV if a step does not converge (the state is then that of the
-   failed iterate). */
+   failed iterate).  The vectors and tables of the cycle that the solver
+   controls select are allocated by the first step that runs it: SULF_ENOMEM if
+   they do not fit (the state is unchanged, and a later step tries again). */
 int sulf_step(sulf_handle h, double dt, int nsteps);
 
 /* Copy the state to caller-owned host arrays of (N+1)^dim entries; any pointer

@@ -362,9 +362,11 @@ struct Coarse {
     // addresses) over the visit, so a phase is a handful of loads and
     // multiply-adds between two barriers.  What a warp executes between two
     // barriers is its latency and what all warps execute the CTA's, so nothing
-    // else is left there and the warps without a row do nothing.  Measured: a
-    // phase of CTA 0 takes 120 cycles at least, one with a cluster barrier and
-    // remote loads 770, of which the barrier's fence is 350.
+    // else is left there and the warps without a row do nothing.  Measured
+    // (clock stamps, levels of 100 to 5000 nodes, a visit of two sweeps and the
+    // defect, its loads of the rows included, per phase): 570 to 680 cycles on
+    // CTA 0 and 1200 to 1300 on the cluster in FP32, 1200 to 1400 and 2000 to
+    // 2150 in FP64.
     template <bool W>
     __device__ __forceinline__ void visit(const CLev& L, int nsw, bool skip_red, bool delta, bool last,
                                           bool dft) const {
@@ -734,9 +736,9 @@ int build_coarse(CoarseSet<T>& S, const LevelGeo* G, const SGeo* SG, const SVec<
     S.rows = false;  // (the caller's note of success)
     if (want < 0 || want > L - 1) return SULF_OK;
     const bool f32 = std::is_same<T, float>::value;
-    // Levels of up to this many nodes run on CTA 0, whose phases are short: 120
-    // cycles against the 770 of a cluster's, while an SM's two FP64 lanes or
-    // the ghosts of 3-D levels make them long sooner.  Two CN steps with 300 /
+    // Levels of up to this many nodes run on CTA 0, whose phases take half as
+    // long as the cluster's (see visit), while an SM's two FP64 lanes or the
+    // ghosts of 3-D levels make them long sooner.  Two CN steps with 300 /
     // 600 / 1200: 257^2 star, mixed 7.49 / 7.47 / 7.77 and 5.81 / 5.81 / 5.70 ms;
     // 1025^2 star, FP64 8.77 / 8.62 / 8.63, mixed 5.92 / 5.79 / 5.80; 321^2 star
     // (Neumann), FP64 8.33 / 7.87 / 7.89; 65^3 box, mixed 17.2 / 18.4 / 18.4;
@@ -1162,7 +1164,6 @@ int build_coarse(CoarseSet<T>& S, const LevelGeo* G, const SGeo* SG, const SVec<
             for (int r = 0; r < C; r++) {
                 CLev& c = lev[(size_t)r * n + n - 1];
                 c.m = m;
-                c.row0 = row0;
                 d.ainv_off[r] = row0 * m;
                 d.ainv_len[r] = c.nx * m;
                 row0 += c.nx;

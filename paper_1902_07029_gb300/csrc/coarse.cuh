@@ -8,8 +8,8 @@
 // l0 .. L-1 are dealt to the CTAs of a cluster in bands of the box order; each
 // CTA keeps its rows, tables and values in shared memory, reads a neighbour's
 // value from its owner's shared memory, and a cluster barrier separates the
-// phases.  Levels too small for that (kNarrow nodes) run on CTA 0 alone with
-// CTA barriers.  The rows (gt, dd, 1/dd, rho, C) and the tables are fixed
+// phases.  Levels too small for that (`narrow` nodes in build_coarse) run on CTA 0
+// alone with CTA barriers.  The rows (gt, dd, 1/dd, rho, C) and the tables are fixed
 // during a linear solve and are copied in while the previous kernel runs.
 #pragma once
 
@@ -42,7 +42,7 @@ struct CLev {
     int cptr, cref, cval;  // rows of the restriction onto the own inside nodes
     CTab c;               // and onto the own ghosts
     int ainv;             // coarsest level: own rows of the inverse (-1: in global memory)
-    int m, row0;          // coarsest level: order of the matrix, first own row
+    int m;                // coarsest level: order of the matrix
 };
 
 template <typename T>

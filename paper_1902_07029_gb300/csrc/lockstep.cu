@@ -7,7 +7,7 @@
 // coarsest solve) is one launch over an (instance, node) work list: CTA b
 // belongs to the instance i with pre[i] <= b < pre[i+1] and takes its nodes
 // from that instance's level.  An instance whose linear solve has converged
-// is masked (its CTAs return at once), so every instance runs exactly the
+// is masked (its CTAs only pass the dependent-launch wait), so every instance runs exactly the
 // cycles it would run alone, with the same per-node stage functions
 // (mg_stages.cuh), hence the same results.
 #include "lockstep.cuh"
@@ -17,17 +17,7 @@ namespace {
 
 constexpr int kBT = 256;
 
-__device__ __forceinline__ int find_instance(const int* __restrict__ pre, int K, int b) {
-    int lo = 0, hi = K;  // pre[0] = 0 <= b < pre[K]
-    while (hi - lo > 1) {
-        const int mid = (lo + hi) >> 1;
-        if (pre[mid] <= b)
-            lo = mid;
-        else
-            hi = mid;
-    }
-    return lo;
-}
+using stages::find_instance;
 
 // block-wide max of non-negative doubles held as bit patterns, one atomicMax
 __device__ __forceinline__ void block_max_to(unsigned long long v, unsigned long long* out) {

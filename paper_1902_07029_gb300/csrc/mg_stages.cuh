@@ -65,6 +65,19 @@ __device__ __forceinline__ void block_max(unsigned long long v, unsigned long lo
     }
 }
 
+// instance of CTA b of a lock-step launch: pre[i] <= b < pre[i+1]
+__device__ __forceinline__ int find_instance(const int* __restrict__ pre, int K, int b) {
+    int lo = 0, hi = K;  // pre[0] = 0 <= b < pre[K]
+    while (hi - lo > 1) {
+        const int mid = (lo + hi) >> 1;
+        if (pre[mid] <= b)
+            lo = mid;
+        else
+            hi = mid;
+    }
+    return lo;
+}
+
 // node of list position t in the concatenation (inside colour 0, inside
 // colour 1, ghosts); kind 1 inside, 2 ghost
 struct Lists {

@@ -45,9 +45,11 @@ extern "C" unsigned long long sulf_estimate_device_bytes(int dim, int N, int coa
     if ((dim != 2 && dim != 3) || N < 2 || coarsest_N < 2) return 0;
     double nn0 = 1;
     for (int a = 0; a < dim; a++) nn0 *= (double)(N + 1);
-    // bytes per box node: FP64 level vectors (Wc, rhs, x, res 64; edges 16 dim;
-    // 2x2 blocks and inverses 64, and their copies and rhs's in list order, at
-    // most 80), geometry (phi, type, maps, lists, marks ~30), the finest
+    // An upper bound for either cycle, from the layout of the two-unknown one,
+    // the larger of the two (domains of both, 17^2 to 2049^2 and 17^3 to 257^3,
+    // hold 0.23 to 0.65 of it).  Bytes per box node: FP64 level vectors (Wc,
+    // rhs, x, res 64; edges 16 dim; 2x2 blocks and inverses 64, and their copies
+    // and rhs's in list order, at most 80), geometry (phi, type, maps, lists, marks ~30), the finest
     // level's W^n, old-time part and staging (49); FP32 vectors (32 + 8 dim +
     // 32 + 32) when mixed; coarser levels add 1/(2^dim - 1)
     double per_level = 208.0 + 16.0 * dim + 30.0;

@@ -10,6 +10,7 @@ namespace sulf {
 
 using stages::abs_bits;
 using stages::block_max;
+using stages::find_instance;
 using stages::fmadd;
 using stages::kGopLanes;
 
@@ -1006,18 +1007,6 @@ template <int D>
 __global__ void __launch_bounds__(kT) k_s_outer(const __grid_constant__ SLev<D, double> L,
                                                  const __grid_constant__ SLev<D, float> U, unsigned long long* norm) {
     s_outer<D>(L, U, blockIdx.x * blockDim.x + threadIdx.x, norm);
-}
-
-__device__ __forceinline__ int find_instance(const int* __restrict__ pre, int K, int b) {
-    int lo = 0, hi = K;  // pre[0] = 0 <= b < pre[K]
-    while (hi - lo > 1) {
-        const int mid = (lo + hi) >> 1;
-        if (pre[mid] <= b)
-            lo = mid;
-        else
-            hi = mid;
-    }
-    return lo;
 }
 
 template <int D, typename T, int PH>

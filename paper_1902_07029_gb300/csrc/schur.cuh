@@ -117,7 +117,6 @@ enum class SPhase { correct, red, black, ghosts, residual, outer, restrict_to, p
 
 // geometry of a level in these terms (precision independent)
 struct SGeo {
-    bool ready = false;
     int H = 0, P = 0, Hn = 0, n0 = 0, n1 = 0, nga = 0, nreg0 = 0, nreg1 = 0, ng1 = 0, ng8 = 0;
     int* hl = nullptr;
     int* gslot = nullptr;
@@ -235,10 +234,13 @@ template <int D, typename T>
 int launch_s_relax(const SLev<D, T>& L, int colour, bool delta, bool snap, bool skip, bool acc, cudaStream_t s);
 template <int D, typename T>
 int launch_s_ghosts(const SLev<D, T>& L, bool skip, bool acc, cudaStream_t s);
-// defect of the red nodes, of the black ones next to a ghost and of the
-// ghosts into R (norm null), or its max-norm only (and *L.skip set to 0)
+// the red half-sweep that opens an FP64 cycle, from the defects that the norm
+// of the cycle before left in R
 template <int D, typename T>
 int launch_s_correct(const SLev<D, T>& L, cudaStream_t s);
+// defect of the red nodes, of the black ones next to a ghost and of the
+// ghosts into R (norm null), or its max-norm, with the red nodes' defects in R
+// and *L.skip set to 0
 template <int D, typename T>
 int launch_s_residual(const SLev<D, T>& L, unsigned long long* norm, cudaStream_t s);
 // mixed precision: the FP64 defect of every row with its max-norm, stored as

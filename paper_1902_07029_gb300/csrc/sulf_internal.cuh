@@ -325,8 +325,13 @@ __host__ __device__ inline double tail_tau_scale(int dim, double h) {
 // the kernel was launched without the attribute), then launch_dependents lets
 // the next kernel's CTAs be scheduled while this one runs.  The next grid
 // therefore waits, resident, for this one instead of paying its launch latency
-// after it; at most two grids of a stream are in flight.  All threads pass the
-// wait before any global access.
+// after it; at most two grids of a stream are in flight.  Every thread passes
+// the wait.  Ahead of it a kernel reads only what no kernel just before it on
+// the stream writes: lists, geometry and the rows of the system, which are fixed
+// during a linear solve.  (What the grid before that one wrote is complete: its
+// successor passed its own wait before this grid was launched.)  Where the kernel
+// before may have written the rows, the set-up of a solve, the launch is made
+// without the attribute.
 __device__ __forceinline__ void pdl_enter() {
     asm volatile("griddepcontrol.wait;" ::: "memory");
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
